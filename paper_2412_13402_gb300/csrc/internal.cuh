@@ -13,8 +13,8 @@
 //     ph-ph segments (a, proc)     -> idx = b | c << pp_bits
 //     every segment is padded with zero-weight entries to a multiple of 4 entries so that a
 //     warp reads 4 entries per lane with one 16-byte load.
-//   work items: <= 512 entries of one segment, processed by one warp, which writes one
-//   compensated partial sum (hi, lo); rows combine their items' partials in item order.
+//   work items: <= 512 entries of one segment, processed by one warp or sub-warp, which writes
+//   one partial sum; rows combine their items' partials in item order.
 #pragma once
 
 #include <cuda_runtime.h>

@@ -150,92 +150,59 @@ __device__ __forceinline__ unsigned comp4(const uint4 &e, int k) {
 
 // Per-lane sum of W*F over one item: each 4-entry vector is summed with an FMA chain and the
 // vector sums are added into (acc, cmp) by lane_add; the warp reduction follows in finish_item.
-template <class R, int VPL>
+// FULL: every lane holds VPL vectors (a whole-warp item of the maximum length), so the vectors
+// carry no bounds tests.
+template <class R, int VPL, bool FULL, class F>
+__device__ __forceinline__ void lane_sum(const Batch<R, VPL> &b, int nv, int sl, int lg, R &acc, R &cmp, F &&factor) {
+    acc = R(0);
+    cmp = R(0);
+#pragma unroll
+    for (int j = 0; j < VPL; ++j) {
+        if (!FULL && sl + (j << lg) >= nv) break;
+        R t = R(0);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) t = fma(b.w(j, k), factor(comp4(b.iv[j], k)), t);
+        if (j == 0) acc = t;
+        else lane_add(acc, cmp, t);
+    }
+}
+
+template <class R, int VPL, bool FULL>
 __device__ __forceinline__ void compute_item(const GroupView<R> &V, const Item &it, const Batch<R, VPL> &b, int sl,
                                              int lg, R &acc, R &cmp) {
     const int nv = it.len >> 2;
-    acc = R(0);
-    cmp = R(0);
     if (V.part == PART_EPH) {
+        // F_em = f(1-f') + N(f-f') = fma(N, f-f', fma(f', -f, f)),
+        // F_abs = N(f-f') - f'(1-f) = fma(N, f-f', fma(f', -(1-f), 0)): one form with the two
+        // coefficients chosen per item, so sub-warps on emission and on absorption items of the
+        // same warp do not diverge
         const unsigned smask = (1u << V.sb) - 1u;
         const R fd = V.s0[it.dest];
-        if (it.proc == 0) {  // F_em = f(1-f') + N(f-f') = fma(N, f-f', fma(f', -f, f))
-#pragma unroll
-            for (int j = 0; j < VPL; ++j) {
-                if (sl + (j << lg) >= nv) continue;
-                R t = R(0);
-#pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    const unsigned e = comp4(b.iv[j], k);
-                    const R fs = V.s0[e & smask], N = V.s1[e >> V.sb];
-                    const R F = fma(N, fd - fs, fma(fs, -fd, fd));
-                    t = fma(b.w(j, k), F, t);
-                }
-                lane_add(acc, cmp, t);
-            }
-        } else {  // F_abs = N(f-f') - f'(1-f)
-            const R u = R(1) - fd;
-#pragma unroll
-            for (int j = 0; j < VPL; ++j) {
-                if (sl + (j << lg) >= nv) continue;
-                R t = R(0);
-#pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    const unsigned e = comp4(b.iv[j], k);
-                    const R fs = V.s0[e & smask], N = V.s1[e >> V.sb];
-                    const R F = fma(N, fd - fs, -fs * u);
-                    t = fma(b.w(j, k), F, t);
-                }
-                lane_add(acc, cmp, t);
-            }
-        }
+        const R cb = it.proc == 0 ? -fd : -(R(1) - fd), c0 = it.proc == 0 ? fd : R(0);
+        lane_sum<R, VPL, FULL>(b, nv, sl, lg, acc, cmp, [&](unsigned e) {
+            const R fs = V.s0[e & smask], N = V.s1[e >> V.sb];
+            return fma(N, fd - fs, fma(fs, cb, c0));
+        });
     } else if (V.part == PART_PHE) {  // F_abs(f_d, f_s, N_p) with N_p per item
         const unsigned smask = (1u << V.sb) - 1u;
         const R Np = b.Np;
-#pragma unroll
-        for (int j = 0; j < VPL; ++j) {
-            if (sl + (j << lg) >= nv) continue;
-            R t = R(0);
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                const unsigned e = comp4(b.iv[j], k);
-                const R fd = V.s0[e & smask], fs = V.s0[e >> V.sb];
-                const R F = fma(Np, fd - fs, -fs * (R(1) - fd));
-                t = fma(b.w(j, k), F, t);
-            }
-            lane_add(acc, cmp, t);
-        }
+        lane_sum<R, VPL, FULL>(b, nv, sl, lg, acc, cmp, [&](unsigned e) {
+            const R fd = V.s0[e & smask], fs = V.s0[e >> V.sb];
+            return fma(Np, fd - fs, -fs * (R(1) - fd));
+        });
     } else {
         const unsigned pmask = (1u << V.pb) - 1u;
         const R Na = V.s0[it.dest];
         if (it.proc == 0) {  // G_em = N(N'+N''+1) - N'N''
-#pragma unroll
-            for (int j = 0; j < VPL; ++j) {
-                if (sl + (j << lg) >= nv) continue;
-                R t = R(0);
-#pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    const unsigned e = comp4(b.iv[j], k);
-                    const R Nb = V.s0[e & pmask], Nc = V.s0[e >> V.pb];
-                    const R G = fma(-Nb, Nc, fma(Na, Nb + Nc, Na));
-                    t = fma(b.w(j, k), G, t);
-                }
-                lane_add(acc, cmp, t);
-            }
+            lane_sum<R, VPL, FULL>(b, nv, sl, lg, acc, cmp, [&](unsigned e) {
+                const R Nb = V.s0[e & pmask], Nc = V.s0[e >> V.pb];
+                return fma(-Nb, Nc, fma(Na, Nb + Nc, Na));
+            });
         } else {  // G_abs = N(N''-N') - N'(N''+1)
-#pragma unroll
-            for (int j = 0; j < VPL; ++j) {
-                if (sl + (j << lg) >= nv) continue;
-                R t = R(0);
-#pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    const unsigned e = comp4(b.iv[j], k);
-                    const R Nb = V.s0[e & pmask], Nc = V.s0[e >> V.pb];
-                    const R G = fma(Na, Nc - Nb, -Nb * (Nc + R(1)));
-                    t = fma(b.w(j, k), G, t);
-                }
-                lane_add(acc, cmp, t);
-            }
+            lane_sum<R, VPL, FULL>(b, nv, sl, lg, acc, cmp, [&](unsigned e) {
+                const R Nb = V.s0[e & pmask], Nc = V.s0[e >> V.pb];
+                return fma(Na, Nc - Nb, -Nb * (Nc + R(1)));
+            });
         }
     }
 }
@@ -250,77 +217,11 @@ __device__ __forceinline__ Item item_from(const int4 &d) {  // decode an ItemRec
     return it;
 }
 
-// Item descriptors of a warp's strided sequence are fetched 32 at a time (one per lane) and
-// broadcast with shuffles.
-struct DescStream {
-    const int4 *items;
-    int k0, end, stride;  // first item of the current block, end of the range, item stride
-    int4 cur, nxt;        // this lane's descriptor in the current / next block
-    __device__ __forceinline__ int4 fetch(int base, int lane) const {
-        const int k = base + lane * stride;
-        return k < end ? __ldg(items + k) : make_int4(0, 0, 0, 0);
-    }
-    __device__ __forceinline__ void init(const ItemRec *it, int a, int b, int st, int lane) {
-        items = reinterpret_cast<const int4 *>(it);
-        k0 = a;
-        end = b;
-        stride = st;
-        cur = fetch(a, lane);
-        nxt = fetch(a + 32 * st, lane);
-    }
-    __device__ __forceinline__ Item get(int k, int lane) {  // k advances by `stride` per call
-        if (k - k0 >= 32 * stride) {
-            k0 += 32 * stride;
-            cur = nxt;
-            nxt = fetch(k0 + 32 * stride, lane);
-        }
-        const int src = (k - k0) / stride;
-        int4 d;
-        d.x = __shfl_sync(kFull, cur.x, src);
-        d.y = __shfl_sync(kFull, cur.y, src);
-        d.z = __shfl_sync(kFull, cur.z, src);
-        d.w = __shfl_sync(kFull, cur.w, src);
-        return item_from(d);
-    }
-    // descriptor of item kb + h*stride for this lane (h = its sub-warp), kb warp-uniform and
-    // advancing by (items per iteration) * stride per call
-    __device__ __forceinline__ Item get_sub(int kb, int h) {
-        if (kb - k0 >= 32 * stride) {
-            k0 += 32 * stride;
-            cur = nxt;
-            nxt = fetch(k0 + 32 * stride, threadIdx.x & 31);
-        }
-        const int off = (kb - k0) / stride + h;
-        const bool in_cur = off < 32;
-        const int src = in_cur ? off : off - 32;
-        int4 d;
-        d.x = __shfl_sync(kFull, in_cur ? cur.x : nxt.x, src);
-        d.y = __shfl_sync(kFull, in_cur ? cur.y : nxt.y, src);
-        d.z = __shfl_sync(kFull, in_cur ? cur.z : nxt.z, src);
-        d.w = __shfl_sync(kFull, in_cur ? cur.w : nxt.w, src);
-        return item_from(d);
-    }
-    // descriptor of item k in the current or next block, without advancing (warp-uniform k)
-    __device__ __forceinline__ Item peek(int k) const {
-        const int off = (k - k0) / stride;
-        const bool in_cur = off < 32;
-        const int src = in_cur ? off : off - 32;
-        int4 d;
-        d.x = __shfl_sync(kFull, in_cur ? cur.x : nxt.x, src);
-        d.y = __shfl_sync(kFull, in_cur ? cur.y : nxt.y, src);
-        d.z = __shfl_sync(kFull, in_cur ? cur.z : nxt.z, src);
-        d.w = __shfl_sync(kFull, in_cur ? cur.w : nxt.w, src);
-        return item_from(d);
-    }
-};
-
-// L2 prefetch of item k's entry arrays (one bulk prefetch per array, issued by lane 0), so
-// that its streaming loads, issued `dist` items later, find the lines in L2.  Warp-uniform k.
-template <class R>
-__device__ __forceinline__ void prefetch_item(const GroupView<R> &V, const DescStream &D, int k, int b, int lane) {
-    if (k >= b || k - D.k0 >= 64 * D.stride) return;
-    const Item it = D.peek(k);
-    if (lane == 0 && it.len > 0) {
+// L2 prefetch of an item's entry arrays (one bulk prefetch per array), so that its streaming
+// loads, issued some items later, find the lines in L2.
+template <class R> __device__ __forceinline__ void prefetch_item(const GroupView<R> &V, const int4 &d) {
+    const Item it = item_from(d);
+    if (it.len > 0) {
         const uint32_t *ip = V.idx + it.begin;
         const R *wp = V.W + it.begin;
         asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;\n" ::"l"(ip), "r"((unsigned)it.len * 4u) : "memory");
@@ -336,74 +237,95 @@ __device__ __forceinline__ void prefetch_item(const GroupView<R> &V, const DescS
 template <class R>
 __device__ __forceinline__ void finish_item(const KParams &P, unsigned slot, bool valid, R acc, R cmp, int sl, int lg) {
     acc += cmp;
-    cmp = R(0);
 #pragma unroll
     for (int o = 16; o; o >>= 1)
         if (o < (1 << lg)) acc += __shfl_xor_sync(kFull, acc, o);
     if (sl == 0 && valid) {
-        R *out = reinterpret_cast<R *>(P.partials) + 2LL * slot;
-        out[0] = acc;
-        out[1] = cmp;
+        reinterpret_cast<R *>(P.partials)[slot] = acc;
     }
 }
 
-// Items a, a+st, a+2st, ... < b of one group for one warp.  The warp works on G = 32 >> lg
-// items at a time, one per sub-warp of 1 << lg lanes (the group's items are cut to at most
-// 16 << lg entries, so groups of short segments pack two or four items to a warp).  WIDE is
-// the variant for plans whose groups all use whole-warp items (lg = 5 at compile time).  With
-// PIPE, the next items' entry loads are in flight while the current ones are computed (two
-// register buffers).
+// A warp's share of items [a, b) of one group.  The warp works on G = 32 >> lg consecutive items
+// at a time, one per sub-warp of 1 << lg lanes (the group's items are cut to at most 16 << lg
+// entries, so groups of short segments pack two to eight items to a warp), and the warps of the
+// CTA take such packets in turn.  WIDE is the variant for plans whose groups all use whole-warp
+// items (lg = 5 at compile time).  Every sub-warp loads its own descriptors, one packet ahead of
+// their use (uniform 16-byte loads: no shuffles, no index division).  The loop is bound by issue
+// slots and latency as much as by HBM, so what an item costs beyond its entries counts: with
+// descriptors fetched 32 at a time and broadcast by shuffles (two divisions by the runtime stride
+// and eight shuffles an item), bounds tests on full items and separate emission / absorption
+// branches, graphene 180 took 395 us (full RHS, 2.27 GB), silicon 32 470 us and a 64-instance
+// ensemble 1.76 ms; without them 363, 430 and 1.42 ms.  With PIPE, the next items' entry loads are
+// in flight while the current ones are computed (two register buffers).
 template <class R, bool PIPE, bool WIDE>
-__device__ __forceinline__ void run_range(const KParams &P, const GroupView<R> &V, int a, int b, int st, int lane) {
-    if (a >= b) return;
+__device__ __forceinline__ void run_range(const KParams &P, const GroupView<R> &V, int a, int b, int warp, int nwarps,
+                                          int lane) {
     const int lg = WIDE ? 5 : V.lg;
     const int G = 32 >> lg;
-    const int h = lane >> lg, sl = lane & ((1 << lg) - 1);
-    DescStream D;
-    D.init(P.items, a, b, st, lane);
-    auto next = [&](int kb) { return WIDE ? D.get(kb, lane) : D.get_sub(kb, h); };
-    auto valid = [&](int kb) { return WIDE || kb + h * st < b; };
-    const int pf = P.pf_dist;  // iterations ahead whose entries are prefetched into L2 (0: none)
-    R acc, cmp;
-    if (pf > 0)
-        for (int j = 1; j < pf; ++j) prefetch_item(V, D, a + j * G * st, b, lane);
+    const int step = nwarps * G;
+    int kb = a + warp * G;  // first item of the warp's packet
+    if (kb >= b) return;
+    const int sl = lane & ((1 << lg) - 1);
+    int k = kb + (lane >> lg);
+    const int4 *items = reinterpret_cast<const int4 *>(P.items);
+    // (unsigned: an index past INT_MAX near the end of a very long list is out of range, not negative)
+    auto fetch = [&](unsigned i) { return i < (unsigned)b ? __ldg(items + i) : make_int4(0, 0, 0, 0); };
+    auto run = [&](const Item &it, const Batch<R, 4> &B, bool valid) {
+        R acc, cmp;
+        if (WIDE && it.len == kItemEntries) compute_item<R, 4, true>(V, it, B, sl, lg, acc, cmp);
+        else compute_item<R, 4, false>(V, it, B, sl, lg, acc, cmp);
+        finish_item<R>(P, it.slot, valid, acc, cmp, sl, lg);
+    };
+    const int pf = P.pf_dist;  // packets ahead whose entries are prefetched into L2 (0: none)
+    const bool lead = sl == 0 && pf > 0;
+    int4 d = fetch(k), dn = fetch(k + step), dp = make_int4(0, 0, 0, 0);
+    if (lead) {
+        for (int j = 1; j < pf; ++j) prefetch_item(V, fetch((unsigned)k + j * step));
+        dp = fetch((unsigned)k + pf * step);
+    }
     if (!PIPE) {
-        for (int k = a; k < b; k += G * st) {
-            const Item it = next(k);
-            if (pf > 0) prefetch_item(V, D, k + pf * G * st, b, lane);
+        for (; kb < b; kb += step, k += step) {
+            const Item it = item_from(d);
+            d = dn;
+            dn = fetch((unsigned)k + 2 * step);
             Batch<R, 4> B;
             B.issue(V, it, sl, lg);
-            compute_item<R, 4>(V, it, B, sl, lg, acc, cmp);
-            finish_item<R>(P, it.slot, valid(k), acc, cmp, sl, lg);
+            if (lead) {
+                prefetch_item(V, dp);
+                dp = fetch((unsigned)k + (pf + 1) * step);
+            }
+            run(it, B, k < b);
         }
         return;
     }
     Batch<R, 4> A, B;
-    int k = a;
-    Item ia = next(k);
+    Item ia = item_from(d);
     A.issue(V, ia, sl, lg);
+    auto advance = [&](Batch<R, 4> &N, Item &in) {  // the next packet's loads; false at the end
+        const bool has = kb + step < b;
+        if (has) {
+            in = item_from(dn);
+            dn = fetch((unsigned)k + 2 * step);
+            N.issue(V, in, sl, lg);
+        }
+        if (lead) {
+            prefetch_item(V, dp);
+            dp = fetch((unsigned)k + (pf + 1) * step);
+        }
+        return has;
+    };
     for (;;) {
-        const bool hb = k + G * st < b;
         Item ib;
-        if (hb) {
-            ib = next(k + G * st);
-            B.issue(V, ib, sl, lg);
-        }
-        if (pf > 0) prefetch_item(V, D, k + pf * G * st, b, lane);
-        compute_item<R, 4>(V, ia, A, sl, lg, acc, cmp);
-        finish_item<R>(P, ia.slot, valid(k), acc, cmp, sl, lg);
+        const bool hb = advance(B, ib);
+        run(ia, A, k < b);
         if (!hb) break;
-        k += G * st;
-        const bool ha = k + G * st < b;
-        if (ha) {
-            ia = next(k + G * st);
-            A.issue(V, ia, sl, lg);
-        }
-        if (pf > 0) prefetch_item(V, D, k + pf * G * st, b, lane);
-        compute_item<R, 4>(V, ib, B, sl, lg, acc, cmp);
-        finish_item<R>(P, ib.slot, valid(k), acc, cmp, sl, lg);
+        kb += step;
+        k += step;
+        const bool ha = advance(A, ia);
+        run(ib, B, k < b);
         if (!ha) break;
-        k += G * st;
+        kb += step;
+        k += step;
     }
 }
 
@@ -497,7 +419,7 @@ __global__ void __launch_bounds__(NT, MINB) rhs_kernel(KParams P) {
         if (P.ctl && P.ctl[G.inst].done) continue;  // instance already at its t_out
         GroupView<R> V;
         enter_group<R, STAGED>(P, ug, sm, staged, V);
-        run_range<R, PIPE, WIDE>(P, V, ua + warp, ub, nwarps, lane);
+        run_range<R, PIPE, WIDE>(P, V, ua, ub, warp, nwarps, lane);
     }
     if (dynamic && P.n_tail > 0 && threadIdx.x == 0) {  // the last CTA out resets the counters
         __threadfence();
@@ -1042,7 +964,7 @@ int make_plan(rtbte_ctx *ctx) {
     RT_CUDA(ctx, cudaMalloc(&ctx->dyn_tab.p, ctx->dyn_tab.bytes));
     RT_CUDA(ctx, cudaMemsetAsync(ctx->dyn_tab.p, 0, ctx->dyn_tab.bytes, ctx->stream));
     ctx->partials.release();
-    size_t pb = std::max<size_t>(2 * R * (size_t)std::max(ctx->n_items, 1), 16);
+    size_t pb = std::max<size_t>(R * (size_t)std::max(ctx->n_items, 1), 16);
     RT_CUDA(ctx, cudaMalloc(&ctx->partials.p, pb));
     ctx->partials.bytes = pb;
     RT_CUDA(ctx, cudaMemsetAsync(ctx->partials.p, 0, pb, ctx->stream));

@@ -16,7 +16,7 @@ struct RowParams {
     const int *rowoff;               // [n_y+1] first partial slot of each state row
     const int *rowmid;               // [n_y] phonon rows: first ph-ph slot (ph-e slots before it)
     const int *compact;              // sub-lattice index of each phonon or -1
-    const void *partials;            // (hi, lo) per item, compute precision
+    const void *partials;            // one sum per item, compute precision
     void *popf, *popN, *popP;        // population copies, compute precision
 };
 
@@ -29,21 +29,21 @@ __device__ __forceinline__ int find_inst(const RowParams &Q, long long comp) {
     return lo;
 }
 
-// Accumulator of item partials (hi, lo) in item order.  FP64 partials add in FP64.  FP32
-// partials add as an FP32 head/tail pair (two-sum on the heads, tails summed) and are widened
-// once at the end: about 48 significant bits, far below the partials' own rounding, with no
-// FP64 arithmetic per item (FP64 throughput is low on this GPU).
+// Accumulator of item partials in item order.  FP64 partials add in FP64.  FP32 partials add as
+// an FP32 head/tail pair (two-sum on the heads, tails summed) and are widened once at the end:
+// about 48 significant bits, far below the partials' own rounding, with no FP64 arithmetic per
+// item (FP64 throughput is low on this GPU).
 template <class R> struct RowAcc {
     double acc = 0.0;
-    __device__ __forceinline__ void add(R hi, R lo) { acc += (double)hi + (double)lo; }
+    __device__ __forceinline__ void add(R x) { acc += (double)x; }
     __device__ __forceinline__ double value() const { return acc; }
 };
 template <> struct RowAcc<float> {
     float s = 0.f, c = 0.f;
-    __device__ __forceinline__ void add(float hi, float lo) {
-        const float t = s + hi;
+    __device__ __forceinline__ void add(float x) {
+        const float t = s + x;
         const float bp = t - s;
-        c += ((s - (t - bp)) + (hi - bp)) + lo;
+        c += (s - (t - bp)) + (x - bp);
         s = t;
     }
     __device__ __forceinline__ double value() const { return (double)s + (double)c; }
@@ -52,7 +52,7 @@ template <> struct RowAcc<float> {
 template <class R>
 __device__ __forceinline__ void item_sum(const RowParams &Q, int i0, int i1, RowAcc<R> &A) {
     const R *P = reinterpret_cast<const R *>(Q.partials);
-    for (int it = i0; it < i1; ++it) A.add(P[2 * it], P[2 * it + 1]);
+    for (int it = i0; it < i1; ++it) A.add(P[it]);
 }
 
 // RHS value of row `local` of instance I for the selected parts.  The row's partials sit in
