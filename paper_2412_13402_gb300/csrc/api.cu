@@ -745,10 +745,11 @@ void rtbte_destroy(rtbte_ctx *ctx) {
                           &I.pp_off_dev};
         for (DevBuf *b : bufs) b->release();
     }
-    ctx->tail_tab.release();
+    ctx->bound_tab.release();
+    ctx->act_tab.release();
     ctx->tail_ctr.release();
     DevBuf *bufs[] = {&ctx->popf, &ctx->popN, &ctx->popP, &ctx->instdev, &ctx->compact, &ctx->items, &ctx->groups,
-                      &ctx->partials, &ctx->rowoff, &ctx->rowmid, &ctx->cta_tab, &ctx->gwt, &ctx->dyn_tab, &ctx->Y[0], &ctx->Y[1],
+                      &ctx->partials, &ctx->rowoff, &ctx->rowmid, &ctx->gwt, &ctx->dyn_tab, &ctx->Y[0], &ctx->Y[1],
                       &ctx->K, &ctx->Fs, &ctx->forcing, &ctx->wrms_part, &ctx->ctl, &ctx->ystage, &ctx->ydstage,
                       &ctx->range_scratch, &ctx->slow_save};
     for (DevBuf *b : bufs) b->release();

@@ -30,8 +30,8 @@ namespace rtbte {
 
 constexpr int kItemEntries = 512;  // 32 lanes x 4 vectors x 4 entries
 constexpr int kSegPad = 4;
-constexpr int kRhsThreads = 512;      // collision kernel, threads per SM: two register buffers of entries per warp
-constexpr int kRhsThreadsDeep = 768;  // FP32 single-buffer form: 24 warps per SM at 80 registers
+constexpr int kRhsThreads = 768;    // collision kernel, threads per SM in FP32 (80 registers)
+constexpr int kRhsThreads64 = 512;  // ... and in FP64 (128 registers)
 constexpr int kMaxModes = 16;
 constexpr int kMaxStages = 5;
 constexpr int kWrmsBlocks = 512;
@@ -100,13 +100,18 @@ struct __align__(16) Ctl {
     int cur, last, fixed, pad_i0;
 };
 
+// What an item costs the warp that runs it.
+struct ItemCost {
+    unsigned short slots;  // entry slots: vectors per lane x lanes x 4
+    unsigned short lanes;  // its share of a warp
+};
+
 // Launch parameters of the collision kernel for one parts mask.
 struct LaunchTuning {
-    int w = 320;                     // work-split weight of an item beyond its entries
-    int pf = 3;                      // L2 prefetch distance in items of a warp's sequence (0: off)
+    int w = 192;                     // work-split weight of a packet (one warp's items) beyond its entries
+    int pf = 1;                      // L2 prefetch distance in packets of a warp's sequence (0: off)
     double sf = 1.0;                 // share of the weight split statically (rest: dynamic chunks)
     double ps[3] = {1.0, 1.0, 1.0};  // relative cost of an entry of each part
-    bool deep = false;               // FP32: the single-buffer form at 24 warps per SM
 };
 
 struct CtlParams {  // constants of one integration (captured into graphs by value)
@@ -233,19 +238,19 @@ struct rtbte_ctx {
     rtbte::DevBuf popf, popN, popP, instdev, compact;
     // execution plan of the RHS
     bool plan_valid = false;
-    rtbte::DevBuf items, groups, partials, rowoff, rowmid, cta_tab, gwt, dyn_tab;  // rowoff/rowmid: slots of each row
+    rtbte::DevBuf items, groups, partials, rowoff, rowmid, gwt, dyn_tab;  // rowoff/rowmid: slots of each row
     int n_rblk = 0;  // several instances: row blocks of the stage kernels (256 rows of one instance each)
     int n_items = 0, n_groups = 0;
     int part_items[3] = {0, 0, 0};
     int part_first[3] = {0, 0, 0};
     int stage_resident = 0;    // stage kernel: blocks resident on the whole GPU at once (its grid)
-    int grid = 0, per_sm = 1;  // collision kernel: CTAs per SM (1, 2 or 4; threads = form's threads per SM / per_sm)
+    int grid = 0, per_sm = 1;  // collision kernel: CTAs per SM (1, 2 or 4; threads = threads per SM / per_sm)
     rtbte::LaunchTuning lt[8];  // collision-kernel launch parameters of each parts mask (1..7)
     unsigned lt_tuned = 0;      // masks the autotuner tuned themselves (kept across plans)
-    std::vector<unsigned short> item_len_h;  // entries per work item (host copy for re-splitting)
-    std::vector<int> group_begin_h;          // first item of each group (host copy)
-    rtbte::DevBuf tail_tab, tail_ctr;        // dynamic chunks {first, end, group, 0} per mask; grab/exit counters
-    int tail_off[8] = {0, 0, 0, 0, 0, 0, 0, 0};  // chunks of mask m: [tail_off[m-1], tail_off[m])
+    std::vector<rtbte::ItemCost> item_cost_h;  // cost of each work item (host copy for re-splitting)
+    std::vector<int> group_begin_h, group_part_h;  // first item and part of each group (host copies)
+    rtbte::DevBuf bound_tab, act_tab, tail_ctr;    // work-unit bounds and group lists per mask; grab/exit counters
+    int bound_off[8] = {}, act_off[8] = {}, tail_n[8] = {};  // per mask: first bound, first listed group, dynamic units
     size_t smem_bytes = 0;
     bool staged = false;
     bool wide = true;  // every group uses whole-warp items (the kernel variant without sub-warps)

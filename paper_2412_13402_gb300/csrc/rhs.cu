@@ -15,10 +15,8 @@
 // written per item to the item's slot -- the slots of one row's items are consecutive -- and
 // the row kernels add a row's partials in slot order (deterministic).  CTAs
 // first run a static share of the items (split by estimated cost), then take the rest in
-// chunks from a counter; warps may prefetch upcoming items' entries into L2.  FP32 launches
-// come in two forms, chosen per parts mask: two register buffers of entries per warp (the next
-// item's loads in flight during the current one's arithmetic) at 16 warps per SM, or one buffer
-// at 24 warps per SM.
+// chunks from a counter; warps may prefetch upcoming items' entries into L2.  FP32 runs at 24 warps
+// per SM, FP64 at 16.
 //
 // Per-entry arithmetic uses the exact algebraic reductions of the paper's factors
 // (Methods A):  F_em = f(1-f') + N(f-f'),  F_abs = N(f-f') - f'(1-f),
@@ -62,16 +60,17 @@ struct KParams {
     const ItemRec *items;
     const Group *groups;
     int n_groups;
-    const int *cta_items;  // [grid+1] first item of each CTA's static range (real item indices)
-    unsigned mask;         // parts evaluated (groups of other parts are skipped)
+    // Work units: unit u is the items from bound[u] up to bound[u + 1] of the groups listed in act,
+    // in order (parts not evaluated and finished instances are not in the list).  Units 0..grid-1
+    // are the CTAs' static ranges, units grid.. are taken from a counter.
+    const int4 *bound;    // {first item, its group, that group's index in act, 0}
+    const int *act;       // groups to evaluate, ascending (-1 ends)
+    int n_tail;           // dynamic units
+    const int *n_tail_d;  // batched integration: their number, set by split_kernel (else null)
     void *partials;
     const void *popf, *popN, *popP;
     const Ctl *ctl;  // per-instance controllers: launches inside an integrator skip finished instances
-    const int *act;      // batched integration: active groups in order (-1 ends), else null
-    const int *cta_act;  // batched integration: index in act[] of each CTA's first group
-    const int4 *tail;  // dynamic chunks {first item, end item, group, 0} after the static ranges
-    int n_tail;
-    int *tail_ctr;     // [0] next chunk to take, [1] CTAs finished (reset by the last one)
+    int *tail_ctr;     // [0] next dynamic unit, [1] CTAs finished (reset by the last one)
     int pf_dist;       // L2 prefetch distance in items of a warp's sequence (0: off)
 };
 
@@ -255,9 +254,8 @@ __device__ __forceinline__ void finish_item(const KParams &P, unsigned slot, boo
 // descriptors fetched 32 at a time and broadcast by shuffles (two divisions by the runtime stride
 // and eight shuffles an item), bounds tests on full items and separate emission / absorption
 // branches, graphene 180 took 395 us (full RHS, 2.27 GB), silicon 32 470 us and a 64-instance
-// ensemble 1.76 ms; without them 363, 430 and 1.42 ms.  With PIPE, the next items' entry loads are
-// in flight while the current ones are computed (two register buffers).
-template <class R, bool PIPE, bool WIDE>
+// ensemble 1.76 ms; without them 363, 430 and 1.42 ms.
+template <class R, bool WIDE>
 __device__ __forceinline__ void run_range(const KParams &P, const GroupView<R> &V, int a, int b, int warp, int nwarps,
                                           int lane) {
     const int lg = WIDE ? 5 : V.lg;
@@ -270,12 +268,6 @@ __device__ __forceinline__ void run_range(const KParams &P, const GroupView<R> &
     const int4 *items = reinterpret_cast<const int4 *>(P.items);
     // (unsigned: an index past INT_MAX near the end of a very long list is out of range, not negative)
     auto fetch = [&](unsigned i) { return i < (unsigned)b ? __ldg(items + i) : make_int4(0, 0, 0, 0); };
-    auto run = [&](const Item &it, const Batch<R, 4> &B, bool valid) {
-        R acc, cmp;
-        if (WIDE && it.len == kItemEntries) compute_item<R, 4, true>(V, it, B, sl, lg, acc, cmp);
-        else compute_item<R, 4, false>(V, it, B, sl, lg, acc, cmp);
-        finish_item<R>(P, it.slot, valid, acc, cmp, sl, lg);
-    };
     const int pf = P.pf_dist;  // packets ahead whose entries are prefetched into L2 (0: none)
     const bool lead = sl == 0 && pf > 0;
     int4 d = fetch(k), dn = fetch(k + step), dp = make_int4(0, 0, 0, 0);
@@ -283,49 +275,20 @@ __device__ __forceinline__ void run_range(const KParams &P, const GroupView<R> &
         for (int j = 1; j < pf; ++j) prefetch_item(V, fetch((unsigned)k + j * step));
         dp = fetch((unsigned)k + pf * step);
     }
-    if (!PIPE) {
-        for (; kb < b; kb += step, k += step) {
-            const Item it = item_from(d);
-            d = dn;
-            dn = fetch((unsigned)k + 2 * step);
-            Batch<R, 4> B;
-            B.issue(V, it, sl, lg);
-            if (lead) {
-                prefetch_item(V, dp);
-                dp = fetch((unsigned)k + (pf + 1) * step);
-            }
-            run(it, B, k < b);
-        }
-        return;
-    }
-    Batch<R, 4> A, B;
-    Item ia = item_from(d);
-    A.issue(V, ia, sl, lg);
-    auto advance = [&](Batch<R, 4> &N, Item &in) {  // the next packet's loads; false at the end
-        const bool has = kb + step < b;
-        if (has) {
-            in = item_from(dn);
-            dn = fetch((unsigned)k + 2 * step);
-            N.issue(V, in, sl, lg);
-        }
+    for (; kb < b; kb += step, k += step) {
+        const Item it = item_from(d);
+        d = dn;
+        dn = fetch((unsigned)k + 2 * step);
+        Batch<R, 4> B;
+        B.issue(V, it, sl, lg);
         if (lead) {
             prefetch_item(V, dp);
             dp = fetch((unsigned)k + (pf + 1) * step);
         }
-        return has;
-    };
-    for (;;) {
-        Item ib;
-        const bool hb = advance(B, ib);
-        run(ia, A, k < b);
-        if (!hb) break;
-        kb += step;
-        k += step;
-        const bool ha = advance(A, ia);
-        run(ib, B, k < b);
-        if (!ha) break;
-        kb += step;
-        k += step;
+        R acc, cmp;
+        if (WIDE && it.len == kItemEntries) compute_item<R, 4, true>(V, it, B, sl, lg, acc, cmp);
+        else compute_item<R, 4, false>(V, it, B, sl, lg, acc, cmp);
+        finish_item<R>(P, it.slot, k < b, acc, cmp, sl, lg);
     }
 }
 
@@ -362,66 +325,42 @@ __device__ __forceinline__ void enter_group(const KParams &P, int g, R *sm, int 
     }
 }
 
-// Persistent collision kernel.  Each CTA first runs its static range of items (cta_items,
-// split by estimated cost), then takes dynamic chunks of the remaining items from a shared
-// counter until none is left, so that SMs that finish early absorb the tail of the work.
-// Items are round-robin over the warps of the CTA; every item writes its own partial, so the
-// result does not depend on which CTA ran it.
-template <class R, bool STAGED, bool PIPE, bool WIDE, int MINB, int NT>
+// Persistent collision kernel.  Each CTA first runs its static unit (ranges of equal estimated
+// cost), then takes dynamic units of the remaining items from a shared counter until none is
+// left, so that SMs that finish early absorb the tail of the work.  Every item writes its own
+// partial, so the result does not depend on which CTA ran it.
+template <class R, bool STAGED, bool WIDE, int MINB, int NT>
 __global__ void __launch_bounds__(NT, MINB) rhs_kernel(KParams P) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ int s_chunk;
+    __shared__ int s_unit;
     R *sm = reinterpret_cast<R *>(smem_raw);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+    const int n_tail = P.n_tail_d ? *P.n_tail_d : P.n_tail;
     int staged = -1;
-    const int ra = P.cta_items[blockIdx.x], rb = P.cta_items[blockIdx.x + 1];
-    int g = P.n_groups;  // next group of the static range (with P.act: next index into act[])
-    if (ra < rb) {
-        if (P.act) {
-            g = P.cta_act[blockIdx.x];
-        } else {
-            int lo = 0, hi = P.n_groups - 1;  // last group with item_begin <= ra
-            while (lo < hi) {
-                int mid = (lo + hi + 1) >> 1;
-                if (P.groups[mid].item_begin <= ra) lo = mid; else hi = mid - 1;
+    for (int u = blockIdx.x;;) {
+        const int4 from = P.bound[u];
+        const int end = P.bound[u + 1].x;
+        for (int a = from.x, g = from.y, at = from.z; a < end;) {
+            const Group &G = P.groups[g];
+            const int b = min(end, G.item_end);
+            if (a < b && !(P.ctl && P.ctl[G.inst].done)) {  // (done: the instance is at its t_out)
+                GroupView<R> V;
+                enter_group<R, STAGED>(P, g, sm, staged, V);
+                run_range<R, WIDE>(P, V, a, b, warp, nwarps, lane);
             }
-            g = lo;
+            if (end <= G.item_end) break;
+            g = P.act[++at];
+            if (g < 0) break;
+            a = P.groups[g].item_begin;
         }
+        if (n_tail == 0) return;
+        __syncthreads();  // every warp is done with the previous unit and with s_unit
+        if (threadIdx.x == 0) s_unit = atomicAdd(P.tail_ctr, 1);
+        __syncthreads();
+        if (s_unit >= n_tail) break;
+        u = gridDim.x + s_unit;
     }
-    bool dynamic = false;
-    for (;;) {
-        int ug, ua, ub;  // next unit of work: items [ua, ub) of group ug
-        if (!dynamic) {
-            const int gg = !P.act ? g : (g < P.n_groups ? P.act[g] : -1);
-            if (gg < 0 || gg >= P.n_groups || P.groups[gg].item_begin >= rb) {
-                dynamic = true;
-                if (P.n_tail == 0) break;
-                continue;
-            }
-            ug = gg;
-            ++g;
-            ua = max(ra, P.groups[ug].item_begin);
-            ub = min(rb, P.groups[ug].item_end);
-            if (ua >= ub) continue;
-        } else {
-            __syncthreads();  // every warp is done with the previous unit and with s_chunk
-            if (threadIdx.x == 0) s_chunk = atomicAdd(P.tail_ctr, 1);
-            __syncthreads();
-            const int c = s_chunk;
-            if (c >= P.n_tail) break;
-            const int4 ch = P.tail[c];
-            ug = ch.z;
-            ua = ch.x;
-            ub = ch.y;
-        }
-        const Group &G = P.groups[ug];
-        if (!(P.mask & (1u << G.part))) continue;
-        if (P.ctl && P.ctl[G.inst].done) continue;  // instance already at its t_out
-        GroupView<R> V;
-        enter_group<R, STAGED>(P, ug, sm, staged, V);
-        run_range<R, PIPE, WIDE>(P, V, ua, ub, warp, nwarps, lane);
-    }
-    if (dynamic && P.n_tail > 0 && threadIdx.x == 0) {  // the last CTA out resets the counters
+    if (threadIdx.x == 0) {  // the last CTA out resets the counters
         __threadfence();
         if (atomicAdd(P.tail_ctr + 1, 1) == (int)gridDim.x - 1) {
             P.tail_ctr[0] = 0;
@@ -434,15 +373,17 @@ __global__ void __launch_bounds__(NT, MINB) rhs_kernel(KParams P) {
 // Work split over the groups still active (instance not done, part in the mask), recomputed
 // on the device before a collision launch inside a batched integration.  One block:
 //   - the active groups are listed in order in act[] (terminated by -1);
-//   - CTA c gets the active weight [c, c+1) * total / grid: out[c] is its first item, found by
-//     interpolating linearly within the active group holding that weight (items of one group
-//     carry similar weights; the split affects balance only, never results), and out_act[c]
-//     the index in act[] of that group;
-//   - out[grid] is the end of the last active group's items.
-// A CTA then visits only the active groups act[out_act[c]], ... overlapping its item range,
-// so finished instances cost it nothing.
+//   - the units' bounds cut the active weight into `grid` static ranges holding 1 - tail_share of
+//     it and, when a CTA's share is above tail_min, kTailUnits x grid equal dynamic units; a
+//     bound's item is found by interpolating linearly within the active group holding its weight
+//     (items of one group carry similar weights; the split affects balance only, never results).
+// Finished instances cost a collision launch nothing.
+constexpr int kTailUnits = 4;  // dynamic units per CTA of a re-split
+constexpr double kResplitTail = 0.2;               // weight left to them
+constexpr long long kResplitTailMin = 2048LL * 300000;  // ... where a CTA's share is at least this
 __global__ void split_kernel(const Group *groups, int n_groups, const long long *gw, const Ctl *ctl, unsigned mask,
-                             int grid, int *out, int *out_act, int *act, int *memo, int n_inst) {
+                             int grid, double tail_share, long long tail_min, int4 *bound, int *act, int *n_tail,
+                             int *memo, int n_inst) {
     __shared__ long long A[1025];   // inclusive prefix of active weight over groups (A[0] = 0)
     __shared__ int Cn[1025];        // active groups before group g
     __shared__ long long wsum[32];
@@ -519,19 +460,23 @@ __global__ void split_kernel(const Group *groups, int n_groups, const long long 
     for (int g = threadIdx.x; g < n_groups; g += T)  // compact list of the active groups
         if (Cn[g + 1] > Cn[g]) act[Cn[g]] = g;
     if (threadIdx.x == 0) act[n_act] = -1;
-    for (int c = threadIdx.x; c <= grid; c += T) {
+    const bool tail = total / grid >= tail_min;
+    const int nt = tail ? kTailUnits * grid : 0;
+    const long long stat = tail ? total - (long long)(tail_share * (double)total) : total;
+    if (threadIdx.x == 0) *n_tail = nt;
+    for (int c = threadIdx.x; c <= grid + nt; c += T) {
         if (total == 0) {
-            out[c] = 0;
-            if (c < grid) out_act[c] = 0;
+            bound[c] = make_int4(0, 0, 0, 0);
             continue;
         }
-        if (c == grid) {  // end of the last active group's items
+        if (c == grid + nt) {  // end of the last active group's items
             int last = n_groups - 1;
             while (last > 0 && Cn[last + 1] == Cn[last]) --last;
-            out[c] = groups[last].item_end;
+            bound[c] = make_int4(groups[last].item_end, last, n_act - 1, 0);
             continue;
         }
-        const long long t = total * c / grid;
+        const long long t = c < grid ? stat / grid * c + stat % grid * c / grid
+                                     : stat + (total - stat) / nt * (c - grid) + (total - stat) % nt * (c - grid) / nt;
         int lo = 0, hi = n_groups - 1;  // group g with A[g] <= t < A[g+1]
         while (lo < hi) {
             int mid = (lo + hi + 1) >> 1;
@@ -541,8 +486,8 @@ __global__ void split_kernel(const Group *groups, int n_groups, const long long 
         const Group &G = groups[lo];
         const long long wg = A[lo + 1] - A[lo];
         const long long ni = G.item_end - G.item_begin;
-        out[c] = G.item_begin + (int)((t - A[lo]) * ni / (wg > 0 ? wg : 1));
-        out_act[c] = Cn[lo];
+        bound[c] = make_int4(G.item_begin + (int)((double)(t - A[lo]) * (double)ni / (double)(wg > 0 ? wg : 1)), lo,
+                             Cn[lo], 0);
     }
     for (int i = threadIdx.x; i < n_inst; i += T) memo[i] = ctl[i].done;
     if (threadIdx.x == 0) {
@@ -581,6 +526,27 @@ template <class T> int upload_vec(rtbte_ctx *ctx, DevBuf &b, const std::vector<T
     return RTBTE_OK;
 }
 
+// Tables of the device re-split in ctx->dyn_tab: unit bounds, active groups, number of dynamic
+// units, and the memo of the last split ([n_inst] done flags it saw, its parts mask, a valid flag).
+struct DynTab {
+    int4 *bound;  // [(1 + kTailUnits) x grid + 1]
+    int *act;     // [n_groups + 1]
+    int *n_tail;  // [1]
+    int *memo;    // [n_inst + 2]
+};
+size_t dyn_tab_bytes(const rtbte_ctx *ctx) {
+    return sizeof(int4) * ((1 + kTailUnits) * (size_t)ctx->grid + 1) +
+           sizeof(int) * ((size_t)ctx->n_groups + 1 + 1 + ctx->inst.size() + 2);
+}
+DynTab dyn_tab(const rtbte_ctx *ctx) {
+    DynTab T;
+    T.bound = ctx->dyn_tab.as<int4>();
+    T.act = reinterpret_cast<int *>(T.bound + (1 + kTailUnits) * (size_t)ctx->grid + 1);
+    T.n_tail = T.act + ctx->n_groups + 1;
+    T.memo = T.n_tail + 1;
+    return T;
+}
+
 }  // namespace
 
 RowParams row_params(rtbte_ctx *ctx) {
@@ -597,92 +563,189 @@ RowParams row_params(rtbte_ctx *ctx) {
     return Q;
 }
 
-// Per-mask work split of the persistent grid.  Item weight = (entries + w) x the part's
-// calibrated cost per entry, with each mask's own w and costs.  The first share sf of a mask's
-// weight is split into equal-weight contiguous CTA ranges (table [mask][grid+1] of real item
-// indices); the rest is
-// cut into dynamic chunks of decreasing weight (half the remaining weight per grid, at least
-// 1/40 of a CTA's share, never across a group boundary), taken by CTAs in order at run time.
+// Per-mask work units of the persistent grid, from item weights: (entry slots + w x the item's
+// share of a warp) x the part's cost per entry, with each mask's own w and part costs.  The slots
+// count the vectors its lanes step through together, used or not (a warp's packet takes as long
+// as its longest lane), and w is the cost of a packet beyond its entries.  The first share sf of a
+// mask's weight is split into equal static ranges, one per CTA; the rest is cut into dynamic
+// units of decreasing weight (half the remaining weight per grid, at least 1/40 of a CTA's share,
+// never across a group boundary), taken by CTAs in order at run time.
 int split_tables(rtbte_ctx *ctx) {
     const int G = ctx->grid;
-    const std::vector<unsigned short> &len = ctx->item_len_h;
-    const int n = (int)len.size();
-    // weight of item k under mask m's parameters: (entries + w) x the part's cost per entry
-    auto weight = [&](const LaunchTuning &L, int part, int k) {
-        const long long sc = (long long)(64.0 * L.ps[part] + 0.5);  // cost per entry-equivalent
-        return sc * (len[k] + L.w);
+    const int n = (int)ctx->item_cost_h.size();
+    const int ng = (int)ctx->group_begin_h.size();
+    auto group_end = [&](int g) { return g + 1 < ng ? ctx->group_begin_h[g + 1] : n; };
+    // prefix of the unscaled weights (32 x slots + w x lanes) over all items, per distinct w
+    std::map<int, std::vector<long long>> prefixes;
+    auto prefix_of = [&](int w) -> const std::vector<long long> & {
+        std::vector<long long> &p = prefixes[w];
+        if (p.empty()) {
+            p.resize(n + 1);
+            p[0] = 0;
+            for (int k = 0; k < n; ++k)
+                p[k + 1] = p[k] + 32LL * ctx->item_cost_h[k].slots + (long long)w * ctx->item_cost_h[k].lanes;
+        }
+        return p;
     };
-    std::vector<int> item_group(n, 0);
-    for (size_t g = 0; g < ctx->group_begin_h.size(); ++g) {
-        const int e = g + 1 < ctx->group_begin_h.size() ? ctx->group_begin_h[g + 1] : n;
-        for (int k = ctx->group_begin_h[g]; k < e; ++k) item_group[k] = (int)g;
-    }
-    std::vector<int> tab(7LL * (G + 1), 0);
-    std::vector<int4> tail;
-    std::vector<long long> apre;  // prefix of the enabled parts' weights, item order
-    std::vector<int> aidx;
+    auto scale = [](const LaunchTuning &L, int part) { return (long long)(64.0 * L.ps[part] + 0.5); };
+    std::vector<int4> bound;
+    std::vector<int> act;
     for (unsigned mask = 1; mask <= 7; ++mask) {
         const LaunchTuning &L = ctx->lt[mask];
-        apre.assign(1, 0);
-        aidx.clear();
+        const std::vector<long long> &pre = prefix_of(L.w);
+        ctx->bound_off[mask] = (int)bound.size();
+        ctx->act_off[mask] = (int)act.size();
+        const int act0 = (int)act.size();
+        // the mask's parts in order: weight before the part, first and last item
+        long long before[4] = {0, 0, 0, 0};
+        int np = 0, parts[3] = {0, 0, 0};
+        std::vector<int> act_at(ng, -1);
         for (int part = 0; part < 3; ++part) {
-            if (!(mask & (1u << part))) continue;
-            for (int k = ctx->part_first[part]; k < ctx->part_first[part] + ctx->part_items[part]; ++k) {
-                apre.push_back(apre.back() + weight(L, part, k));
-                aidx.push_back(k);
-            }
+            if (!(mask & (1u << part)) || ctx->part_items[part] == 0) continue;
+            const int f = ctx->part_first[part], e = f + ctx->part_items[part];
+            before[np + 1] = before[np] + scale(L, part) * (pre[e] - pre[f]);
+            parts[np++] = part;
         }
-        const long long total = apre.back();
-        const int na = (int)aidx.size();
-        const long long split = L.sf >= 1.0 ? total : (long long)(L.sf * (double)total);
-        const int js = (int)(std::lower_bound(apre.begin(), apre.end(), split) - apre.begin());  // first tail item
-        int *t = tab.data() + (long long)(mask - 1) * (G + 1);
-        for (int c = 0; c <= G; ++c) {
-            if (na == 0) {
-                t[c] = 0;
-                continue;
-            }
-            if (c == G) {
-                t[c] = js >= na ? n : aidx[js];
-                continue;
-            }
-            const long long target = split * c / G;
-            const int j = (int)(std::lower_bound(apre.begin(), apre.end(), target) - apre.begin());
-            t[c] = c == 0 ? 0 : (j >= na ? n : (j >= js ? aidx[js] : aidx[j]));
+        for (int g = 0; g < ng; ++g) {
+            const int part = ctx->group_part_h[g];
+            if (!(mask & (1u << part)) || group_end(g) == ctx->group_begin_h[g]) continue;
+            act_at[g] = (int)act.size() - act0;
+            act.push_back(g);
         }
-        const long long wmin = std::max<long long>(1, total / (40LL * G));
-        for (int j = js; j < na;) {
-            const long long remaining = total - apre[j];
-            const long long want = std::max(wmin, remaining / (2LL * G));
-            const int g = item_group[aidx[j]];
-            int j2 = j + 1;
-            while (j2 < na && item_group[aidx[j2]] == g && aidx[j2] == aidx[j2 - 1] + 1 && apre[j2] - apre[j] < want)
-                ++j2;
-            tail.push_back(make_int4(aidx[j], aidx[j2 - 1] + 1, g, 0));
-            j = j2;
+        act.push_back(-1);
+        const long long total = before[np];
+        const int last = total > 0 ? ctx->part_first[parts[np - 1]] + ctx->part_items[parts[np - 1]] : 0;
+        int g_hint = 0;  // bounds ascend, and so do their groups
+        auto add = [&](int item) {
+            while (g_hint + 1 < ng && ctx->group_begin_h[g_hint + 1] <= item) ++g_hint;
+            bound.push_back(make_int4(item, g_hint, act_at[g_hint] < 0 ? 0 : act_at[g_hint], 0));
+        };
+        // first item at or after weight t
+        auto item_at = [&](long long t) {
+            int q = 0;
+            while (q + 1 < np && before[q + 1] <= t) ++q;
+            const int f = ctx->part_first[parts[q]], e = f + ctx->part_items[parts[q]];
+            const long long want = pre[f] + (t - before[q] + scale(L, parts[q]) - 1) / scale(L, parts[q]);
+            const int k = (int)(std::lower_bound(pre.begin() + f, pre.begin() + e, want) - pre.begin());
+            return k < e ? k : (q + 1 < np ? ctx->part_first[parts[q + 1]] : last);
+        };
+        auto weight_at = [&](int item) {  // weight before an item of the mask
+            for (int q = 0; q < np; ++q) {
+                const int f = ctx->part_first[parts[q]], e = f + ctx->part_items[parts[q]];
+                if (item >= f && item < e) return before[q] + scale(L, parts[q]) * (pre[item] - pre[f]);
+            }
+            return total;
+        };
+        int n_tail = 0;
+        if (total == 0) {
+            for (int c = 0; c <= G; ++c) bound.push_back(make_int4(0, 0, 0, 0));
+        } else {
+            const long long split = L.sf >= 1.0 ? total : (long long)(L.sf * (double)total);
+            const int js = split >= total ? last : item_at(split);
+            for (int c = 0; c < G; ++c) add(std::min(item_at(split / G * c + split % G * c / G), js));
+            const long long wmin = std::max<long long>(1, total / (40LL * G));
+            for (int j = js; j < last;) {
+                add(j);
+                ++n_tail;
+                const long long wj = weight_at(j), remaining = total - wj;
+                const int ge = group_end(g_hint);
+                int j2 = std::max(j + 1, item_at(std::min(total, wj + std::max(wmin, remaining / (2LL * G)))));
+                if (j2 >= ge) {  // on to the next group of the mask
+                    const int nx = act[act0 + act_at[g_hint] + 1];
+                    j2 = nx < 0 ? last : ctx->group_begin_h[nx];
+                }
+                j = j2;
+            }
+            add(last);
         }
-        ctx->tail_off[mask] = (int)tail.size();
+        ctx->tail_n[mask] = n_tail;
     }
     // per-group weights for the device re-split of batched integrations (full-RHS parameters)
-    std::vector<long long> wpre(n + 1, 0);
-    for (int part = 0; part < 3; ++part)
-        for (int k = ctx->part_first[part]; k < ctx->part_first[part] + ctx->part_items[part]; ++k)
-            wpre[k + 1] = weight(ctx->lt[7], part, k);
-    for (int k = 0; k < n; ++k) wpre[k + 1] += wpre[k];
-    std::vector<long long> gwt(ctx->group_begin_h.size());  // weight of each group's items
-    for (size_t g = 0; g < gwt.size(); ++g) {
-        const int e = g + 1 < ctx->group_begin_h.size() ? ctx->group_begin_h[g + 1] : n;
-        gwt[g] = wpre[e] - wpre[ctx->group_begin_h[g]];
-    }
+    std::vector<long long> gwt(ng);
+    const std::vector<long long> &pre7 = prefix_of(ctx->lt[7].w);
+    for (int g = 0; g < ng; ++g)
+        gwt[g] = scale(ctx->lt[7], ctx->group_part_h[g]) * (pre7[group_end(g)] - pre7[ctx->group_begin_h[g]]);
     int rc;
     if ((rc = upload_vec(ctx, ctx->gwt, gwt))) return rc;
     // the device re-split's memo no longer matches the weights: clear its valid flag
-    const size_t valid_at = 2 * (size_t)ctx->grid + 1 + ctx->n_groups + 1 + ctx->inst.size() + 1;
-    if (ctx->dyn_tab.p && (valid_at + 1) * sizeof(int) <= ctx->dyn_tab.bytes)
-        RT_CUDA(ctx, cudaMemsetAsync(ctx->dyn_tab.as<int>() + valid_at, 0, sizeof(int), ctx->stream));
-    if (tail.empty()) tail.push_back(make_int4(0, 0, 0, 0));
-    if ((rc = upload_vec(ctx, ctx->tail_tab, tail))) return rc;
-    return upload_vec(ctx, ctx->cta_tab, tab);
+    if (ctx->dyn_tab.p) {
+        const DynTab T = dyn_tab(ctx);
+        RT_CUDA(ctx, cudaMemsetAsync(T.memo + ctx->inst.size() + 1, 0, sizeof(int), ctx->stream));
+    }
+    if ((rc = upload_vec(ctx, ctx->act_tab, act))) return rc;
+    return upload_vec(ctx, ctx->bound_tab, bound);
+}
+
+// The collision kernel of a plan and its threads per SM (per CTA in the form that reads
+// populations from global memory, at two CTAs per SM).
+const void *collision_kernel(const rtbte_ctx *ctx) {
+    const bool fp64 = ctx->precision == RTBTE_PREC_FP64;
+    if (!ctx->staged)
+        return fp64 ? (const void *)rhs_kernel<double, false, false, 2, kRhsThreads64>
+                    : (const void *)rhs_kernel<float, false, false, 2, kRhsThreads64>;
+    if (fp64)
+        return ctx->wide ? (const void *)rhs_kernel<double, true, true, 1, kRhsThreads64>
+                         : (const void *)rhs_kernel<double, true, false, 1, kRhsThreads64>;
+    return ctx->wide ? (const void *)rhs_kernel<float, true, true, 1, kRhsThreads>
+                     : (const void *)rhs_kernel<float, true, false, 1, kRhsThreads>;
+}
+int collision_threads(const rtbte_ctx *ctx) {
+    return ctx->staged && ctx->precision != RTBTE_PREC_FP64 ? kRhsThreads : kRhsThreads64;
+}
+
+// Launch parameters of the masks the autotuner has not set.  A prefetch distance of one packet is
+// the fastest or within 2% of it at every FP32 size measured (graphene 36-180, silicon 16-32, 2-64
+// instances: none costs 15-30%, two packets up to 4%); FP64, bound by its arithmetic, is 2% faster
+// without and with w = 96 (graphene 120: 728 against 745 us).  The share split statically: dynamic
+// units even out what the weights do not model, at ~1 us and a staging copy each, which pays in
+// launches above ~250 us (FP32: 0.9 against 1.0, graphene 180 365 / 384 us, silicon 32 421 / 437 us,
+// but graphene 150 202 / 198 us; FP64, bound by its arithmetic, already at 90 us: graphene 63 93 / 99
+// us) and with several instances, whose groups differ most (0.5: 64 instances 990 / 1175 us, 16
+// instances 389 / 440 us; fewer groups than ~100, 0.8: 6 instances 167 / 186 us).
+void default_tuning(rtbte_ctx *ctx) {
+    const bool fp64 = ctx->precision == RTBTE_PREC_FP64;
+    double slots[3] = {0, 0, 0};
+    for (int part = 0; part < 3; ++part)
+        for (int k = ctx->part_first[part]; k < ctx->part_first[part] + ctx->part_items[part]; ++k)
+            slots[part] += ctx->item_cost_h[k].slots;
+    for (unsigned m = 0; m < 8; ++m) {
+        if (ctx->lt_tuned) continue;  // a tuned mask's parameters serve the others
+        LaunchTuning L;
+        if (fp64) {
+            L.w = 96;
+            L.pf = 0;
+        }
+        double tot = 0;
+        for (int part = 0; part < 3; ++part) tot += (m & (1u << part)) ? slots[part] : 0.0;
+        if (ctx->inst.size() > 1) L.sf = tot < 4e6 ? 1.0 : ctx->n_groups >= 100 ? 0.5 : 0.8;
+        else L.sf = tot > (fp64 ? 4e6 : 2e8) ? 0.9 : 1.0;
+        ctx->lt[m] = L;
+    }
+}
+
+// Vectors a lane steps through for an item of `len` entries on 1 << lg lanes (1..4).
+int item_rounds(int len, int lg) { return std::max(1, ((len >> 2) + (1 << lg) - 1) >> lg); }
+
+// Order of the items of groups with several items to a warp: a packet's sub-warps run in step, so
+// a packet costs its longest item and, for ph-ph, one pass per process present in it.  Within
+// windows of kSortWindow items (which keep the entry stream local) the items are ordered by
+// process and by vectors per lane, longest first, so that packets hold alike items.  The partials'
+// slots are already set: sums do not depend on the order.
+constexpr int kSortWindow = 1024;
+void order_packets(std::vector<ItemRec> &items, const std::vector<Group> &groups) {
+    std::vector<ItemRec> tmp(kSortWindow);
+    for (const Group &G : groups) {
+        if (G.lanes_log2 == 5) continue;
+        for (int w0 = G.item_begin; w0 < G.item_end; w0 += kSortWindow) {
+            const int n = std::min(kSortWindow, G.item_end - w0);
+            int at[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
+            auto key = [&](const ItemRec &it) { return 4 * (it.proc != 0) + 4 - item_rounds(it.len, G.lanes_log2); };
+            for (int i = 0; i < n; ++i) ++at[key(items[w0 + i]) + 1];
+            for (int b = 0; b < 8; ++b) at[b + 1] += at[b];
+            for (int i = 0; i < n; ++i) tmp[at[key(items[w0 + i])]++] = items[w0 + i];
+            std::copy(tmp.begin(), tmp.begin() + n, items.begin() + w0);
+        }
+    }
 }
 
 // Build the work items, staging groups, per-row partial slots and per-CTA work ranges.
@@ -866,6 +929,7 @@ int make_plan(rtbte_ctx *ctx) {
         rowoff[ctx->n_y] = (int)next;
         if (next != (long long)items.size()) return fail(ctx, RTBTE_E_UNSUPPORTED, "work items not covered by rows");
     }
+    order_packets(items, groups);
     ctx->n_items = (int)items.size();
     ctx->n_groups = (int)groups.size();
     ctx->wide = std::all_of(groups.begin(), groups.end(), [](const Group &G) { return G.lanes_log2 == 5; });
@@ -892,50 +956,35 @@ int make_plan(rtbte_ctx *ctx) {
     // overlaps the others' streaming
     ctx->staged = max_stage + 64 <= ctx->smem_optin;  // 64 B left for the kernel's static shared memory
     ctx->smem_bytes = ctx->staged ? std::max<size_t>(max_stage, 16) : 0;
-    // Two forms of the FP32 kernel: two register buffers of entries per warp at 16 warps per SM
-    // (128 registers), or one buffer at 24 warps per SM (80 registers), which hides the gather and
-    // arithmetic latency better on the e-ph part.  Both must fit the chosen CTAs per SM.
     int per_sm = 1;
-    const bool fp64 = ctx->precision == RTBTE_PREC_FP64;
+    const void *fn = collision_kernel(ctx);
+    const int nt = collision_threads(ctx);
     if (ctx->staged) {
-        std::vector<std::pair<const void *, int>> kfns;  // (kernel, threads per SM)
-        if (fp64) {
-            kfns.push_back({ctx->wide ? (const void *)rhs_kernel<double, true, false, true, 1, kRhsThreads>
-                                      : (const void *)rhs_kernel<double, true, false, false, 1, kRhsThreads>,
-                            kRhsThreads});
-        } else {
-            kfns.push_back({ctx->wide ? (const void *)rhs_kernel<float, true, true, true, 1, kRhsThreads>
-                                      : (const void *)rhs_kernel<float, true, true, false, 1, kRhsThreads>,
-                            kRhsThreads});
-            kfns.push_back({ctx->wide ? (const void *)rhs_kernel<float, true, false, true, 1, kRhsThreadsDeep>
-                                      : (const void *)rhs_kernel<float, true, false, false, 1, kRhsThreadsDeep>,
-                            kRhsThreadsDeep});
-        }
-        for (auto &kf : kfns) {
-            RT_CUDA(ctx, allow_max_dynamic_smem(kf.first));
-            RT_CUDA(ctx, cudaFuncSetAttribute(kf.first, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
-        }
+        RT_CUDA(ctx, allow_max_dynamic_smem(fn));
+        RT_CUDA(ctx, cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
         for (int k : {4, 2}) {
-            bool fits = true;
-            for (auto &kf : kfns) {
-                int nb = 0;
-                RT_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kf.first, kf.second / k, ctx->smem_bytes));
-                fits = fits && nb >= k;
-            }
-            if (fits) {
+            int nb = 0;
+            RT_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fn, nt / k, ctx->smem_bytes));
+            if (nb >= k) {
                 per_sm = k;
                 break;
             }
         }
     }
     ctx->per_sm = per_sm;
-    for (unsigned m = 0; m < 8; ++m)  // default: the 768-thread form where e-ph work is in the launch
-        if (!(ctx->lt_tuned & (1u << m))) ctx->lt[m].deep = !fp64 && (m & (1u << PART_EPH));
     ctx->grid = ctx->num_sms * (ctx->staged ? per_sm : 2);
-    ctx->item_len_h.resize(items.size());
-    for (size_t k = 0; k < items.size(); ++k) ctx->item_len_h[k] = items[k].len;
+    ctx->item_cost_h.resize(items.size());
+    for (const Group &G : groups)
+        for (int k = G.item_begin; k < G.item_end; ++k)
+            ctx->item_cost_h[k] = {(unsigned short)(item_rounds(items[k].len, G.lanes_log2) << (G.lanes_log2 + 2)),
+                                   (unsigned short)(1 << G.lanes_log2)};
     ctx->group_begin_h.resize(groups.size());
-    for (size_t g = 0; g < groups.size(); ++g) ctx->group_begin_h[g] = groups[g].item_begin;
+    ctx->group_part_h.resize(groups.size());
+    for (size_t g = 0; g < groups.size(); ++g) {
+        ctx->group_begin_h[g] = groups[g].item_begin;
+        ctx->group_part_h[g] = groups[g].part;
+    }
+    default_tuning(ctx);
     int rc;
     if (!ctx->tail_ctr.p) {
         RT_CUDA(ctx, cudaMalloc(&ctx->tail_ctr.p, 16));
@@ -957,10 +1006,8 @@ int make_plan(rtbte_ctx *ctx) {
     ctx->dyn_tab.release();  // reallocated below for this plan's sizes
     if ((rc = split_tables(ctx))) return rc;
     if (ctx->n_groups > 1024) return fail(ctx, RTBTE_E_UNSUPPORTED, "more than 1024 staging groups");
-    // device re-split tables: [grid+1] item bounds, [grid] act indices, [n_groups+1] active groups,
-    // then the memo of the last split: [n_inst] done flags it saw, its parts mask, a valid flag
     ctx->dyn_tab.release();
-    ctx->dyn_tab.bytes = sizeof(int) * (2 * ctx->grid + 1 + ctx->n_groups + 1 + ctx->inst.size() + 2);
+    ctx->dyn_tab.bytes = dyn_tab_bytes(ctx);
     RT_CUDA(ctx, cudaMalloc(&ctx->dyn_tab.p, ctx->dyn_tab.bytes));
     RT_CUDA(ctx, cudaMemsetAsync(ctx->dyn_tab.p, 0, ctx->dyn_tab.bytes, ctx->stream));
     ctx->partials.release();
@@ -994,23 +1041,22 @@ static int launch_core_t(rtbte_ctx *ctx, unsigned parts, const Ctl *ctl, cudaStr
     P.items = ctx->items.as<ItemRec>();
     P.groups = ctx->groups.as<Group>();
     P.n_groups = ctx->n_groups;
-    P.mask = parts;
     P.pf_dist = ctx->lt[parts].pf;
+    P.tail_ctr = ctx->tail_ctr.as<int>();
     if (ctl && ctx->inst.size() > 1) {  // batched integration: balance over the active instances
-        int *dt = ctx->dyn_tab.as<int>();  // [grid+1] item bounds, [grid] act indices, [n_groups+1] act, memo
+        const DynTab T = dyn_tab(ctx);
         split_kernel<<<1, 256, 0, s>>>(ctx->groups.as<Group>(), ctx->n_groups, ctx->gwt.as<long long>(), ctl, parts,
-                                       ctx->grid, dt, dt + ctx->grid + 1, dt + 2 * ctx->grid + 1,
-                                       dt + 2 * ctx->grid + 1 + ctx->n_groups + 1, (int)ctx->inst.size());
+                                       ctx->grid, kResplitTail, kResplitTailMin, T.bound, T.act, T.n_tail, T.memo,
+                                       (int)ctx->inst.size());
         RT_CUDA(ctx, cudaGetLastError());
         ctx->launches++;
-        P.cta_items = dt;
-        P.cta_act = dt + ctx->grid + 1;
-        P.act = dt + 2 * ctx->grid + 1;
+        P.bound = T.bound;
+        P.act = T.act;
+        P.n_tail_d = T.n_tail;
     } else {
-        P.cta_items = ctx->cta_tab.as<int>() + (long long)(parts - 1) * (ctx->grid + 1);
-        P.tail = ctx->tail_tab.as<int4>() + ctx->tail_off[parts - 1];
-        P.n_tail = ctx->tail_off[parts] - ctx->tail_off[parts - 1];
-        P.tail_ctr = ctx->tail_ctr.as<int>();
+        P.bound = ctx->bound_tab.as<int4>() + ctx->bound_off[parts];
+        P.act = ctx->act_tab.as<int>() + ctx->act_off[parts];
+        P.n_tail = ctx->tail_n[parts];
     }
     P.partials = ctx->partials.p;
     P.popf = ctx->popf.p;
@@ -1034,29 +1080,10 @@ static int launch_core_t(rtbte_ctx *ctx, unsigned parts, const Ctl *ctl, cudaStr
             RT_CUDA(ctx, cudaEventRecord(e0, s));
         }
     }
-    if (!ctx->staged) {
-        rhs_kernel<R, false, false, false, 2, kRhsThreads><<<ctx->grid, kRhsThreads, 0, s>>>(P);
-    } else if constexpr (sizeof(R) == 4) {
-        if (ctx->lt[parts].deep) {
-            const int nt = kRhsThreadsDeep / ctx->per_sm;
-            if (ctx->wide)
-                rhs_kernel<R, true, false, true, 1, kRhsThreadsDeep><<<ctx->grid, nt, ctx->smem_bytes, s>>>(P);
-            else
-                rhs_kernel<R, true, false, false, 1, kRhsThreadsDeep><<<ctx->grid, nt, ctx->smem_bytes, s>>>(P);
-        } else {
-            const int nt = kRhsThreads / ctx->per_sm;
-            if (ctx->wide)
-                rhs_kernel<R, true, true, true, 1, kRhsThreads><<<ctx->grid, nt, ctx->smem_bytes, s>>>(P);
-            else
-                rhs_kernel<R, true, true, false, 1, kRhsThreads><<<ctx->grid, nt, ctx->smem_bytes, s>>>(P);
-        }
-    } else {
-        const int nt = kRhsThreads / ctx->per_sm;
-        if (ctx->wide)
-            rhs_kernel<R, true, false, true, 1, kRhsThreads><<<ctx->grid, nt, ctx->smem_bytes, s>>>(P);
-        else
-            rhs_kernel<R, true, false, false, 1, kRhsThreads><<<ctx->grid, nt, ctx->smem_bytes, s>>>(P);
-    }
+    void *args[] = {&P};
+    RT_CUDA(ctx, cudaLaunchKernel(collision_kernel(ctx), dim3(ctx->grid),
+                                  dim3(collision_threads(ctx) / (ctx->staged ? ctx->per_sm : 1)), args,
+                                  ctx->staged ? ctx->smem_bytes : 0, s));
     RT_CUDA(ctx, cudaGetLastError());
     ctx->launches++;
     if (e0) {
@@ -1087,11 +1114,11 @@ int time_launches(rtbte_ctx *ctx, unsigned parts, cudaEvent_t e0, cudaEvent_t e1
     return RTBTE_OK;
 }
 
-// Tuning of mask `parts`'s work split for its current kernel form: per-item weight, per-part
+// Tuning of mask `parts`'s work split: packet weight, per-part
 // entry costs, L2 prefetch distance and static share, each timed over 3 launches and the
 // fastest kept.
 int tune_split(rtbte_ctx *ctx, unsigned parts, cudaEvent_t e0, cudaEvent_t e1) {
-    static const int cand[] = {32, 96, 192, 320, 512, 800, 1280, 2048};
+    static const int cand[] = {32, 96, 192, 320, 512, 1024};
     LaunchTuning &L = ctx->lt[parts];
     int best = L.w, rc = RTBTE_OK;
     float best_ms = 1e30f;
@@ -1114,7 +1141,7 @@ int tune_split(rtbte_ctx *ctx, unsigned parts, cudaEvent_t e0, cudaEvent_t e1) {
     for (int part = 0; part < 3; ++part) {
         if (!(parts & (1u << part)) || ctx->part_items[part] == 0 || (parts == (1u << part))) continue;
         for (int k = ctx->part_first[part]; k < ctx->part_first[part] + ctx->part_items[part]; ++k)
-            wsum[part] += ctx->item_len_h[k] + best;
+            wsum[part] += ctx->item_cost_h[k].slots + best * ctx->item_cost_h[k].lanes / 32.0;
         const unsigned pm = 1u << part;
         const LaunchTuning keep = ctx->lt[pm];
         ctx->lt[pm] = L;
@@ -1146,7 +1173,7 @@ int tune_split(rtbte_ctx *ctx, unsigned parts, cudaEvent_t e0, cudaEvent_t e1) {
     }
     // L2 prefetch distance, then the share of the work split statically (the rest is taken
     // dynamically by CTAs that finish early)
-    static const int dists[] = {0, 2, 3, 4, 6, 8};
+    static const int dists[] = {0, 1, 2, 3, 4};
     int best_d = L.pf;
     float best_d_ms = 1e30f;
     for (int d : dists) {
@@ -1159,7 +1186,7 @@ int tune_split(rtbte_ctx *ctx, unsigned parts, cudaEvent_t e0, cudaEvent_t e1) {
         }
     }
     L.pf = best_d;
-    static const double fracs[] = {1.0, 0.9, 0.8, 0.7, 0.6};
+    static const double fracs[] = {1.0, 0.9, 0.8, 0.6, 0.4};
     double best_f = 1.0;
     float best_f_ms = 1e30f;
     for (double f : fracs) {
@@ -1177,38 +1204,19 @@ int tune_split(rtbte_ctx *ctx, unsigned parts, cudaEvent_t e0, cudaEvent_t e1) {
 
 }  // namespace
 
-// Autotuner of the collision launch of one parts mask.  FP32 has two kernel forms (two entry
-// buffers per warp at 16 warps per SM, or one buffer at 24): the work split is tuned for each
-// form from the same starting point, the two tuned launches are timed over 10 launches each
-// (they often differ by ~2%, less than the spread of 3-launch timings) and the faster is kept.
-// The result belongs to this mask; masks never tuned themselves take its work split (not its
-// form) as their own.
+// Autotuner of the collision launch of one parts mask.  The result belongs to this mask; masks
+// never tuned themselves take it as their own.
 int autotune(rtbte_ctx *ctx, unsigned parts, int *chosen) {
     cudaEvent_t e0, e1;
     RT_CUDA(ctx, cudaEventCreate(&e0));
     RT_CUDA(ctx, cudaEventCreate(&e1));
-    const bool two_forms = ctx->staged && ctx->precision != RTBTE_PREC_FP64;
     const LaunchTuning start = ctx->lt[parts];
-    LaunchTuning res[2] = {start, start};
-    float ms10[2] = {0.f, 0.f};
-    int rc = RTBTE_OK, nf = two_forms ? 2 : 1;
-    for (int f = 0; f < nf && !rc; ++f) {
-        ctx->lt[parts] = start;
-        if (two_forms) ctx->lt[parts].deep = f == 1;
-        if ((rc = tune_split(ctx, parts, e0, e1))) break;
-        if (two_forms && (rc = time_launches(ctx, parts, e0, e1, 10, &ms10[f]))) break;
-        res[f] = ctx->lt[parts];
-    }
-    const int pick = (!rc && two_forms && ms10[1] < ms10[0]) ? 1 : 0;
-    ctx->lt[parts] = rc ? start : res[pick];
+    const int rc = tune_split(ctx, parts, e0, e1);
+    if (rc) ctx->lt[parts] = start;
     if (!rc) {
         ctx->lt_tuned |= 1u << parts;
-        for (unsigned m = 1; m <= 7; ++m) {
-            if (m == parts || (ctx->lt_tuned & (1u << m))) continue;
-            const bool deep = ctx->lt[m].deep;
-            ctx->lt[m] = ctx->lt[parts];
-            ctx->lt[m].deep = deep;
-        }
+        for (unsigned m = 1; m <= 7; ++m)
+            if (!(ctx->lt_tuned & (1u << m))) ctx->lt[m] = ctx->lt[parts];
     }
     const int rc2 = split_tables(ctx);
     cudaEventDestroy(e0);
