@@ -48,14 +48,6 @@ template <class R> __device__ __forceinline__ void two_sum(R &s, R &c, R x) {
     c += e;
 }
 
-// A lane's sum of its (at most 4) vector sums within an item: compensated in FP32; a plain
-// addition in FP64, whose rounding over 4 terms is far below the FP64 study's needs and whose
-// arithmetic this GPU runs at a low rate (the compensated form cost FP64 mode ~20% of its time).
-template <class R> __device__ __forceinline__ void lane_add(R &s, R &c, R x) {
-    if constexpr (sizeof(R) == 8) s += x;
-    else two_sum(s, c, x);
-}
-
 struct KParams {
     const ItemRec *items;
     const Group *groups;
@@ -147,8 +139,11 @@ __device__ __forceinline__ unsigned comp4(const uint4 &e, int k) {
     return k == 0 ? e.x : k == 1 ? e.y : k == 2 ? e.z : e.w;
 }
 
-// Per-lane sum of W*F over one item: each 4-entry vector is summed with an FMA chain and the
-// vector sums are added into (acc, cmp) by lane_add; the warp reduction follows in finish_item.
+// Per-lane sum of W*F over one item.  FP32: each 4-entry vector is summed with an FMA chain and the
+// vector sums are added into (acc, cmp) with two-sum; FP64: one FMA chain.  The warp reduction
+// follows in finish_item.  The FP64 pipe (2 lanes per clock per SM) bounds FP64 launches -- 86%
+// busy at graphene 120 -- so there the factors take the forms with the fewest operations (4 per
+// entry with the weight) and no additions beyond the chain (728 -> 615 us).
 // FULL: every lane holds VPL vectors (a whole-warp item of the maximum length), so the vectors
 // carry no bounds tests.
 template <class R, int VPL, bool FULL, class F>
@@ -158,11 +153,11 @@ __device__ __forceinline__ void lane_sum(const Batch<R, VPL> &b, int nv, int sl,
 #pragma unroll
     for (int j = 0; j < VPL; ++j) {
         if (!FULL && sl + (j << lg) >= nv) break;
-        R t = R(0);
+        R t = sizeof(R) == 8 ? acc : R(0);
 #pragma unroll
         for (int k = 0; k < 4; ++k) t = fma(b.w(j, k), factor(comp4(b.iv[j], k)), t);
-        if (j == 0) acc = t;
-        else lane_add(acc, cmp, t);
+        if (sizeof(R) == 8 || j == 0) acc = t;
+        else two_sum(acc, cmp, t);
     }
 }
 
@@ -187,7 +182,8 @@ __device__ __forceinline__ void compute_item(const GroupView<R> &V, const Item &
         const R Np = b.Np;
         lane_sum<R, VPL, FULL>(b, nv, sl, lg, acc, cmp, [&](unsigned e) {
             const R fd = V.s0[e & smask], fs = V.s0[e >> V.sb];
-            return fma(Np, fd - fs, -fs * (R(1) - fd));
+            if constexpr (sizeof(R) == 8) return fma(Np, fd - fs, fma(fs, fd, -fs));
+            else return fma(Np, fd - fs, -fs * (R(1) - fd));
         });
     } else {
         const unsigned pmask = (1u << V.pb) - 1u;
@@ -200,7 +196,8 @@ __device__ __forceinline__ void compute_item(const GroupView<R> &V, const Item &
         } else {  // G_abs = N(N''-N') - N'(N''+1)
             lane_sum<R, VPL, FULL>(b, nv, sl, lg, acc, cmp, [&](unsigned e) {
                 const R Nb = V.s0[e & pmask], Nc = V.s0[e >> V.pb];
-                return fma(Na, Nc - Nb, -Nb * (Nc + R(1)));
+                if constexpr (sizeof(R) == 8) return fma(Na, Nc - Nb, fma(-Nb, Nc, -Nb));
+                else return fma(Na, Nc - Nb, -Nb * (Nc + R(1)));
             });
         }
     }
@@ -229,20 +226,60 @@ template <class R> __device__ __forceinline__ void prefetch_item(const GroupView
     }
 }
 
-// Item sum: the lane's compensated sum (acc + cmp) is rounded once, then added over the
-// sub-warp by a butterfly in a fixed order (every lane ends with the same bits).  The RHS error
-// is set by the conversion of the populations to FP32 (about 5e-8 relative on the parity
-// models), not by this tree: the compensated tree measured the same to two digits.
-template <class R>
-__device__ __forceinline__ void finish_item(const KParams &P, unsigned slot, bool valid, R acc, R cmp, int sl, int lg) {
-    acc += cmp;
+// Item sum in FP32: the lane's compensated sum, rounded once, added over the sub-warp by a
+// butterfly in a fixed order (every lane ends with the same bits).  The RHS error is set by the
+// conversion of the populations to FP32 (about 5e-8 relative on the parity models), not by this
+// tree: the compensated tree measured the same to two digits.
+__device__ __forceinline__ void finish_item(const KParams &P, unsigned slot, bool valid, float acc, int sl, int lg) {
 #pragma unroll
     for (int o = 16; o; o >>= 1)
         if (o < (1 << lg)) acc += __shfl_xor_sync(kFull, acc, o);
-    if (sl == 0 && valid) {
-        reinterpret_cast<R *>(P.partials)[slot] = acc;
-    }
+    if (sl == 0 && valid) reinterpret_cast<float *>(P.partials)[slot] = acc;
 }
+
+// Item sums in FP64, four packets at a time.  The butterfly of one packet costs lg additions on
+// the FP64 pipe, which bounds these launches; four packets share them: at the first level (lanes
+// L/2 apart, L the lanes per item) two packets' sums go to the two halves of the sub-warp, at the
+// second two such pairs to its quarters, and the rest runs once, 6 additions for 4 packets of 32
+// lanes instead of 20 (graphene 120: 615 -> 575 us).  Every item's terms meet in the order of the
+// single butterfly, so the sums are the same.
+struct ItemSum4 {
+    double held0, held1;
+    unsigned slot;  // where this lane writes its quarter's sum (kNoSlot: nowhere)
+    int n;          // packets held
+    static constexpr unsigned kNoSlot = 0xffffffffu;
+    __device__ __forceinline__ ItemSum4() : held0(0), held1(0), slot(kNoSlot), n(0) {}
+    static __device__ __forceinline__ double merge(double first, double second, int half, int sl) {
+        const bool up = sl & half;
+        const double mine = up ? second : first, other = up ? first : second;
+        return mine + __shfl_xor_sync(kFull, other, half);
+    }
+    // every lane of the warp; n advances alike in all
+    __device__ __forceinline__ void add(const KParams &P, unsigned s, bool valid, double acc, int sl, int lg) {
+        const int L2 = 1 << (lg - 1), L4 = L2 >> 1;
+        if ((sl & (L4 - 1)) == 0 && ((sl & L2) ? 1 : 0) + ((sl & L4) ? 2 : 0) == n) slot = valid ? s : kNoSlot;
+        ++n;
+        if (n & 1) {
+            held0 = acc;
+            return;
+        }
+        const double m = merge(held0, acc, L2, sl);
+        if (n == 2) {
+            held1 = m;
+            return;
+        }
+        double r = merge(held1, m, L4, sl);
+#pragma unroll
+        for (int o = 4; o; o >>= 1)
+            if (o < L4) r += __shfl_xor_sync(kFull, r, o);
+        if (slot != kNoSlot) reinterpret_cast<double *>(P.partials)[slot] = r;
+        slot = kNoSlot;
+        n = 0;
+    }
+    __device__ __forceinline__ void flush(const KParams &P, int sl, int lg) {  // the packets still held
+        while (n) add(P, 0, false, 0.0, sl, lg);
+    }
+};
 
 // A warp's share of items [a, b) of one group.  The warp works on G = 32 >> lg consecutive items
 // at a time, one per sub-warp of 1 << lg lanes (the group's items are cut to at most 16 << lg
@@ -275,6 +312,7 @@ __device__ __forceinline__ void run_range(const KParams &P, const GroupView<R> &
         for (int j = 1; j < pf; ++j) prefetch_item(V, fetch((unsigned)k + j * step));
         dp = fetch((unsigned)k + pf * step);
     }
+    ItemSum4 sums;  // (FP64)
     for (; kb < b; kb += step, k += step) {
         const Item it = item_from(d);
         d = dn;
@@ -288,8 +326,10 @@ __device__ __forceinline__ void run_range(const KParams &P, const GroupView<R> &
         R acc, cmp;
         if (WIDE && it.len == kItemEntries) compute_item<R, 4, true>(V, it, B, sl, lg, acc, cmp);
         else compute_item<R, 4, false>(V, it, B, sl, lg, acc, cmp);
-        finish_item<R>(P, it.slot, k < b, acc, cmp, sl, lg);
+        if constexpr (sizeof(R) == 8) sums.add(P, it.slot, k < b, acc, sl, lg);
+        else finish_item(P, it.slot, k < b, acc + cmp, sl, lg);
     }
+    if constexpr (sizeof(R) == 8) sums.flush(P, sl, lg);
 }
 
 // Point V at group g's populations, staging them in shared memory unless this CTA already
@@ -677,11 +717,12 @@ int split_tables(rtbte_ctx *ctx) {
 }
 
 // The collision kernel of a plan and its threads per SM (per CTA in the form that reads
-// populations from global memory, at two CTAs per SM).
+// populations from global memory: two CTAs per SM in FP32; one in FP64, where two at 64 registers
+// spill -- silicon at 80^3 / 40^3, 2.1e9 entries: 16.1 ms with two, 15.4 with one).
 const void *collision_kernel(const rtbte_ctx *ctx) {
     const bool fp64 = ctx->precision == RTBTE_PREC_FP64;
     if (!ctx->staged)
-        return fp64 ? (const void *)rhs_kernel<double, false, false, 2, kRhsThreads64>
+        return fp64 ? (const void *)rhs_kernel<double, false, false, 1, kRhsThreads64>
                     : (const void *)rhs_kernel<float, false, false, 2, kRhsThreads64>;
     if (fp64)
         return ctx->wide ? (const void *)rhs_kernel<double, true, true, 1, kRhsThreads64>
@@ -957,6 +998,7 @@ int make_plan(rtbte_ctx *ctx) {
     ctx->staged = max_stage + 64 <= ctx->smem_optin;  // 64 B left for the kernel's static shared memory
     ctx->smem_bytes = ctx->staged ? std::max<size_t>(max_stage, 16) : 0;
     int per_sm = 1;
+    const bool fp64 = ctx->precision == RTBTE_PREC_FP64;
     const void *fn = collision_kernel(ctx);
     const int nt = collision_threads(ctx);
     if (ctx->staged) {
@@ -972,7 +1014,7 @@ int make_plan(rtbte_ctx *ctx) {
         }
     }
     ctx->per_sm = per_sm;
-    ctx->grid = ctx->num_sms * (ctx->staged ? per_sm : 2);
+    ctx->grid = ctx->num_sms * (ctx->staged ? per_sm : fp64 ? 1 : 2);
     ctx->item_cost_h.resize(items.size());
     for (const Group &G : groups)
         for (int k = G.item_begin; k < G.item_end; ++k)
