@@ -1274,24 +1274,110 @@ int autotune(rtbte_ctx *ctx, unsigned parts, int *chosen) {
 // (Eq. ph-ph with G_em, G_abs differentiated in the destination population; W as stored,
 // pair and absorption factors included), from the compute-precision sub-lattice copy popP,
 // summed in FP64 per lane then a fixed butterfly; written to rates[y_off + n_c + full(a)].
-template <class R>
-__global__ void pp_rates_kernel(const uint32_t *idx, const R *W, const long long *off, const R *P, const int *pp_full,
-                                int pp_bits, long long M, long long row0, double *rates) {
+// The FP64 pipe bounds it (2 or 3 operations per entry: 0.35 ms for graphene 180's 8.8e7 entries;
+// the list streams in 0.16 ms).  STAGED: one CTA per SM holds the populations in shared memory;
+// lanes read four entries with a 16-byte load, four such vectors in flight, and the next
+// destination's entries are prefetched into L2 (graphene 180, FP64 lists: 1043 us with one entry
+// per lane and load and gathers from global memory, 489 us so).
+constexpr int kRateThreads = 512;
+template <class R, bool STAGED>
+__global__ void __launch_bounds__(kRateThreads) pp_rates_kernel(const uint32_t *idx, const R *W, const long long *off,
+                                                                const R *popP, int n_stage, const int *pp_full,
+                                                                int pp_bits, int M, long long row0, double *rates) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const R *P = popP;
+    if (STAGED) {
+        R *sm = reinterpret_cast<R *>(smem_raw);
+        stage_copy<R>(sm, popP, n_stage);
+        asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;\n" ::: "memory");
+        __syncthreads();
+        P = sm;
+    }
     const int lane = threadIdx.x & 31;
     const unsigned pmask = (1u << pp_bits) - 1u;
-    const long long nw = ((long long)gridDim.x * blockDim.x) >> 5;
-    for (long long a = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5; a < M; a += nw) {
-        double acc = 0.0;
-        for (int proc = 0; proc < 2; ++proc)
-            for (long long e = off[2 * a + proc] + lane; e < off[2 * a + proc + 1]; e += 32) {
-                const uint32_t x = idx[e];
-                const double Nb = (double)P[x & pmask], Nc = (double)P[x >> pp_bits];
-                acc += (double)W[e] * (proc == 0 ? Nb + Nc + 1.0 : Nc - Nb);
+    // destinations dealt over the CTAs first: neighbouring segments have alike lengths
+    const int step = gridDim.x * (kRateThreads >> 5);
+    for (int a = (threadIdx.x >> 5) * gridDim.x + blockIdx.x; a < M; a += step) {
+        const long long o0 = off[2 * a], o1 = off[2 * a + 1], o2 = off[2 * a + 2];
+        if (a < M - step && lane == 0) {
+            const long long p0 = off[2 * (a + step)], p1 = off[2 * (a + step) + 2];
+            if (p1 > p0) {
+                asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;\n" ::"l"(idx + p0),
+                             "r"((unsigned)((p1 - p0) * 4)) : "memory");
+                asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;\n" ::"l"(W + p0),
+                             "r"((unsigned)((p1 - p0) * sizeof(R))) : "memory");
             }
+        }
+        double acc = 0.0;
+        // sum of W (N' + N'' + 1), or W (N'' - N'), over a segment: FP64 lists in FP64; FP32 lists
+        // as exact sums and products in FP32 head/tail pairs (two-sum, FMA residual), widened once
+        // per 16 entries -- converting every value cost more than the arithmetic (graphene 180, FP32
+        // lists: 1579 us before, 1046 with conversions, 237 so)
+        auto segment = [&](long long b, long long e, auto emission) {
+            constexpr bool EM = decltype(emission)::value;
+            const int nv = (int)((e - b) >> 2);  // segments are padded to whole vectors
+            GroupView<R> V;
+            V.idx = idx;
+            V.W = W;
+            V.part = PART_PP;
+            Item it;
+            it.len = 0;
+            for (int v0 = 0; v0 < nv; v0 += 128) {
+                it.begin = b + 4LL * v0;
+                it.len = (unsigned short)(4 * min(nv - v0, 128));
+                Batch<R, 4> B;
+                B.issue(V, it, lane, 5);
+                [[maybe_unused]] R hi = R(0), lo = R(0);
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    if (lane + 32 * j >= (it.len >> 2)) break;
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        const unsigned x = comp4(B.iv[j], k);
+                        const R w = B.w(j, k), Nb = P[x & pmask], Nc = P[x >> pp_bits];
+                        if constexpr (sizeof(R) == 8) {
+                            acc = fma(w, EM ? Nb + Nc + 1.0 : Nc - Nb, acc);
+                        } else {
+                            R t = Nc, c = R(0);
+                            two_sum(t, c, EM ? Nb : -Nb);
+                            if (EM) two_sum(t, c, R(1));
+                            const R p = w * t;
+                            two_sum(hi, lo, p);
+                            lo += fma(w, c, fma(w, t, -p));
+                        }
+                    }
+                }
+                // (an infinite sum has no tail: its two-sum residual is not a number)
+                if constexpr (sizeof(R) == 4) acc += (double)hi + (isfinite(hi) ? (double)lo : 0.0);
+            }
+        };
+        segment(o0, o1, std::true_type{});
+        segment(o1, o2, std::false_type{});
 #pragma unroll
         for (int m = 16; m; m >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, m);
         if (lane == 0) rates[row0 + pp_full[a]] = acc;
     }
+}
+
+template <class R> static int launch_pp_rates_t(rtbte_ctx *ctx, InstHost &I, double *rates, cudaStream_t s) {
+    const size_t bytes = sizeof(R) * (size_t)I.M_pad;
+    const bool staged = bytes + 64 <= ctx->smem_optin;
+    const uint32_t *idx = I.pp_idx.as<uint32_t>();
+    const R *P = reinterpret_cast<const R *>(ctx->popP.p) + I.P_off;
+    const int grid = (int)std::min<long long>((I.M + 7) / 8, (long long)ctx->num_sms);
+    if (staged) {
+        RT_CUDA(ctx, allow_max_dynamic_smem((const void *)pp_rates_kernel<R, true>));
+        pp_rates_kernel<R, true><<<grid, kRateThreads, bytes, s>>>(idx, I.pp_W.as<R>(), I.pp_off_dev.as<long long>(), P,
+                                                                   I.M_pad, I.t_ppfull.as<int>(), I.pp_bits, (int)I.M,
+                                                                   I.y_off + I.d.n_c, rates);
+    } else {
+        pp_rates_kernel<R, false><<<grid, kRateThreads, 0, s>>>(idx, I.pp_W.as<R>(), I.pp_off_dev.as<long long>(), P, 0,
+                                                                I.t_ppfull.as<int>(), I.pp_bits, (int)I.M,
+                                                                I.y_off + I.d.n_c, rates);
+    }
+    RT_CUDA(ctx, cudaGetLastError());
+    ctx->launches++;
+    return RTBTE_OK;
 }
 
 int launch_pp_rates(rtbte_ctx *ctx, int inst, double *rates, cudaStream_t s) {
@@ -1302,19 +1388,8 @@ int launch_pp_rates(rtbte_ctx *ctx, int inst, double *rates, cudaStream_t s) {
         I.pp_off_dev.bytes = sizeof(long long) * I.pp_off.size();
         RT_CUDA(ctx, cudaMemcpyAsync(I.pp_off_dev.p, I.pp_off.data(), I.pp_off_dev.bytes, cudaMemcpyHostToDevice, s));
     }
-    const int blocks = (int)std::min<long long>((I.M + 7) / 8, 8LL * ctx->num_sms);
-    if (ctx->precision == RTBTE_PREC_FP64)
-        pp_rates_kernel<double><<<blocks, 256, 0, s>>>(I.pp_idx.as<uint32_t>(), I.pp_W.as<double>(),
-                                                       I.pp_off_dev.as<long long>(),
-                                                       ctx->popP.as<double>() + I.P_off, I.t_ppfull.as<int>(),
-                                                       I.pp_bits, I.M, I.y_off + I.d.n_c, rates);
-    else
-        pp_rates_kernel<float><<<blocks, 256, 0, s>>>(I.pp_idx.as<uint32_t>(), I.pp_W.as<float>(),
-                                                      I.pp_off_dev.as<long long>(), ctx->popP.as<float>() + I.P_off,
-                                                      I.t_ppfull.as<int>(), I.pp_bits, I.M, I.y_off + I.d.n_c, rates);
-    RT_CUDA(ctx, cudaGetLastError());
-    ctx->launches++;
-    return RTBTE_OK;
+    return ctx->precision == RTBTE_PREC_FP64 ? launch_pp_rates_t<double>(ctx, I, rates, s)
+                                             : launch_pp_rates_t<float>(ctx, I, rates, s);
 }
 
 int launch_rows(rtbte_ctx *ctx, unsigned parts, double *out, const double *forcing, cudaStream_t s) {
