@@ -37,11 +37,12 @@ constexpr int kLayers = 4;
 
 // C[M x N] (+)= op(A)[M x K] * op(B)[K x N]; A(m,k) = TA ? A[k*lda+m] : A[m*lda+k],
 // B(k,n) = TB ? B[n*ldb+k] : B[k*ldb+n].  Split-K: blockIdx.z takes K range z, writing to
-// C + z*M*ldc.  Epilogue (split 1 only): + bias[n], tanh if act, BF16 copy if Cb.
+// C + z*M*ldc.  Epilogue (split 1 only): + bias[n], tanh if act, times 1 - back^2 (the gradient
+// through tanh), BF16 copy if Cb.
 template <bool TA, bool TB>
 __global__ void __launch_bounds__(kGemmThreads) gemm_bf16(const bf16 *A, int lda, const bf16 *B, int ldb, float *C,
                                                           int ldc, int M, int N, int K, int kchunk, const float *bias,
-                                                          int act, bf16 *Cb) {
+                                                          int act, bf16 *Cb, const float *back) {
     __shared__ __align__(16) bf16 As[kBM][kBK + 8];
     __shared__ __align__(16) bf16 Bt[kBN][kBK + 8];  // transposed: n-major, k contiguous
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -113,6 +114,10 @@ __global__ void __launch_bounds__(kGemmThreads) gemm_bf16(const bf16 *A, int lda
                 float v = acc[mi][ni][r];
                 if (bias) v += bias[col];
                 if (act) v = tanhf(v);
+                if (back) {
+                    const float h = back[(long long)row * ldc + col];
+                    v = v * (1.f - h * h);
+                }
                 Cz[(long long)row * ldc + col] = v;
                 if (Cb) Cb[(long long)row * ldc + col] = __float2bfloat16(v);
             }
@@ -127,23 +132,42 @@ __global__ void sum_splits(const float *part, int splits, long long n, float *ou
     }
 }
 
-// im2col with periodic padding: col[p][tap*C + c] = act[b, (y+dy)%ny, (x+dx)%nx, c], zero pad to kpad.
+// im2col with periodic padding: col[p][tap*C + c] = act[b, (y+dy)%ny, (x+dx)%nx, c], zero pad to
+// kpad (a multiple of 8).  A thread writes 8 columns with one 16-byte store -- one 16-byte load too
+// where C is a multiple of 8 and the 8 columns share a tap (64 channels, batch 8 of 60 x 60: 98 us
+// with one element per thread; bound by the 33 MB it writes).
 __global__ void im2col(const bf16 *act, int C, int ny, int nx, long long P, bf16 *col, int kpad) {
-    const long long total = P * kpad;
+    const int nv = kpad >> 3;
+    const long long total = P * nv;
     const long long per = (long long)ny * nx;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x) {
-        const long long p = i / kpad;
-        const int k = (int)(i - p * kpad);
-        bf16 v = __float2bfloat16(0.f);
-        if (k < 9 * C) {
-            const int tap = k / C, c = k - tap * C;
-            const int dy = tap / 3 - 1, dx = tap % 3 - 1;
-            const long long b = p / per;
-            const int yx = (int)(p - b * per), y = yx / nx, x = yx - y * nx;
-            const int ys = (y + dy + ny) % ny, xs = (x + dx + nx) % nx;
-            v = act[(b * per + (long long)ys * nx + xs) * C + c];
+        const long long p = i / nv;
+        const int k0 = (int)(i - p * nv) << 3;
+        const long long b = p / per;
+        const int yx = (int)(p - b * per), y = yx / nx, x = yx - y * nx;
+        auto at = [&](int tap) {
+            const int ys = (y + tap / 3 - 1 + ny) % ny, xs = (x + tap % 3 - 1 + nx) % nx;
+            return act + (b * per + (long long)ys * nx + xs) * C;
+        };
+        uint4 u = make_uint4(0u, 0u, 0u, 0u);
+        if ((C & 7) == 0) {
+            if (k0 < 9 * C) {
+                const int tap = k0 / C;
+                u = *reinterpret_cast<const uint4 *>(at(tap) + (k0 - tap * C));
+            }
+        } else {
+            unsigned short h[8];
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                const int k = k0 + j, tap = k / C;
+                h[j] = k < 9 * C ? __bfloat16_as_ushort(at(tap)[k - tap * C]) : (unsigned short)0;
+            }
+            u.x = h[0] | (unsigned)h[1] << 16;
+            u.y = h[2] | (unsigned)h[3] << 16;
+            u.z = h[4] | (unsigned)h[5] << 16;
+            u.w = h[6] | (unsigned)h[7] << 16;
         }
-        col[i] = v;
+        *reinterpret_cast<uint4 *>(col + p * kpad + k0) = u;
     }
 }
 
@@ -190,13 +214,141 @@ __global__ void col_sums(const float *G, long long M, int N, float *out) {
     if (threadIdx.x == 0) out[col] = red[0];
 }
 
-// mean-square loss: g = 2 (out - t)/n, per-block partial losses
-__global__ void mse(const float *out, const float *t, long long n, float *g, float *part) {
+// Gradients of the weights and biases that the other kernels left as partial sums.
+//   weights: the split-K partials of every matrix, summed in split order;
+//   biases: column sums of the layers' gz [P][64] and of g_out [P][C] -- 256 interleaved row chains
+//   per column (bias_chains), then a halving tree over them (finish_grads).
+// One launch of each per step instead of a sum per matrix and a strided column pass per layer
+// (16 us each): the chains' loads are coalesced across columns and all layers run at once.
+struct GradSums {
+    const float *part[6];
+    float *out[6];
+    int splits[6], n[6];  // matrix elements
+    const float *G[6];    // bias column sources [P][cols]
+    int cols[6];
+    float *bias[6];
+    float *chains;        // [6][256][64]
+    long long P;
+};
+
+__global__ void __launch_bounds__(256) bias_chains(GradSums a) {
+    const int l = blockIdx.y, col = threadIdx.x & 63, t = blockIdx.x * 4 + (threadIdx.x >> 6);
+    const int N = a.cols[l];
+    if (col >= N) return;
+    const float *G = a.G[l] + col;
+    float s = 0.f;
+#pragma unroll 16
+    for (long long r = t; r < a.P; r += 256) s += G[r * N];
+    a.chains[(l * 256 + t) * 64 + col] = s;
+}
+
+__global__ void __launch_bounds__(256) finish_grads(GradSums a, int nbias) {
+    if ((int)blockIdx.x < nbias) {  // one bias column
+        __shared__ float red[256];
+        int l = 0, col = blockIdx.x;
+        while (col >= a.cols[l]) col -= a.cols[l++];
+        red[threadIdx.x] = a.chains[(l * 256 + threadIdx.x) * 64 + col];
+        __syncthreads();
+        for (int o = 128; o > 0; o >>= 1) {
+            if (threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
+            __syncthreads();
+        }
+        if (threadIdx.x == 0) a.bias[l][col] = red[0];
+        return;
+    }
+    int i = ((int)blockIdx.x - nbias) * 256 + threadIdx.x;
+    for (int l = 0; l < 6; ++l) {
+        if (i < a.n[l]) {
+            float s = 0.f;
+#pragma unroll 16
+            for (int z = 0; z < a.splits[l]; ++z) s += a.part[l][(long long)z * a.n[l] + i];
+            a.out[l][i] = s;
+            return;
+        }
+        i -= a.n[l];
+    }
+}
+
+// Split-K partials of the output layer's weight gradient, part[z][64][C] = A^T B over the split's
+// points, A [P][64], B [P][C] BF16, C <= 16, with the mma.sync steps (16 points each, in order) of
+// gemm_bf16; the points pass through shared memory in blocks of kHeadRows, 16 bytes a copy, the
+// next block in flight during the current one's steps (a 64 x 64 tile loaded element by element per
+// 32 points: 91 us at batch 8 of 60 x 60).
+constexpr int kHeadRows = 256, kHeadLdA = 72, kHeadLdB = kHeadRows + 8;
+constexpr size_t kHeadSmem = 2 * sizeof(bf16) * (kHeadRows * kHeadLdA + 16 * kHeadLdB);
+__global__ void __launch_bounds__(128) head_grad(const bf16 *A, const bf16 *B, int C, int P, int kchunk, float *part) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    bf16 *As = reinterpret_cast<bf16 *>(smem), *Bt = As + 2 * kHeadRows * kHeadLdA;
+    const int tid = threadIdx.x, lane = tid & 31, g = lane >> 2, t4 = lane & 3;
+    const int m = (tid >> 5) * 16 + g;
+    const int kb = blockIdx.x * kchunk, ke = min(P, kb + kchunk);
+    const int nblk = (ke - kb + kHeadRows - 1) / kHeadRows, nt = (C + 7) / 8;
+    auto load = [&](int i) {  // rows [kb + i * kHeadRows, ..) of A and, transposed, of B; zeros past ke
+        const int k0 = kb + i * kHeadRows;
+        bf16 *Ad = As + (i & 1) * kHeadRows * kHeadLdA, *Bd = Bt + (i & 1) * 16 * kHeadLdB;
+        for (int e = tid; e < kHeadRows * 8; e += 128) {
+            const int r = e >> 3, ch = e & 7;
+            umma::cp_async16(umma::smem_u32(Ad + r * kHeadLdA + ch * 8), A + (long long)min(k0 + r, P - 1) * 64 + ch * 8,
+                             k0 + r < ke);
+        }
+        asm volatile("cp.async.commit_group;\n" ::: "memory");
+        for (int e = tid; e < kHeadRows * 8 * nt; e += 128) {
+            const int r = e / (8 * nt), n = e - r * 8 * nt;
+            Bd[n * kHeadLdB + r] = n < C && k0 + r < ke ? B[(long long)(k0 + r) * C + n] : __float2bfloat16(0.f);
+        }
+    };
+    float acc[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
+    if (nblk > 0) load(0);
+    for (int i = 0; i < nblk; ++i) {
+        if (i + 1 < nblk) {
+            load(i + 1);
+            asm volatile("cp.async.wait_group 1;\n" ::: "memory");
+        } else {
+            asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+        }
+        __syncthreads();
+        const unsigned short *Ab = reinterpret_cast<const unsigned short *>(As + (i & 1) * kHeadRows * kHeadLdA);
+        const bf16 *Bb = Bt + (i & 1) * 16 * kHeadLdB;
+        const int steps = (min(ke - kb - i * kHeadRows, kHeadRows) + 15) / 16;
+        for (int kk = 0; kk < 16 * steps; kk += 16) {
+            auto pair = [&](int k, int row) {
+                return (unsigned)Ab[k * kHeadLdA + row] | (unsigned)Ab[(k + 1) * kHeadLdA + row] << 16;
+            };
+            const int k = kk + 2 * t4;
+            const unsigned a0 = pair(k, m), a1 = pair(k, m + 8), a2 = pair(k + 8, m), a3 = pair(k + 8, m + 8);
+#pragma unroll
+            for (int ni = 0; ni < 2; ++ni) {
+                if (ni >= nt) break;
+                const bf16 *b = Bb + (ni * 8 + g) * kHeadLdB + k;
+                const unsigned b0 = *reinterpret_cast<const unsigned *>(b), b1 = *reinterpret_cast<const unsigned *>(b + 8);
+                asm volatile(
+                    "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
+                    "{%0,%1,%2,%3};\n"
+                    : "+f"(acc[ni][0]), "+f"(acc[ni][1]), "+f"(acc[ni][2]), "+f"(acc[ni][3])
+                    : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+            }
+        }
+        __syncthreads();  // the buffer is free for block i + 2
+    }
+    float *out = part + (long long)blockIdx.x * 64 * C;
+#pragma unroll
+    for (int ni = 0; ni < 2; ++ni)
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            const int row = m + (r >= 2 ? 8 : 0), col = ni * 8 + 2 * t4 + (r & 1);
+            if (col < C) out[row * C + col] = acc[ni][r];
+        }
+}
+
+// mean-square loss: g = 2 (out - t)/n (FP32 and BF16), per-block partial losses
+__global__ void mse(const float *out, const float *t, long long n, float *g, bf16 *gb, float *part) {
     __shared__ float red[256];
     float s = 0.f;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
         const float d = out[i] - t[i];
-        g[i] = 2.f * d / (float)n;
+        const float v = 2.f * d / (float)n;
+        g[i] = v;
+        gb[i] = __float2bfloat16(v);
         s += d * d;
     }
     red[threadIdx.x] = s;
@@ -213,9 +365,15 @@ __global__ void to_bf16(const float *x, long long n, bf16 *y) {
         y[i] = __float2bfloat16(x[i]);
 }
 
-// Adam on the FP32 master weights; refresh the BF16 copy.
+// Adam on the FP32 master weights; refreshes the BF16 copy and, with L.wt, the K-major BF16 copies
+// of the weight matrices (one launch instead of one per matrix).
+struct WeightLayout {
+    bf16 *wt;  // null: no K-major copies
+    long long begin[6], out[6];
+    int K[6], N[6];
+};
 __global__ void adam(float *w, const float *g, float *m, float *v, long long n, float lr, float b1, float b2, float eps,
-                     float c1, float c2, bf16 *wb) {
+                     float c1, float c2, bf16 *wb, WeightLayout L) {
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
         const float gi = g[i];
         const float mi = b1 * m[i] + (1.f - b1) * gi;
@@ -225,6 +383,14 @@ __global__ void adam(float *w, const float *g, float *m, float *v, long long n, 
         const float wi = w[i] - lr * (mi / c1) / (sqrtf(vi / c2) + eps);
         w[i] = wi;
         wb[i] = __float2bfloat16(wi);
+        if (L.wt) {
+            for (int l = 0; l < 6; ++l) {
+                const long long e = i - L.begin[l];
+                if (e < 0 || e >= (long long)L.K[l] * L.N[l]) continue;
+                const int k = (int)(e / L.N[l]), c = (int)(e - (long long)k * L.N[l]);
+                L.wt[L.out[l] + (long long)c * L.K[l] + k] = __float2bfloat16(wi);
+            }
+        }
     }
 }
 
@@ -322,13 +488,16 @@ __global__ void judge_cv(const float *out, float *out_ref, double *Eref, const d
 
 // difference loss for pairs (sample b, sample b + B): d = (out_b - out_{b+B}) - (t_b - t_{b+B});
 // loss = mean(d^2) over the first half; g_b = 2d/n, g_{b+B} = -2d/n
-__global__ void mse_diff(const float *out, const float *t, long long n, float *g, float *part) {
+__global__ void mse_diff(const float *out, const float *t, long long n, float *g, bf16 *gb, float *part) {
     __shared__ float red[256];
     float s = 0.f;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
         const float d = (out[i] - out[i + n]) - (t[i] - t[i + n]);
-        g[i] = 2.f * d / (float)n;
+        const float v = 2.f * d / (float)n;
+        g[i] = v;
         g[i + n] = -2.f * d / (float)n;
+        gb[i] = __float2bfloat16(v);
+        gb[i + n] = __float2bfloat16(-2.f * d / (float)n);
         s += d * d;
     }
     red[threadIdx.x] = s;
@@ -554,6 +723,7 @@ struct rtbte_surrogate {
     DevBuf wbt, a0, a1;           // transposed BF16 weights and activations of the fused inference path
     DevBuf wtt, tcerr;            // K-major BF16 weights of the tensor-core GEMMs (W_l^T, M1^T, M2^T); error word
     long long off_tt[kLayers + 2] = {0, 0, 0, 0, 0, 0};
+    DevBuf gzl, chains;           // implicit-convolution training: gz of each layer [5][P][64], bias chain sums
     int engine = 0;               // 0: tcgen05 GEMMs where both operands are K-major; 1: mma.sync everywhere
     long long off_t[kLayers + 1] = {0, 0, 0, 0, 0};
     bool has_ref = false, fused = false, smem_set = false;
@@ -591,18 +761,19 @@ int salloc(rtbte_surrogate *s, DevBuf &b, size_t bytes) {
 
 template <bool TA, bool TB>
 int gemm(rtbte_surrogate *s, const bf16 *A, int lda, const bf16 *B, int ldb, float *C, int ldc, int M, int N, int K,
-         const float *bias, int act, bf16 *Cb, int splits = 1) {
+         const float *bias, int act, bf16 *Cb, int splits = 1, const float *back = nullptr) {
     cudaStream_t st = s->ctx->stream;
     if (splits <= 1) {
         dim3 grid((M + kBM - 1) / kBM, (N + kBN - 1) / kBN, 1);
-        gemm_bf16<TA, TB><<<grid, kGemmThreads, 0, st>>>(A, lda, B, ldb, C, ldc, M, N, K, K, bias, act, Cb);
+        gemm_bf16<TA, TB><<<grid, kGemmThreads, 0, st>>>(A, lda, B, ldb, C, ldc, M, N, K, K, bias, act, Cb, back);
     } else {
         int kchunk = (K + splits - 1) / splits;
         kchunk = (kchunk + kBK - 1) / kBK * kBK;
         splits = (K + kchunk - 1) / kchunk;
         dim3 grid((M + kBM - 1) / kBM, (N + kBN - 1) / kBN, splits);
         float *part = s->split.as<float>();
-        gemm_bf16<TA, TB><<<grid, kGemmThreads, 0, st>>>(A, lda, B, ldb, part, ldc, M, N, K, kchunk, nullptr, 0, nullptr);
+        gemm_bf16<TA, TB><<<grid, kGemmThreads, 0, st>>>(A, lda, B, ldb, part, ldc, M, N, K, kchunk, nullptr, 0, nullptr,
+                                                           nullptr);
         sum_splits<<<blocks_for((long long)M * ldc), 256, 0, st>>>(part, splits, (long long)M * ldc, C);
     }
     S_CUDA(s, cudaGetLastError());
@@ -648,7 +819,7 @@ bool kmajor_map(CUtensorMap *m, const bf16 *ptr, long long rows, long long cols,
 
 // C[M x N] = A[M x K] B[N x K]^T (+ bias, tanh, BF16 copy) on the tensor cores, A and B K-major
 int gemm_tc(rtbte_surrogate *s, const bf16 *A, int lda, const bf16 *B, int ldb, float *C, int ldc, int M, int N, int K,
-            const float *bias, int act, bf16 *Cb) {
+            const float *bias, int act, bf16 *Cb, const float *back = nullptr) {
     const int bn_full = (N + 15) / 16 * 16;
     const int bn = std::min(bn_full, 256);
     CUtensorMap ta, tb;
@@ -662,6 +833,7 @@ int gemm_tc(rtbte_surrogate *s, const bf16 *A, int lda, const bf16 *B, int ldb, 
     a.bn = bn;
     a.ldc = ldc;
     a.act = act;
+    a.back = back;
     a.bias = bias;
     a.C = C;
     a.Cb = Cb;
@@ -689,21 +861,28 @@ int gemm_tc(rtbte_surrogate *s, const bf16 *A, int lda, const bf16 *B, int ldb, 
     return RTBTE_OK;
 }
 
+// K range of one split of a weight-gradient GEMM: about two CTAs per SM, at most 64 splits, each a
+// whole number of 64-wide K slices
+long long split_chunk(const rtbte_surrogate *s, int M, int K) {
+    const int mt = (M + umma::kTM - 1) / umma::kTM;
+    const int want = std::max(1, std::min(64, (2 * s->ctx->num_sms + mt - 1) / mt));
+    const long long kc = ((long long)K + want - 1) / want;
+    return (kc + umma::kTK - 1) / umma::kTK * umma::kTK;
+}
+
 // C[M x N] = A^T B on the tensor cores for A stored [K][M] (row stride lda) and B stored [K][N]
 // (row stride ldb), both MN-major, N a multiple of 64: K split over CTAs in multiples of 64, the
-// partial products summed in a fixed order (the weight gradients, a contraction over points)
+// partial products summed in a fixed order (the weight gradients, a contraction over points), or left
+// in part [*nsplit][M][ldc] for the caller to sum
 int gemm_tc_mn(rtbte_surrogate *s, const bf16 *A, int lda, const bf16 *B, int ldb, float *C, int ldc, int M, int N,
-               int K) {
+               int K, float *part = nullptr, int *nsplit = nullptr) {
     if (N % 64 || N > 256) return sfail(s, RTBTE_E_UNSUPPORTED, "tensor-core GEMM: MN-major N must be 64..256 by 64");
     CUtensorMap ta, tb;
     if ((lda * (int)sizeof(bf16)) % 16 || (ldb * (int)sizeof(bf16)) % 16 || !kmajor_map(&ta, A, K, M, lda, 64) ||
         !kmajor_map(&tb, B, K, N, ldb, 64))
         return sfail(s, RTBTE_E_UNSUPPORTED, "tensor-core GEMM: operand layout not expressible as a TMA map");
     const int mt = (M + umma::kTM - 1) / umma::kTM;
-    // about two CTAs per SM, at most 64 slices, each a whole number of 64-wide K slices
-    const int want = std::max(1, std::min(64, (2 * s->ctx->num_sms + mt - 1) / mt));
-    long long kc = ((long long)K + want - 1) / want;
-    kc = (kc + umma::kTK - 1) / umma::kTK * umma::kTK;
+    const long long kc = split_chunk(s, M, K);
     const int splits = (int)((K + kc - 1) / kc);
     umma::Args a{};
     a.M = M;
@@ -712,7 +891,8 @@ int gemm_tc_mn(rtbte_surrogate *s, const bf16 *A, int lda, const bf16 *B, int ld
     a.bn = N;
     a.ldc = ldc;
     a.act = 0;
-    a.C = splits > 1 ? s->split.as<float>() : C;
+    a.C = part ? part : splits > 1 ? s->split.as<float>() : C;
+    if (nsplit) *nsplit = splits;
     a.err = s->tcerr.as<int>();
     a.a_mn = a.b_mn = 1;
     a.k_base = 0;
@@ -724,7 +904,7 @@ int gemm_tc_mn(rtbte_surrogate *s, const bf16 *A, int lda, const bf16 *B, int ld
     else umma::gemm_tc<256, 2><<<grid, umma::kThreads, umma::smem_bytes(N), st>>>(ta, tb, a);
     S_CUDA(s, cudaGetLastError());
     s->ctx->launches++;
-    if (splits > 1) {
+    if (splits > 1 && !part) {
         sum_splits<<<blocks_for((long long)M * ldc), 256, 0, st>>>(s->split.as<float>(), splits, (long long)M * ldc, C);
         S_CUDA(s, cudaGetLastError());
         s->ctx->launches++;
@@ -761,6 +941,33 @@ int check_tc(rtbte_surrogate *s) {
     return RTBTE_OK;
 }
 
+// Convolutions of layers 1..3 gather their operand slices themselves (umma::conv_tc) where a K
+// slice of 64 lies within a tap: 64 channels on the tcgen05 engine.  Other widths take im2col.
+bool implicit_conv(const rtbte_surrogate *s) { return s->engine == 0 && s->width == umma::kConvC; }
+
+// One implicit convolution over B samples; `mat` is the kernel's TMA operand [rows][cols].
+template <int MODE>
+int conv(rtbte_surrogate *s, umma::ConvArgs a, int B, const bf16 *mat, long long rows, long long cols, int splits = 1) {
+    a.P = (int)((long long)B * s->Pq);
+    a.ny = s->ny;
+    a.nx = s->nx;
+    a.err = s->tcerr.as<int>();
+    CUtensorMap tb;
+    if (!kmajor_map(&tb, mat, rows, cols, cols, 64))
+        return sfail(s, RTBTE_E_UNSUPPORTED, "tensor-core convolution: operand layout not expressible as a TMA map");
+    static bool attr_set = false;  // the shared-memory limit is a per-function attribute: set once
+    if (!attr_set) {
+        S_CUDA(s, allow_max_dynamic_smem((const void *)umma::conv_tc<MODE>));
+        attr_set = true;
+    }
+    const int mrows = MODE == umma::CONV_WEIGHT ? 9 * umma::kConvC : a.P;
+    const dim3 grid((mrows + umma::kTM - 1) / umma::kTM, splits);
+    umma::conv_tc<MODE><<<grid, umma::kThreads, umma::conv_smem_bytes(), s->ctx->stream>>>(tb, a);
+    S_CUDA(s, cudaGetLastError());
+    s->ctx->launches++;
+    return RTBTE_OK;
+}
+
 // forward of B samples whose normalised input is in s->xb ([B*Pq][C] BF16); output FP32 in s->out
 int forward(rtbte_surrogate *s, int B) {
     cudaStream_t st = s->ctx->stream;
@@ -768,7 +975,18 @@ int forward(rtbte_surrogate *s, int B) {
     const bf16 *in = s->xb.as<bf16>();
     int C = s->C, rc;
     for (int l = 0; l < kLayers; ++l) {
-        im2col<<<blocks_for(P * s->kpad[l]), 256, 0, st>>>(in, C, s->ny, s->nx, P, s->cols[l].as<bf16>(), s->kpad[l]);
+        if (l > 0 && implicit_conv(s)) {
+            umma::ConvArgs a{};
+            a.src = in;
+            a.bias = s->w.as<float>() + s->off_b[l];
+            a.out = s->acts[l + 1].as<float>();
+            a.outb = s->actb[l + 1].as<bf16>();
+            if ((rc = conv<umma::CONV_FORWARD>(s, a, B, s->wtt.as<bf16>() + s->off_tt[l], s->width, s->kpad[l]))) return rc;
+            in = s->actb[l + 1].as<bf16>();
+            continue;
+        }
+        im2col<<<blocks_for(P * s->kpad[l] / 8), 256, 0, st>>>(in, C, s->ny, s->nx, P, s->cols[l].as<bf16>(),
+                                                               s->kpad[l]);
         S_CUDA(s, cudaGetLastError());
         s->ctx->launches++;
         if (s->engine == 0)
@@ -801,6 +1019,108 @@ int forward(rtbte_surrogate *s, int B) {
                               nullptr);
 }
 
+int read_loss(rtbte_surrogate *s, int nb, float *loss) {
+    std::vector<float> lp(nb);
+    S_CUDA(s, cudaMemcpyAsync(lp.data(), s->lossp.p, sizeof(float) * nb, cudaMemcpyDeviceToHost, s->ctx->stream));
+    S_CUDA(s, cudaStreamSynchronize(s->ctx->stream));
+    double acc = 0;
+    for (float x : lp) acc += x;
+    *loss = (float)acc;
+    return RTBTE_OK;
+}
+
+// Gradients (s->g) of a 64-channel network on the tcgen05 engine from g_out (s->gout, s->goutb):
+// the gradient through tanh is applied where the gradient of the activation is produced, every
+// layer keeps its own gz, and all split-K partials and bias columns are summed by one launch.
+int backward_conv(rtbte_surrogate *s, int B) {
+    cudaStream_t st = s->ctx->stream;
+    const long long P = (long long)B * s->Pq;
+    const int Wd = s->width, C = s->C;
+    int rc;
+    float *g = s->g.as<float>();
+    float *gz[kLayers + 1];  // gz[l], l < kLayers: convolution l; gz[kLayers]: the pointwise layer
+    for (int l = 0; l <= kLayers; ++l) gz[l] = s->gzl.as<float>() + (long long)l * P * Wd;
+    bf16 *gb[2] = {s->gzb.as<bf16>(), s->gzb.as<bf16>() + P * Wd};  // BF16 gz of the current and the next layer
+    float *part = s->split.as<float>();
+    GradSums q{};
+    int nq = 0;
+    auto sums = [&](float *p, int splits, int n, float *out) {  // partials for finish_grads
+        q.part[nq] = p;
+        q.splits[nq] = splits;
+        q.n[nq] = n;
+        q.out[nq++] = out;
+        part = p + (long long)splits * n;
+    };
+    // out = h5 M2 + c2: the splits of gemm over points (s->split), FP32 columns of g_out
+    int splits = (int)std::min<long long>(64, std::max<long long>(1, P / 1024));
+    const int kchunk = (int)(((P + splits - 1) / splits + kBK - 1) / kBK * kBK);
+    splits = (int)((P + kchunk - 1) / kchunk);
+    static bool attr_set = false;
+    if (!attr_set) {
+        S_CUDA(s, allow_max_dynamic_smem((const void *)head_grad));
+        attr_set = true;
+    }
+    head_grad<<<splits, 128, kHeadSmem, st>>>(s->actb[0].as<bf16>(), s->goutb.as<bf16>(), C, (int)P, kchunk, part);
+    S_CUDA(s, cudaGetLastError());
+    sums(part, splits, Wd * C, g + s->off_M2);
+    // gz5 = (g_out M2^T)(1 - h5^2)
+    if ((rc = gemm<false, true>(s, s->goutb.as<bf16>(), C, s->wb.as<bf16>() + s->off_M2, C, gz[kLayers], Wd, (int)P, Wd,
+                                C, nullptr, 0, gb[0], 1, s->acts[0].as<float>())))
+        return rc;
+    int ns = 0;
+    if ((rc = gemm_tc_mn(s, s->actb[kLayers].as<bf16>(), Wd, gb[0], Wd, nullptr, Wd, Wd, Wd, (int)P, part, &ns)))
+        return rc;
+    sums(part, ns, Wd * Wd, g + s->off_M1);
+    // gz4 = (gz5 M1^T)(1 - h4^2) (M1 itself is the K-major [n][k] operand)
+    if ((rc = gemm_tc(s, gb[0], Wd, s->wb.as<bf16>() + s->off_M1, Wd, gz[kLayers - 1], Wd, (int)P, Wd, Wd, nullptr, 0,
+                      gb[1], s->acts[kLayers].as<float>())))
+        return rc;
+    int cur = 1;
+    for (int l = kLayers - 1; l >= 0; --l) {
+        if (l == 0) {
+            if ((rc = gemm_tc_mn(s, s->cols[0].as<bf16>(), s->kpad[0], gb[cur], Wd, nullptr, Wd, s->kpad[0], Wd, (int)P,
+                                 part, &ns)))
+                return rc;
+            sums(part, ns, s->kpad[0] * Wd, g + s->off_W[0]);
+            break;
+        }
+        umma::ConvArgs a{};
+        a.src = s->actb[l].as<bf16>();
+        a.kchunk = (int)split_chunk(s, s->kpad[l], (int)P);
+        a.out = part;
+        ns = (int)((P + a.kchunk - 1) / a.kchunk);
+        if ((rc = conv<umma::CONV_WEIGHT>(s, a, B, gb[cur], P, Wd, ns))) return rc;
+        sums(part, ns, s->kpad[l] * Wd, g + s->off_W[l]);
+        umma::ConvArgs b{};
+        b.src = gb[cur];
+        b.back = s->acts[l].as<float>();
+        b.out = gz[l - 1];
+        b.outb = gb[cur ^ 1];
+        if ((rc = conv<umma::CONV_BACK>(s, b, B, s->wb.as<bf16>() + s->off_W[l], s->kpad[l], Wd))) return rc;
+        cur ^= 1;
+    }
+    for (int l = 0; l <= kLayers; ++l) {
+        q.G[l] = gz[l];
+        q.cols[l] = Wd;
+        q.bias[l] = l < kLayers ? g + s->off_b[l] : g + s->off_c1;
+    }
+    q.G[kLayers + 1] = s->gout.as<float>();
+    q.cols[kLayers + 1] = C;
+    q.bias[kLayers + 1] = g + s->off_c2;
+    q.chains = s->chains.as<float>();
+    q.P = P;
+    bias_chains<<<dim3(64, kLayers + 2), 256, 0, st>>>(q);
+    int nbias = 0, elems = 0;
+    for (int l = 0; l < kLayers + 2; ++l) {
+        nbias += q.cols[l];
+        elems += q.n[l];
+    }
+    finish_grads<<<nbias + (elems + 255) / 256, 256, 0, st>>>(q, nbias);
+    S_CUDA(s, cudaGetLastError());
+    s->ctx->launches += 3;
+    return RTBTE_OK;
+}
+
 // loss and gradients (FP32, s->g) for targets s->t of the B samples in s->xb
 int loss_grad(rtbte_surrogate *s, int B, float *loss, bool diff = false) {
     cudaStream_t st = s->ctx->stream;
@@ -810,12 +1130,16 @@ int loss_grad(rtbte_surrogate *s, int B, float *loss, bool diff = false) {
     const int nb = blocks_for(diff ? nout / 2 : nout);
     if (diff)  // samples b and b + B/2 form a pair
         mse_diff<<<nb, 256, 0, st>>>(s->out.as<float>(), s->t.as<float>(), nout / 2, s->gout.as<float>(),
-                                     s->lossp.as<float>());
+                                     s->goutb.as<bf16>(), s->lossp.as<float>());
     else
-        mse<<<nb, 256, 0, st>>>(s->out.as<float>(), s->t.as<float>(), nout, s->gout.as<float>(), s->lossp.as<float>());
-    to_bf16<<<nb, 256, 0, st>>>(s->gout.as<float>(), nout, s->goutb.as<bf16>());
+        mse<<<nb, 256, 0, st>>>(s->out.as<float>(), s->t.as<float>(), nout, s->gout.as<float>(), s->goutb.as<bf16>(),
+                                s->lossp.as<float>());
     S_CUDA(s, cudaGetLastError());
-    s->ctx->launches += 2;
+    s->ctx->launches++;
+    if (implicit_conv(s)) {
+        if ((rc = backward_conv(s, B))) return rc;
+        return loss ? read_loss(s, nb, loss) : RTBTE_OK;
+    }
     float *g = s->g.as<float>();
     const int Wd = s->width;
     const int splitsP = (int)std::min<long long>(64, std::max<long long>(1, P / 1024));
@@ -872,15 +1196,7 @@ int loss_grad(rtbte_surrogate *s, int B, float *loss, bool diff = false) {
     }
     S_CUDA(s, cudaGetLastError());
     s->ctx->launches += 4 + 3 * kLayers;
-    if (loss) {
-        std::vector<float> lp(nb);
-        S_CUDA(s, cudaMemcpyAsync(lp.data(), s->lossp.p, sizeof(float) * nb, cudaMemcpyDeviceToHost, st));
-        S_CUDA(s, cudaStreamSynchronize(st));
-        double acc = 0;
-        for (float x : lp) acc += x;
-        *loss = (float)acc;
-    }
-    return RTBTE_OK;
+    return loss ? read_loss(s, nb, loss) : RTBTE_OK;
 }
 
 // host <-> device parameter copies in the logical layout (W_l rows 0..9*C_in-1)
@@ -913,10 +1229,15 @@ int params_io(rtbte_surrogate *s, float *host, bool to_device) {
     return RTBTE_OK;
 }
 
-// largest weight-gradient matrix (the split-K partial buffer holds 64 of them)
-long long split_elems(const rtbte_surrogate *s) {
-    long long e = (long long)s->width * std::max(s->width, s->C);
-    for (int l = 0; l < kLayers; ++l) e = std::max(e, (long long)s->kpad[l] * s->width);
+// elements of the split-K partial buffer per split (at most 64): the largest weight-gradient
+// matrix, or all of them side by side
+long long split_elems(const rtbte_surrogate *s, bool all) {
+    const long long m1 = (long long)s->width * s->width, m2 = (long long)s->width * s->C;
+    long long e = all ? m1 + m2 : std::max(m1, m2);
+    for (int l = 0; l < kLayers; ++l) {
+        const long long w = (long long)s->kpad[l] * s->width;
+        e = all ? e + w : std::max(e, w);
+    }
     return e;
 }
 
@@ -924,17 +1245,20 @@ int ensure_batch(rtbte_surrogate *s, int B) {
     if (B <= s->max_batch) return RTBTE_OK;
     const long long P = (long long)B * s->Pq;
     const int Wd = s->width;
+    const bool conv = implicit_conv(s);
     int rc;
     if ((rc = salloc(s, s->xb, sizeof(bf16) * P * s->C)) || (rc = salloc(s, s->t, sizeof(float) * P * s->C)) ||
         (rc = salloc(s, s->out, sizeof(float) * P * s->C)) || (rc = salloc(s, s->gout, sizeof(float) * P * s->C)) ||
         (rc = salloc(s, s->goutb, sizeof(bf16) * P * s->C)) || (rc = salloc(s, s->ga, sizeof(float) * P * Wd)) ||
-        (rc = salloc(s, s->gz, sizeof(float) * P * Wd)) || (rc = salloc(s, s->gzb, sizeof(bf16) * P * Wd)) ||
-        (rc = salloc(s, s->gcol, sizeof(float) * P * s->kpad[1])) ||
-        (rc = salloc(s, s->split, sizeof(float) * 64LL * split_elems(s))) ||
+        (rc = salloc(s, s->gz, sizeof(float) * P * Wd)) || (rc = salloc(s, s->gzb, sizeof(bf16) * 2 * P * Wd)) ||
+        (rc = salloc(s, s->gcol, conv ? 0 : sizeof(float) * P * s->kpad[1])) ||
+        (rc = salloc(s, s->gzl, conv ? sizeof(float) * (kLayers + 1) * P * Wd : 0)) ||
+        (rc = salloc(s, s->chains, conv ? sizeof(float) * 6 * 256 * 64 : 0)) ||
+        (rc = salloc(s, s->split, sizeof(float) * 64LL * split_elems(s, conv))) ||
         (rc = salloc(s, s->lossp, sizeof(float) * 4096)) || (rc = salloc(s, s->idx, sizeof(int) * B)))
         return rc;
     for (int l = 0; l < kLayers; ++l)
-        if ((rc = salloc(s, s->cols[l], sizeof(bf16) * P * s->kpad[l]))) return rc;
+        if ((rc = salloc(s, s->cols[l], conv && l > 0 ? 0 : sizeof(bf16) * P * s->kpad[l]))) return rc;
     for (int l = 0; l <= kLayers; ++l)
         if ((rc = salloc(s, s->acts[l], sizeof(float) * P * Wd)) || (rc = salloc(s, s->actb[l], sizeof(bf16) * P * Wd)))
             return rc;
@@ -1299,6 +1623,16 @@ int rtbte_surrogate_train(rtbte_surrogate *s, int steps, int batch, int horizon,
     for (size_t i = 0; i < perm.size(); ++i) perm[i] = (int)i;
     size_t pos = perm.size();
     std::vector<int> bidx(nsamp);
+    WeightLayout layout{};
+    if (s->engine == 0) {
+        layout.wt = s->wtt.as<bf16>();
+        for (int l = 0; l < kLayers + 2; ++l) {
+            layout.begin[l] = l < kLayers ? s->off_W[l] : l == kLayers ? s->off_M1 : s->off_M2;
+            layout.out[l] = s->off_tt[l];
+            layout.K[l] = l < kLayers ? s->kpad[l] : s->width;
+            layout.N[l] = l <= kLayers ? s->width : s->C;
+        }
+    }
     float last = 0.f;
     for (int it = 0; it < steps; ++it) {
         for (int b = 0; b < batch; ++b) {
@@ -1321,10 +1655,9 @@ int rtbte_surrogate_train(rtbte_surrogate *s, int steps, int batch, int horizon,
         const float b1 = 0.9f, b2 = 0.999f;
         adam<<<blocks_for(s->nparam), 256, 0, ctx->stream>>>(
             s->w.as<float>(), s->g.as<float>(), s->m.as<float>(), s->v.as<float>(), s->nparam, lr, b1, b2, 1e-8f,
-            1.f - powf(b1, (float)s->adam_t), 1.f - powf(b2, (float)s->adam_t), s->wb.as<bf16>());
+            1.f - powf(b1, (float)s->adam_t), 1.f - powf(b2, (float)s->adam_t), s->wb.as<bf16>(), layout);
         S_CUDA(s, cudaGetLastError());
         ctx->launches++;
-        if ((rc = refresh_training_layout(s))) return rc;
     }
     if ((rc = refresh_inference(s))) return rc;
     S_CUDA(s, cudaStreamSynchronize(ctx->stream));
@@ -1378,6 +1711,7 @@ int rtbte_surrogate_set_gemm(rtbte_surrogate *s, int engine) {
         cudaDeviceGetAttribute(&cc, cudaDevAttrComputeCapabilityMajor, s->ctx->device);
         if (cc < 10 || !encode_tiled()) return sfail(s, RTBTE_E_UNSUPPORTED, "no tcgen05 tensor cores or TMA maps");
     }
+    if (engine != s->engine) s->max_batch = 0;  // the engines' batch buffers differ
     s->engine = engine;
     int rc;
     if ((rc = refresh_training_layout(s))) return rc;
@@ -1431,7 +1765,7 @@ void rtbte_surrogate_destroy(rtbte_surrogate *s) {
     DevBuf *bufs[] = {&s->w,  &s->wb,  &s->g,     &s->m,    &s->v,     &s->stats, &s->ppfull, &s->Ns,
                       &s->Is, &s->idx, &s->xb,    &s->t,    &s->out,   &s->gout,  &s->goutb,  &s->ga,
                       &s->gz, &s->gzb, &s->gcol,  &s->split, &s->lossp, &s->ydot, &s->Eref,   &s->out_ref,
-                      &s->normp, &s->wbt, &s->a0,  &s->a1, &s->wtt, &s->tcerr};
+                      &s->normp, &s->wbt, &s->a0,  &s->a1, &s->wtt, &s->tcerr, &s->gzl, &s->chains};
     for (DevBuf *b : bufs) b->release();
     for (int l = 0; l < kLayers; ++l) s->cols[l].release();
     for (int l = 0; l <= kLayers; ++l) {

@@ -37,6 +37,7 @@ constexpr uint32_t kMnLbo = kTK * 128, kMnSbo = 1024;
 struct Args {
     int M, N, K, bn;
     int ldc, act;
+    const float *back;    // [M][ldc] activations a: C = acc (1 - a^2) (the gradient through tanh), or null
     const float *bias;
     float *C;
     __nv_bfloat16 *Cb;
@@ -225,6 +226,10 @@ __global__ void __launch_bounds__(kThreads) gemm_tc(const __grid_constant__ CUte
                 v[j] = __uint_as_float(r[j]);
                 if (a.bias && col0 + j < a.N) v[j] += a.bias[col0 + j];
                 if (a.act) v[j] = tanhf(v[j]);
+                if (a.back && col0 + j < a.N) {
+                    const float h = a.back[(long long)row * a.ldc + col0 + j];
+                    v[j] = v[j] * (1.f - h * h);
+                }
             }
             float *cr = a.C + (long long)blockIdx.z * a.c_split + (long long)row * a.ldc + col0;
             __nv_bfloat16 *br = a.Cb ? a.Cb + (long long)row * a.ldc + col0 : nullptr;
@@ -263,6 +268,268 @@ __global__ void __launch_bounds__(kThreads) gemm_tc(const __grid_constant__ CUte
     if (warp == 0)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(NCOLS) : "memory");
 }
+
+// ---- periodic 3x3 convolutions of 64 channels as implicit GEMMs ---------------------------------
+// The K slices of a convolution's GEMM over (tap, channel) are its taps: a slice of the A operand
+// is the 128 points' neighbours of one tap, 128 bytes of channels each.  These kernels gather the
+// slices from the activations themselves (cp.async, 16 bytes a thread, eight threads a row, written
+// in the 128-byte swizzle that TMA would write) instead of from an im2col matrix nine times their
+// size, so a layer reads 3.7 MB instead of writing and reading 33 MB (batch 8 of 60 x 60), and the
+// input gradient adds its nine taps in registers instead of through a 66 MB column matrix.  The
+// slices, their order and every rounding are those of the GEMMs over im2col columns.
+constexpr int kConvC = 64;      // channels in and out
+constexpr int kConvStages = 4;  // ring of A (16 KB) and B (8 KB) slices: two CTAs per SM
+constexpr int kConvA = kTM * kTK * 2, kConvB = kConvC * kTK * 2;
+
+struct ConvArgs {
+    const __nv_bfloat16 *src;  // [P][64] gathered operand
+    int P, ny, nx;             // points of the batch, sample grid
+    int kchunk;                // weight gradient: points per split
+    const float *bias;         // forward
+    const float *back;         // input gradient: [P][64] activations a, out = sum (1 - a^2)
+    float *out;                // [P][64], or the weight gradient's partials [split][576][64]
+    __nv_bfloat16 *outb;       // [P][64] BF16 copy of out
+    int *err;
+};
+
+__device__ __forceinline__ void cp_async16(uint32_t dst, const void *src, bool valid) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(dst), "l"(src), "r"(valid ? 16 : 0) : "memory");
+}
+
+// A point of the batch as (first point of its sample, y, x).
+struct Point {
+    int b0, y, x;
+    __device__ __forceinline__ void set(int p, int ny, int nx) {
+        const int per = ny * nx, b = p / per, yx = p - b * per;
+        b0 = b * per;
+        y = yx / nx;
+        x = yx - y * nx;
+    }
+    // its neighbour across tap (dy + 1) * 3 + dx + 1 (periodic)
+    __device__ __forceinline__ int at(int dy, int dx, int ny, int nx) const {
+        int ys = y + dy, xs = x + dx;
+        ys += ys < 0 ? ny : 0;
+        ys -= ys >= ny ? ny : 0;
+        xs += xs < 0 ? nx : 0;
+        xs -= xs >= nx ? nx : 0;
+        return b0 + ys * nx + xs;
+    }
+};
+
+enum { CONV_FORWARD = 0, CONV_BACK = 1, CONV_WEIGHT = 2 };
+
+// CONV_FORWARD  out[p][n] = tanh(sum_tap sum_c src[p + tap][c] W[tap, c][n] + bias[n]), tB: W^T [64][576]
+// CONV_BACK     out[p][c] = (sum_tap sum_n src[p - tap][n] W[tap, c][n]) (1 - a[p][c]^2), tB: W [576][64];
+//               each tap's product is rounded to FP32 and the nine are added in tap order
+// CONV_WEIGHT   part[z][(tap, c)][n] = sum over the split's points of src[p + tap][c] g[p][n],
+//               tB: g [P][64]; both operands MN-major, two taps a tile
+// Every barrier wait is bounded; after one that gave up nothing more is issued and *err is set.
+template <int MODE>
+__global__ void __launch_bounds__(kThreads) conv_tc(const __grid_constant__ CUtensorMap tB, ConvArgs a) {
+    extern __shared__ unsigned char smem_raw[];
+    constexpr int NS = kConvStages;
+    constexpr uint32_t kCols = MODE == CONV_BACK ? 256u : 64u;  // CONV_BACK: four accumulators in turn
+    const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
+    const uint32_t bars = base + NS * (kConvA + kConvB);  // full[NS] (B slices), used[NS] (MMAs done), TMEM slot
+    auto sA = [&](int s) { return base + (uint32_t)s * kConvA; };
+    auto sB = [&](int s) { return base + NS * kConvA + (uint32_t)s * kConvB; };
+    auto full = [&](int s) { return bars + 8u * s; };
+    auto used = [&](int s) { return bars + 8u * (NS + s); };
+    const uint32_t tslot = bars + 16 * NS;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int m0 = blockIdx.x * kTM;  // first point, or first (tap, channel) row
+    const int k0 = MODE == CONV_WEIGHT ? blockIdx.y * a.kchunk : 0;
+    const int nk = MODE == CONV_WEIGHT ? a.kchunk / kTK : 9;
+    bool bad = false;  // this thread saw a wait give up
+
+    if (tid == 0) {
+        for (int i = 0; i < NS; ++i) {
+            mbar_init(full(i), 1);
+            mbar_init(used(i), 1);
+        }
+        asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+    }
+    if (warp == 0) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(tslot), "r"(kCols)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+    uint32_t tmem;
+    asm volatile("ld.shared.b32 %0, [%1];\n" : "=r"(tmem) : "r"(tslot) : "memory");
+
+    // gather role: chunk c of rows r0 + 16 i; all of a thread's rows have the same row mod 8
+    const int c = tid & 7, r0 = tid >> 3;
+    const uint32_t gdst = (uint32_t)r0 * 128u + ((uint32_t)(c ^ (r0 & 7)) << 4);
+    Point pt[8];  // the tile's points (forward and input gradient)
+    if (MODE != CONV_WEIGHT) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) pt[i].set(min(m0 + r0 + 16 * i, a.P - 1), a.ny, a.nx);
+    }
+    // start slice kt's copies into stage s: thread 0 the B slice, every thread its rows of the A slice
+    auto load = [&](int s, int kt) {
+        if (tid == 0) {
+            mbar_expect_tx(full(s), kConvB);
+            if (MODE == CONV_FORWARD) tma_load_2d(sB(s), &tB, kt * kTK, 0, full(s));
+            if (MODE == CONV_BACK) tma_load_2d(sB(s), &tB, 0, kt * kConvC, full(s));
+            if (MODE == CONV_WEIGHT) tma_load_2d(sB(s), &tB, 0, k0 + kt * kTK, full(s));
+        }
+        if (MODE != CONV_WEIGHT) {
+            const int dy = MODE == CONV_BACK ? 1 - kt / 3 : kt / 3 - 1, dx = MODE == CONV_BACK ? 1 - kt % 3 : kt % 3 - 1;
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+                cp_async16(sA(s) + gdst + 2048u * i, a.src + (long long)pt[i].at(dy, dx, a.ny, a.nx) * kConvC + 8 * c,
+                           m0 + r0 + 16 * i < a.P);
+        } else {
+            const int t0 = m0 / kConvC;  // two taps: blocks of 64 points x 128 bytes
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const int p = k0 + kt * kTK + r0 + 16 * i;
+                Point q;
+                q.set(min(p, a.P - 1), a.ny, a.nx);
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const int tap = min(t0 + h, 8);  // (rows of a tenth tap are not stored)
+                    cp_async16(sA(s) + (uint32_t)h * 8192u + gdst + 2048u * i,
+                               a.src + (long long)q.at(tap / 3 - 1, tap % 3 - 1, a.ny, a.nx) * kConvC + 8 * c, p < a.P);
+                }
+            }
+        }
+    };
+    auto give_up = [&](int code) {
+        bad = true;
+        atomicExch(a.err, code);
+    };
+    float sum[kConvC];  // CONV_BACK: this thread's row
+    auto add_tap = [&](int kt) {
+#pragma unroll
+        for (int c0 = 0; c0 < kConvC; c0 += 16) {
+            uint32_t r[16];
+            asm volatile(
+                "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, "
+                "[%16];\n"
+                : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+                  "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+                : "r"(tmem + ((uint32_t)(32 * warp) << 16) + (uint32_t)(MODE == CONV_BACK ? 64 * (kt & 3) : 0) +
+                      (uint32_t)c0));
+            asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
+#pragma unroll
+            for (int j = 0; j < 16; ++j) {
+                const float v = __uint_as_float(r[j]);
+                sum[c0 + j] = MODE == CONV_BACK && kt > 0 ? sum[c0 + j] + v : v;
+            }
+        }
+    };
+
+    int loaded = 0;  // slices whose copies were started
+    for (; loaded < NS - 1 && loaded < nk; ++loaded) {
+        load(loaded, loaded);
+        asm volatile("cp.async.commit_group;\n" ::: "memory");
+    }
+    for (int i = loaded; i < NS - 1; ++i) asm volatile("cp.async.commit_group;\n" ::: "memory");
+    const uint32_t idesc = idesc_bf16(kTM, kConvC, MODE == CONV_WEIGHT, MODE == CONV_WEIGHT);
+    for (int kt = 0; kt < nk; ++kt) {
+        const int s = kt % NS;
+        // slice kt is the oldest of the NS - 1 groups in flight; its bytes become visible to the
+        // tensor core through the proxy fence of the threads that wrote them
+        asm volatile("cp.async.wait_group %0;\n" ::"n"(NS - 2) : "memory");
+        asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+        asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+        if (__syncthreads_or(bad)) break;
+        if (tid == 0) {
+            asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+            if (!mbar_wait(full(s), (uint32_t)((kt / NS) & 1))) give_up(3);
+            else {
+                const uint32_t d = tmem + (MODE == CONV_BACK ? 64u * (kt & 3) : 0u);
+#pragma unroll
+                for (int k16 = 0; k16 < kTK / 16; ++k16) {
+                    const uint64_t da = MODE == CONV_WEIGHT ? sw128_desc(sA(s) + 2048u * k16, kMnLbo, kMnSbo)
+                                                            : sw128_desc(sA(s) + 32u * k16);
+                    const uint64_t db = MODE == CONV_WEIGHT ? sw128_desc(sB(s) + 2048u * k16, kMnLbo, kMnSbo)
+                                                            : sw128_desc(sB(s) + 32u * k16);
+                    const uint32_t acc = ((MODE != CONV_BACK && kt > 0) || k16 > 0) ? 1u : 0u;
+                    asm volatile(
+                        "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
+                        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d),
+                        "l"(da), "l"(db), "r"(idesc), "r"(acc)
+                        : "memory");
+                }
+                asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(
+                                 used(s))
+                             : "memory");
+            }
+        }
+        // the previous slice's MMAs: their stage is free, and (CONV_BACK) their product complete
+        if (kt > 0) {
+            if (!mbar_wait(used((kt - 1) % NS), (uint32_t)(((kt - 1) / NS) & 1))) give_up(4);
+            if (MODE == CONV_BACK) {
+                asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+                __syncwarp();
+                add_tap(kt - 1);
+            }
+        }
+        if (loaded < nk && !bad) {  // into the stage slice kt - 1 used (slice NS - 1: unused so far)
+            load(loaded % NS, loaded);
+            ++loaded;
+        }
+        asm volatile("cp.async.commit_group;\n" ::: "memory");
+    }
+    asm volatile("cp.async.wait_all;\n" ::: "memory");
+    bool any = __syncthreads_or(bad);
+    if (!any) {
+        if (!mbar_wait(used((nk - 1) % NS), (uint32_t)(((nk - 1) / NS) & 1))) give_up(5);
+        any = __syncthreads_or(bad);
+    }
+    if (any) {  // copies of B slices started but never waited for land before the CTA leaves
+        if (tid == 0)
+            for (int kt = 0; kt < loaded; ++kt) mbar_wait(full(kt % NS), (uint32_t)((kt / NS) & 1));
+        __syncthreads();
+    } else {
+        asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+        add_tap(nk - 1);
+        const int row = m0 + 32 * warp + lane;
+        if (row < (MODE == CONV_WEIGHT ? 9 * kConvC : a.P)) {
+            float *o = a.out + ((long long)(MODE == CONV_WEIGHT ? blockIdx.y * (9 * kConvC) : 0) + row) * kConvC;
+#pragma unroll
+            for (int j = 0; j < kConvC; j += 4) {
+                if (MODE == CONV_FORWARD) {
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) sum[j + i] = tanhf(sum[j + i] + a.bias[j + i]);
+                }
+                if (MODE == CONV_BACK) {
+                    const float4 h = *reinterpret_cast<const float4 *>(a.back + (long long)row * kConvC + j);
+                    sum[j] = sum[j] * (1.f - h.x * h.x);
+                    sum[j + 1] = sum[j + 1] * (1.f - h.y * h.y);
+                    sum[j + 2] = sum[j + 2] * (1.f - h.z * h.z);
+                    sum[j + 3] = sum[j + 3] * (1.f - h.w * h.w);
+                }
+                *reinterpret_cast<float4 *>(o + j) = make_float4(sum[j], sum[j + 1], sum[j + 2], sum[j + 3]);
+            }
+            if (MODE != CONV_WEIGHT) {
+                __nv_bfloat16 *ob = a.outb + (long long)row * kConvC;
+#pragma unroll
+                for (int j = 0; j < kConvC; j += 8) {
+                    uint4 u;
+                    __nv_bfloat162 h0 = __floats2bfloat162_rn(sum[j], sum[j + 1]), h1 = __floats2bfloat162_rn(sum[j + 2], sum[j + 3]),
+                                   h2 = __floats2bfloat162_rn(sum[j + 4], sum[j + 5]), h3 = __floats2bfloat162_rn(sum[j + 6], sum[j + 7]);
+                    u.x = *reinterpret_cast<uint32_t *>(&h0);
+                    u.y = *reinterpret_cast<uint32_t *>(&h1);
+                    u.z = *reinterpret_cast<uint32_t *>(&h2);
+                    u.w = *reinterpret_cast<uint32_t *>(&h3);
+                    *reinterpret_cast<uint4 *>(ob + j) = u;
+                }
+            }
+        }
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+    __syncthreads();
+    if (warp == 0)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(kCols) : "memory");
+}
+
+inline size_t conv_smem_bytes() { return 1024 + (size_t)kConvStages * (kConvA + kConvB) + 16 * kConvStages + 16; }
 
 // Stages of the ring: four while they fit beside each other in 128 KB, else two.
 inline int stages_for(int bn) { return 4 * ((size_t)(kTM * kTK * 2) + (size_t)bn * kTK * 2) <= 131072 ? 4 : 2; }
