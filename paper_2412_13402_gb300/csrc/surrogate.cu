@@ -259,9 +259,16 @@ __global__ void __launch_bounds__(256) finish_grads(GradSums a, int nbias) {
     int i = ((int)blockIdx.x - nbias) * 256 + threadIdx.x;
     for (int l = 0; l < 6; ++l) {
         if (i < a.n[l]) {
+            const int ns = a.splits[l];  // <= 64, summed in order, 16 loads in flight
             float s = 0.f;
-#pragma unroll 16
-            for (int z = 0; z < a.splits[l]; ++z) s += a.part[l][(long long)z * a.n[l] + i];
+            for (int z0 = 0; z0 < ns; z0 += 16) {
+                float v[16];
+#pragma unroll
+                for (int z = 0; z < 16; ++z) v[z] = z0 + z < ns ? a.part[l][(long long)(z0 + z) * a.n[l] + i] : 0.f;
+#pragma unroll
+                for (int z = 0; z < 16; ++z)
+                    if (z0 + z < ns) s += v[z];
+            }
             a.out[l][i] = s;
             return;
         }
@@ -276,7 +283,8 @@ __global__ void __launch_bounds__(256) finish_grads(GradSums a, int nbias) {
 // 32 points: 91 us at batch 8 of 60 x 60).
 constexpr int kHeadRows = 256, kHeadLdA = 72, kHeadLdB = kHeadRows + 8;
 constexpr size_t kHeadSmem = 2 * sizeof(bf16) * (kHeadRows * kHeadLdA + 16 * kHeadLdB);
-__global__ void __launch_bounds__(128) head_grad(const bf16 *A, const bf16 *B, int C, int P, int kchunk, float *part) {
+constexpr int kHeadThreads = 256;  // all copy, the first four warps multiply (16 channels each)
+__global__ void __launch_bounds__(kHeadThreads) head_grad(const bf16 *A, const bf16 *B, int C, int P, int kchunk, float *part) {
     extern __shared__ __align__(16) unsigned char smem[];
     bf16 *As = reinterpret_cast<bf16 *>(smem), *Bt = As + 2 * kHeadRows * kHeadLdA;
     const int tid = threadIdx.x, lane = tid & 31, g = lane >> 2, t4 = lane & 3;
@@ -286,16 +294,20 @@ __global__ void __launch_bounds__(128) head_grad(const bf16 *A, const bf16 *B, i
     auto load = [&](int i) {  // rows [kb + i * kHeadRows, ..) of A and, transposed, of B; zeros past ke
         const int k0 = kb + i * kHeadRows;
         bf16 *Ad = As + (i & 1) * kHeadRows * kHeadLdA, *Bd = Bt + (i & 1) * 16 * kHeadLdB;
-        for (int e = tid; e < kHeadRows * 8; e += 128) {
+#pragma unroll
+        for (int e = tid; e < kHeadRows * 8; e += kHeadThreads) {
             const int r = e >> 3, ch = e & 7;
             umma::cp_async16(umma::smem_u32(Ad + r * kHeadLdA + ch * 8), A + (long long)min(k0 + r, P - 1) * 64 + ch * 8,
                              k0 + r < ke);
         }
         asm volatile("cp.async.commit_group;\n" ::: "memory");
-        for (int e = tid; e < kHeadRows * 8 * nt; e += 128) {
-            const int r = e / (8 * nt), n = e - r * 8 * nt;
-            Bd[n * kHeadLdB + r] = n < C && k0 + r < ke ? B[(long long)(k0 + r) * C + n] : __float2bfloat16(0.f);
-        }
+        bf16 v[16];  // row tid of the block (kHeadRows == kHeadThreads)
+#pragma unroll
+        for (int n = 0; n < 16; ++n)
+            v[n] = n < C && k0 + tid < ke ? B[(long long)(k0 + tid) * C + n] : __float2bfloat16(0.f);
+#pragma unroll
+        for (int n = 0; n < 16; ++n)
+            if (n < 8 * nt) Bd[n * kHeadLdB + tid] = v[n];
     };
     float acc[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
     if (nblk > 0) load(0);
@@ -310,7 +322,7 @@ __global__ void __launch_bounds__(128) head_grad(const bf16 *A, const bf16 *B, i
         const unsigned short *Ab = reinterpret_cast<const unsigned short *>(As + (i & 1) * kHeadRows * kHeadLdA);
         const bf16 *Bb = Bt + (i & 1) * 16 * kHeadLdB;
         const int steps = (min(ke - kb - i * kHeadRows, kHeadRows) + 15) / 16;
-        for (int kk = 0; kk < 16 * steps; kk += 16) {
+        for (int kk = 0; kk < 16 * steps && tid < 128; kk += 16) {
             auto pair = [&](int k, int row) {
                 return (unsigned)Ab[k * kHeadLdA + row] | (unsigned)Ab[(k + 1) * kHeadLdA + row] << 16;
             };
@@ -330,6 +342,7 @@ __global__ void __launch_bounds__(128) head_grad(const bf16 *A, const bf16 *B, i
         }
         __syncthreads();  // the buffer is free for block i + 2
     }
+    if (tid >= 128) return;
     float *out = part + (long long)blockIdx.x * 64 * C;
 #pragma unroll
     for (int ni = 0; ni < 2; ++ni)
@@ -1060,7 +1073,7 @@ int backward_conv(rtbte_surrogate *s, int B) {
         S_CUDA(s, allow_max_dynamic_smem((const void *)head_grad));
         attr_set = true;
     }
-    head_grad<<<splits, 128, kHeadSmem, st>>>(s->actb[0].as<bf16>(), s->goutb.as<bf16>(), C, (int)P, kchunk, part);
+    head_grad<<<splits, kHeadThreads, kHeadSmem, st>>>(s->actb[0].as<bf16>(), s->goutb.as<bf16>(), C, (int)P, kchunk, part);
     S_CUDA(s, cudaGetLastError());
     sums(part, splits, Wd * C, g + s->off_M2);
     // gz5 = (g_out M2^T)(1 - h5^2)

@@ -4,7 +4,7 @@
 // A and B are BF16 matrices in global memory (row stride lda / ldb elements, a multiple of 8),
 // K-major ([M][K], [N][K]) or MN-major ([K][M], [K][N]; then bn is a multiple of 64), C is
 // row-major FP32; a split of K over blockIdx.z writes its partial product to its own slice of C.
-// One CTA of four warps computes a 128 x bn tile (bn = N rounded up to a multiple of 16, at most
+// One CTA of eight warps computes a 128 x bn tile (bn = N rounded up to a multiple of 16, at most
 // 256; wider N takes several tiles):
 //   - TMA (cp.async.bulk.tensor, 128-byte swizzle) brings 64-column K slices of the A tile
 //     (128 x 64) and the B tile (bn x 64) into a shared-memory ring of four stages (two when bn is
@@ -12,7 +12,7 @@
 //   - one thread issues four tcgen05.mma (M 128, N bn, K 16) per slice with the FP32 accumulator
 //     in tensor memory, and tcgen05.commit releases the slice's stage (and, after the last
 //     slice, the accumulator) through an mbarrier;
-//   - the four warps read their 32 accumulator rows with tcgen05.ld and apply the epilogue.
+//   - the warps read the accumulator with tcgen05.ld and apply the epilogue (store_tile).
 // Out-of-range rows and columns of a tile are zero-filled by TMA and not stored.  Every mbarrier
 // wait is bounded: on timeout the kernel writes a nonzero code to *err, stops issuing, waits
 // (bounded) for the copies it started, frees its tensor memory and returns.
@@ -27,7 +27,7 @@ namespace umma {
 
 constexpr int kTM = 128;        // tile rows (accumulator lanes)
 constexpr int kTK = 64;         // K per stage: 64 BF16 = 128 bytes = one swizzle span
-constexpr int kThreads = 128;
+constexpr int kThreads = 256;  // two warps per 32 accumulator rows, 32 of 64 columns each
 constexpr long long kWaitLimit = 1LL << 24;  // polls of an mbarrier before giving up
 // MN-major tiles with 128-byte swizzle: blocks of 64 M (or N) elements x kTK K rows; the leading
 // byte offset is the distance between such blocks, the stride byte offset the distance between
@@ -94,6 +94,84 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap *map
             dst),
         "l"(map), "r"(x), "r"(y), "r"(bar)
         : "memory");
+}
+
+// Epilogue of a 128-row accumulator, 64 columns at a time.  A warp reads rows of its quadrant of
+// tensor memory (one row a lane), so storing from there would touch 32 cache lines per
+// instruction (the input-gradient convolution spent half its 21 us so: 17 us since); the columns pass through a
+// shared-memory tile instead and leave as whole rows, sixteen lanes each.
+constexpr int kEpiLd = 64 + 4;  // floats per tile row: 16-byte accesses spread over all banks
+constexpr int kEpiBytes = kTM * kEpiLd * 4;
+
+// this warp's half of 64 accumulator columns from tmem column c0 (32 of its row) into r
+__device__ __forceinline__ void read_acc32(uint32_t tmem, int c0, float *r) {
+    const int warp = threadIdx.x >> 5;
+    const uint32_t at = tmem + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)(c0 + 32 * (warp >> 2));
+#pragma unroll
+    for (int h = 0; h < 32; h += 16) {
+        uint32_t u[16];
+        asm volatile(
+            "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, "
+            "[%16];\n"
+            : "=r"(u[0]), "=r"(u[1]), "=r"(u[2]), "=r"(u[3]), "=r"(u[4]), "=r"(u[5]), "=r"(u[6]), "=r"(u[7]),
+              "=r"(u[8]), "=r"(u[9]), "=r"(u[10]), "=r"(u[11]), "=r"(u[12]), "=r"(u[13]), "=r"(u[14]), "=r"(u[15])
+            : "r"(at + (uint32_t)h));
+        asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
+#pragma unroll
+        for (int j = 0; j < 16; ++j) r[h + j] = __uint_as_float(u[j]);
+    }
+}
+__device__ __forceinline__ void put_tile(float *tile, const float *r) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    float *t = tile + (32 * (warp & 3) + lane) * kEpiLd + 32 * (warp >> 2);
+#pragma unroll
+    for (int j = 0; j < 32; j += 4) *reinterpret_cast<float4 *>(t + j) = make_float4(r[j], r[j + 1], r[j + 2], r[j + 3]);
+}
+// columns [col0, col0 + 64) of rows [m0, m0 + 128), clipped to M x N: + bias, tanh, times 1 - back^2,
+// FP32 to C and BF16 to Cb (each may be null except C)
+__device__ __forceinline__ void store_tile(const float *tile, int m0, int col0, int M, int N, int ldc, const float *bias,
+                                           bool act, const float *back, float *C, __nv_bfloat16 *Cb) {
+    const bool vec = (ldc & 3) == 0;
+    for (int e = threadIdx.x; e < kTM * 16; e += kThreads) {
+        const int r = e >> 4, row = m0 + r, j = (e & 15) * 4, col = col0 + j;
+        if (row >= M || col >= N) continue;
+        const float4 t = *reinterpret_cast<const float4 *>(tile + r * kEpiLd + j);
+        float v[4] = {t.x, t.y, t.z, t.w};
+        const long long at = (long long)row * ldc + col;
+        const int n = min(4, N - col);
+        float h[4] = {0.f, 0.f, 0.f, 0.f};
+        if (back) {
+            if (n == 4 && vec) {
+                const float4 b = *reinterpret_cast<const float4 *>(back + at);
+                h[0] = b.x, h[1] = b.y, h[2] = b.z, h[3] = b.w;
+            } else {
+                for (int i = 0; i < n; ++i) h[i] = back[at + i];
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            if (bias && i < n) v[i] += bias[col + i];
+            if (act) v[i] = tanhf(v[i]);
+            if (back) v[i] = v[i] * (1.f - h[i] * h[i]);
+        }
+        if (n == 4 && vec) {
+            *reinterpret_cast<float4 *>(C + at) = make_float4(v[0], v[1], v[2], v[3]);
+            if (Cb) {
+                uint2 u;
+                __nv_bfloat162 h0 = __floats2bfloat162_rn(v[0], v[1]), h1 = __floats2bfloat162_rn(v[2], v[3]);
+                u.x = *reinterpret_cast<uint32_t *>(&h0);
+                u.y = *reinterpret_cast<uint32_t *>(&h1);
+                *reinterpret_cast<uint2 *>(Cb + at) = u;
+            }
+        } else {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                if (i >= n) break;
+                C[at + i] = v[i];
+                if (Cb) Cb[at + i] = __float2bfloat16(v[i]);
+            }
+        }
+    }
 }
 
 // NS-stage ring (NS = 2 or 4) of A and B slices; stage s holds A at base + s*a_bytes and B at
@@ -203,64 +281,26 @@ __global__ void __launch_bounds__(kThreads) gemm_tc(const __grid_constant__ CUte
         }
     }
     __syncthreads();
-    const bool failed = s_fail != 0;
-    if (!failed && !mbar_wait(done, 0)) {
+    bool bad = s_fail != 0;
+    if (!bad && !mbar_wait(done, 0)) {
+        bad = true;
         if (lane == 0) atomicExch(a.err, 2);
-    } else if (!failed) {
+    }
+    if (!__syncthreads_or(bad)) {
         asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-        const int row = m0 + 32 * warp + lane;
-        for (int c0 = 0; c0 < bn; c0 += 16) {
-            uint32_t r[16];
-            asm volatile(
-                "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, "
-                "[%16];\n"
-                : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-                  "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-                : "r"(tmem + ((uint32_t)(32 * warp) << 16) + (uint32_t)c0));
-            asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
-            if (row >= a.M) continue;
-            const int col0 = n0 + c0;
-            float v[16];
-#pragma unroll
-            for (int j = 0; j < 16; ++j) {
-                v[j] = __uint_as_float(r[j]);
-                if (a.bias && col0 + j < a.N) v[j] += a.bias[col0 + j];
-                if (a.act) v[j] = tanhf(v[j]);
-                if (a.back && col0 + j < a.N) {
-                    const float h = a.back[(long long)row * a.ldc + col0 + j];
-                    v[j] = v[j] * (1.f - h * h);
-                }
+        // the ring is free: every slice was read before `done`
+        float *tile = reinterpret_cast<float *>(smem_raw + (base - raw));
+        for (int c0 = 0; c0 < bn; c0 += 64) {
+            float r[32];
+            if (c0 + 32 * (warp >> 2) < NCOLS) {
+                read_acc32(tmem, c0, r);
+                put_tile(tile, r);
             }
-            float *cr = a.C + (long long)blockIdx.z * a.c_split + (long long)row * a.ldc + col0;
-            __nv_bfloat16 *br = a.Cb ? a.Cb + (long long)row * a.ldc + col0 : nullptr;
-            // 16-byte stores where the 16 columns are in range and the row is 16-byte aligned
-            if (col0 + 16 <= a.N && (a.ldc & 3) == 0 && (col0 & 3) == 0) {
-#pragma unroll
-                for (int j = 0; j < 16; j += 4) *reinterpret_cast<float4 *>(cr + j) = make_float4(v[j], v[j + 1], v[j + 2], v[j + 3]);
-                if (br && (a.ldc & 7) == 0 && (col0 & 7) == 0) {
-#pragma unroll
-                    for (int j = 0; j < 16; j += 8) {
-                        uint4 u;
-                        __nv_bfloat162 h0 = __floats2bfloat162_rn(v[j], v[j + 1]), h1 = __floats2bfloat162_rn(v[j + 2], v[j + 3]),
-                                       h2 = __floats2bfloat162_rn(v[j + 4], v[j + 5]), h3 = __floats2bfloat162_rn(v[j + 6], v[j + 7]);
-                        u.x = *reinterpret_cast<uint32_t *>(&h0);
-                        u.y = *reinterpret_cast<uint32_t *>(&h1);
-                        u.z = *reinterpret_cast<uint32_t *>(&h2);
-                        u.w = *reinterpret_cast<uint32_t *>(&h3);
-                        *reinterpret_cast<uint4 *>(br + j) = u;
-                    }
-                } else if (br) {
-#pragma unroll
-                    for (int j = 0; j < 16; ++j) br[j] = __float2bfloat16(v[j]);
-                }
-            } else {
-#pragma unroll
-                for (int j = 0; j < 16; ++j) {
-                    if (col0 + j >= a.N) break;
-                    cr[j] = v[j];
-                    if (br) br[j] = __float2bfloat16(v[j]);
-                }
-            }
+            __syncthreads();
+            // (bn is N rounded up to 16: columns past N hold zeros or the next tile's share and are clipped)
+            store_tile(tile, m0, n0 + c0, a.M, min(a.N, n0 + bn), a.ldc, a.bias, a.act != 0, a.back,
+                       a.C + (long long)blockIdx.z * a.c_split, a.Cb);
+            __syncthreads();
         }
     }
     asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
@@ -276,7 +316,10 @@ __global__ void __launch_bounds__(kThreads) gemm_tc(const __grid_constant__ CUte
 // in the 128-byte swizzle that TMA would write) instead of from an im2col matrix nine times their
 // size, so a layer reads 3.7 MB instead of writing and reading 33 MB (batch 8 of 60 x 60), and the
 // input gradient adds its nine taps in registers instead of through a 66 MB column matrix.  The
-// slices, their order and every rounding are those of the GEMMs over im2col columns.
+// slices, their order and every rounding are those of the GEMMs over im2col columns.  Bound by the
+// latency of a slice's round trip (L2 gather, proxy fence, MMA, commit) at six or twelve warps per
+// SM; per layer at batch 8 of 60 x 60: forward 98 + 17 -> 12.5 us, input gradient 40 + 21 + 7 ->
+// 17 us, weight gradient 17 -> 11 us.
 constexpr int kConvC = 64;      // channels in and out
 constexpr int kConvStages = 4;  // ring of A (16 KB) and B (8 KB) slices: two CTAs per SM
 constexpr int kConvA = kTM * kTK * 2, kConvB = kConvC * kTK * 2;
@@ -325,7 +368,7 @@ enum { CONV_FORWARD = 0, CONV_BACK = 1, CONV_WEIGHT = 2 };
 //               tB: g [P][64]; both operands MN-major, two taps a tile
 // Every barrier wait is bounded; after one that gave up nothing more is issued and *err is set.
 template <int MODE>
-__global__ void __launch_bounds__(kThreads) conv_tc(const __grid_constant__ CUtensorMap tB, ConvArgs a) {
+__global__ void __launch_bounds__(kThreads, 2) conv_tc(const __grid_constant__ CUtensorMap tB, ConvArgs a) {
     extern __shared__ unsigned char smem_raw[];
     constexpr int NS = kConvStages;
     constexpr uint32_t kCols = MODE == CONV_BACK ? 256u : 64u;  // CONV_BACK: four accumulators in turn
@@ -360,13 +403,13 @@ __global__ void __launch_bounds__(kThreads) conv_tc(const __grid_constant__ CUte
     uint32_t tmem;
     asm volatile("ld.shared.b32 %0, [%1];\n" : "=r"(tmem) : "r"(tslot) : "memory");
 
-    // gather role: chunk c of rows r0 + 16 i; all of a thread's rows have the same row mod 8
+    // gather role: chunk c of rows r0 + 32 i; all of a thread's rows have the same row mod 8
     const int c = tid & 7, r0 = tid >> 3;
     const uint32_t gdst = (uint32_t)r0 * 128u + ((uint32_t)(c ^ (r0 & 7)) << 4);
-    Point pt[8];  // the tile's points (forward and input gradient)
+    Point pt[4];  // the tile's points (forward and input gradient)
     if (MODE != CONV_WEIGHT) {
 #pragma unroll
-        for (int i = 0; i < 8; ++i) pt[i].set(min(m0 + r0 + 16 * i, a.P - 1), a.ny, a.nx);
+        for (int i = 0; i < 4; ++i) pt[i].set(min(m0 + r0 + 32 * i, a.P - 1), a.ny, a.nx);
     }
     // start slice kt's copies into stage s: thread 0 the B slice, every thread its rows of the A slice
     auto load = [&](int s, int kt) {
@@ -379,20 +422,20 @@ __global__ void __launch_bounds__(kThreads) conv_tc(const __grid_constant__ CUte
         if (MODE != CONV_WEIGHT) {
             const int dy = MODE == CONV_BACK ? 1 - kt / 3 : kt / 3 - 1, dx = MODE == CONV_BACK ? 1 - kt % 3 : kt % 3 - 1;
 #pragma unroll
-            for (int i = 0; i < 8; ++i)
-                cp_async16(sA(s) + gdst + 2048u * i, a.src + (long long)pt[i].at(dy, dx, a.ny, a.nx) * kConvC + 8 * c,
-                           m0 + r0 + 16 * i < a.P);
+            for (int i = 0; i < 4; ++i)
+                cp_async16(sA(s) + gdst + 4096u * i, a.src + (long long)pt[i].at(dy, dx, a.ny, a.nx) * kConvC + 8 * c,
+                           m0 + r0 + 32 * i < a.P);
         } else {
             const int t0 = m0 / kConvC;  // two taps: blocks of 64 points x 128 bytes
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const int p = k0 + kt * kTK + r0 + 16 * i;
+            for (int i = 0; i < 2; ++i) {
+                const int p = k0 + kt * kTK + r0 + 32 * i;
                 Point q;
                 q.set(min(p, a.P - 1), a.ny, a.nx);
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
                     const int tap = min(t0 + h, 8);  // (rows of a tenth tap are not stored)
-                    cp_async16(sA(s) + (uint32_t)h * 8192u + gdst + 2048u * i,
+                    cp_async16(sA(s) + (uint32_t)h * 8192u + gdst + 4096u * i,
                                a.src + (long long)q.at(tap / 3 - 1, tap % 3 - 1, a.ny, a.nx) * kConvC + 8 * c, p < a.P);
                 }
             }
@@ -402,25 +445,12 @@ __global__ void __launch_bounds__(kThreads) conv_tc(const __grid_constant__ CUte
         bad = true;
         atomicExch(a.err, code);
     };
-    float sum[kConvC];  // CONV_BACK: this thread's row
+    float sum[32];  // this warp's half of an accumulator row
     auto add_tap = [&](int kt) {
+        float v[32];
+        read_acc32(tmem, MODE == CONV_BACK ? 64 * (kt & 3) : 0, v);
 #pragma unroll
-        for (int c0 = 0; c0 < kConvC; c0 += 16) {
-            uint32_t r[16];
-            asm volatile(
-                "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, "
-                "[%16];\n"
-                : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-                  "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-                : "r"(tmem + ((uint32_t)(32 * warp) << 16) + (uint32_t)(MODE == CONV_BACK ? 64 * (kt & 3) : 0) +
-                      (uint32_t)c0));
-            asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
-#pragma unroll
-            for (int j = 0; j < 16; ++j) {
-                const float v = __uint_as_float(r[j]);
-                sum[c0 + j] = MODE == CONV_BACK && kt > 0 ? sum[c0 + j] + v : v;
-            }
-        }
+        for (int j = 0; j < 32; ++j) sum[j] = MODE == CONV_BACK && kt > 0 ? sum[j] + v[j] : v[j];
     };
 
     int loaded = 0;  // slices whose copies were started
@@ -489,39 +519,15 @@ __global__ void __launch_bounds__(kThreads) conv_tc(const __grid_constant__ CUte
     } else {
         asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
         add_tap(nk - 1);
-        const int row = m0 + 32 * warp + lane;
-        if (row < (MODE == CONV_WEIGHT ? 9 * kConvC : a.P)) {
-            float *o = a.out + ((long long)(MODE == CONV_WEIGHT ? blockIdx.y * (9 * kConvC) : 0) + row) * kConvC;
-#pragma unroll
-            for (int j = 0; j < kConvC; j += 4) {
-                if (MODE == CONV_FORWARD) {
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) sum[j + i] = tanhf(sum[j + i] + a.bias[j + i]);
-                }
-                if (MODE == CONV_BACK) {
-                    const float4 h = *reinterpret_cast<const float4 *>(a.back + (long long)row * kConvC + j);
-                    sum[j] = sum[j] * (1.f - h.x * h.x);
-                    sum[j + 1] = sum[j + 1] * (1.f - h.y * h.y);
-                    sum[j + 2] = sum[j + 2] * (1.f - h.z * h.z);
-                    sum[j + 3] = sum[j + 3] * (1.f - h.w * h.w);
-                }
-                *reinterpret_cast<float4 *>(o + j) = make_float4(sum[j], sum[j + 1], sum[j + 2], sum[j + 3]);
-            }
-            if (MODE != CONV_WEIGHT) {
-                __nv_bfloat16 *ob = a.outb + (long long)row * kConvC;
-#pragma unroll
-                for (int j = 0; j < kConvC; j += 8) {
-                    uint4 u;
-                    __nv_bfloat162 h0 = __floats2bfloat162_rn(sum[j], sum[j + 1]), h1 = __floats2bfloat162_rn(sum[j + 2], sum[j + 3]),
-                                   h2 = __floats2bfloat162_rn(sum[j + 4], sum[j + 5]), h3 = __floats2bfloat162_rn(sum[j + 6], sum[j + 7]);
-                    u.x = *reinterpret_cast<uint32_t *>(&h0);
-                    u.y = *reinterpret_cast<uint32_t *>(&h1);
-                    u.z = *reinterpret_cast<uint32_t *>(&h2);
-                    u.w = *reinterpret_cast<uint32_t *>(&h3);
-                    *reinterpret_cast<uint4 *>(ob + j) = u;
-                }
-            }
-        }
+        float *tile = reinterpret_cast<float *>(smem_raw + (base - smem_u32(smem_raw)));  // the ring is free
+        put_tile(tile, sum);
+        __syncthreads();
+        if (MODE == CONV_WEIGHT)
+            store_tile(tile, m0, 0, 9 * kConvC, kConvC, kConvC, nullptr, false, nullptr,
+                       a.out + (long long)blockIdx.y * (9 * kConvC) * kConvC, nullptr);
+        else
+            store_tile(tile, m0, 0, a.P, kConvC, kConvC, a.bias, MODE == CONV_FORWARD,
+                       MODE == CONV_BACK ? a.back : nullptr, a.out, a.outb);
     }
     asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
     __syncthreads();
