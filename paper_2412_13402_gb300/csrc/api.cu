@@ -378,6 +378,17 @@ int ensure_plan(rtbte_ctx *ctx) {
     return RTBTE_OK;
 }
 
+// RHS of a device state: one launch for a small instance, else populations, collision sums and
+// rows.  (The one launch reads y while it writes ydot, so overlapping vectors take the three.)
+int device_rhs(rtbte_ctx *ctx, const double *y, double *ydot, unsigned parts) {
+    if (ctx->small_grid > 0 && (y + ctx->n_y <= ydot || ydot + ctx->n_y <= y))
+        return launch_small_rhs(ctx, parts, y, ydot, ctx->stream);
+    int rc;
+    if ((rc = launch_prep_from_y(ctx, y, ctx->stream))) return rc;
+    if ((rc = launch_rhs_core(ctx, parts, nullptr, ctx->stream))) return rc;
+    return launch_rows(ctx, parts, ydot, nullptr, ctx->stream);
+}
+
 }  // namespace
 }  // namespace rtbte
 
@@ -518,18 +529,12 @@ int rtbte_rhs(rtbte_ctx *ctx, double t, const double *y, double *ydot, unsigned 
     if ((rc = ensure_plan(ctx))) return rc;
     const bool dy = ptr_is_device(y), dd = ptr_is_device(ydot);
     if (dy != dd) return fail(ctx, RTBTE_E_INVALID_ARG, "y and ydot must both be device or both be host pointers");
-    if (dy) {
-        if ((rc = launch_prep_from_y(ctx, y, ctx->stream))) return rc;
-        if ((rc = launch_rhs_core(ctx, parts, nullptr, ctx->stream))) return rc;
-        return launch_rows(ctx, parts, ydot, nullptr, ctx->stream);
-    }
+    if (dy) return device_rhs(ctx, y, ydot, parts);
     const size_t nb = sizeof(double) * ctx->n_y;
     if (!ctx->ystage.p && (rc = dev_alloc(ctx, ctx->ystage, nb, false))) return rc;
     if (!ctx->ydstage.p && (rc = dev_alloc(ctx, ctx->ydstage, nb, false))) return rc;
     RT_CUDA(ctx, cudaMemcpyAsync(ctx->ystage.p, y, nb, cudaMemcpyHostToDevice, ctx->stream));
-    if ((rc = launch_prep_from_y(ctx, ctx->ystage.as<double>(), ctx->stream))) return rc;
-    if ((rc = launch_rhs_core(ctx, parts, nullptr, ctx->stream))) return rc;
-    if ((rc = launch_rows(ctx, parts, ctx->ydstage.as<double>(), nullptr, ctx->stream))) return rc;
+    if ((rc = device_rhs(ctx, ctx->ystage.as<double>(), ctx->ydstage.as<double>(), parts))) return rc;
     RT_CUDA(ctx, cudaMemcpyAsync(ydot, ctx->ydstage.p, nb, cudaMemcpyDeviceToHost, ctx->stream));
     RT_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
     return RTBTE_OK;
@@ -751,7 +756,8 @@ void rtbte_destroy(rtbte_ctx *ctx) {
     DevBuf *bufs[] = {&ctx->popf, &ctx->popN, &ctx->popP, &ctx->instdev, &ctx->compact, &ctx->items, &ctx->groups,
                       &ctx->partials, &ctx->rowoff, &ctx->rowmid, &ctx->gwt, &ctx->dyn_tab, &ctx->Y[0], &ctx->Y[1],
                       &ctx->K, &ctx->Fs, &ctx->forcing, &ctx->wrms_part, &ctx->ctl, &ctx->ystage, &ctx->ydstage,
-                      &ctx->range_scratch, &ctx->slow_save};
+                      &ctx->range_scratch, &ctx->slow_save, &ctx->small_items, &ctx->small_runs, &ctx->small_rows,
+                      &ctx->small_off, &ctx->small_pops, &ctx->small_sync};
     for (DevBuf *b : bufs) b->release();
     for (auto &pr : ctx->ev_pending) {
         ctx->ev_pool.push_back(pr.first);
@@ -759,6 +765,7 @@ void rtbte_destroy(rtbte_ctx *ctx) {
     }
     for (cudaEvent_t e : ctx->ev_pool) cudaEventDestroy(e);
     if (ctx->ctl_host) cudaFreeHost(ctx->ctl_host);
+    if (ctx->small_sync_host) cudaFreeHost(ctx->small_sync_host);
     if (ctx->cap_stream) cudaStreamDestroy(ctx->cap_stream);
     delete ctx;
 }

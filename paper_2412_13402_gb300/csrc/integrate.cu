@@ -26,14 +26,13 @@
 
 #include "internal.cuh"
 #include "rows.cuh"
+#include "step.cuh"
 
 namespace rtbte {
 
 RowParams row_params(rtbte_ctx *ctx);
 
 namespace {
-
-constexpr int kRedThreads = 256;
 
 // ---- Butcher tableaux (as exact fractions in double) --------------------------------
 Tableau tableau_of(int method) {
@@ -82,67 +81,6 @@ Mis mis_kw3() {
         for (int j = 0; j < 3; ++j) M.Om[i][j] = A[i][j] - A[i - 1][j];
     for (int j = 0; j < 3; ++j) M.Om[3][j] = b[j] - A[2][j];
     return M;
-}
-
-struct StageArgs {
-    Tableau T;
-    CtlParams cp;
-    Ctl *ctl;  // one controller per instance
-    double *Y0, *Y1, *K;
-    const double *forcing;
-    double *wsq;  // per-row squared weighted error of the last stage
-    unsigned long long *range;  // per instance: rows of the attempted state out of range
-    long long n;
-    unsigned parts;
-    int stage;         // -1: populations <- y; 0..S-1: combine stage `stage`
-    int respect_done;  // inside an attempt sequence: skip instances whose integration is done
-    int batched;       // several instances: rows visited by row blocks of active instances only
-};
-
-__device__ __forceinline__ double atol_of(const CtlParams &cp, const InstDev &I, long long local) {
-    return local < I.n_c ? cp.atol_c : cp.atol_ph;
-}
-
-template <class R>
-__device__ __forceinline__ void stage_row(const RowParams &Q, const StageArgs &a, int ii, const InstDev &I, long long c) {
-    const int S = a.T.S, i = a.stage;
-    const Ctl *C = a.ctl + ii;
-    const long long local = c - I.y_off;
-    const double *y = C->cur ? a.Y1 : a.Y0;
-    if (i < 0) {
-        write_pops<R>(Q, I, local, y[c]);
-        return;
-    }
-    const double h = C->h_try;
-    double k = row_value<R>(Q, I, local, a.parts);
-    if (a.forcing) k += a.forcing[c];
-    a.K[(long long)i * a.n + c] = k;
-    if (i < S - 1) {
-        double acc = 0.0;
-        for (int j = 0; j <= i; ++j) acc += a.T.A[i + 1][j] * a.K[(long long)j * a.n + c];
-        write_pops<R>(Q, I, local, (R)(y[c] + h * acc));
-    } else {
-        double s1 = 0.0, s2 = 0.0;
-        for (int j = 0; j < S; ++j) {
-            const double kj = a.K[(long long)j * a.n + c];
-            s1 += a.T.b[j] * kj;
-            s2 += (a.T.b[j] - a.T.bt[j]) * kj;
-        }
-        const double ynew = y[c] + h * s1;
-        (C->cur ? a.Y0 : a.Y1)[c] = ynew;
-        // populations outside their physical range (f in [0,1], N >= 0) beyond the absolute
-        // tolerance: counted per attempt, added to the instance's total if it is accepted
-        const bool out = local < I.n_c ? (ynew < -a.cp.atol_c || ynew > 1.0 + a.cp.atol_c) : (ynew < -a.cp.atol_ph);
-        if (out && a.range) atomicAdd(a.range + ii, 1ULL);
-        double x2 = 0.0;
-        if (a.T.has_emb) {  // error weight and weighted error in FP64 (step acceptance reads them)
-            const double w = 1.0 / (a.cp.rtol * fabs(y[c]) + atol_of(a.cp, I, local));
-            const double x = h * s2 * w;
-            x2 = x * x;
-        }
-        if (!isfinite(ynew)) x2 = __longlong_as_double(0x7ff8000000000000LL);
-        a.wsq[c] = x2;
-    }
 }
 
 // Exclusive prefix of v over the threads of the block (thread order); *total = the block's sum.
@@ -220,37 +158,6 @@ __global__ void __launch_bounds__(kRedThreads) stage_kernel(RowParams Q, StageAr
     }
 }
 
-// Fixed-order sum of v[b .. b+n) by one block: strided per-thread sums, a butterfly within each
-// warp (both partners of a pair add the same two values, so every lane holds the same bits), then
-// the warp sums in warp order.  Every thread returns the sum.
-__device__ double block_sum(const double *v, long long b, long long n) {
-    __shared__ double ws[kRedThreads / 32];
-    double acc = 0.0;
-    for (long long r = threadIdx.x; r < n; r += blockDim.x) acc += v[b + r];
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if ((threadIdx.x & 31) == 0) ws[threadIdx.x >> 5] = acc;
-    __syncthreads();
-    double r = 0.0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) r += ws[w];
-    __syncthreads();  // ws is free for the next call
-    return r;
-}
-
-__device__ __forceinline__ void arm(Ctl *c) {
-    double hk = c->h;
-    c->last = 0;
-    if (c->fixed) {  // classical fixed steps: last step ends exactly at t_out
-        c->last = (c->steps + 1 >= c->max_steps) ? 1 : 0;
-        c->h_try = c->last ? c->t_out - c->t : hk;
-        return;
-    }
-    if (c->t + hk >= c->t_out) {
-        hk = c->t_out - c->t;
-        c->last = 1;
-    }
-    c->h_try = hk;
-}
-
 // One block per instance: WRMS norm (Eq. wrms_norm) of its rows, accept/reject, PID proposal.
 // Per-instance partial sums of a state-size vector: block (c, i) adds chunk c of instance i's
 // rows (fixed chunk boundaries and order, so the norms are deterministic); finished instances
@@ -275,91 +182,10 @@ __global__ void controller_kernel(RowParams Q, Ctl *ctl, CtlParams cp, const dou
     const long long ni = (long long)I.n_c + I.n_ph;
     const double sum = block_sum(part, (long long)blockIdx.x * kWrmsChunks, kWrmsChunks);
     if (threadIdx.x >= 32) return;
-    const double eps = sqrt(sum / (double)ni);
-    // logarithms of the three PID factors, one per lane, ahead of the scalar logic of thread 0:
-    // FP64 transcendental functions are slow in a single thread on this GPU, and the three are
-    // independent (lane 0: the floored error norm, lanes 1-2: the two previous ones)
-    double lg = 0.0;
-    if (threadIdx.x < 3) lg = log(threadIdx.x == 0 ? fmax(eps, 1e-10) : threadIdx.x == 1 ? c->eps1 : c->eps2);
-    const double lg1 = __shfl_sync(0xffffffffu, lg, 1), lg2 = __shfl_sync(0xffffffffu, lg, 2);
-    if (threadIdx.x != 0) return;
-    const double lg0 = lg;
     const unsigned long long nr = range[blockIdx.x];
-    range[blockIdx.x] = 0;
-    c->attempts++;
-    if (!isfinite(eps)) {
-        c->status = RTBTE_E_NONFINITE;
-        c->done = 1;
-        return;
-    }
-    if (c->fixed) {
-        c->cur ^= 1;
-        c->t = c->last ? c->t_out : c->t + c->h_try;
-        c->steps++;
-        c->range_viol += (long long)nr;
-        c->h_last = c->h_try;
-        if (c->last) c->done = 1;
-        else arm(c);
-        return;
-    }
-    const double p = (double)cp.p;
-    c->eps = eps;
-    if (eps <= 1.0) {
-        c->cur ^= 1;
-        c->t = c->last ? c->t_out : c->t + c->h_try;
-        c->steps++;
-        c->range_viol += (long long)nr;
-        const double e = eps > 1e-10 ? eps : 1e-10;
-        // e^(-a1/p) eps1^(+-a2/p) eps2^(-a3/p) as one exponential of the lanes' logarithms
-        const double x2 = cp.pid_sign_mode == 0 ? cp.a2 / p : -cp.a2 / p;
-        double eta = exp((-cp.a1 / p) * lg0 + x2 * lg1 + (-cp.a3 / p) * lg2);
-        eta *= cp.safety;
-        double cap = c->first ? cp.growth_first : cp.growth;
-        if (c->nef > 0 && cap > 1.0) cap = 1.0;
-        if (eta > cap) eta = cap;
-        double h = c->h_try * eta;
-        if (cp.hmax > 0 && h > cp.hmax) h = cp.hmax;
-        c->h = h;
-        c->eps2 = c->eps1;
-        c->eps1 = e;
-        c->first = 0;
-        c->nef = 0;
-        c->h_last = c->h_try;
-        if (c->t >= c->t_out) {
-            c->done = 1;
-            return;
-        }
-        if (!(c->t + h > c->t)) {  // the proposed step no longer advances time
-            c->status = RTBTE_E_STEP_UNDERFLOW;
-            c->done = 1;
-            return;
-        }
-        if (c->steps - c->steps_base >= c->max_steps) {
-            c->status = RTBTE_E_TOO_MANY_STEPS;
-            c->done = 1;
-            return;
-        }
-    } else {
-        c->fails++;
-        c->nef++;
-        if (c->nef >= cp.max_nef) {
-            c->status = RTBTE_E_ERR_TEST_FAIL;
-            c->done = 1;
-            return;
-        }
-        double eta = cp.safety * exp((-1.0 / p) * lg0);  // eps^(-1/p); eps > 1 here, so lg0 = log(eps)
-        if (eta < cp.etamin) eta = cp.etamin;
-        if (eta > 1.0) eta = 1.0;
-        if (c->nef >= cp.small_nef && eta > cp.etamxf) eta = cp.etamxf;
-        const double h = c->h_try * eta;
-        c->h = h;
-        if (h < cp.hmin || !(c->t + h > c->t)) {
-            c->status = RTBTE_E_STEP_UNDERFLOW;
-            c->done = 1;
-            return;
-        }
-    }
-    arm(c);
+    __syncwarp();
+    if (threadIdx.x == 0) range[blockIdx.x] = 0;
+    control(c, cp, sum, ni, nr);
 }
 
 // ---- Hairer-Norsett-Wanner starting step, per instance --------------------------------
@@ -693,6 +519,17 @@ int run_attempts(rtbte_ctx *ctx, int method, const CtlParams &cp, unsigned parts
         if (attempts_out) *attempts_out = sum_attempts(ctx) - a0;
         return RTBTE_OK;
     }
+    if (ctx->small_grid > 0) {  // a small instance: up to cap attempts in one launch
+        const StageArgs a = stage_args(ctx, tableau_of(method), cp, parts, forcing);
+        for (;;) {
+            if ((rc = launch_small_attempts(ctx, &a, cap, ctx->stream)) || (rc = read_small(ctx))) return rc;
+            if ((rc = read_ctl(ctx))) return rc;
+            if (all_done(ctx)) break;
+            if (small_attempts_run(ctx) <= 0) return fail(ctx, RTBTE_E_TIMEOUT, "a grid barrier gave up");
+        }
+        if (attempts_out) *attempts_out = sum_attempts(ctx) - a0;
+        return RTBTE_OK;
+    }
     cudaGraphExec_t ex;
     int nl;
     if ((rc = attempt_graph(ctx, method, cp, parts, forcing, cap, &ex, &nl))) return rc;
@@ -753,9 +590,10 @@ CtlParams ctl_params(const rtbte_integ *o, int p) {
     cp.rtol = o->rtol;
     cp.atol_c = o->atol_c;
     cp.atol_ph = o->atol_ph;
-    cp.a1 = o->a1;
-    cp.a2 = o->a2;
-    cp.a3 = o->a3;
+    cp.x1 = -o->a1 / (double)p;
+    cp.x2 = o->pid_sign_mode == 0 ? o->a2 / (double)p : -o->a2 / (double)p;
+    cp.x3 = -o->a3 / (double)p;
+    cp.xf = -1.0 / (double)p;
     cp.safety = o->safety > 0 ? o->safety : 0.96;
     cp.growth = o->growth > 0 ? o->growth : 20.0;
     cp.growth_first = o->growth_first > 0 ? o->growth_first : 1e4;
@@ -764,7 +602,6 @@ CtlParams ctl_params(const rtbte_integ *o, int p) {
     cp.hmin = o->hmin;
     cp.hmax = o->hmax;
     cp.p = p;
-    cp.pid_sign_mode = o->pid_sign_mode;
     cp.small_nef = o->small_nef > 0 ? o->small_nef : 2;
     cp.max_nef = o->max_nef > 0 ? o->max_nef : 7;
     return cp;
@@ -947,6 +784,13 @@ int advance_to(rtbte_ctx *ctx, double t_out, double *y, const rtbte_integ *o, rt
         }
         auto slow_exact = [&](double *dst) -> int {
             int r2;
+            if (ctx->small_grid > 0) {
+                if ((r2 = launch_small_rhs(ctx, RTBTE_SLOW, ctx->Y[ctx->ctl_host[0].cur].as<double>(), dst, ctx->stream)))
+                    return r2;
+                st->rhs_slow += NI;
+                st->slow_exact += NI;
+                return RTBTE_OK;
+            }
             if ((r2 = stage(ctx, a, ctx->stream))) return r2;
             if ((r2 = launch_rhs_core(ctx, RTBTE_SLOW, nullptr, ctx->stream))) return r2;
             if ((r2 = launch_rows(ctx, RTBTE_SLOW, dst, nullptr, ctx->stream))) return r2;

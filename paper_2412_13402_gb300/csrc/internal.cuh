@@ -37,7 +37,8 @@ constexpr int kMaxStages = 5;
 constexpr int kWrmsBlocks = 512;
 constexpr int kWrmsChunks = 128;  // per-instance blocks of the WRMS reduction before the controller
 constexpr int kMaxBatch = 1024;  // instances per context (shared-memory tables of the batched kernels)
-constexpr int kLoopCap = 64;     // attempts per launch of an attempt-loop graph (default)
+constexpr int kLoopCap = 64;     // attempts per launch of an attempt loop (default)
+constexpr double kSmallSlots = 1.2e7;  // entry slots up to which a single instance takes the one-launch kernels
 
 enum { PART_EPH = 0, PART_PHE = 1, PART_PP = 2 };
 // Lanes working on one item are chosen per staging group (Group::lanes_log2): 4, 8, 16 or 32 lanes,
@@ -116,8 +117,9 @@ struct LaunchTuning {
 
 struct CtlParams {  // constants of one integration (captured into graphs by value)
     double rtol, atol_c, atol_ph;
-    double a1, a2, a3, safety, growth, growth_first, etamxf, etamin, hmin, hmax;
-    int p, pid_sign_mode, small_nef, max_nef;
+    double x1, x2, x3, xf;  // exponents of the PID proposal: -a1/p, +-a2/p (pid_sign_mode), -a3/p; -1/p
+    double safety, growth, growth_first, etamxf, etamin, hmin, hmax;
+    int p, small_nef, max_nef, pad;
 };
 
 struct Tableau {
@@ -254,6 +256,10 @@ struct rtbte_ctx {
     size_t smem_bytes = 0;
     bool staged = false;
     bool wide = true;  // every group uses whole-warp items (the kernel variant without sub-warps)
+    // one-launch kernels of a small single instance (small.cu); small_grid 0: not taken
+    rtbte::DevBuf small_items, small_runs, small_rows, small_off, small_pops, small_sync;
+    int small_grid = 0, small_max_items = 0, small_max_rows = 0, small_max_runs = 0;
+    void *small_sync_host = nullptr;  // pinned mirror of small_sync
     int num_sms = 0;
     size_t smem_optin = 0;
     // integrator work buffers
@@ -292,6 +298,15 @@ int launch_rhs_core(rtbte_ctx *ctx, unsigned parts, const Ctl *ctl, cudaStream_t
 int launch_rows(rtbte_ctx *ctx, unsigned parts, double *out, const double *forcing, cudaStream_t s);
 int split_tables(rtbte_ctx *ctx);
 int autotune(rtbte_ctx *ctx, unsigned parts, int *chosen);
+int timing_begin(rtbte_ctx *ctx, cudaStream_t s, std::pair<cudaEvent_t, cudaEvent_t> *ev);  // .first null: not timed
+int timing_end(rtbte_ctx *ctx, cudaStream_t s, const std::pair<cudaEvent_t, cudaEvent_t> &ev);
+// small.cu
+int make_small_plan(rtbte_ctx *ctx, const std::vector<ItemRec> &items, const std::vector<Group> &groups,
+                    const std::vector<int> &rowoff, const std::vector<int> &rowmid);
+int launch_small_rhs(rtbte_ctx *ctx, unsigned parts, const double *y, double *ydot, cudaStream_t s);
+int launch_small_attempts(rtbte_ctx *ctx, const void *stage_args, int cap, cudaStream_t s);
+int small_attempts_run(const rtbte_ctx *ctx);  // by the last launch, once its counters were read back
+int read_small(rtbte_ctx *ctx);                // enqueue that read-back
 // integrate.cu
 int advance_to(rtbte_ctx *ctx, double t_out, double *y, const rtbte_integ *opt, rtbte_stats *st);
 void destroy_graphs(rtbte_ctx *ctx);

@@ -1,0 +1,602 @@
+// small.cu -- RHS evaluations and adaptive attempts of small instances in one launch each.
+//
+// The launch sequence of a small instance is latency: three launches for an RHS, fourteen for an
+// attempted Zonneveld step, each a few microseconds for work that would take one.  Where the
+// populations of the single instance of a context fit in shared memory together (f, every mode's
+// N and the sub-lattice N), each CTA can own a set of state rows: it holds a copy of all
+// populations, runs every work item of its rows -- whatever their part and mode -- and sums them
+// itself, so no partial leaves the SM and the only exchange between CTAs is the new populations.
+//   - rhs_small: one launch per RHS, populations straight from y, rows straight to ydot;
+//   - attempts_small: up to `cap` attempted steps per launch on a cooperative grid, two grid
+//     barriers per stage less one: S - 1 to exchange stage populations, one before and one after
+//     the chunk sums of the WRMS norm; every CTA then runs the controller on its own copy.
+// Items, their lanes and entry order, the order of a row's items, the norm's chunks and the
+// controller are those of the launch sequence (collide.cuh, rows.cuh, step.cuh), so both give the
+// same results bit for bit.
+#include <algorithm>
+#include <cstring>
+#include <numeric>
+
+#include "collide.cuh"
+#include "internal.cuh"
+#include "rows.cuh"
+#include "step.cuh"
+
+namespace rtbte {
+
+namespace {
+
+// A run of items of one group that a CTA owns: items [a, b) of the plan's own item array, whose
+// slots index the CTA's partials, with what the item loop needs of the group.
+struct __align__(16) SmallRun {
+    const uint32_t *idx;
+    const void *W;
+    int a, b;
+    short part, sb, pb, lg;
+    int N_at, pad[3];  // e-ph: the mode's first population in the CTA's N
+};
+// A state row that a CTA owns: its partials (ph-e before mid, ph-ph from mid; an electron's all
+// before mid) and where its value goes in the population copies.
+struct __align__(16) SmallRow {
+    int row, p0, mid, p1;
+    int f, N, P, pad;  // index in f / N / the sub-lattice N, or -1
+};
+struct SmallPlan {
+    const SmallRun *runs;  // [CTA][max_runs] (empty runs fill up)
+    const SmallRow *rows;
+    const int *row_off;    // [CTAs + 1]
+    int max_runs, max_items, max_rows;  // largest CTA's
+    int n_f, n_N, n_P;     // populations held: f, all modes' N (mode stride N_q_pad), sub-lattice N
+    const int *pp_full;    // [M] phonon of each sub-lattice state
+};
+
+template <class R> struct SmallMem {  // shared memory of a CTA
+    R *f, *N, *P, *partials;
+    SmallRun *runs;
+    // attempts only:
+    SmallRow *rows;
+    double *y;  // [2][max_rows] state of the owned rows: current and attempted, in turn
+    double *K;  // [stages][max_rows]
+    __device__ __forceinline__ SmallMem(unsigned char *raw, const SmallPlan &S) {
+        runs = reinterpret_cast<SmallRun *>(raw);
+        f = reinterpret_cast<R *>(runs + S.max_runs);
+        N = f + S.n_f;
+        P = N + S.n_N;
+        partials = P + S.n_P;
+        rows = reinterpret_cast<SmallRow *>(partials + S.max_items);
+        y = reinterpret_cast<double *>(rows + S.max_rows);
+        K = y + 2 * S.max_rows;
+    }
+};
+size_t small_smem(size_t R, const SmallPlan &S, bool attempts) {  // every array a multiple of 16 bytes
+    return sizeof(SmallRun) * S.max_runs + R * (size_t)(S.n_f + S.n_N + S.n_P + S.max_items) +
+           (attempts ? (sizeof(SmallRow) + sizeof(double) * (2 + kMaxStages)) * S.max_rows : 0);
+}
+
+template <class T> __device__ __forceinline__ void copy_in(T *dst, const T *src, int n) {  // 16-byte units
+    const int m = n * (int)(sizeof(T) / 16);
+    for (int i = threadIdx.x; i < m; i += blockDim.x)
+        reinterpret_cast<int4 *>(dst)[i] = __ldg(reinterpret_cast<const int4 *>(src) + i);
+}
+
+// Every item of this CTA's rows whose part is in the mask, by `nwarps` warps of which this is
+// number `warp`.  Warps take packets in turn across the runs, so short runs do not all fall to the
+// first warps.
+template <class R, bool CACHED>
+__device__ __forceinline__ void own_items(const KParams &P, const SmallPlan &S, const SmallMem<R> &M, unsigned parts,
+                                          int warp, int nwarps) {
+    const int lane = threadIdx.x & 31;
+    KParams L = P;
+    L.partials = M.partials;
+    for (int u = 0; u < S.max_runs; ++u) {
+        const SmallRun &run = M.runs[u];
+        const int a = run.a, b = run.b;
+        if (a >= b || !(parts & (1u << run.part))) continue;
+        GroupView<R> V;
+        V.idx = run.idx;
+        V.W = reinterpret_cast<const R *>(run.W);
+        V.part = run.part;
+        V.sb = run.sb;
+        V.pb = run.pb;
+        V.lg = run.lg;
+        V.s0 = V.part == PART_PP ? M.P : M.f;
+        V.s1 = M.N + run.N_at;
+        V.Nglob = M.N;
+        run_range<R, false, CACHED>(L, V, a, b, warp, nwarps, lane);
+        const int packets = (b - a + (32 >> V.lg) - 1) >> (5 - V.lg);
+        warp -= packets;
+        while (warp < 0) warp += nwarps;
+    }
+}
+
+// RHS value of an owned row from the CTA's partials (row_value of rows.cuh).
+template <class R>
+__device__ __forceinline__ double own_row(const R *partials, const SmallRow &row, unsigned parts) {
+    RowAcc<R> A;
+    auto sum = [&](int i0, int i1) {
+        for (int i = i0; i < i1; ++i) A.add(partials[i]);
+    };
+    if (row.f >= 0) {
+        if (!(parts & RTBTE_EPH)) return 0.0;
+        sum(row.p0, row.p1);
+        return -A.value();
+    }
+    if (parts & RTBTE_PHE) sum(row.p0, row.mid);
+    if (parts & RTBTE_PHPH) sum(row.mid, row.p1);
+    return -A.value();
+}
+
+// One RHS of the state y (FP64): populations converted into shared memory, own items, own rows.
+template <class R, int NT>
+__global__ void __launch_bounds__(NT) rhs_small(KParams P, SmallPlan S, const InstDev *inst, unsigned parts,
+                                                const double *y, double *ydot) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const SmallMem<R> M(smem_raw, S);
+    copy_in(M.runs, S.runs + (long long)blockIdx.x * S.max_runs, S.max_runs);
+    const int r0 = __ldg(S.row_off + blockIdx.x) + threadIdx.x, r1 = __ldg(S.row_off + blockIdx.x + 1);
+    const InstDev I = *inst;
+    for (int i = threadIdx.x; i < I.n_c; i += NT) M.f[i] = (R)y[i];
+    const double *yN = y + I.n_c;
+    if (I.N_q == I.N_q_pad) {
+        for (int p = threadIdx.x; p < I.n_ph; p += NT) M.N[p] = (R)yN[p];
+    } else {
+        for (int p = threadIdx.x; p < I.n_ph; p += NT) {
+            const int nu = p / I.N_q;
+            M.N[nu * I.N_q_pad + (p - nu * I.N_q)] = (R)yN[p];
+        }
+    }
+    if (parts & RTBTE_PHPH)
+        for (int a = threadIdx.x; a < I.M; a += NT) M.P[a] = (R)yN[__ldg(S.pp_full + a)];
+    __syncthreads();
+    own_items<R, false>(P, S, M, parts, threadIdx.x >> 5, NT / 32);
+    __syncthreads();
+    for (int r = r0; r < r1; r += NT) {
+        const SmallRow row = S.rows[r];
+        ydot[row.row] = own_row<R>(M.partials, row, parts);
+    }
+}
+
+// ---- attempt loop ---------------------------------------------------------------------------------
+struct SmallSync {
+    unsigned arrived;          // barrier arrivals so far
+    int failed;                // a barrier wait gave up
+    unsigned long long range;  // rows out of range in all attempts so far
+    int attempts;              // attempts run
+    int pad;
+};
+constexpr int kBarrierPolls = 1 << 22;
+
+// Grid barrier (arrivals reach `target`); false in every thread if the wait gave up.
+__device__ __forceinline__ bool grid_barrier(SmallSync *sync, unsigned target) {
+    __shared__ int s_ok;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        int ok = 0;
+        asm volatile("red.release.gpu.global.add.u32 [%0], 1;\n" ::"l"(&sync->arrived) : "memory");
+        for (int i = 0; i < kBarrierPolls; ++i) {
+            unsigned v;
+            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];\n" : "=r"(v) : "l"(&sync->arrived) : "memory");
+            if ((int)(v - target) >= 0) {
+                ok = 1;
+                break;
+            }
+        }
+        if (!ok) atomicExch(&sync->failed, 1);
+        s_ok = ok;
+    }
+    __syncthreads();
+    return s_ok != 0;
+}
+
+// Population copies of three states: the current one (kept while attempts from it are rejected)
+// and two that the stages alternate between.
+struct SmallPops {
+    void *f[3], *N[3], *P[3];
+};
+
+// Sum of the squared weighted errors of all rows, in the order of wrms_chunks and the controller:
+// 128 chunks of L rows, each by the butterfly of its first warp, then the butterfly of 128.  For
+// L <= 8, by the first four warps, one chunk a thread: of a chunk's 256 strided terms only the
+// first L are not 0, and adding zeros is exact, so its butterfly is a tree over 8 values.  The
+// first warp returns the sum.
+__device__ __forceinline__ double small_wrms(const double *wsq, long long ni, int L) {
+    __shared__ double ws[4];
+    const int t = threadIdx.x;
+    if (t < kWrmsChunks) {
+        double v[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            const long long r = (long long)t * L + j;
+            v[j] = j < L && r < ni ? __ldcg(wsq + r) : 0.0;
+        }
+        double s = ((v[0] + v[4]) + (v[2] + v[6])) + ((v[1] + v[5]) + (v[3] + v[7]));
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if ((t & 31) == 0) ws[t >> 5] = s;
+    }
+    __syncthreads();
+    return t < 32 ? ((ws[0] + ws[1]) + ws[2]) + ws[3] : 0.0;
+}
+
+template <class R, int NT>
+__global__ void __launch_bounds__(NT) attempts_small(KParams P, SmallPlan S, SmallPops B, StageArgs a, double *chunks,
+                                                     int cap, SmallSync *sync) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ Ctl C;
+    __shared__ int s_accept;
+    const SmallMem<R> M(smem_raw, S);
+    const int row0 = __ldg(S.row_off + blockIdx.x), nrows = __ldg(S.row_off + blockIdx.x + 1) - row0;
+    if (threadIdx.x == 0) C = a.ctl[0];
+    copy_in(M.runs, S.runs + (long long)blockIdx.x * S.max_runs, S.max_runs);
+    copy_in(M.rows, S.rows + row0, nrows);
+    __syncthreads();
+    if (C.done) return;  // (alike in every CTA)
+    const long long ni = a.n;
+    const int L = (int)((ni + kWrmsChunks - 1) / kWrmsChunks);  // rows of a chunk
+    const int warp = threadIdx.x >> 5;
+    unsigned barriers = 0;
+    unsigned long long range_seen = 0;
+    int cur = 0, n = 0;  // population set of the current state, attempts run
+    int yc = 0;          // which of M.y is the current state
+    bool ok = true;
+    auto put = [&](int set, const SmallRow &row, R v) {  // into a set of population copies
+        if (row.f >= 0) {
+            reinterpret_cast<R *>(B.f[set])[row.f] = v;
+        } else {
+            reinterpret_cast<R *>(B.N[set])[row.N] = v;
+            if (row.P >= 0) reinterpret_cast<R *>(B.P[set])[row.P] = v;
+        }
+    };
+    {
+        const double *y = C.cur ? a.Y1 : a.Y0;
+        for (int r = threadIdx.x; r < nrows; r += NT) {
+            const double v = y[M.rows[r].row];
+            M.y[r] = v;
+            put(0, M.rows[r], (R)v);
+        }
+        ok = grid_barrier(sync, ++barriers * gridDim.x);
+    }
+    bool pending = false;  // the last attempt's controller runs beside the first stage of the next
+    double sum = 0.0;
+    while (ok) {
+        int in = cur;
+        for (int i = 0; i < a.T.S && ok; ++i) {
+            // This stage's populations (written by every CTA before the last barrier: L2 copies) and
+            // items.  With a controller pending the first warp runs it meanwhile -- its logarithms
+            // and exponential in FP64 take longer than these small sums -- and the others do both.
+            const bool split = i == 0 && pending;
+            if (split && warp == 0) {
+                unsigned long long r = 0;
+                if (threadIdx.x == 0) r = __ldcg(&sync->range);
+                control(&C, a.cp, sum, ni, r - range_seen);
+                if (threadIdx.x == 0) range_seen = r;
+            } else {
+                const int t0 = split ? 32 : 0;
+                stage_part<R>(M.f, reinterpret_cast<const R *>(B.f[in]), S.n_f, t0);
+                stage_part<R>(M.N, reinterpret_cast<const R *>(B.N[in]), S.n_N, t0);
+                if (a.parts & RTBTE_PHPH) stage_part<R>(M.P, reinterpret_cast<const R *>(B.P[in]), S.n_P, t0);
+                asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;\n" ::: "memory");
+                if (split) asm volatile("bar.sync 1, %0;\n" ::"n"(NT - 32) : "memory");
+                else __syncthreads();
+                own_items<R, true>(P, S, M, a.parts, warp - t0 / 32, (NT - t0) / 32);
+            }
+            __syncthreads();
+            if (split) {
+                pending = false;
+                if (C.done || n == cap) {  // that attempt was the last one
+                    ok = false;
+                    break;
+                }
+            }
+            const double h = C.h_try;
+            int out = 0;  // a set neither current nor being read
+            while (out == cur || out == in) ++out;
+            for (int r = threadIdx.x; r < nrows; r += NT) {
+                const SmallRow row = M.rows[r];
+                double k = own_row<R>(M.partials, row, a.parts);
+                if (a.forcing) k += __ldg(a.forcing + row.row);
+                M.K[i * S.max_rows + r] = k;
+                auto K = [&](int j) { return M.K[j * S.max_rows + r]; };
+                const double y = M.y[yc * S.max_rows + r];
+                double z;
+                if (i < a.T.S - 1) {
+                    z = stage_next(a.T, i, h, y, K);
+                } else {
+                    double x2;
+                    bool beyond;
+                    z = stage_last(a, row.f >= 0, h, y, K, &x2, &beyond);
+                    M.y[(yc ^ 1) * S.max_rows + r] = z;
+                    a.wsq[row.row] = x2;
+                    if (beyond) atomicAdd(&sync->range, 1ULL);
+                }
+                put(out, row, (R)z);
+            }
+            in = out;
+            ok = grid_barrier(sync, ++barriers * gridDim.x);
+        }
+        if (!ok) break;
+        if (L <= 8) {
+            sum = small_wrms(a.wsq, ni, L);
+        } else {
+            for (int ch = blockIdx.x; ch < kWrmsChunks; ch += gridDim.x) {
+                const long long b = (long long)ch * L, e = b + L < ni ? b + L : ni;
+                const double s = block_sum<true>(a.wsq, b, e > b ? e - b : 0);
+                if (threadIdx.x == 0) chunks[ch] = s;
+            }
+            if (!(ok = grid_barrier(sync, ++barriers * gridDim.x))) break;
+            sum = small_wrms(chunks, kWrmsChunks, 1);
+        }
+        // accepted or not decides which state the next attempt starts from; the rest of the
+        // controller follows beside its first stage
+        if (warp == 0) {
+            const double eps = sqrt(sum / (double)ni);
+            if (threadIdx.x == 0) s_accept = isfinite(eps) && (C.fixed || eps <= 1.0);
+        }
+        __syncthreads();
+        if (s_accept) {
+            cur = in;
+            yc ^= 1;
+        }
+        pending = true;
+        ++n;
+    }
+    __syncthreads();
+    if (!C.done && n != cap && blockIdx.x == 0 && threadIdx.x == 0) {  // a barrier wait gave up
+        C.status = RTBTE_E_TIMEOUT;
+        C.done = 1;
+    }
+    double *y = C.cur ? a.Y1 : a.Y0;
+    for (int r = threadIdx.x; r < nrows; r += NT) y[M.rows[r].row] = M.y[yc * S.max_rows + r];
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        a.ctl[0] = C;
+        sync->attempts = n;
+    }
+}
+
+constexpr int kSmallThreads = 768, kSmallThreads64 = 512;  // RHS; attempts: kSmallThreads64
+
+KParams small_params(rtbte_ctx *ctx) {
+    KParams P;
+    std::memset(&P, 0, sizeof(P));
+    P.items = ctx->small_items.as<ItemRec>();
+    P.groups = ctx->groups.as<Group>();
+    P.n_groups = ctx->n_groups;
+    return P;
+}
+
+SmallPlan small_plan(rtbte_ctx *ctx) {
+    SmallPlan S;
+    const InstHost &I = ctx->inst[0];
+    S.runs = ctx->small_runs.as<SmallRun>();
+    S.rows = ctx->small_rows.as<SmallRow>();
+    S.row_off = ctx->small_off.as<int>();
+    S.max_runs = ctx->small_max_runs;
+    S.max_items = ctx->small_max_items;
+    S.max_rows = ctx->small_max_rows;
+    S.n_f = I.n_c_pad;
+    S.n_N = I.d.nmodes * I.N_q_pad;
+    S.n_P = I.M_pad;
+    S.pp_full = I.t_ppfull.as<int>();
+    return S;
+}
+
+const void *rhs_fn(const rtbte_ctx *ctx) {
+    return ctx->precision == RTBTE_PREC_FP64 ? (const void *)rhs_small<double, kSmallThreads64>
+                                             : (const void *)rhs_small<float, kSmallThreads>;
+}
+const void *attempts_fn(const rtbte_ctx *ctx) {
+    return ctx->precision == RTBTE_PREC_FP64 ? (const void *)attempts_small<double, kSmallThreads64>
+                                             : (const void *)attempts_small<float, kSmallThreads64>;
+}
+int small_threads(const rtbte_ctx *ctx) {
+    return ctx->precision == RTBTE_PREC_FP64 ? kSmallThreads64 : kSmallThreads;
+}
+
+template <class T> int upload(rtbte_ctx *ctx, DevBuf &b, const std::vector<T> &h) {
+    b.release();
+    RT_CUDA(ctx, cudaMalloc(&b.p, std::max<size_t>(h.size() * sizeof(T), 16)));
+    b.bytes = h.size() * sizeof(T);
+    if (!h.empty()) RT_CUDA(ctx, cudaMemcpyAsync(b.p, h.data(), b.bytes, cudaMemcpyHostToDevice, ctx->stream));
+    return RTBTE_OK;
+}
+
+}  // namespace
+
+// Row ownership of a single small instance, or none (ctx->small_grid = 0).  `items` in launch
+// order with their row-major slots, `rowoff` / `rowmid` the rows' slots.
+int make_small_plan(rtbte_ctx *ctx, const std::vector<ItemRec> &items, const std::vector<Group> &groups,
+                    const std::vector<int> &rowoff, const std::vector<int> &rowmid) {
+    ctx->small_grid = 0;
+    if (ctx->inst.size() != 1 || ctx->sliced || items.empty()) return RTBTE_OK;
+    const InstHost &I = ctx->inst[0];
+    const size_t R = ctx->real_size;
+    const size_t pops = R * ((size_t)I.n_c_pad + (size_t)I.d.nmodes * I.N_q_pad + I.M_pad);
+    double slots = 0;
+    for (const ItemCost &c : ctx->item_cost_h) slots += c.slots;
+    if (pops > 160 * 1024 || slots > kSmallSlots) return RTBTE_OK;
+    const int n = (int)items.size();
+    std::vector<int> by_slot(n), group_of(n);
+    for (size_t g = 0; g < groups.size(); ++g)
+        for (int k = groups[g].item_begin; k < groups[g].item_end; ++k) {
+            by_slot[items[k].slot] = k;
+            group_of[k] = (int)g;
+        }
+    // Rows dealt to the CTAs family by family (electrons, sub-lattice phonons, other phonons: so
+    // every parts mask is spread evenly), back and forth; dearest first where a CTA gets only a few
+    // (many rows average out, and sorting them would cost more than it evens).
+    const int ny = (int)ctx->n_y, nc = I.d.n_c;
+    const int G = (int)std::max(1.0, std::min((double)ctx->num_sms, std::ceil(slots / 64.0)));
+    std::vector<std::vector<int>> own(G);
+    for (auto &o : own) o.reserve(ny / G + 3);
+    int at = 0, dir = 1;
+    std::vector<std::pair<long long, int>> rows_of[3];  // (-cost, row)
+    for (int c = 0; c < ny; ++c) {
+        const int f = c < nc ? 0 : (I.M > 0 && I.compact[c - nc] >= 0 ? 1 : 2);
+        long long cost = 0;
+        if (ny < 32 * G)
+            for (int s = rowoff[c]; s < rowoff[c + 1]; ++s) cost -= ctx->item_cost_h[by_slot[s]].slots;
+        rows_of[f].push_back({cost, c});
+    }
+    for (auto &rows : rows_of) {
+        if (ny < 32 * G) std::sort(rows.begin(), rows.end());
+        for (const auto &r : rows) {
+            own[at].push_back(r.second);
+            at += dir;
+            if (at == G || at < 0) {
+                dir = -dir;
+                at += dir;
+            }
+        }
+    }
+    std::vector<ItemRec> out;
+    std::vector<std::vector<SmallRun>> runs(G);
+    std::vector<SmallRow> rows;
+    std::vector<int> off(G + 1, 0);
+    out.reserve(n);
+    rows.reserve(ny);
+    int max_items = 0, max_rows = 0, max_runs = 0;
+    // a CTA's items by group and, within it, alike ones together (the packets of order_packets in
+    // rhs.cu): counting sort over (group, process, vectors per lane)
+    const int nb = 8 * (int)groups.size();
+    std::vector<int> count(nb + 1), keys;
+    std::vector<ItemRec> mine;
+    for (int b = 0; b < G; ++b) {
+        off[b] = (int)rows.size();
+        mine.clear();
+        keys.clear();
+        std::fill(count.begin(), count.end(), 0);
+        for (int c : own[b]) {
+            SmallRow r{};
+            r.row = c;
+            r.p0 = (int)mine.size();
+            r.mid = r.p0 + rowmid[c] - rowoff[c];
+            for (int s = rowoff[c]; s < rowoff[c + 1]; ++s) {
+                const int k = by_slot[s], g = group_of[k], lanes = ctx->item_cost_h[k].lanes;
+                mine.push_back(items[k]);
+                mine.back().slot = (unsigned)mine.size() - 1;
+                keys.push_back(8 * g + 4 * (mine.back().proc != 0) + 4 - ctx->item_cost_h[k].slots / (4 * lanes));
+                ++count[keys.back() + 1];
+            }
+            r.p1 = (int)mine.size();
+            const int p = c - nc;
+            r.f = c < nc ? c : -1;
+            r.N = c < nc ? -1 : (int)((p / I.N_q) * I.N_q_pad + p % I.N_q);
+            r.P = c < nc || I.M == 0 ? -1 : I.compact[p];
+            rows.push_back(r);
+        }
+        max_items = std::max(max_items, (int)mine.size());
+        max_rows = std::max(max_rows, (int)own[b].size());
+        for (int k = 0; k < nb; ++k) count[k + 1] += count[k];
+        const int base = (int)out.size();
+        for (size_t g = 0; g < groups.size(); ++g) {
+            if (count[8 * (g + 1)] == count[8 * g]) continue;
+            const Group &Q = groups[g];
+            SmallRun r{};
+            r.idx = Q.idx;
+            r.W = Q.W;
+            r.a = base + count[8 * g];
+            r.b = base + count[8 * (g + 1)];
+            r.part = (short)Q.part;
+            r.sb = (short)Q.s_bits;
+            r.pb = (short)Q.pp_bits;
+            r.lg = (short)Q.lanes_log2;
+            r.N_at = Q.nu * Q.n_q_pad;
+            runs[b].push_back(r);
+        }
+        out.resize(base + mine.size());
+        for (size_t k = 0; k < mine.size(); ++k) out[base + count[keys[k]]++] = mine[k];
+        max_runs = std::max(max_runs, (int)runs[b].size());
+    }
+    off[G] = (int)rows.size();
+    std::vector<SmallRun> run_tab((size_t)G * max_runs, SmallRun{});
+    for (int b = 0; b < G; ++b) std::copy(runs[b].begin(), runs[b].end(), run_tab.begin() + (size_t)b * max_runs);
+    ctx->small_max_items = (int)round_up(max_items, 4);
+    ctx->small_max_rows = (int)round_up(max_rows, 2);
+    ctx->small_max_runs = max_runs;
+    int rc;
+    if ((rc = upload(ctx, ctx->small_items, out)) || (rc = upload(ctx, ctx->small_runs, run_tab)) ||
+        (rc = upload(ctx, ctx->small_rows, rows)) || (rc = upload(ctx, ctx->small_off, off)))
+        return rc;
+    ctx->small_grid = G;
+    SmallPlan S = small_plan(ctx);
+    if (small_smem(R, S, true) + 2048 > ctx->smem_optin) {
+        ctx->small_grid = 0;
+        return RTBTE_OK;
+    }
+    for (const void *f : {rhs_fn(ctx), attempts_fn(ctx)}) RT_CUDA(ctx, allow_max_dynamic_smem(f));
+    ctx->small_pops.release();  // (of another plan)
+    RT_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
+    return RTBTE_OK;
+}
+
+int launch_small_rhs(rtbte_ctx *ctx, unsigned parts, const double *y, double *ydot, cudaStream_t s) {
+    KParams P = small_params(ctx);
+    SmallPlan S = small_plan(ctx);
+    const InstDev *inst = ctx->instdev.as<InstDev>();
+    void *args[] = {&P, &S, &inst, &parts, &y, &ydot};
+    std::pair<cudaEvent_t, cudaEvent_t> ev;
+    int rc;
+    if ((rc = timing_begin(ctx, s, &ev))) return rc;
+    RT_CUDA(ctx, cudaLaunchKernel(rhs_fn(ctx), dim3(ctx->small_grid), dim3(small_threads(ctx)), args,
+                                  small_smem(ctx->real_size, S, false), s));
+    ctx->launches++;
+    return timing_end(ctx, s, ev);
+}
+
+int read_small(rtbte_ctx *ctx) {
+    RT_CUDA(ctx, cudaMemcpyAsync(ctx->small_sync_host, ctx->small_sync.p, sizeof(SmallSync), cudaMemcpyDeviceToHost,
+                                 ctx->stream));
+    return RTBTE_OK;
+}
+int small_attempts_run(const rtbte_ctx *ctx) { return reinterpret_cast<const SmallSync *>(ctx->small_sync_host)->attempts; }
+
+namespace {
+// Buffers of the attempt loop, made on its first use.
+int ensure_attempts(rtbte_ctx *ctx) {
+    if (ctx->small_pops.p) return RTBTE_OK;
+    const size_t R = ctx->real_size;
+    // two more sets of population copies beside popf / popN / popP, and the barrier
+    const size_t bf = R * (size_t)(ctx->popf_len + 4), bN = R * (size_t)(ctx->popN_len + 4), bP = R * (size_t)(ctx->popP_len + 4);
+    const size_t al = 256, set = (bf + al - 1) / al * al + (bN + al - 1) / al * al + (bP + al - 1) / al * al;
+    RT_CUDA(ctx, cudaMalloc(&ctx->small_pops.p, 2 * set));
+    ctx->small_pops.bytes = 2 * set;
+    RT_CUDA(ctx, cudaMemsetAsync(ctx->small_pops.p, 0, 2 * set, ctx->stream));
+    if (!ctx->small_sync.p) {
+        RT_CUDA(ctx, cudaMalloc(&ctx->small_sync.p, sizeof(SmallSync)));
+        ctx->small_sync.bytes = sizeof(SmallSync);
+    }
+    if (!ctx->small_sync_host) RT_CUDA(ctx, cudaMallocHost(&ctx->small_sync_host, sizeof(SmallSync)));
+    return RTBTE_OK;
+}
+}  // namespace
+
+int launch_small_attempts(rtbte_ctx *ctx, const void *stage_args, int cap, cudaStream_t s) {
+    int rc;
+    if ((rc = ensure_attempts(ctx))) return rc;
+    KParams P = small_params(ctx);
+    SmallPlan S = small_plan(ctx);
+    StageArgs a = *reinterpret_cast<const StageArgs *>(stage_args);
+    const size_t R = ctx->real_size, al = 256;
+    SmallPops B;
+    B.f[0] = ctx->popf.p;
+    B.N[0] = ctx->popN.p;
+    B.P[0] = ctx->popP.p;
+    char *p = ctx->small_pops.as<char>();
+    for (int k = 1; k < 3; ++k) {
+        B.f[k] = p;
+        p += (R * (size_t)(ctx->popf_len + 4) + al - 1) / al * al;
+        B.N[k] = p;
+        p += (R * (size_t)(ctx->popN_len + 4) + al - 1) / al * al;
+        B.P[k] = p;
+        p += (R * (size_t)(ctx->popP_len + 4) + al - 1) / al * al;
+    }
+    double *chunks = ctx->wrms_part.as<double>() + 2 * ctx->n_y;
+    SmallSync *sync = ctx->small_sync.as<SmallSync>();
+    RT_CUDA(ctx, cudaMemsetAsync(sync, 0, sizeof(SmallSync), s));
+    void *args[] = {&P, &S, &B, &a, &chunks, &cap, &sync};
+    RT_CUDA(ctx, cudaLaunchCooperativeKernel(attempts_fn(ctx), dim3(ctx->small_grid), dim3(kSmallThreads64), args,
+                                             small_smem(R, S, true), s));
+    ctx->launches++;
+    return RTBTE_OK;
+}
+
+}  // namespace rtbte
