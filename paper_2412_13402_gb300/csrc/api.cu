@@ -756,8 +756,7 @@ void rtbte_destroy(rtbte_ctx *ctx) {
     DevBuf *bufs[] = {&ctx->popf, &ctx->popN, &ctx->popP, &ctx->instdev, &ctx->compact, &ctx->items, &ctx->groups,
                       &ctx->partials, &ctx->rowoff, &ctx->rowmid, &ctx->gwt, &ctx->dyn_tab, &ctx->Y[0], &ctx->Y[1],
                       &ctx->K, &ctx->Fs, &ctx->forcing, &ctx->wrms_part, &ctx->ctl, &ctx->ystage, &ctx->ydstage,
-                      &ctx->range_scratch, &ctx->slow_save, &ctx->small_items, &ctx->small_runs, &ctx->small_rows,
-                      &ctx->small_off, &ctx->small_pops, &ctx->small_sync};
+                      &ctx->range_scratch, &ctx->slow_save, &ctx->small_tab, &ctx->small_pops, &ctx->small_sync};
     for (DevBuf *b : bufs) b->release();
     for (auto &pr : ctx->ev_pending) {
         ctx->ev_pool.push_back(pr.first);

@@ -20,8 +20,13 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <algorithm>
+#include <atomic>
 #include <map>
+#include <memory>
 #include <string>
+#include <system_error>
+#include <thread>
 #include <vector>
 
 #include "rtbte.h"
@@ -38,7 +43,6 @@ constexpr int kWrmsBlocks = 512;
 constexpr int kWrmsChunks = 128;  // per-instance blocks of the WRMS reduction before the controller
 constexpr int kMaxBatch = 1024;  // instances per context (shared-memory tables of the batched kernels)
 constexpr int kLoopCap = 64;     // attempts per launch of an attempt loop (default)
-constexpr double kSmallSlots = 1.2e7;  // entry slots up to which a single instance takes the one-launch kernels
 
 enum { PART_EPH = 0, PART_PHE = 1, PART_PP = 2 };
 // Lanes working on one item are chosen per staging group (Group::lanes_log2): 4, 8, 16 or 32 lanes,
@@ -165,6 +169,26 @@ inline cudaError_t allow_max_dynamic_smem(const void *f) {
     return e;
 }
 
+// f(0) .. f(n - 1), over host threads when there is enough to do.  f must not throw; where threads
+// cannot be started the caller does everything itself.
+template <class F> void parallel_for(int n, bool threads, F &&f) {
+    std::atomic<int> next{0};
+    auto work = [&] {
+        for (int i; (i = next.fetch_add(1)) < n;) f(i);
+    };
+    std::thread t[7];
+    int nt = 0;
+    if (threads) {
+        const int want = std::min({7, n - 1, (int)std::thread::hardware_concurrency() - 1});
+        try {
+            for (; nt < want; ++nt) t[nt] = std::thread(work);
+        } catch (const std::system_error &) {
+        }
+    }
+    work();
+    for (int i = 0; i < nt; ++i) t[i].join();
+}
+
 // ---- device buffer ----------------------------------------------------------
 struct DevBuf {
     void *p = nullptr;
@@ -249,7 +273,8 @@ struct rtbte_ctx {
     int grid = 0, per_sm = 1;  // collision kernel: CTAs per SM (1, 2 or 4; threads = threads per SM / per_sm)
     rtbte::LaunchTuning lt[8];  // collision-kernel launch parameters of each parts mask (1..7)
     unsigned lt_tuned = 0;      // masks the autotuner tuned themselves (kept across plans)
-    std::vector<rtbte::ItemCost> item_cost_h;  // cost of each work item (host copy for re-splitting)
+    std::unique_ptr<rtbte::ItemCost[]> item_cost_h;  // cost of each work item (host copy for re-splitting)
+    long long part_slots[3] = {0, 0, 0};             // entry slots of each part's items
     std::vector<int> group_begin_h, group_part_h;  // first item and part of each group (host copies)
     rtbte::DevBuf bound_tab, act_tab, tail_ctr;    // work-unit bounds and group lists per mask; grab/exit counters
     int bound_off[8] = {}, act_off[8] = {}, tail_n[8] = {};  // per mask: first bound, first listed group, dynamic units
@@ -257,7 +282,8 @@ struct rtbte_ctx {
     bool staged = false;
     bool wide = true;  // every group uses whole-warp items (the kernel variant without sub-warps)
     // one-launch kernels of a small single instance (small.cu); small_grid 0: not taken
-    rtbte::DevBuf small_items, small_runs, small_rows, small_off, small_pops, small_sync;
+    rtbte::DevBuf small_tab, small_pops, small_sync;  // small_tab: items, runs, rows, row offsets at small_at[0..3]
+    size_t small_at[4] = {0, 0, 0, 0};
     int small_grid = 0, small_max_items = 0, small_max_rows = 0, small_max_runs = 0;
     void *small_sync_host = nullptr;  // pinned mirror of small_sync
     int num_sms = 0;
@@ -301,7 +327,7 @@ int autotune(rtbte_ctx *ctx, unsigned parts, int *chosen);
 int timing_begin(rtbte_ctx *ctx, cudaStream_t s, std::pair<cudaEvent_t, cudaEvent_t> *ev);  // .first null: not timed
 int timing_end(rtbte_ctx *ctx, cudaStream_t s, const std::pair<cudaEvent_t, cudaEvent_t> &ev);
 // small.cu
-int make_small_plan(rtbte_ctx *ctx, const std::vector<ItemRec> &items, const std::vector<Group> &groups,
+int make_small_plan(rtbte_ctx *ctx, const ItemRec *items, int n, const std::vector<Group> &groups,
                     const std::vector<int> &rowoff, const std::vector<int> &rowmid);
 int launch_small_rhs(rtbte_ctx *ctx, unsigned parts, const double *y, double *ydot, cudaStream_t s);
 int launch_small_attempts(rtbte_ctx *ctx, const void *stage_args, int cap, cudaStream_t s);

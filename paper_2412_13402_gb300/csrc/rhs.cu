@@ -258,13 +258,16 @@ __global__ void rows_kernel(RowParams Q, unsigned parts, double *out, const doub
     }
 }
 
-template <class T> int upload_vec(rtbte_ctx *ctx, DevBuf &b, const std::vector<T> &h) {
+int upload_raw(rtbte_ctx *ctx, DevBuf &b, const void *h, size_t n) {
     b.release();
-    size_t bytes = std::max<size_t>(h.size() * sizeof(T), 16);
+    const size_t bytes = std::max<size_t>(n, 16);
     RT_CUDA(ctx, cudaMalloc(&b.p, bytes));
     b.bytes = bytes;
-    if (!h.empty()) RT_CUDA(ctx, cudaMemcpyAsync(b.p, h.data(), h.size() * sizeof(T), cudaMemcpyHostToDevice, ctx->stream));
+    if (n) RT_CUDA(ctx, cudaMemcpyAsync(b.p, h, n, cudaMemcpyHostToDevice, ctx->stream));
     return RTBTE_OK;
+}
+template <class T> int upload_vec(rtbte_ctx *ctx, DevBuf &b, const std::vector<T> &h) {
+    return upload_raw(ctx, b, h.data(), h.size() * sizeof(T));
 }
 
 // Tables of the device re-split in ctx->dyn_tab: unit bounds, active groups, number of dynamic
@@ -312,100 +315,127 @@ RowParams row_params(rtbte_ctx *ctx) {
 // units of decreasing weight (half the remaining weight per grid, at least 1/40 of a CTA's share,
 // never across a group boundary), taken by CTAs in order at run time.
 int split_tables(rtbte_ctx *ctx) {
-    const int G = ctx->grid;
-    const int n = (int)ctx->item_cost_h.size();
+    const int G = ctx->grid, n = ctx->n_items;
     const int ng = (int)ctx->group_begin_h.size();
+    const ItemCost *cost = ctx->item_cost_h.get();
     auto group_end = [&](int g) { return g + 1 < ng ? ctx->group_begin_h[g + 1] : n; };
-    // prefix of the unscaled weights (32 x slots + w x lanes) over all items, per distinct w
-    std::map<int, std::vector<long long>> prefixes;
-    auto prefix_of = [&](int w) -> const std::vector<long long> & {
-        std::vector<long long> &p = prefixes[w];
+    // sums of the unscaled weights (32 x slots + w x lanes) of blocks of 64 items, per distinct w
+    auto raw = [&](int w, int k) { return 32LL * cost[k].slots + (long long)w * cost[k].lanes; };
+    std::map<int, std::vector<long long>> block_sums;
+    auto blocks_of = [&](int w) -> const std::vector<long long> & {
+        std::vector<long long> &p = block_sums[w];
         if (p.empty()) {
-            p.resize(n + 1);
-            p[0] = 0;
-            for (int k = 0; k < n; ++k)
-                p[k + 1] = p[k] + 32LL * ctx->item_cost_h[k].slots + (long long)w * ctx->item_cost_h[k].lanes;
+            p.resize(n / 64 + 1);
+            parallel_for((n / 64 + 1023) / 1024, n > 500000, [&](int c) {
+                for (int b = 1024 * c; b < std::min(1024 * (c + 1), n / 64); ++b) {
+                    long long s = 0;
+                    for (int k = 64 * b; k < 64 * (b + 1); ++k) s += raw(w, k);
+                    p[b] = s;
+                }
+            });
         }
         return p;
     };
+    auto sum_of = [&](int w, int k0, int k1) {  // items [k0, k1)
+        const std::vector<long long> &p = blocks_of(w);
+        long long s = 0;
+        while (k0 < k1) {
+            if ((k0 & 63) == 0 && k0 + 64 <= k1) {
+                s += p[k0 >> 6];
+                k0 += 64;
+            } else {
+                s += raw(w, k0++);
+            }
+        }
+        return s;
+    };
     auto scale = [](const LaunchTuning &L, int part) { return (long long)(64.0 * L.ps[part] + 0.5); };
+    std::map<int, std::vector<long long>> group_sums;  // raw weight of each group, per w
+    auto groups_of = [&](int w) -> const std::vector<long long> & {
+        std::vector<long long> &p = group_sums[w];
+        if (p.empty()) {
+            p.resize(std::max(ng, 1));
+            for (int g = 0; g < ng; ++g) p[g] = sum_of(w, ctx->group_begin_h[g], group_end(g));
+        }
+        return p;
+    };
     std::vector<int4> bound;
     std::vector<int> act;
+    std::vector<long long> start;  // weight of the mask's items before each of its groups, and the total
     for (unsigned mask = 1; mask <= 7; ++mask) {
         const LaunchTuning &L = ctx->lt[mask];
-        const std::vector<long long> &pre = prefix_of(L.w);
+        const std::vector<long long> &blocks = blocks_of(L.w), &gsum = groups_of(L.w);
         ctx->bound_off[mask] = (int)bound.size();
         ctx->act_off[mask] = (int)act.size();
         const int act0 = (int)act.size();
-        // the mask's parts in order: weight before the part, first and last item
-        long long before[4] = {0, 0, 0, 0};
-        int np = 0, parts[3] = {0, 0, 0};
-        std::vector<int> act_at(ng, -1);
-        for (int part = 0; part < 3; ++part) {
-            if (!(mask & (1u << part)) || ctx->part_items[part] == 0) continue;
-            const int f = ctx->part_first[part], e = f + ctx->part_items[part];
-            before[np + 1] = before[np] + scale(L, part) * (pre[e] - pre[f]);
-            parts[np++] = part;
-        }
+        start.assign(1, 0);
         for (int g = 0; g < ng; ++g) {
             const int part = ctx->group_part_h[g];
             if (!(mask & (1u << part)) || group_end(g) == ctx->group_begin_h[g]) continue;
-            act_at[g] = (int)act.size() - act0;
             act.push_back(g);
+            start.push_back(start.back() + scale(L, part) * gsum[g]);
         }
+        const int na = (int)act.size() - act0;
         act.push_back(-1);
-        const long long total = before[np];
-        const int last = total > 0 ? ctx->part_first[parts[np - 1]] + ctx->part_items[parts[np - 1]] : 0;
-        int g_hint = 0;  // bounds ascend, and so do their groups
-        auto add = [&](int item) {
-            while (g_hint + 1 < ng && ctx->group_begin_h[g_hint + 1] <= item) ++g_hint;
-            bound.push_back(make_int4(item, g_hint, act_at[g_hint] < 0 ? 0 : act_at[g_hint], 0));
+        const long long total = start.back();
+        // a position among the mask's items that moves forward only: item `at` of its group number
+        // `ai`, with weight `before` in front of it (ai == na: past the last item)
+        int ai = 0, at = 0;
+        long long before = 0;
+        auto enter = [&](int k) {
+            ai = k;
+            before = start[k];
+            at = k < na ? ctx->group_begin_h[act[act0 + k]] : group_end(act[act0 + na - 1]);
         };
-        // first item at or after weight t
-        auto item_at = [&](long long t) {
-            int q = 0;
-            while (q + 1 < np && before[q + 1] <= t) ++q;
-            const int f = ctx->part_first[parts[q]], e = f + ctx->part_items[parts[q]];
-            const long long want = pre[f] + (t - before[q] + scale(L, parts[q]) - 1) / scale(L, parts[q]);
-            const int k = (int)(std::lower_bound(pre.begin() + f, pre.begin() + e, want) - pre.begin());
-            return k < e ? k : (q + 1 < np ? ctx->part_first[parts[q + 1]] : last);
-        };
-        auto weight_at = [&](int item) {  // weight before an item of the mask
-            for (int q = 0; q < np; ++q) {
-                const int f = ctx->part_first[parts[q]], e = f + ctx->part_items[parts[q]];
-                if (item >= f && item < e) return before[q] + scale(L, parts[q]) * (pre[item] - pre[f]);
+        auto move_to = [&](long long t) {  // the first item with weight t or more in front
+            if (ai < na && start[ai + 1] <= t) {
+                int k = ai + 1;
+                while (k < na && start[k + 1] <= t) ++k;
+                enter(k);
             }
-            return total;
+            if (ai == na) return;
+            const int g = act[act0 + ai], end = group_end(g);
+            const long long sc = scale(L, ctx->group_part_h[g]);
+            while (at < end && before < t) {
+                if ((at & 63) == 0 && at + 64 <= end && before + sc * blocks[at >> 6] <= t) {
+                    before += sc * blocks[at >> 6];
+                    at += 64;
+                } else {
+                    before += sc * raw(L.w, at++);
+                }
+            }
+            if (at == end) enter(ai + 1);
+        };
+        auto add = [&] {
+            const int k = std::min(ai, na - 1);
+            bound.push_back(make_int4(at, act[act0 + k], k, 0));
         };
         int n_tail = 0;
-        if (total == 0) {
+        if (na == 0) {
             for (int c = 0; c <= G; ++c) bound.push_back(make_int4(0, 0, 0, 0));
         } else {
             const long long split = L.sf >= 1.0 ? total : (long long)(L.sf * (double)total);
-            const int js = split >= total ? last : item_at(split);
-            for (int c = 0; c < G; ++c) add(std::min(item_at(split / G * c + split % G * c / G), js));
-            const long long wmin = std::max<long long>(1, total / (40LL * G));
-            for (int j = js; j < last;) {
-                add(j);
-                ++n_tail;
-                const long long wj = weight_at(j), remaining = total - wj;
-                const int ge = group_end(g_hint);
-                int j2 = std::max(j + 1, item_at(std::min(total, wj + std::max(wmin, remaining / (2LL * G)))));
-                if (j2 >= ge) {  // on to the next group of the mask
-                    const int nx = act[act0 + act_at[g_hint] + 1];
-                    j2 = nx < 0 ? last : ctx->group_begin_h[nx];
-                }
-                j = j2;
+            enter(0);
+            for (int c = 0; c < G; ++c) {
+                move_to(split / G * c + split % G * c / G);
+                add();
             }
-            add(last);
+            move_to(split);
+            const long long wmin = std::max<long long>(1, total / (40LL * G));
+            while (ai < na) {
+                add();
+                ++n_tail;
+                const int k = ai;
+                move_to(before + std::max(wmin, (total - before) / (2LL * G)));
+                if (ai > k) enter(k + 1);  // units end with their group
+            }
+            add();
         }
         ctx->tail_n[mask] = n_tail;
     }
     // per-group weights for the device re-split of batched integrations (full-RHS parameters)
     std::vector<long long> gwt(ng);
-    const std::vector<long long> &pre7 = prefix_of(ctx->lt[7].w);
-    for (int g = 0; g < ng; ++g)
-        gwt[g] = scale(ctx->lt[7], ctx->group_part_h[g]) * (pre7[group_end(g)] - pre7[ctx->group_begin_h[g]]);
+    for (int g = 0; g < ng; ++g) gwt[g] = scale(ctx->lt[7], ctx->group_part_h[g]) * groups_of(ctx->lt[7].w)[g];
     int rc;
     if ((rc = upload_vec(ctx, ctx->gwt, gwt))) return rc;
     // the device re-split's memo no longer matches the weights: clear its valid flag
@@ -446,10 +476,6 @@ int collision_threads(const rtbte_ctx *ctx) {
 // instances 389 / 440 us; fewer groups than ~100, 0.8: 6 instances 167 / 186 us).
 void default_tuning(rtbte_ctx *ctx) {
     const bool fp64 = ctx->precision == RTBTE_PREC_FP64;
-    double slots[3] = {0, 0, 0};
-    for (int part = 0; part < 3; ++part)
-        for (int k = ctx->part_first[part]; k < ctx->part_first[part] + ctx->part_items[part]; ++k)
-            slots[part] += ctx->item_cost_h[k].slots;
     for (unsigned m = 0; m < 8; ++m) {
         if (ctx->lt_tuned) continue;  // a tuned mask's parameters serve the others
         LaunchTuning L;
@@ -458,7 +484,7 @@ void default_tuning(rtbte_ctx *ctx) {
             L.pf = 0;
         }
         double tot = 0;
-        for (int part = 0; part < 3; ++part) tot += (m & (1u << part)) ? slots[part] : 0.0;
+        for (int part = 0; part < 3; ++part) tot += (m & (1u << part)) ? (double)ctx->part_slots[part] : 0.0;
         if (ctx->inst.size() > 1) L.sf = tot < 4e6 ? 1.0 : ctx->n_groups >= 100 ? 0.5 : 0.8;
         else L.sf = tot > (fp64 ? 4e6 : 2e8) ? 0.9 : 1.0;
         ctx->lt[m] = L;
@@ -474,63 +500,54 @@ int item_rounds(int len, int lg) { return std::max(1, ((len >> 2) + (1 << lg) - 
 // process and by vectors per lane, longest first, so that packets hold alike items.  The partials'
 // slots are already set: sums do not depend on the order.
 constexpr int kSortWindow = 1024;
-void order_packets(std::vector<ItemRec> &items, const std::vector<Group> &groups) {
-    std::vector<ItemRec> tmp(kSortWindow);
-    for (const Group &G : groups) {
-        if (G.lanes_log2 == 5) continue;
-        for (int w0 = G.item_begin; w0 < G.item_end; w0 += kSortWindow) {
-            const int n = std::min(kSortWindow, G.item_end - w0);
-            int at[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
-            auto key = [&](const ItemRec &it) { return 4 * (it.proc != 0) + 4 - item_rounds(it.len, G.lanes_log2); };
-            for (int i = 0; i < n; ++i) ++at[key(items[w0 + i]) + 1];
-            for (int b = 0; b < 8; ++b) at[b + 1] += at[b];
-            for (int i = 0; i < n; ++i) tmp[at[key(items[w0 + i])]++] = items[w0 + i];
-            std::copy(tmp.begin(), tmp.begin() + n, items.begin() + w0);
-        }
+void order_packets(ItemRec *items, const Group &G) {
+    if (G.lanes_log2 == 5) return;
+    ItemRec tmp[kSortWindow];
+    for (int w0 = G.item_begin; w0 < G.item_end; w0 += kSortWindow) {
+        const int n = std::min(kSortWindow, G.item_end - w0);
+        int at[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
+        auto key = [&](const ItemRec &it) { return 4 * (it.proc != 0) + 4 - item_rounds(it.len, G.lanes_log2); };
+        for (int i = 0; i < n; ++i) ++at[key(items[w0 + i]) + 1];
+        for (int b = 0; b < 8; ++b) at[b + 1] += at[b];
+        for (int i = 0; i < n; ++i) tmp[at[key(items[w0 + i])]++] = items[w0 + i];
+        std::copy(tmp, tmp + n, items + w0);
     }
 }
 
 // Build the work items, staging groups, per-row partial slots and per-CTA work ranges.
 int make_plan(rtbte_ctx *ctx) {
     const size_t R = ctx->real_size;
-    std::vector<ItemRec> items;
+    const size_t NI = ctx->inst.size();
     std::vector<Group> groups;
-    std::vector<int> eoff, poff, ppoff;  // item offsets per row (host only: they order the slots)
-    std::vector<long long> eoff_base(ctx->inst.size()), poff_base(ctx->inst.size()), ppoff_base(ctx->inst.size());
-    std::vector<InstDev> idev(ctx->inst.size());
-    bool begin_overflow = false;
-    int cut = 512;  // entries per item at most (16 << the current group's lanes_log2)
-    // lanes per item of a group: from the mean padded length of its non-empty segments [s0, s1),
-    // counted over every row (also those outside a row slice, so that a sliced context cuts
-    // its items as a full one does), so that a sub-warp's item holds about one segment
-    auto lanes_log2 = [](const std::vector<long long> &plen, long long s0, long long s1) {
-        long long tot = 0, n = 0;
-        for (long long s = s0; s < s1; ++s)
-            if (plen[s] > 0) {
-                tot += plen[s];
-                ++n;
-            }
-        const double mean = n ? (double)tot / (double)n : 0.0;
-        return mean <= 64.0 ? 2 : mean <= 128.0 ? 3 : mean <= 256.0 ? 4 : 5;
-    };
-    auto add_seg = [&](long long b, long long e, int dest, int proc) {
-        for (long long x = b; x < e; x += cut) {
-            ItemRec it;
-            begin_overflow = begin_overflow || x >= (1LL << 40);
-            it.begin_lo = (unsigned)(x & 0xffffffffLL);
-            it.begin_hi = (unsigned char)((x >> 32) & 0xff);
-            it.slot = 0;  // set once every item exists
-            it.dest = dest;
-            it.len = (unsigned short)std::min<long long>(cut, e - x);
-            it.proc = (unsigned char)proc;
-            items.push_back(it);
-        }
-    };
+    std::vector<InstDev> idev(NI);
     size_t max_stage = 0;
-    // e-ph groups (instance, mode)
-    for (size_t i = 0; i < ctx->inst.size(); ++i) {
-        InstHost &I = ctx->inst[i];
-        eoff_base[i] = (long long)eoff.size();
+    // Staging groups in item order: e-ph (instance, mode, q-block), ph-e (instance), ph-ph (instance).
+    // Each comes with its destinations' segments: destination r holds segments [r * nproc, ...) of
+    // off (from segment seg0), the first of them of process proc0; dest_of maps r to the items' dest.
+    struct Source {
+        const std::vector<long long> *off, *plen;
+        long long seg0, rows;
+        int nproc, proc0, N_q, N_q_pad;  // ph-e: destinations are stored by mode with a padded stride
+        long long at;                    // first entry of this group's row offsets in row_items
+        long long slots;                 // entry slots of its items
+    };
+    std::vector<Source> src;
+    std::vector<long long> eoff_base(NI), poff_base(NI), ppoff_base(NI);
+    long long n_row_items = 0;
+    auto add_group = [&](Group &G, const InstHost &I, Source S) {
+        G.f_inst = I.f_off;
+        G.N_inst = I.N_off;
+        G.P_inst = I.P_off;
+        S.at = n_row_items;
+        n_row_items += S.rows + 1;
+        groups.push_back(G);
+        src.push_back(S);
+        max_stage = std::max(max_stage, (size_t)(G.stage0_len + G.stage1_len) * R);
+    };
+    int part_group[4] = {0, 0, 0, 0};  // first group of each part
+    for (size_t i = 0; i < NI; ++i) {
+        const InstHost &I = ctx->inst[i];
+        eoff_base[i] = n_row_items;
         const int nqb = std::max(I.eph_nqb, 1);
         const int qblk = I.eph_qblk > 0 ? I.eph_qblk : I.N_q_pad;
         for (int blk = 0; blk < I.d.nmodes * nqb; ++blk) {  // (mode, q-block)
@@ -539,7 +556,6 @@ int make_plan(rtbte_ctx *ctx) {
             Group G{};
             G.idx = I.eph_idx.as<uint32_t>();
             G.W = I.eph_W.p;
-            G.item_begin = (int)items.size();
             G.part = PART_EPH;
             G.inst = (int)i;
             G.nu = nu;
@@ -550,129 +566,158 @@ int make_plan(rtbte_ctx *ctx) {
             G.stage1_len = q_len;
             G.stage1_src = I.N_off + (long long)nu * I.N_q_pad + q_lo;
             G.stage1_q0 = q_lo;
-            G.lanes_log2 = lanes_log2(I.eph_plen, 2LL * blk * I.d.n_c, 2LL * (blk + 1) * I.d.n_c);
-            cut = 16 << G.lanes_log2;
-            G.f_inst = I.f_off;
-            G.N_inst = I.N_off;
-            G.P_inst = I.P_off;
-            for (int d = 0; d < I.d.n_c; ++d) {
-                eoff.push_back((int)items.size());
-                long long g = ((long long)blk * I.d.n_c + d) * 2;
-                
-                add_seg(I.eph_off[g], I.eph_off[g + 1], d, 0);
-                add_seg(I.eph_off[g + 1], I.eph_off[g + 2], d, 1);
-            }
-            eoff.push_back((int)items.size());
-            G.item_end = (int)items.size();
-            groups.push_back(G);
-            max_stage = std::max(max_stage, (size_t)(G.stage0_len + G.stage1_len) * R);
+            add_group(G, I, {&I.eph_off, &I.eph_plen, 2LL * blk * I.d.n_c, I.d.n_c, 2, 0, 0, 0, 0, 0});
         }
     }
-    ctx->part_first[PART_EPH] = 0;
-    ctx->part_items[PART_EPH] = (int)items.size();
-    // ph-e groups (instance)
-    for (size_t i = 0; i < ctx->inst.size(); ++i) {
-        InstHost &I = ctx->inst[i];
-        poff_base[i] = (long long)poff.size();
+    part_group[PART_PHE] = (int)groups.size();
+    for (size_t i = 0; i < NI; ++i) {
+        const InstHost &I = ctx->inst[i];
+        poff_base[i] = n_row_items;
         Group G{};
         G.idx = I.phe_idx.as<uint32_t>();
         G.W = I.phe_W.p;
-        G.item_begin = (int)items.size();
         G.part = PART_PHE;
         G.inst = (int)i;
         G.s_bits = I.s_bits;
         G.n_q_pad = I.N_q_pad;
         G.stage0_len = I.n_c_pad;
         G.stage0_src = I.f_off;
-        G.lanes_log2 = lanes_log2(I.phe_plen, 0, I.n_ph);
-        cut = 16 << G.lanes_log2;
-        G.f_inst = I.f_off;
-        G.N_inst = I.N_off;
-        G.P_inst = I.P_off;
-        for (long long p = 0; p < I.n_ph; ++p) {
-            poff.push_back((int)items.size());
-            int nu = (int)(p / I.N_q);
-            long long q = p - (long long)nu * I.N_q;
-            
-            add_seg(I.phe_off[p], I.phe_off[p + 1], (int)((long long)nu * I.N_q_pad + q), 1);
-        }
-        poff.push_back((int)items.size());
-        G.item_end = (int)items.size();
-        groups.push_back(G);
-        max_stage = std::max(max_stage, (size_t)G.stage0_len * R);
+        add_group(G, I, {&I.phe_off, &I.phe_plen, 0, I.n_ph, 1, 1, (int)I.N_q, I.N_q_pad, 0, 0});
     }
-    ctx->part_first[PART_PHE] = ctx->part_items[PART_EPH];
-    ctx->part_items[PART_PHE] = (int)items.size() - ctx->part_first[PART_PHE];
-    // ph-ph groups (instance)
-    for (size_t i = 0; i < ctx->inst.size(); ++i) {
-        InstHost &I = ctx->inst[i];
-        ppoff_base[i] = (long long)ppoff.size();
+    part_group[PART_PP] = (int)groups.size();
+    for (size_t i = 0; i < NI; ++i) {
+        const InstHost &I = ctx->inst[i];
+        ppoff_base[i] = n_row_items;
         if (I.M == 0) continue;
         Group G{};
         G.idx = I.pp_idx.as<uint32_t>();
         G.W = I.pp_W.p;
-        G.item_begin = (int)items.size();
         G.part = PART_PP;
         G.inst = (int)i;
         G.pp_bits = I.pp_bits;
         G.stage0_len = I.M_pad;
         G.stage0_src = I.P_off;
-        G.lanes_log2 = lanes_log2(I.pp_plen, 0, 2 * I.M);
-        cut = 16 << G.lanes_log2;
-        G.f_inst = I.f_off;
-        G.N_inst = I.N_off;
-        G.P_inst = I.P_off;
-        for (long long a = 0; a < I.M; ++a) {
-            ppoff.push_back((int)items.size());
-            
-            add_seg(I.pp_off[2 * a], I.pp_off[2 * a + 1], (int)a, 0);
-            add_seg(I.pp_off[2 * a + 1], I.pp_off[2 * a + 2], (int)a, 1);
-        }
-        ppoff.push_back((int)items.size());
-        G.item_end = (int)items.size();
-        groups.push_back(G);
-        max_stage = std::max(max_stage, (size_t)G.stage0_len * R);
+        add_group(G, I, {&I.pp_off, &I.pp_plen, 0, I.M, 2, 0, 0, 0, 0, 0});
     }
-    ctx->part_first[PART_PP] = ctx->part_first[PART_PHE] + ctx->part_items[PART_PHE];
-    ctx->part_items[PART_PP] = (int)items.size() - ctx->part_first[PART_PP];
-    if (items.size() >= (size_t)INT32_MAX) return fail(ctx, RTBTE_E_UNSUPPORTED, "too many work items");
-    if (begin_overflow) return fail(ctx, RTBTE_E_UNSUPPORTED, "channel list longer than 2^40 entries");
+    part_group[3] = (int)groups.size();
+    // Lanes per item of each group -- from the mean padded length of its non-empty segments, counted
+    // over every row (also those outside a row slice, so that a sliced context cuts its items as a
+    // full one does), so that a sub-warp's item holds about one segment -- and its items per row.
+    std::vector<int> row_items(n_row_items);  // first item of each row of each group, from its own 0
+    std::vector<long long> group_items(groups.size());
+    const bool threads = n_row_items > 100000;
+    parallel_for((int)groups.size(), threads, [&](int g) {
+        const Source &S = src[g];
+        long long tot = 0, n = 0;
+        for (long long s = S.seg0; s < S.seg0 + S.rows * S.nproc; ++s)
+            if ((*S.plen)[s] > 0) {
+                tot += (*S.plen)[s];
+                ++n;
+            }
+        const double mean = n ? (double)tot / (double)n : 0.0;
+        const int lg = mean <= 64.0 ? 2 : mean <= 128.0 ? 3 : mean <= 256.0 ? 4 : 5, sh = lg + 4;
+        groups[g].lanes_log2 = lg;
+        const long long *off = S.off->data() + S.seg0;
+        long long k = 0;
+        for (long long r = 0; r < S.rows; ++r) {
+            row_items[S.at + r] = (int)k;
+            for (int p = 0; p < S.nproc; ++p, ++off) k += (off[1] - off[0] + (1 << sh) - 1) >> sh;
+        }
+        row_items[S.at + S.rows] = (int)k;
+        group_items[g] = k;
+    });
+    long long total_items = 0;
+    for (size_t g = 0; g < groups.size(); ++g) {
+        const long long k = group_items[g];
+        if (total_items + k >= (long long)INT32_MAX) return fail(ctx, RTBTE_E_UNSUPPORTED, "too many work items");
+        groups[g].item_begin = (int)total_items;
+        total_items += k;
+        groups[g].item_end = (int)total_items;
+    }
+    const int n_items = (int)total_items;
+    for (const Source &S : src)
+        if ((*S.off)[S.seg0 + S.rows * S.nproc] > (1LL << 40))
+            return fail(ctx, RTBTE_E_UNSUPPORTED, "channel list longer than 2^40 entries");
+    for (int part = 0; part < 3; ++part) {
+        const int g0 = part_group[part], g1 = part_group[part + 1];
+        ctx->part_first[part] = g0 < (int)groups.size() ? groups[g0].item_begin : n_items;
+        ctx->part_items[part] = g1 > g0 ? groups[g1 - 1].item_end - groups[g0].item_begin : 0;
+    }
+    // the items themselves (arrays left uninitialised: every element is written below)
+    std::unique_ptr<ItemRec[]> items_h(new ItemRec[std::max(n_items, 1)]);
+    ItemRec *items = items_h.get();
+    parallel_for((int)groups.size(), threads, [&](int g) {
+        const Source &S = src[g];
+        const int cut = 16 << groups[g].lanes_log2;  // entries per item at most
+        ItemRec *it = items + groups[g].item_begin;
+        const long long *off = S.off->data() + S.seg0;
+        for (long long r = 0; r < S.rows; ++r) {
+            const int dest = S.N_q > 0 ? (int)((int)r / S.N_q * S.N_q_pad + (int)r % S.N_q) : (int)r;
+            for (int p = 0; p < S.nproc; ++p, ++off)
+                for (long long x = off[0]; x < off[1]; x += cut, ++it) {
+                    it->begin_lo = (unsigned)(x & 0xffffffffLL);
+                    it->begin_hi = (unsigned char)((x >> 32) & 0xff);
+                    it->slot = 0;  // set below
+                    it->dest = dest;
+                    it->len = (unsigned short)std::min<long long>(cut, off[1] - x);
+                    it->proc = (unsigned char)(S.proc0 + p);
+                }
+        }
+        for (long long r = 0; r <= S.rows; ++r) row_items[S.at + r] += groups[g].item_begin;
+    });
     // partial slots, row-major: every row's items get consecutive slots in the order the row
     // adds them (an electron row: its (mode, q-block) blocks in turn, emission then absorption
     // items of each; a phonon row: its ph-e items, then its ph-ph items if it is a sub-lattice
     // phonon), so a row kernel reads one offset pair and one contiguous run of partials
     std::vector<int> rowoff(ctx->n_y + 1, 0), rowmid(std::max<long long>(ctx->n_y, 1), 0);
-    {
-        long long next = 0;
-        auto take = [&](int i0, int i1) {
-            for (int k = i0; k < i1; ++k) items[k].slot = (unsigned)next++;
+    std::vector<long long> first_slot(NI + 1, 0);
+    for (size_t g = 0; g < groups.size(); ++g) first_slot[groups[g].inst + 1] += groups[g].item_end - groups[g].item_begin;
+    for (size_t i = 0; i < NI; ++i) first_slot[i + 1] += first_slot[i];
+    std::atomic<bool> covered{true};
+    parallel_for((int)NI, threads, [&](int i) {
+        const InstHost &I = ctx->inst[i];
+        const int nc = I.d.n_c, nblk = I.d.nmodes * std::max(I.eph_nqb, 1);
+        long long next = first_slot[i];
+        auto take = [&](long long o) {
+            for (int k = row_items[o]; k < row_items[o + 1]; ++k) items[k].slot = (unsigned)next++;
         };
-        for (size_t i = 0; i < ctx->inst.size(); ++i) {
-            const InstHost &I = ctx->inst[i];
-            const int nc = I.d.n_c, nblk = I.d.nmodes * std::max(I.eph_nqb, 1);
-            for (int d = 0; d < nc; ++d) {
-                const long long c = I.y_off + d;
-                rowoff[c] = (int)next;
-                for (int blk = 0; blk < nblk; ++blk) {
-                    const long long o = eoff_base[i] + (long long)blk * (nc + 1) + d;
-                    take(eoff[o], eoff[o + 1]);
-                }
-                rowmid[c] = (int)next;
-            }
-            for (long long p = 0; p < I.n_ph; ++p) {
-                const long long c = I.y_off + nc + p;
-                rowoff[c] = (int)next;
-                take(poff[poff_base[i] + p], poff[poff_base[i] + p + 1]);
-                rowmid[c] = (int)next;
-                const int a = I.M > 0 ? I.compact[p] : -1;
-                if (a >= 0) take(ppoff[ppoff_base[i] + a], ppoff[ppoff_base[i] + a + 1]);
-            }
+        for (int d = 0; d < nc; ++d) {
+            const long long c = I.y_off + d;
+            rowoff[c] = (int)next;
+            for (int blk = 0; blk < nblk; ++blk) take(eoff_base[i] + (long long)blk * (nc + 1) + d);
+            rowmid[c] = (int)next;
         }
-        rowoff[ctx->n_y] = (int)next;
-        if (next != (long long)items.size()) return fail(ctx, RTBTE_E_UNSUPPORTED, "work items not covered by rows");
+        for (long long p = 0; p < I.n_ph; ++p) {
+            const long long c = I.y_off + nc + p;
+            rowoff[c] = (int)next;
+            take(poff_base[i] + p);
+            rowmid[c] = (int)next;
+            const int a = I.M > 0 ? I.compact[p] : -1;
+            if (a >= 0) take(ppoff_base[i] + a);
+        }
+        if (next != first_slot[i + 1]) covered = false;
+    });
+    rowoff[ctx->n_y] = n_items;
+    if (!covered) return fail(ctx, RTBTE_E_UNSUPPORTED, "work items not covered by rows");
+    // item order within groups of several items to a warp, and what each item costs
+    ctx->item_cost_h.reset(new ItemCost[std::max(n_items, 1)]);
+    ItemCost *cost = ctx->item_cost_h.get();
+    parallel_for((int)groups.size(), threads, [&](int g) {
+        const Group &G = groups[g];
+        order_packets(items, G);
+        long long slots = 0;
+        for (int k = G.item_begin; k < G.item_end; ++k) {
+            cost[k] = {(unsigned short)(item_rounds(items[k].len, G.lanes_log2) << (G.lanes_log2 + 2)),
+                       (unsigned short)(1 << G.lanes_log2)};
+            slots += cost[k].slots;
+        }
+        src[g].slots = slots;
+    });
+    for (int part = 0; part < 3; ++part) {
+        ctx->part_slots[part] = 0;
+        for (int g = part_group[part]; g < part_group[part + 1]; ++g) ctx->part_slots[part] += src[g].slots;
     }
-    order_packets(items, groups);
-    ctx->n_items = (int)items.size();
+    ctx->n_items = n_items;
     ctx->n_groups = (int)groups.size();
     ctx->wide = std::all_of(groups.begin(), groups.end(), [](const Group &G) { return G.lanes_log2 == 5; });
     // instance layout for the row kernels
@@ -716,11 +761,6 @@ int make_plan(rtbte_ctx *ctx) {
     }
     ctx->per_sm = per_sm;
     ctx->grid = ctx->num_sms * (ctx->staged ? per_sm : fp64 ? 1 : 2);
-    ctx->item_cost_h.resize(items.size());
-    for (const Group &G : groups)
-        for (int k = G.item_begin; k < G.item_end; ++k)
-            ctx->item_cost_h[k] = {(unsigned short)(item_rounds(items[k].len, G.lanes_log2) << (G.lanes_log2 + 2)),
-                                   (unsigned short)(1 << G.lanes_log2)};
     ctx->group_begin_h.resize(groups.size());
     ctx->group_part_h.resize(groups.size());
     for (size_t g = 0; g < groups.size(); ++g) {
@@ -734,7 +774,7 @@ int make_plan(rtbte_ctx *ctx) {
         ctx->tail_ctr.bytes = 16;
         RT_CUDA(ctx, cudaMemsetAsync(ctx->tail_ctr.p, 0, 16, ctx->stream));
     }
-    if ((rc = upload_vec(ctx, ctx->items, items))) return rc;
+    if ((rc = upload_raw(ctx, ctx->items, items, sizeof(ItemRec) * (size_t)n_items))) return rc;
     if ((rc = upload_vec(ctx, ctx->groups, groups))) return rc;
     if ((rc = upload_vec(ctx, ctx->rowoff, rowoff))) return rc;
     if ((rc = upload_vec(ctx, ctx->rowmid, rowmid))) return rc;
@@ -760,7 +800,7 @@ int make_plan(rtbte_ctx *ctx) {
     RT_CUDA(ctx, cudaMemsetAsync(ctx->partials.p, 0, pb, ctx->stream));
     RT_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
     if ((rc = init_stage_grid(ctx))) return rc;
-    if ((rc = make_small_plan(ctx, items, groups, rowoff, rowmid))) return rc;
+    if ((rc = make_small_plan(ctx, items, n_items, groups, rowoff, rowmid))) return rc;
     ctx->plan_valid = true;
     return RTBTE_OK;
 }

@@ -12,10 +12,12 @@
 //     the chunk sums of the WRMS norm; every CTA then runs the controller on its own copy.
 // Items, their lanes and entry order, the order of a row's items, the norm's chunks and the
 // controller are those of the launch sequence (collide.cuh, rows.cuh, step.cuh), so both give the
-// same results bit for bit.
+// same results bit for bit.  The 12 x 12 toy model in FP64 (15 174 entries): RHS 18.9 -> 8.2 us a
+// call, Bogacki-Shampine attempts 62 -> 31 us.  What is left of an attempt is latency: a grid barrier
+// 2.5 us, the items of a stage 2 us, its rows 0.9 us, the populations' copy 0.6 us.
 #include <algorithm>
 #include <cstring>
-#include <numeric>
+#include <memory>
 
 #include "collide.cuh"
 #include "internal.cuh"
@@ -357,7 +359,7 @@ constexpr int kSmallThreads = 768, kSmallThreads64 = 512;  // RHS; attempts: kSm
 KParams small_params(rtbte_ctx *ctx) {
     KParams P;
     std::memset(&P, 0, sizeof(P));
-    P.items = ctx->small_items.as<ItemRec>();
+    P.items = reinterpret_cast<const ItemRec *>(ctx->small_tab.as<char>() + ctx->small_at[0]);
     P.groups = ctx->groups.as<Group>();
     P.n_groups = ctx->n_groups;
     return P;
@@ -366,9 +368,10 @@ KParams small_params(rtbte_ctx *ctx) {
 SmallPlan small_plan(rtbte_ctx *ctx) {
     SmallPlan S;
     const InstHost &I = ctx->inst[0];
-    S.runs = ctx->small_runs.as<SmallRun>();
-    S.rows = ctx->small_rows.as<SmallRow>();
-    S.row_off = ctx->small_off.as<int>();
+    const char *tab = ctx->small_tab.as<char>();
+    S.runs = reinterpret_cast<const SmallRun *>(tab + ctx->small_at[1]);
+    S.rows = reinterpret_cast<const SmallRow *>(tab + ctx->small_at[2]);
+    S.row_off = reinterpret_cast<const int *>(tab + ctx->small_at[3]);
     S.max_runs = ctx->small_max_runs;
     S.max_items = ctx->small_max_items;
     S.max_rows = ctx->small_max_rows;
@@ -391,53 +394,56 @@ int small_threads(const rtbte_ctx *ctx) {
     return ctx->precision == RTBTE_PREC_FP64 ? kSmallThreads64 : kSmallThreads;
 }
 
-template <class T> int upload(rtbte_ctx *ctx, DevBuf &b, const std::vector<T> &h) {
-    b.release();
-    RT_CUDA(ctx, cudaMalloc(&b.p, std::max<size_t>(h.size() * sizeof(T), 16)));
-    b.bytes = h.size() * sizeof(T);
-    if (!h.empty()) RT_CUDA(ctx, cudaMemcpyAsync(b.p, h.data(), b.bytes, cudaMemcpyHostToDevice, ctx->stream));
-    return RTBTE_OK;
-}
-
 }  // namespace
+
+// Entry slots up to which a single instance takes the one-launch kernels: about where what they
+// save over a few evaluations no longer covers building their plan (FP32 one-launch / launch
+// sequence, per RHS and per Zonneveld attempt: graphene 24, 0.23M entries, 10.3 / 16.5 and 59 / 80 us;
+// graphene 36, 0.96M, 12.4 / 19.5 and 65 / 89 us, plan 0.27 ms; graphene 48, 2.6M, 16.5 / 22.6 and
+// 88 / 111 us, plan 0.6 ms beside 0.6; graphene 63, 7.1M, 26.8 / 28.5 and 130 / 147 us; FP64, where the
+// arithmetic dominates sooner: graphene 36, 20.6 / 26.7 and 126 / 135 us; graphene 48, 41 / 45 and
+// 237 / 224 us).
+constexpr double kSmallSlots = 2e6, kSmallSlots64 = 1.5e6;
 
 // Row ownership of a single small instance, or none (ctx->small_grid = 0).  `items` in launch
 // order with their row-major slots, `rowoff` / `rowmid` the rows' slots.
-int make_small_plan(rtbte_ctx *ctx, const std::vector<ItemRec> &items, const std::vector<Group> &groups,
+int make_small_plan(rtbte_ctx *ctx, const ItemRec *items, int n, const std::vector<Group> &groups,
                     const std::vector<int> &rowoff, const std::vector<int> &rowmid) {
     ctx->small_grid = 0;
-    if (ctx->inst.size() != 1 || ctx->sliced || items.empty()) return RTBTE_OK;
+    if (ctx->inst.size() != 1 || ctx->sliced || n == 0) return RTBTE_OK;
     const InstHost &I = ctx->inst[0];
     const size_t R = ctx->real_size;
     const size_t pops = R * ((size_t)I.n_c_pad + (size_t)I.d.nmodes * I.N_q_pad + I.M_pad);
-    double slots = 0;
-    for (const ItemCost &c : ctx->item_cost_h) slots += c.slots;
-    if (pops > 160 * 1024 || slots > kSmallSlots) return RTBTE_OK;
-    const int n = (int)items.size();
-    std::vector<int> by_slot(n), group_of(n);
-    for (size_t g = 0; g < groups.size(); ++g)
+    const double slots = (double)(ctx->part_slots[0] + ctx->part_slots[1] + ctx->part_slots[2]);
+    if (pops > 160 * 1024 || slots > (R == 8 ? kSmallSlots64 : kSmallSlots) || groups.size() > 64) return RTBTE_OK;
+    constexpr bool threads = false;  // (starting threads takes longer than these plans)
+    std::unique_ptr<int[]> by_slot(new int[n]);
+    std::unique_ptr<short[]> group_of(new short[n]);
+    parallel_for((int)groups.size(), threads, [&](int g) {
         for (int k = groups[g].item_begin; k < groups[g].item_end; ++k) {
             by_slot[items[k].slot] = k;
-            group_of[k] = (int)g;
+            group_of[k] = (short)g;
         }
+    });
     // Rows dealt to the CTAs family by family (electrons, sub-lattice phonons, other phonons: so
     // every parts mask is spread evenly), back and forth; dearest first where a CTA gets only a few
     // (many rows average out, and sorting them would cost more than it evens).
-    const int ny = (int)ctx->n_y, nc = I.d.n_c;
+    const int ny = (int)ctx->n_y, nc = I.d.n_c, Nq = (int)I.N_q, ng = (int)groups.size();
     const int G = (int)std::max(1.0, std::min((double)ctx->num_sms, std::ceil(slots / 64.0)));
-    std::vector<std::vector<int>> own(G);
-    for (auto &o : own) o.reserve(ny / G + 3);
-    int at = 0, dir = 1;
+    const ItemCost *cost = ctx->item_cost_h.get();
     std::vector<std::pair<long long, int>> rows_of[3];  // (-cost, row)
     for (int c = 0; c < ny; ++c) {
         const int f = c < nc ? 0 : (I.M > 0 && I.compact[c - nc] >= 0 ? 1 : 2);
-        long long cost = 0;
-        if (ny < 32 * G)
-            for (int s = rowoff[c]; s < rowoff[c + 1]; ++s) cost -= ctx->item_cost_h[by_slot[s]].slots;
-        rows_of[f].push_back({cost, c});
+        long long w = 0;
+        if (ny < 8 * G)
+            for (int s = rowoff[c]; s < rowoff[c + 1]; ++s) w -= cost[by_slot[s]].slots;
+        rows_of[f].push_back({w, c});
     }
+    std::vector<std::vector<int>> own(G);
+    for (auto &o : own) o.reserve(ny / G + 3);
+    int at = 0, dir = 1;
     for (auto &rows : rows_of) {
-        if (ny < 32 * G) std::sort(rows.begin(), rows.end());
+        if (ny < 8 * G) std::sort(rows.begin(), rows.end());
         for (const auto &r : rows) {
             own[at].push_back(r.second);
             at += dir;
@@ -447,75 +453,89 @@ int make_small_plan(rtbte_ctx *ctx, const std::vector<ItemRec> &items, const std
             }
         }
     }
-    std::vector<ItemRec> out;
-    std::vector<std::vector<SmallRun>> runs(G);
-    std::vector<SmallRow> rows;
-    std::vector<int> off(G + 1, 0);
-    out.reserve(n);
-    rows.reserve(ny);
-    int max_items = 0, max_rows = 0, max_runs = 0;
+    // where each CTA's rows and items start; items [first[b], first[b + 1]) are CTA b's
+    std::vector<int> off(G + 1, 0), first(G + 1, 0);
+    int max_items = 0, max_rows = 0;
+    for (int b = 0; b < G; ++b) {
+        int m = 0;
+        for (int c : own[b]) m += rowoff[c + 1] - rowoff[c];
+        off[b + 1] = off[b] + (int)own[b].size();
+        first[b + 1] = first[b] + m;
+        max_items = std::max(max_items, m);
+        max_rows = std::max(max_rows, (int)own[b].size());
+    }
+    // one buffer, copied at once: items, runs, rows, row offsets
+    const size_t len[4] = {sizeof(ItemRec) * n, sizeof(SmallRun) * (size_t)G * ng, sizeof(SmallRow) * ny,
+                           sizeof(int) * (G + 1)};
+    size_t bytes = 0;
+    for (int k = 0; k < 4; ++k) {
+        ctx->small_at[k] = bytes;
+        bytes += (len[k] + 15) / 16 * 16;
+    }
+    std::unique_ptr<char[]> tab(new char[bytes]);
+    ItemRec *out = reinterpret_cast<ItemRec *>(tab.get() + ctx->small_at[0]);
+    SmallRun *runs = reinterpret_cast<SmallRun *>(tab.get() + ctx->small_at[1]);
+    SmallRow *rows = reinterpret_cast<SmallRow *>(tab.get() + ctx->small_at[2]);
+    std::memcpy(tab.get() + ctx->small_at[3], off.data(), len[3]);
+    std::memset(runs, 0, len[1]);
     // a CTA's items by group and, within it, alike ones together (the packets of order_packets in
     // rhs.cu): counting sort over (group, process, vectors per lane)
-    const int nb = 8 * (int)groups.size();
-    std::vector<int> count(nb + 1), keys;
-    std::vector<ItemRec> mine;
-    for (int b = 0; b < G; ++b) {
-        off[b] = (int)rows.size();
-        mine.clear();
-        keys.clear();
-        std::fill(count.begin(), count.end(), 0);
+    std::unique_ptr<int[]> counts(new int[(size_t)G * (8 * ng + 1)]), keys(new int[n]);
+    parallel_for(G, threads, [&](int b) {
+        int *count = counts.get() + (size_t)b * (8 * ng + 1), *key = keys.get() + first[b];
+        std::fill(count, count + 8 * ng + 1, 0);
+        int m = 0;
+        SmallRow *r = rows + off[b];
         for (int c : own[b]) {
-            SmallRow r{};
-            r.row = c;
-            r.p0 = (int)mine.size();
-            r.mid = r.p0 + rowmid[c] - rowoff[c];
-            for (int s = rowoff[c]; s < rowoff[c + 1]; ++s) {
-                const int k = by_slot[s], g = group_of[k], lanes = ctx->item_cost_h[k].lanes;
-                mine.push_back(items[k]);
-                mine.back().slot = (unsigned)mine.size() - 1;
-                keys.push_back(8 * g + 4 * (mine.back().proc != 0) + 4 - ctx->item_cost_h[k].slots / (4 * lanes));
-                ++count[keys.back() + 1];
+            r->row = c;
+            r->p0 = m;
+            r->mid = m + rowmid[c] - rowoff[c];
+            for (int s = rowoff[c]; s < rowoff[c + 1]; ++s, ++m) {
+                const int k = by_slot[s];
+                key[m] = 8 * group_of[k] + 4 * (items[k].proc != 0) + 4 - cost[k].slots / (4 * cost[k].lanes);
+                ++count[key[m] + 1];
             }
-            r.p1 = (int)mine.size();
+            r->p1 = m;
             const int p = c - nc;
-            r.f = c < nc ? c : -1;
-            r.N = c < nc ? -1 : (int)((p / I.N_q) * I.N_q_pad + p % I.N_q);
-            r.P = c < nc || I.M == 0 ? -1 : I.compact[p];
-            rows.push_back(r);
+            r->f = c < nc ? c : -1;
+            r->N = c < nc ? -1 : p / Nq * I.N_q_pad + p % Nq;
+            r->P = c < nc || I.M == 0 ? -1 : I.compact[p];
+            r->pad = 0;
+            ++r;
         }
-        max_items = std::max(max_items, (int)mine.size());
-        max_rows = std::max(max_rows, (int)own[b].size());
-        for (int k = 0; k < nb; ++k) count[k + 1] += count[k];
-        const int base = (int)out.size();
-        for (size_t g = 0; g < groups.size(); ++g) {
+        for (int k = 0; k < 8 * ng; ++k) count[k + 1] += count[k];
+        SmallRun *q = runs + (size_t)b * ng;
+        for (int g = 0; g < ng; ++g) {
             if (count[8 * (g + 1)] == count[8 * g]) continue;
             const Group &Q = groups[g];
-            SmallRun r{};
-            r.idx = Q.idx;
-            r.W = Q.W;
-            r.a = base + count[8 * g];
-            r.b = base + count[8 * (g + 1)];
-            r.part = (short)Q.part;
-            r.sb = (short)Q.s_bits;
-            r.pb = (short)Q.pp_bits;
-            r.lg = (short)Q.lanes_log2;
-            r.N_at = Q.nu * Q.n_q_pad;
-            runs[b].push_back(r);
+            q->idx = Q.idx;
+            q->W = Q.W;
+            q->a = first[b] + count[8 * g];
+            q->b = first[b] + count[8 * (g + 1)];
+            q->part = (short)Q.part;
+            q->sb = (short)Q.s_bits;
+            q->pb = (short)Q.pp_bits;
+            q->lg = (short)Q.lanes_log2;
+            q->N_at = Q.nu * Q.n_q_pad;
+            ++q;
         }
-        out.resize(base + mine.size());
-        for (size_t k = 0; k < mine.size(); ++k) out[base + count[keys[k]]++] = mine[k];
-        max_runs = std::max(max_runs, (int)runs[b].size());
-    }
-    off[G] = (int)rows.size();
-    std::vector<SmallRun> run_tab((size_t)G * max_runs, SmallRun{});
-    for (int b = 0; b < G; ++b) std::copy(runs[b].begin(), runs[b].end(), run_tab.begin() + (size_t)b * max_runs);
+        m = 0;
+        for (int c : own[b])
+            for (int s = rowoff[c]; s < rowoff[c + 1]; ++s, ++m) {
+                ItemRec &it = out[first[b] + count[key[m]]++];
+                it = items[by_slot[s]];
+                it.slot = (unsigned)m;
+            }
+    });
     ctx->small_max_items = (int)round_up(max_items, 4);
     ctx->small_max_rows = (int)round_up(max_rows, 2);
-    ctx->small_max_runs = max_runs;
-    int rc;
-    if ((rc = upload(ctx, ctx->small_items, out)) || (rc = upload(ctx, ctx->small_runs, run_tab)) ||
-        (rc = upload(ctx, ctx->small_rows, rows)) || (rc = upload(ctx, ctx->small_off, off)))
-        return rc;
+    ctx->small_max_runs = ng;
+    if (ctx->small_tab.bytes < bytes) {
+        ctx->small_tab.release();
+        RT_CUDA(ctx, cudaMalloc(&ctx->small_tab.p, bytes));
+        ctx->small_tab.bytes = bytes;
+    }
+    RT_CUDA(ctx, cudaMemcpyAsync(ctx->small_tab.p, tab.get(), bytes, cudaMemcpyHostToDevice, ctx->stream));
     ctx->small_grid = G;
     SmallPlan S = small_plan(ctx);
     if (small_smem(R, S, true) + 2048 > ctx->smem_optin) {

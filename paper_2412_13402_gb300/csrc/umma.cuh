@@ -379,7 +379,7 @@ __global__ void __launch_bounds__(kThreads, 2) conv_tc(const __grid_constant__ C
     auto full = [&](int s) { return bars + 8u * s; };
     auto used = [&](int s) { return bars + 8u * (NS + s); };
     const uint32_t tslot = bars + 16 * NS;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = tid >> 5;
     const int m0 = blockIdx.x * kTM;  // first point, or first (tap, channel) row
     const int k0 = MODE == CONV_WEIGHT ? blockIdx.y * a.kchunk : 0;
     const int nk = MODE == CONV_WEIGHT ? a.kchunk / kTK : 9;
