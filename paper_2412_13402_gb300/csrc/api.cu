@@ -754,7 +754,7 @@ void rtbte_destroy(rtbte_ctx *ctx) {
     ctx->act_tab.release();
     ctx->tail_ctr.release();
     DevBuf *bufs[] = {&ctx->popf, &ctx->popN, &ctx->popP, &ctx->instdev, &ctx->compact, &ctx->items, &ctx->groups,
-                      &ctx->partials, &ctx->rowoff, &ctx->rowmid, &ctx->gwt, &ctx->dyn_tab, &ctx->Y[0], &ctx->Y[1],
+                      &ctx->partials, &ctx->rowoff, &ctx->rowmid, &ctx->gwt, &ctx->dyn_tab, &ctx->row_blocks, &ctx->Y[0], &ctx->Y[1],
                       &ctx->K, &ctx->Fs, &ctx->forcing, &ctx->wrms_part, &ctx->ctl, &ctx->ystage, &ctx->ydstage,
                       &ctx->range_scratch, &ctx->slow_save, &ctx->small_tab, &ctx->small_pops, &ctx->small_sync};
     for (DevBuf *b : bufs) b->release();

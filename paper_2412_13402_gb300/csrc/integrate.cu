@@ -192,9 +192,7 @@ __global__ void controller_kernel(RowParams Q, Ctl *ctl, CtlParams cp, const dou
 __global__ void __launch_bounds__(kRedThreads) h0_norms(RowParams Q, CtlParams cp, const Ctl *ctl, const double *Y0,
                                                          const double *Y1, const double *K0, const double *K1,
                                                          double *wsq, int second, long long n) {
-    for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < n; c += (long long)gridDim.x * blockDim.x) {
-        const int ii = Q.n_inst > 1 ? find_inst(Q, c) : 0;
-        const InstDev I = Q.inst[ii];
+    for_rows(Q, n, [&](int ii, const InstDev &I, long long c) {
         const double *y = ctl[ii].cur ? Y1 : Y0;
         const double w = 1.0 / (cp.rtol * fabs(y[c]) + atol_of(cp, I, c - I.y_off));
         if (!second) {
@@ -205,7 +203,7 @@ __global__ void __launch_bounds__(kRedThreads) h0_norms(RowParams Q, CtlParams c
             const double d = (K1[c] - K0[c]) * w;
             wsq[c] = d * d;
         }
-    }
+    });
 }
 
 __global__ void h0_first(RowParams Q, Ctl *ctl, const double *part0, const double *part1, double span) {
@@ -224,12 +222,10 @@ __global__ void h0_first(RowParams Q, Ctl *ctl, const double *part0, const doubl
 
 template <class R>
 __global__ void h0_probe(RowParams Q, const Ctl *ctl, const double *Y0, const double *Y1, const double *K0, long long n) {
-    for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < n; c += (long long)gridDim.x * blockDim.x) {
-        const int ii = Q.n_inst > 1 ? find_inst(Q, c) : 0;
-        const InstDev I = Q.inst[ii];
+    for_rows(Q, n, [&](int ii, const InstDev &I, long long c) {
         const double *y = ctl[ii].cur ? Y1 : Y0;
-        write_pops<R>(Q, I, c - I.y_off, y[c] + ctl[ii].h0tmp * K0[c]);
-    }
+        write_pops<R>(Q, I, c - I.y_off, (R)(y[c] + ctl[ii].h0tmp * K0[c]));
+    });
 }
 
 __global__ void h0_second(RowParams Q, Ctl *ctl, CtlParams cp, const double *part, double span) {
@@ -290,11 +286,10 @@ __global__ void mri_forcing(double *r, const double *Fs, double om0, double om1,
 // Tolerance-chosen MRI (step doubling on the MIS step): copy each instance's rows between its
 // current state buffer and buf (to_buf: current -> buf, else buf -> current).
 __global__ void copy_cur(RowParams Q, const Ctl *ctl, double *Y0, double *Y1, double *buf, long long n, int to_buf) {
-    for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < n; c += (long long)gridDim.x * blockDim.x) {
-        const int ii = Q.n_inst > 1 ? find_inst(Q, c) : 0;
+    for_rows(Q, n, [&](int ii, const InstDev &, long long c) {
         double *y = ctl[ii].cur ? Y1 : Y0;
         if (to_buf) buf[c] = y[c]; else y[c] = buf[c];
-    }
+    });
 }
 
 // Squared weighted local-error estimate of the two-half-step result y_2 (the current state):
@@ -302,14 +297,12 @@ __global__ void copy_cur(RowParams Q, const Ctl *ctl, double *Y0, double *Y1, do
 __global__ void __launch_bounds__(kRedThreads) slow_err_sq(RowParams Q, CtlParams cp, const Ctl *ctl, const double *Y0,
                                                              const double *Y1, const double *yn, const double *y1,
                                                              double *wsq, long long n) {
-    for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < n; c += (long long)gridDim.x * blockDim.x) {
-        const int ii = Q.n_inst > 1 ? find_inst(Q, c) : 0;
-        const InstDev I = Q.inst[ii];
+    for_rows(Q, n, [&](int ii, const InstDev &I, long long c) {
         const double y2 = (ctl[ii].cur ? Y1 : Y0)[c];
         const double w = 1.0 / (cp.rtol * fabs(yn[c]) + atol_of(cp, I, c - I.y_off));
         const double d = (y1[c] - y2) / 7.0 * w;
         wsq[c] = d * d;
-    }
+    });
 }
 
 // Per-instance WRMS norm (Eq. wrms_norm) from the chunk sums of wrms_chunks.
@@ -364,7 +357,7 @@ int enqueue_attempt(rtbte_ctx *ctx, const Tableau &T, const CtlParams &cp, unsig
     a.stage = -1;
     a.respect_done = 1;
     int rc;
-    if ((rc = stage(ctx, a, s))) return rc;
+    if ((rc = stage(ctx, a, s)) || (rc = launch_resplit(ctx, parts, ctx->ctl.as<Ctl>(), s))) return rc;
     for (int i = 0; i < T.S; ++i) {
         if ((rc = launch_rhs_core(ctx, parts, ctx->ctl.as<Ctl>(), s))) return rc;
         a.stage = i;

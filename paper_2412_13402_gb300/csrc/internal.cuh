@@ -264,7 +264,7 @@ struct rtbte_ctx {
     rtbte::DevBuf popf, popN, popP, instdev, compact;
     // execution plan of the RHS
     bool plan_valid = false;
-    rtbte::DevBuf items, groups, partials, rowoff, rowmid, gwt, dyn_tab;  // rowoff/rowmid: slots of each row
+    rtbte::DevBuf items, groups, partials, rowoff, rowmid, gwt, dyn_tab, row_blocks;  // rowoff/rowmid: slots of each row
     int n_rblk = 0;  // several instances: row blocks of the stage kernels (256 rows of one instance each)
     int n_items = 0, n_groups = 0;
     int part_items[3] = {0, 0, 0};
@@ -321,6 +321,7 @@ int upload_tables(rtbte_ctx *ctx, int inst);
 int make_plan(rtbte_ctx *ctx);
 int launch_prep_from_y(rtbte_ctx *ctx, const double *y, cudaStream_t s);
 int launch_rhs_core(rtbte_ctx *ctx, unsigned parts, const Ctl *ctl, cudaStream_t s);
+int launch_resplit(rtbte_ctx *ctx, unsigned parts, const Ctl *ctl, cudaStream_t s);
 int launch_rows(rtbte_ctx *ctx, unsigned parts, double *out, const double *forcing, cudaStream_t s);
 int split_tables(rtbte_ctx *ctx);
 int autotune(rtbte_ctx *ctx, unsigned parts, int *chosen);

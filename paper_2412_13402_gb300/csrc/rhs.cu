@@ -112,7 +112,7 @@ __global__ void __launch_bounds__(NT, MINB) rhs_kernel(KParams P) {
 }
 
 // Work split over the groups still active (instance not done, part in the mask), recomputed
-// on the device before a collision launch inside a batched integration.  One block:
+// on the device before the collision launches of an attempt of a batched integration.  One block:
 //   - the active groups are listed in order in act[] (terminated by -1);
 //   - the units' bounds cut the active weight into `grid` static ranges holding 1 - tail_share of
 //     it and, when a CTA's share is above tail_min, kTailUnits x grid equal dynamic units; a
@@ -239,23 +239,18 @@ __global__ void split_kernel(const Group *groups, int n_groups, const long long 
 
 // y (FP64) -> population copies in the compute precision
 template <class R>
-__global__ void prep_kernel(RowParams Q, const double *y, long long n) {
-    for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < n; c += (long long)gridDim.x * blockDim.x) {
-        const int i = Q.n_inst > 1 ? find_inst(Q, c) : 0;
-        const InstDev I = Q.inst[i];
-        write_pops<R>(Q, I, c - I.y_off, y[c]);
-    }
+__global__ void __launch_bounds__(256) prep_kernel(RowParams Q, const double *y, long long n) {
+    for_rows(Q, n, [&](int, const InstDev &I, long long c) { write_pops<R>(Q, I, c - I.y_off, (R)y[c]); });
 }
 
 template <class R>
-__global__ void rows_kernel(RowParams Q, unsigned parts, double *out, const double *forcing, long long n) {
-    for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < n; c += (long long)gridDim.x * blockDim.x) {
-        const int i = Q.n_inst > 1 ? find_inst(Q, c) : 0;
-        const InstDev I = Q.inst[i];
+__global__ void __launch_bounds__(256) rows_kernel(RowParams Q, unsigned parts, double *out, const double *forcing,
+                                                   long long n) {
+    for_rows(Q, n, [&](int, const InstDev &I, long long c) {
         double v = row_value<R>(Q, I, c - I.y_off, parts);
         if (forcing) v += forcing[c];
         out[c] = v;
-    }
+    });
 }
 
 int upload_raw(rtbte_ctx *ctx, DevBuf &b, const void *h, size_t n) {
@@ -300,6 +295,8 @@ RowParams row_params(rtbte_ctx *ctx) {
     Q.rowoff = ctx->rowoff.as<int>();
     Q.rowmid = ctx->rowmid.as<int>();
     Q.compact = ctx->compact.as<int>();
+    Q.blocks = ctx->row_blocks.as<int2>();
+    Q.n_blocks = ctx->n_rblk;
     Q.partials = ctx->partials.p;
     Q.popf = ctx->popf.p;
     Q.popN = ctx->popN.p;
@@ -782,10 +779,12 @@ int make_plan(rtbte_ctx *ctx) {
     if ((rc = upload_vec(ctx, ctx->compact, compact))) return rc;
     if (ctx->n_y >= (long long)INT32_MAX) return fail(ctx, RTBTE_E_UNSUPPORTED, "state vector too long");
     if (ctx->inst.size() > (size_t)kMaxBatch) return fail(ctx, RTBTE_E_UNSUPPORTED, "more than 1024 instances");
-    long long nrb = 0;  // row blocks of 256 rows of one instance (batched stage kernels)
-    if (ctx->inst.size() > 1)
-        for (const InstHost &I : ctx->inst) nrb += (I.d.n_c + I.n_ph + 255) / 256;
-    ctx->n_rblk = (int)nrb;
+    std::vector<int2> rblk;  // several instances: blocks of 256 rows of one instance
+    if (NI > 1)
+        for (size_t i = 0; i < NI; ++i)
+            for (long long r = 0; r < ctx->inst[i].d.n_c + ctx->inst[i].n_ph; r += 256) rblk.push_back(make_int2((int)i, (int)r));
+    ctx->n_rblk = (int)rblk.size();
+    if ((rc = upload_vec(ctx, ctx->row_blocks, rblk))) return rc;
     ctx->dyn_tab.release();  // reallocated below for this plan's sizes
     if ((rc = split_tables(ctx))) return rc;
     if (ctx->n_groups > 1024) return fail(ctx, RTBTE_E_UNSUPPORTED, "more than 1024 staging groups");
@@ -805,14 +804,33 @@ int make_plan(rtbte_ctx *ctx) {
     return RTBTE_OK;
 }
 
+// Blocks of the row kernels: at most 8 per SM, one pass each otherwise.
+static int row_grid(const rtbte_ctx *ctx) {
+    const long long want = ctx->inst.size() > 1 ? ctx->n_rblk : (ctx->n_y + 255) / 256;
+    return (int)std::max<long long>(1, std::min<long long>(want, 8LL * ctx->num_sms));
+}
+
 int launch_prep_from_y(rtbte_ctx *ctx, const double *y, cudaStream_t s) {
     RowParams Q = row_params(ctx);
     const int threads = 256;
-    const int blocks = (int)std::min<long long>((ctx->n_y + threads - 1) / threads, 8LL * ctx->num_sms);
+    const int blocks = row_grid(ctx);
     if (ctx->precision == RTBTE_PREC_FP64)
         prep_kernel<double><<<blocks, threads, 0, s>>>(Q, y, ctx->n_y);
     else
         prep_kernel<float><<<blocks, threads, 0, s>>>(Q, y, ctx->n_y);
+    RT_CUDA(ctx, cudaGetLastError());
+    ctx->launches++;
+    return RTBTE_OK;
+}
+
+// Units of the collision launches of one attempt of a batched integration (the set of instances
+// still integrating changes only after it).
+int launch_resplit(rtbte_ctx *ctx, unsigned parts, const Ctl *ctl, cudaStream_t s) {
+    if (ctx->inst.size() <= 1) return RTBTE_OK;
+    const DynTab T = dyn_tab(ctx);
+    split_kernel<<<1, 256, 0, s>>>(ctx->groups.as<Group>(), ctx->n_groups, ctx->gwt.as<long long>(), ctl, parts,
+                                   ctx->grid, kResplitTail, kResplitTailMin, T.bound, T.act, T.n_tail, T.memo,
+                                   (int)ctx->inst.size());
     RT_CUDA(ctx, cudaGetLastError());
     ctx->launches++;
     return RTBTE_OK;
@@ -853,13 +871,8 @@ static int launch_core_t(rtbte_ctx *ctx, unsigned parts, const Ctl *ctl, cudaStr
     P.n_groups = ctx->n_groups;
     P.pf_dist = ctx->lt[parts].pf;
     P.tail_ctr = ctx->tail_ctr.as<int>();
-    if (ctl && ctx->inst.size() > 1) {  // batched integration: balance over the active instances
+    if (ctl && ctx->inst.size() > 1) {  // batched integration: units over the active instances (launch_resplit)
         const DynTab T = dyn_tab(ctx);
-        split_kernel<<<1, 256, 0, s>>>(ctx->groups.as<Group>(), ctx->n_groups, ctx->gwt.as<long long>(), ctl, parts,
-                                       ctx->grid, kResplitTail, kResplitTailMin, T.bound, T.act, T.n_tail, T.memo,
-                                       (int)ctx->inst.size());
-        RT_CUDA(ctx, cudaGetLastError());
-        ctx->launches++;
         P.bound = T.bound;
         P.act = T.act;
         P.n_tail_d = T.n_tail;
@@ -1145,7 +1158,7 @@ int launch_pp_rates(rtbte_ctx *ctx, int inst, double *rates, cudaStream_t s) {
 int launch_rows(rtbte_ctx *ctx, unsigned parts, double *out, const double *forcing, cudaStream_t s) {
     RowParams Q = row_params(ctx);
     const int threads = 256;
-    const int blocks = (int)std::min<long long>((ctx->n_y + threads - 1) / threads, 8LL * ctx->num_sms);
+    const int blocks = row_grid(ctx);
     if (ctx->precision == RTBTE_PREC_FP64)
         rows_kernel<double><<<blocks, threads, 0, s>>>(Q, parts, out, forcing, ctx->n_y);
     else
