@@ -113,7 +113,7 @@ struct ItemCost {
 
 // Launch parameters of the collision kernel for one parts mask.
 struct LaunchTuning {
-    int w = 192;                     // work-split weight of a packet (one warp's items) beyond its entries
+    int w = 384;                     // work-split weight of a packet (one warp's items) beyond its entries
     int pf = 1;                      // L2 prefetch distance in packets of a warp's sequence (0: off)
     double sf = 1.0;                 // share of the weight split statically (rest: dynamic chunks)
     double ps[3] = {1.0, 1.0, 1.0};  // relative cost of an entry of each part
@@ -154,6 +154,27 @@ inline int bits_for(long long n) {  // bits needed for indices 0..n-1
     return b;
 }
 inline long long round_up(long long x, long long m) { return (x + m - 1) / m * m; }
+
+// Programmatic dependent launch: the kernel may start while the one before it on the stream is
+// still running (once all of that one's blocks have called pdl_begin or ended), so its launch
+// and prologue are hidden; it must call pdl_wait, which returns when the kernel before has ended
+// and its writes are visible, before it touches any memory that one reads or writes.
+template <class... P, class... A>
+inline cudaError_t launch_pdl(void (*f)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A &&...args) {
+    cudaLaunchConfig_t c{};
+    c.gridDim = grid;
+    c.blockDim = block;
+    c.dynamicSmemBytes = smem;
+    c.stream = s;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    c.attrs = &at;
+    c.numAttrs = 1;
+    return cudaLaunchKernelEx(&c, f, static_cast<P>(args)...);
+}
+__device__ __forceinline__ void pdl_begin() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
 
 // The dynamic shared-memory limit is an attribute of the kernel function, shared by every
 // context (and surrogate) of the process: it is set to the device's opt-in maximum less the

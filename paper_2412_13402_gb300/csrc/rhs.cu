@@ -465,7 +465,9 @@ int collision_threads(const rtbte_ctx *ctx) {
 // Launch parameters of the masks the autotuner has not set.  A prefetch distance of one packet is
 // the fastest or within 2% of it at every FP32 size measured (graphene 36-180, silicon 16-32, 2-64
 // instances: none costs 15-30%, two packets up to 4%); FP64, bound by its arithmetic, is 2% faster
-// without and with w = 96 (graphene 120: 728 against 745 us).  The share split statically: dynamic
+// without (graphene 120: 728 against 745 us).  Packet weight and part costs come from static launches
+// (sf 1) over w 64-384 and costs 0.9-1.3: graphene 75 32.6 -> 31.4 us, graphene 90 49.7 -> 47.4, three
+// instances 98 -> 92, FP64 graphene 63 79.9 -> 75.9, against w 192 and equal costs.  The share split statically: dynamic
 // units even out what the weights do not model, at ~1 us and a staging copy each, which pays in
 // launches above ~250 us (FP32: 0.9 against 1.0, graphene 180 365 / 384 us, silicon 32 421 / 437 us,
 // but graphene 150 202 / 198 us; FP64, bound by its arithmetic, already at 90 us: graphene 63 93 / 99
@@ -477,8 +479,11 @@ void default_tuning(rtbte_ctx *ctx) {
         if (ctx->lt_tuned) continue;  // a tuned mask's parameters serve the others
         LaunchTuning L;
         if (fp64) {
-            L.w = 96;
+            L.w = 64;
             L.pf = 0;
+        } else {  // a ph-e entry takes two gathers of f and one operation more, a ph-ph entry two of N
+            L.ps[PART_PHE] = 1.1;
+            L.ps[PART_PP] = 1.05;
         }
         double tot = 0;
         for (int part = 0; part < 3; ++part) tot += (m & (1u << part)) ? (double)ctx->part_slots[part] : 0.0;

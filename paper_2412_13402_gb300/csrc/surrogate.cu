@@ -43,6 +43,8 @@ template <bool TA, bool TB>
 __global__ void __launch_bounds__(kGemmThreads) gemm_bf16(const bf16 *A, int lda, const bf16 *B, int ldb, float *C,
                                                           int ldc, int M, int N, int K, int kchunk, const float *bias,
                                                           int act, bf16 *Cb, const float *back) {
+    pdl_begin();
+    pdl_wait();
     __shared__ __align__(16) bf16 As[kBM][kBK + 8];
     __shared__ __align__(16) bf16 Bt[kBN][kBK + 8];  // transposed: n-major, k contiguous
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -137,6 +139,8 @@ __global__ void sum_splits(const float *part, int splits, long long n, float *ou
 // where C is a multiple of 8 and the 8 columns share a tap (64 channels, batch 8 of 60 x 60: 98 us
 // with one element per thread; bound by the 33 MB it writes).
 __global__ void im2col(const bf16 *act, int C, int ny, int nx, long long P, bf16 *col, int kpad) {
+    pdl_begin();
+    pdl_wait();
     const int nv = kpad >> 3;
     const long long total = P * nv;
     const long long per = (long long)ny * nx;
@@ -232,6 +236,8 @@ struct GradSums {
 };
 
 __global__ void __launch_bounds__(256) bias_chains(GradSums a) {
+    pdl_begin();
+    pdl_wait();
     const int l = blockIdx.y, col = threadIdx.x & 63, t = blockIdx.x * 4 + (threadIdx.x >> 6);
     const int N = a.cols[l];
     if (col >= N) return;
@@ -243,6 +249,8 @@ __global__ void __launch_bounds__(256) bias_chains(GradSums a) {
 }
 
 __global__ void __launch_bounds__(256) finish_grads(GradSums a, int nbias) {
+    pdl_begin();
+    pdl_wait();
     if ((int)blockIdx.x < nbias) {  // one bias column
         __shared__ float red[256];
         int l = 0, col = blockIdx.x;
@@ -285,6 +293,8 @@ constexpr int kHeadRows = 256, kHeadLdA = 72, kHeadLdB = kHeadRows + 8;
 constexpr size_t kHeadSmem = 2 * sizeof(bf16) * (kHeadRows * kHeadLdA + 16 * kHeadLdB);
 constexpr int kHeadThreads = 256;  // all copy, the first four warps multiply (16 channels each)
 __global__ void __launch_bounds__(kHeadThreads) head_grad(const bf16 *A, const bf16 *B, int C, int P, int kchunk, float *part) {
+    pdl_begin();
+    pdl_wait();
     extern __shared__ __align__(16) unsigned char smem[];
     bf16 *As = reinterpret_cast<bf16 *>(smem), *Bt = As + 2 * kHeadRows * kHeadLdA;
     const int tid = threadIdx.x, lane = tid & 31, g = lane >> 2, t4 = lane & 3;
@@ -355,6 +365,8 @@ __global__ void __launch_bounds__(kHeadThreads) head_grad(const bf16 *A, const b
 
 // mean-square loss: g = 2 (out - t)/n (FP32 and BF16), per-block partial losses
 __global__ void mse(const float *out, const float *t, long long n, float *g, bf16 *gb, float *part) {
+    pdl_begin();
+    pdl_wait();
     __shared__ float red[256];
     float s = 0.f;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
@@ -387,6 +399,8 @@ struct WeightLayout {
 };
 __global__ void adam(float *w, const float *g, float *m, float *v, long long n, float lr, float b1, float b2, float eps,
                      float c1, float c2, bf16 *wb, WeightLayout L) {
+    pdl_begin();
+    pdl_wait();
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
         const float gi = g[i];
         const float mi = b1 * m[i] + (1.f - b1) * gi;
@@ -434,6 +448,8 @@ __global__ void gather_pair(const double *y, const double *ydot, const int *pp_f
 // minibatch assembly from stored pairs: x = (N - mu)/sd (BF16), t = I/so
 __global__ void gather_batch(const float *Ns, const float *Is, const int *idx, int B, int C, long long Pq, const float *mu,
                              const float *sd, const float *so, bf16 *xb, float *t) {
+    pdl_begin();
+    pdl_wait();
     const long long per = Pq * C;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < (long long)B * per;
          i += (long long)gridDim.x * blockDim.x) {
@@ -502,6 +518,8 @@ __global__ void judge_cv(const float *out, float *out_ref, double *Eref, const d
 // difference loss for pairs (sample b, sample b + B): d = (out_b - out_{b+B}) - (t_b - t_{b+B});
 // loss = mean(d^2) over the first half; g_b = 2d/n, g_{b+B} = -2d/n
 __global__ void mse_diff(const float *out, const float *t, long long n, float *g, bf16 *gb, float *part) {
+    pdl_begin();
+    pdl_wait();
     __shared__ float red[256];
     float s = 0.f;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
@@ -778,7 +796,8 @@ int gemm(rtbte_surrogate *s, const bf16 *A, int lda, const bf16 *B, int ldb, flo
     cudaStream_t st = s->ctx->stream;
     if (splits <= 1) {
         dim3 grid((M + kBM - 1) / kBM, (N + kBN - 1) / kBN, 1);
-        gemm_bf16<TA, TB><<<grid, kGemmThreads, 0, st>>>(A, lda, B, ldb, C, ldc, M, N, K, K, bias, act, Cb, back);
+        S_CUDA(s, launch_pdl(gemm_bf16<TA, TB>, grid, dim3(kGemmThreads), 0, st, A, lda, B, ldb, C, ldc, M, N, K, K, bias,
+                             act, Cb, back));
     } else {
         int kchunk = (K + splits - 1) / splits;
         kchunk = (kchunk + kBK - 1) / kBK * kBK;
@@ -865,11 +884,12 @@ int gemm_tc(rtbte_surrogate *s, const bf16 *A, int lda, const bf16 *B, int ldb, 
         attr_set = true;
     }
     static_assert(umma::kTM * umma::kTK * 2 + 128 * umma::kTK * 2 <= 32768, "four stages for bn <= 128");
-    if (bn <= 32) umma::gemm_tc<32, 4><<<grid, umma::kThreads, sm, st>>>(ta, tb, a);
-    else if (bn <= 64) umma::gemm_tc<64, 4><<<grid, umma::kThreads, sm, st>>>(ta, tb, a);
-    else if (bn <= 128) umma::gemm_tc<128, 4><<<grid, umma::kThreads, sm, st>>>(ta, tb, a);
-    else umma::gemm_tc<256, 2><<<grid, umma::kThreads, sm, st>>>(ta, tb, a);
-    S_CUDA(s, cudaGetLastError());
+    cudaError_t e;
+    if (bn <= 32) e = launch_pdl(umma::gemm_tc<32, 4>, grid, dim3(umma::kThreads), sm, st, ta, tb, a);
+    else if (bn <= 64) e = launch_pdl(umma::gemm_tc<64, 4>, grid, dim3(umma::kThreads), sm, st, ta, tb, a);
+    else if (bn <= 128) e = launch_pdl(umma::gemm_tc<128, 4>, grid, dim3(umma::kThreads), sm, st, ta, tb, a);
+    else e = launch_pdl(umma::gemm_tc<256, 2>, grid, dim3(umma::kThreads), sm, st, ta, tb, a);
+    S_CUDA(s, e);
     s->ctx->launches++;
     return RTBTE_OK;
 }
@@ -912,10 +932,11 @@ int gemm_tc_mn(rtbte_surrogate *s, const bf16 *A, int lda, const bf16 *B, int ld
     a.c_split = (long long)M * ldc;
     const dim3 grid(mt, 1, splits);
     cudaStream_t st = s->ctx->stream;
-    if (N <= 64) umma::gemm_tc<64, 4><<<grid, umma::kThreads, umma::smem_bytes(64), st>>>(ta, tb, a);
-    else if (N <= 128) umma::gemm_tc<128, 4><<<grid, umma::kThreads, umma::smem_bytes(128), st>>>(ta, tb, a);
-    else umma::gemm_tc<256, 2><<<grid, umma::kThreads, umma::smem_bytes(N), st>>>(ta, tb, a);
-    S_CUDA(s, cudaGetLastError());
+    cudaError_t e;
+    if (N <= 64) e = launch_pdl(umma::gemm_tc<64, 4>, grid, dim3(umma::kThreads), umma::smem_bytes(64), st, ta, tb, a);
+    else if (N <= 128) e = launch_pdl(umma::gemm_tc<128, 4>, grid, dim3(umma::kThreads), umma::smem_bytes(128), st, ta, tb, a);
+    else e = launch_pdl(umma::gemm_tc<256, 2>, grid, dim3(umma::kThreads), umma::smem_bytes(N), st, ta, tb, a);
+    S_CUDA(s, e);
     s->ctx->launches++;
     if (splits > 1 && !part) {
         sum_splits<<<blocks_for((long long)M * ldc), 256, 0, st>>>(s->split.as<float>(), splits, (long long)M * ldc, C);
@@ -975,8 +996,7 @@ int conv(rtbte_surrogate *s, umma::ConvArgs a, int B, const bf16 *mat, long long
     }
     const int mrows = MODE == umma::CONV_WEIGHT ? 9 * umma::kConvC : a.P;
     const dim3 grid((mrows + umma::kTM - 1) / umma::kTM, splits);
-    umma::conv_tc<MODE><<<grid, umma::kThreads, umma::conv_smem_bytes(), s->ctx->stream>>>(tb, a);
-    S_CUDA(s, cudaGetLastError());
+    S_CUDA(s, launch_pdl(umma::conv_tc<MODE>, grid, dim3(umma::kThreads), umma::conv_smem_bytes(), s->ctx->stream, tb, a));
     s->ctx->launches++;
     return RTBTE_OK;
 }
@@ -998,9 +1018,8 @@ int forward(rtbte_surrogate *s, int B) {
             in = s->actb[l + 1].as<bf16>();
             continue;
         }
-        im2col<<<blocks_for(P * s->kpad[l] / 8), 256, 0, st>>>(in, C, s->ny, s->nx, P, s->cols[l].as<bf16>(),
-                                                               s->kpad[l]);
-        S_CUDA(s, cudaGetLastError());
+        S_CUDA(s, launch_pdl(im2col, dim3(blocks_for(P * s->kpad[l] / 8)), dim3(256), 0, st, in, C, s->ny, s->nx, P,
+                             s->cols[l].as<bf16>(), s->kpad[l]));
         s->ctx->launches++;
         if (s->engine == 0)
             rc = gemm_tc(s, s->cols[l].as<bf16>(), s->kpad[l], s->wtt.as<bf16>() + s->off_tt[l], s->kpad[l],
@@ -1073,8 +1092,8 @@ int backward_conv(rtbte_surrogate *s, int B) {
         S_CUDA(s, allow_max_dynamic_smem((const void *)head_grad));
         attr_set = true;
     }
-    head_grad<<<splits, kHeadThreads, kHeadSmem, st>>>(s->actb[0].as<bf16>(), s->goutb.as<bf16>(), C, (int)P, kchunk, part);
-    S_CUDA(s, cudaGetLastError());
+    S_CUDA(s, launch_pdl(head_grad, dim3(splits), dim3(kHeadThreads), kHeadSmem, st, s->actb[0].as<bf16>(), s->goutb.as<bf16>(), C,
+                         (int)P, kchunk, part));
     sums(part, splits, Wd * C, g + s->off_M2);
     // gz5 = (g_out M2^T)(1 - h5^2)
     if ((rc = gemm<false, true>(s, s->goutb.as<bf16>(), C, s->wb.as<bf16>() + s->off_M2, C, gz[kLayers], Wd, (int)P, Wd,
@@ -1122,14 +1141,13 @@ int backward_conv(rtbte_surrogate *s, int B) {
     q.bias[kLayers + 1] = g + s->off_c2;
     q.chains = s->chains.as<float>();
     q.P = P;
-    bias_chains<<<dim3(64, kLayers + 2), 256, 0, st>>>(q);
+    S_CUDA(s, launch_pdl(bias_chains, dim3(64, kLayers + 2), dim3(256), 0, st, q));
     int nbias = 0, elems = 0;
     for (int l = 0; l < kLayers + 2; ++l) {
         nbias += q.cols[l];
         elems += q.n[l];
     }
-    finish_grads<<<nbias + (elems + 255) / 256, 256, 0, st>>>(q, nbias);
-    S_CUDA(s, cudaGetLastError());
+    S_CUDA(s, launch_pdl(finish_grads, dim3(nbias + (elems + 255) / 256), dim3(256), 0, st, q, nbias));
     s->ctx->launches += 3;
     return RTBTE_OK;
 }
@@ -1142,12 +1160,11 @@ int loss_grad(rtbte_surrogate *s, int B, float *loss, bool diff = false) {
     const long long P = (long long)B * s->Pq, nout = P * s->C;
     const int nb = blocks_for(diff ? nout / 2 : nout);
     if (diff)  // samples b and b + B/2 form a pair
-        mse_diff<<<nb, 256, 0, st>>>(s->out.as<float>(), s->t.as<float>(), nout / 2, s->gout.as<float>(),
-                                     s->goutb.as<bf16>(), s->lossp.as<float>());
+        S_CUDA(s, launch_pdl(mse_diff, dim3(nb), dim3(256), 0, st, s->out.as<float>(), s->t.as<float>(), nout / 2,
+                             s->gout.as<float>(), s->goutb.as<bf16>(), s->lossp.as<float>()));
     else
-        mse<<<nb, 256, 0, st>>>(s->out.as<float>(), s->t.as<float>(), nout, s->gout.as<float>(), s->goutb.as<bf16>(),
-                                s->lossp.as<float>());
-    S_CUDA(s, cudaGetLastError());
+        S_CUDA(s, launch_pdl(mse, dim3(nb), dim3(256), 0, st, s->out.as<float>(), s->t.as<float>(), nout, s->gout.as<float>(),
+                             s->goutb.as<bf16>(), s->lossp.as<float>()));
     s->ctx->launches++;
     if (implicit_conv(s)) {
         if ((rc = backward_conv(s, B))) return rc;
@@ -1658,18 +1675,16 @@ int rtbte_surrogate_train(rtbte_surrogate *s, int steps, int batch, int horizon,
             if (horizon > 0) bidx[batch + b] = u.second;
         }
         S_CUDA(s, cudaMemcpyAsync(s->idx.p, bidx.data(), sizeof(int) * nsamp, cudaMemcpyHostToDevice, ctx->stream));
-        gather_batch<<<blocks_for(nsamp * per), 256, 0, ctx->stream>>>(s->Ns.as<float>(), s->Is.as<float>(),
-                                                                      s->idx.as<int>(), nsamp, s->C, s->Pq, mu, sd, so,
-                                                                      s->xb.as<bf16>(), s->t.as<float>());
-        S_CUDA(s, cudaGetLastError());
+        S_CUDA(s, launch_pdl(gather_batch, dim3(blocks_for(nsamp * per)), dim3(256), 0, ctx->stream, s->Ns.as<float>(),
+                             s->Is.as<float>(), s->idx.as<int>(), nsamp, s->C, s->Pq, mu, sd, so, s->xb.as<bf16>(),
+                             s->t.as<float>()));
         ctx->launches++;
         if ((rc = loss_grad(s, nsamp, it == steps - 1 ? &last : nullptr, horizon > 0))) return rc;
         s->adam_t++;
         const float b1 = 0.9f, b2 = 0.999f;
-        adam<<<blocks_for(s->nparam), 256, 0, ctx->stream>>>(
-            s->w.as<float>(), s->g.as<float>(), s->m.as<float>(), s->v.as<float>(), s->nparam, lr, b1, b2, 1e-8f,
-            1.f - powf(b1, (float)s->adam_t), 1.f - powf(b2, (float)s->adam_t), s->wb.as<bf16>(), layout);
-        S_CUDA(s, cudaGetLastError());
+        S_CUDA(s, launch_pdl(
+            adam, dim3(blocks_for(s->nparam)), dim3(256), 0, ctx->stream, s->w.as<float>(), s->g.as<float>(), s->m.as<float>(), s->v.as<float>(), s->nparam, lr, b1, b2, 1e-8f,
+            1.f - powf(b1, (float)s->adam_t), 1.f - powf(b2, (float)s->adam_t), s->wb.as<bf16>(), layout));
         ctx->launches++;
     }
     if ((rc = refresh_inference(s))) return rc;

@@ -22,6 +22,8 @@
 #include <cuda_bf16.h>
 #include <stdint.h>
 
+#include "internal.cuh"
+
 namespace rtbte {
 namespace umma {
 
@@ -234,6 +236,8 @@ __global__ void __launch_bounds__(kThreads) gemm_tc(const __grid_constant__ CUte
     uint32_t tmem;
     asm volatile("ld.shared.b32 %0, [%1];\n" : "=r"(tmem) : "r"(tslot) : "memory");
 
+    pdl_begin();  // (after the allocation: the next kernel's cannot come between this grid's)
+    pdl_wait();
     __shared__ int s_fail;
     if (threadIdx.x == 0) {
         s_fail = 0;
@@ -403,6 +407,7 @@ __global__ void __launch_bounds__(kThreads, 2) conv_tc(const __grid_constant__ C
     uint32_t tmem;
     asm volatile("ld.shared.b32 %0, [%1];\n" : "=r"(tmem) : "r"(tslot) : "memory");
 
+    pdl_begin();  // (after the allocation: the next kernel's cannot come between this grid's)
     // gather role: chunk c of rows r0 + 32 i; all of a thread's rows have the same row mod 8
     const int c = tid & 7, r0 = tid >> 3;
     const uint32_t gdst = (uint32_t)r0 * 128u + ((uint32_t)(c ^ (r0 & 7)) << 4);
@@ -453,6 +458,7 @@ __global__ void __launch_bounds__(kThreads, 2) conv_tc(const __grid_constant__ C
         for (int j = 0; j < 32; ++j) sum[j] = MODE == CONV_BACK && kt > 0 ? sum[j] + v[j] : v[j];
     };
 
+    pdl_wait();
     int loaded = 0;  // slices whose copies were started
     for (; loaded < NS - 1 && loaded < nk; ++loaded) {
         load(loaded, loaded);
