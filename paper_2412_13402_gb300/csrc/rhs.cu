@@ -70,7 +70,7 @@ __device__ __forceinline__ void enter_group(const KParams &P, int g, R *sm, int 
 // cost), then takes dynamic units of the remaining items from a shared counter until none is
 // left, so that SMs that finish early absorb the tail of the work.  Every item writes its own
 // partial, so the result does not depend on which CTA ran it.
-template <class R, bool STAGED, bool WIDE, int MINB, int NT>
+template <class R, bool STAGED, bool WIDE, bool CACHED, int MINB, int NT>
 __global__ void __launch_bounds__(NT, MINB) rhs_kernel(KParams P) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ int s_unit;
@@ -87,7 +87,7 @@ __global__ void __launch_bounds__(NT, MINB) rhs_kernel(KParams P) {
             if (a < b && !(P.ctl && P.ctl[G.inst].done)) {  // (done: the instance is at its t_out)
                 GroupView<R> V;
                 enter_group<R, STAGED>(P, g, sm, staged, V);
-                run_range<R, WIDE>(P, V, a, b, warp, nwarps, lane);
+                run_range<R, WIDE, CACHED>(P, V, a, b, warp, nwarps, lane);
             }
             if (end <= G.item_end) break;
             g = P.act[++at];
@@ -447,16 +447,32 @@ int split_tables(rtbte_ctx *ctx) {
 // The collision kernel of a plan and its threads per SM (per CTA in the form that reads
 // populations from global memory: two CTAs per SM in FP32; one in FP64, where two at 64 registers
 // spill -- silicon at 80^3 / 40^3, 2.1e9 entries: 16.1 ms with two, 15.4 with one).
-const void *collision_kernel(const rtbte_ctx *ctx) {
+template <bool CACHED> const void *collision_kernel_of(const rtbte_ctx *ctx) {
     const bool fp64 = ctx->precision == RTBTE_PREC_FP64;
     if (!ctx->staged)
-        return fp64 ? (const void *)rhs_kernel<double, false, false, 1, kRhsThreads64>
-                    : (const void *)rhs_kernel<float, false, false, 2, kRhsThreads64>;
+        return fp64 ? (const void *)rhs_kernel<double, false, false, CACHED, 1, kRhsThreads64>
+                    : (const void *)rhs_kernel<float, false, false, CACHED, 2, kRhsThreads64>;
     if (fp64)
-        return ctx->wide ? (const void *)rhs_kernel<double, true, true, 1, kRhsThreads64>
-                         : (const void *)rhs_kernel<double, true, false, 1, kRhsThreads64>;
-    return ctx->wide ? (const void *)rhs_kernel<float, true, true, 1, kRhsThreads>
-                     : (const void *)rhs_kernel<float, true, false, 1, kRhsThreads>;
+        return ctx->wide ? (const void *)rhs_kernel<double, true, true, CACHED, 1, kRhsThreads64>
+                         : (const void *)rhs_kernel<double, true, false, CACHED, 1, kRhsThreads64>;
+    return ctx->wide ? (const void *)rhs_kernel<float, true, true, CACHED, 1, kRhsThreads>
+                     : (const void *)rhs_kernel<float, true, false, CACHED, 1, kRhsThreads>;
+}
+// Ordinary or streaming loads of the lists.  Inside an integration the same lists are read again
+// at once: below kKeepBytes they stay in L2 (129 MB) with ordinary loads (57 MB: 22.4 -> 20.7 us a
+// launch, 79 MB: 27.0 -> 25.0), and several instances take ordinary loads whatever their size, since
+// what is read shrinks as they finish (16-instance window: 32.2 -> 31.1 ms of collision time).
+// Otherwise streaming loads, whose lines are evicted first, keep a part of the stream for the next
+// reading where ordinary ones would evict all of it (105 MB: 33.0 us, 37.1 with ordinary loads; three
+// contexts of 57 MB in turn: 31.1 / 32.2 us a call), up to sizes where no part matters and ordinary
+// loads are 1-2% faster again (2.27 GB: 348.6 -> 345.0 us, 2.78 GB: 413 -> 406).
+constexpr double kKeepBytes = 85e6, kStreamBytes = 1e9;
+const void *collision_kernel(const rtbte_ctx *ctx, unsigned parts, bool integrating) {
+    double bytes = 0;
+    for (int part = 0; part < 3; ++part)
+        if (parts & (1u << part)) bytes += (double)ctx->part_slots[part] * (4 + ctx->real_size);
+    const bool ordinary = bytes >= kStreamBytes || (integrating && (ctx->inst.size() > 1 || bytes <= kKeepBytes));
+    return ordinary ? collision_kernel_of<true>(ctx) : collision_kernel_of<false>(ctx);
 }
 int collision_threads(const rtbte_ctx *ctx) {
     return ctx->staged && ctx->precision != RTBTE_PREC_FP64 ? kRhsThreads : kRhsThreads64;
@@ -747,15 +763,18 @@ int make_plan(rtbte_ctx *ctx) {
     ctx->smem_bytes = ctx->staged ? std::max<size_t>(max_stage, 16) : 0;
     int per_sm = 1;
     const bool fp64 = ctx->precision == RTBTE_PREC_FP64;
-    const void *fn = collision_kernel(ctx);
+    const void *fns[2] = {collision_kernel_of<false>(ctx), collision_kernel_of<true>(ctx)};
     const int nt = collision_threads(ctx);
     if (ctx->staged) {
-        RT_CUDA(ctx, allow_max_dynamic_smem(fn));
-        RT_CUDA(ctx, cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
+        for (const void *fn : fns) {
+            RT_CUDA(ctx, allow_max_dynamic_smem(fn));
+            RT_CUDA(ctx, cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
+        }
         for (int k : {4, 2}) {
-            int nb = 0;
-            RT_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fn, nt / k, ctx->smem_bytes));
-            if (nb >= k) {
+            int nb = 0, nb2 = 0;
+            RT_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fns[0], nt / k, ctx->smem_bytes));
+            RT_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb2, fns[1], nt / k, ctx->smem_bytes));
+            if (std::min(nb, nb2) >= k) {
                 per_sm = k;
                 break;
             }
@@ -895,7 +914,7 @@ static int launch_core_t(rtbte_ctx *ctx, unsigned parts, const Ctl *ctl, cudaStr
     int rc;
     if ((rc = timing_begin(ctx, s, &ev))) return rc;
     void *args[] = {&P};
-    RT_CUDA(ctx, cudaLaunchKernel(collision_kernel(ctx), dim3(ctx->grid),
+    RT_CUDA(ctx, cudaLaunchKernel(collision_kernel(ctx, parts, ctl != nullptr), dim3(ctx->grid),
                                   dim3(collision_threads(ctx) / (ctx->staged ? ctx->per_sm : 1)), args,
                                   ctx->staged ? ctx->smem_bytes : 0, s));
     RT_CUDA(ctx, cudaGetLastError());
