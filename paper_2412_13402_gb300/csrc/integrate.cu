@@ -115,6 +115,8 @@ __device__ int block_excl_scan(int v, int *total) {
 // instance: a grid-stride loop over its rows.
 template <class R>
 __global__ void __launch_bounds__(kRedThreads) stage_kernel(RowParams Q, StageArgs a) {
+    pdl_begin();
+    pdl_wait();
     if (a.batched) {
         __shared__ int s_pre[kMaxBatch + 1];  // s_pre[i]: first active row block of instance i
         const int NI = Q.n_inst;              // <= kMaxBatch (checked on the host)
@@ -163,6 +165,8 @@ __global__ void __launch_bounds__(kRedThreads) stage_kernel(RowParams Q, StageAr
 // rows (fixed chunk boundaries and order, so the norms are deterministic); finished instances
 // are skipped when respect_done.
 __global__ void wrms_chunks(RowParams Q, const Ctl *ctl, const double *wsq, double *part, int respect_done) {
+    pdl_begin();
+    pdl_wait();
     const int i = blockIdx.y;
     if (respect_done && ctl[i].done) return;
     const InstDev I = Q.inst[i];
@@ -176,6 +180,8 @@ __global__ void wrms_chunks(RowParams Q, const Ctl *ctl, const double *wsq, doub
 
 __global__ void controller_kernel(RowParams Q, Ctl *ctl, CtlParams cp, const double *part,
                                   unsigned long long *range) {
+    pdl_begin();
+    pdl_wait();
     Ctl *c = ctl + blockIdx.x;
     if (c->done) return;
     const InstDev I = Q.inst[blockIdx.x];
@@ -322,8 +328,7 @@ int launch_stage(rtbte_ctx *ctx, const StageArgs &a, cudaStream_t s) {
     const long long want = a.batched ? ctx->n_rblk : (ctx->n_y + kRedThreads - 1) / kRedThreads;
     const int grid = (int)std::max<long long>(1, std::min<long long>(want, ctx->stage_resident > 0 ? ctx->stage_resident
                                                                                                : 2 * ctx->num_sms));
-    stage_kernel<R><<<grid, kRedThreads, 0, s>>>(row_params(ctx), a);
-    RT_CUDA(ctx, cudaGetLastError());
+    RT_CUDA(ctx, launch_pdl(stage_kernel<R>, dim3(grid), dim3(kRedThreads), 0, s, row_params(ctx), a));
     ctx->launches++;
     return RTBTE_OK;
 }
@@ -364,11 +369,10 @@ int enqueue_attempt(rtbte_ctx *ctx, const Tableau &T, const CtlParams &cp, unsig
         if ((rc = stage(ctx, a, s))) return rc;
     }
     double *chunks = ctx->wrms_part.as<double>() + 2 * ctx->n_y;
-    wrms_chunks<<<dim3(kWrmsChunks, n_inst(ctx)), kRedThreads, 0, s>>>(row_params(ctx), ctx->ctl.as<Ctl>(),
-                                                                      ctx->wrms_part.as<double>(), chunks, 1);
-    controller_kernel<<<n_inst(ctx), kRedThreads, 0, s>>>(row_params(ctx), ctx->ctl.as<Ctl>(), cp, chunks,
-                                                          ctx->range_scratch.as<unsigned long long>());
-    RT_CUDA(ctx, cudaGetLastError());
+    RT_CUDA(ctx, launch_pdl(wrms_chunks, dim3(kWrmsChunks, n_inst(ctx)), dim3(kRedThreads), 0, s, row_params(ctx),
+                            ctx->ctl.as<Ctl>(), ctx->wrms_part.as<double>(), chunks, 1));
+    RT_CUDA(ctx, launch_pdl(controller_kernel, dim3(n_inst(ctx)), dim3(kRedThreads), 0, s, row_params(ctx),
+                            ctx->ctl.as<Ctl>(), cp, chunks, ctx->range_scratch.as<unsigned long long>()));
     ctx->launches += 2;
     return RTBTE_OK;
 }
@@ -386,6 +390,8 @@ long long graph_key(int method, unsigned parts, bool forcing, const CtlParams &c
 // so the loop ends after at most `cap` attempts whatever the other kernels do.
 __global__ void loop_guard(const Ctl *ctl, int n_inst, int *iter, int cap, cudaGraphConditionalHandle h) {
     __shared__ int active;
+    pdl_begin();
+    pdl_wait();
     if (threadIdx.x == 0) active = 0;
     __syncthreads();
     for (int i = threadIdx.x; i < n_inst; i += blockDim.x)
@@ -447,8 +453,8 @@ int attempt_graph(rtbte_ctx *ctx, int method, const CtlParams &cp, unsigned part
     e = cudaStreamBeginCaptureToGraph(ctx->cap_stream, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal);
     if (e != cudaSuccess) return bail(e, "cudaStreamBeginCaptureToGraph");
     int rc = enqueue_attempt(ctx, T, cp, parts, forcing, ctx->cap_stream);
-    loop_guard<<<1, 256, 0, ctx->cap_stream>>>(ctx->ctl.as<Ctl>(), n_inst(ctx), iter, cap, h);
-    cudaError_t el = cudaGetLastError();
+    const cudaError_t el = launch_pdl(loop_guard, dim3(1), dim3(256), 0, ctx->cap_stream, ctx->ctl.as<Ctl>(), n_inst(ctx),
+                                      iter, cap, h);
     e = cudaStreamEndCapture(ctx->cap_stream, &body);
     ctx->graph_launches[key] = (int)(ctx->launches - before) + 1;  // kernels per attempt, guard included
     ctx->launches = before;                                       // captured, not executed

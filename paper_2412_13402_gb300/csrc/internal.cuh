@@ -27,6 +27,7 @@
 #include <string>
 #include <system_error>
 #include <thread>
+#include <tuple>
 #include <vector>
 
 #include "rtbte.h"
@@ -159,8 +160,7 @@ inline long long round_up(long long x, long long m) { return (x + m - 1) / m * m
 // still running (once all of that one's blocks have called pdl_begin or ended), so its launch
 // and prologue are hidden; it must call pdl_wait, which returns when the kernel before has ended
 // and its writes are visible, before it touches any memory that one reads or writes.
-template <class... P, class... A>
-inline cudaError_t launch_pdl(void (*f)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A &&...args) {
+inline cudaError_t launch_pdl_fn(const void *f, dim3 grid, dim3 block, size_t smem, cudaStream_t s, void **args) {
     cudaLaunchConfig_t c{};
     c.gridDim = grid;
     c.blockDim = block;
@@ -171,7 +171,15 @@ inline cudaError_t launch_pdl(void (*f)(P...), dim3 grid, dim3 block, size_t sme
     at.val.programmaticStreamSerializationAllowed = 1;
     c.attrs = &at;
     c.numAttrs = 1;
-    return cudaLaunchKernelEx(&c, f, static_cast<P>(args)...);
+    return cudaLaunchKernelExC(&c, f, args);
+}
+template <class... P, class... A>
+inline cudaError_t launch_pdl(void (*f)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A &&...args) {
+    std::tuple<P...> vals(static_cast<P>(args)...);  // the arguments in the kernel's own types
+    void *ptrs[sizeof...(P)];
+    size_t n = 0;
+    std::apply([&](auto &...v) { ((ptrs[n++] = (void *)&v), ...); }, vals);
+    return launch_pdl_fn((const void *)f, grid, block, smem, s, ptrs);
 }
 __device__ __forceinline__ void pdl_begin() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }

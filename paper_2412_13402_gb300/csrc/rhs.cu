@@ -76,8 +76,24 @@ __global__ void __launch_bounds__(NT, MINB) rhs_kernel(KParams P) {
     __shared__ int s_unit;
     R *sm = reinterpret_cast<R *>(smem_raw);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
-    const int n_tail = P.n_tail_d ? *P.n_tail_d : P.n_tail;
     int staged = -1;
+    // (no pdl_begin: blocks of the row kernel behind this one, waiting on SMs that finish early, slow the
+    // others down -- graphene 180 345 -> 361 us, 64 instances 991 -> 1090)
+    if (!P.n_tail_d) {  // (a device re-split writes the bounds just before)
+        // the first packets' entries on their way to L2 while the populations are still computed
+        const int4 from = P.bound[blockIdx.x];
+        const Group &G = P.groups[from.y];
+        const int lg = WIDE ? 5 : G.lanes_log2;
+        const int k = from.x + warp * (32 >> lg) + (lane >> lg);
+        if ((lane & ((1 << lg) - 1)) == 0 && k < min(P.bound[blockIdx.x + 1].x, G.item_end)) {
+            GroupView<R> V;
+            V.idx = G.idx;
+            V.W = reinterpret_cast<const R *>(G.W);
+            prefetch_item(V, __ldg(reinterpret_cast<const int4 *>(P.items) + k));
+        }
+    }
+    pdl_wait();
+    const int n_tail = P.n_tail_d ? *P.n_tail_d : P.n_tail;
     for (int u = blockIdx.x;;) {
         const int4 from = P.bound[u];
         const int end = P.bound[u + 1].x;
@@ -131,6 +147,8 @@ __global__ void split_kernel(const Group *groups, int n_groups, const long long 
     __shared__ int csum[32];
     __shared__ int s_same;
     const int T = blockDim.x;  // 256 threads, n_groups <= 1024 (checked on the host)
+    pdl_begin();
+    pdl_wait();
     // the tables of the last split still hold when the same instances are active for the same
     // parts (memo: the done flags and mask it was made for, and a flag the host clears whenever
     // the item weights change)
@@ -240,12 +258,16 @@ __global__ void split_kernel(const Group *groups, int n_groups, const long long 
 // y (FP64) -> population copies in the compute precision
 template <class R>
 __global__ void __launch_bounds__(256) prep_kernel(RowParams Q, const double *y, long long n) {
+    pdl_begin();
+    pdl_wait();
     for_rows(Q, n, [&](int, const InstDev &I, long long c) { write_pops<R>(Q, I, c - I.y_off, (R)y[c]); });
 }
 
 template <class R>
 __global__ void __launch_bounds__(256) rows_kernel(RowParams Q, unsigned parts, double *out, const double *forcing,
                                                    long long n) {
+    pdl_begin();
+    pdl_wait();
     for_rows(Q, n, [&](int, const InstDev &I, long long c) {
         double v = row_value<R>(Q, I, c - I.y_off, parts);
         if (forcing) v += forcing[c];
@@ -838,11 +860,8 @@ int launch_prep_from_y(rtbte_ctx *ctx, const double *y, cudaStream_t s) {
     RowParams Q = row_params(ctx);
     const int threads = 256;
     const int blocks = row_grid(ctx);
-    if (ctx->precision == RTBTE_PREC_FP64)
-        prep_kernel<double><<<blocks, threads, 0, s>>>(Q, y, ctx->n_y);
-    else
-        prep_kernel<float><<<blocks, threads, 0, s>>>(Q, y, ctx->n_y);
-    RT_CUDA(ctx, cudaGetLastError());
+    RT_CUDA(ctx, launch_pdl(ctx->precision == RTBTE_PREC_FP64 ? prep_kernel<double> : prep_kernel<float>, dim3(blocks),
+                            dim3(threads), 0, s, Q, y, ctx->n_y));
     ctx->launches++;
     return RTBTE_OK;
 }
@@ -852,10 +871,9 @@ int launch_prep_from_y(rtbte_ctx *ctx, const double *y, cudaStream_t s) {
 int launch_resplit(rtbte_ctx *ctx, unsigned parts, const Ctl *ctl, cudaStream_t s) {
     if (ctx->inst.size() <= 1) return RTBTE_OK;
     const DynTab T = dyn_tab(ctx);
-    split_kernel<<<1, 256, 0, s>>>(ctx->groups.as<Group>(), ctx->n_groups, ctx->gwt.as<long long>(), ctl, parts,
-                                   ctx->grid, kResplitTail, kResplitTailMin, T.bound, T.act, T.n_tail, T.memo,
-                                   (int)ctx->inst.size());
-    RT_CUDA(ctx, cudaGetLastError());
+    RT_CUDA(ctx, launch_pdl(split_kernel, dim3(1), dim3(256), 0, s, ctx->groups.as<Group>(), ctx->n_groups,
+                            ctx->gwt.as<long long>(), ctl, parts, ctx->grid, kResplitTail, kResplitTailMin, T.bound, T.act,
+                            T.n_tail, T.memo, (int)ctx->inst.size()));
     ctx->launches++;
     return RTBTE_OK;
 }
@@ -914,9 +932,9 @@ static int launch_core_t(rtbte_ctx *ctx, unsigned parts, const Ctl *ctl, cudaStr
     int rc;
     if ((rc = timing_begin(ctx, s, &ev))) return rc;
     void *args[] = {&P};
-    RT_CUDA(ctx, cudaLaunchKernel(collision_kernel(ctx, parts, ctl != nullptr), dim3(ctx->grid),
-                                  dim3(collision_threads(ctx) / (ctx->staged ? ctx->per_sm : 1)), args,
-                                  ctx->staged ? ctx->smem_bytes : 0, s));
+    RT_CUDA(ctx, launch_pdl_fn(collision_kernel(ctx, parts, ctl != nullptr), dim3(ctx->grid),
+                               dim3(collision_threads(ctx) / (ctx->staged ? ctx->per_sm : 1)),
+                               ctx->staged ? ctx->smem_bytes : 0, s, args));
     RT_CUDA(ctx, cudaGetLastError());
     ctx->launches++;
     return timing_end(ctx, s, ev);
@@ -1183,11 +1201,8 @@ int launch_rows(rtbte_ctx *ctx, unsigned parts, double *out, const double *forci
     RowParams Q = row_params(ctx);
     const int threads = 256;
     const int blocks = row_grid(ctx);
-    if (ctx->precision == RTBTE_PREC_FP64)
-        rows_kernel<double><<<blocks, threads, 0, s>>>(Q, parts, out, forcing, ctx->n_y);
-    else
-        rows_kernel<float><<<blocks, threads, 0, s>>>(Q, parts, out, forcing, ctx->n_y);
-    RT_CUDA(ctx, cudaGetLastError());
+    RT_CUDA(ctx, launch_pdl(ctx->precision == RTBTE_PREC_FP64 ? rows_kernel<double> : rows_kernel<float>, dim3(blocks),
+                            dim3(threads), 0, s, Q, parts, out, forcing, ctx->n_y));
     ctx->launches++;
     return RTBTE_OK;
 }

@@ -137,6 +137,8 @@ __global__ void __launch_bounds__(NT) rhs_small(KParams P, SmallPlan S, const In
     copy_in(M.runs, S.runs + (long long)blockIdx.x * S.max_runs, S.max_runs);
     const int r0 = __ldg(S.row_off + blockIdx.x) + threadIdx.x, r1 = __ldg(S.row_off + blockIdx.x + 1);
     const InstDev I = *inst;
+    pdl_begin();
+    pdl_wait();
     for (int i = threadIdx.x; i < I.n_c; i += NT) M.f[i] = (R)y[i];
     const double *yN = y + I.n_c;
     if (I.N_q == I.N_q_pad) {
@@ -556,8 +558,8 @@ int launch_small_rhs(rtbte_ctx *ctx, unsigned parts, const double *y, double *yd
     std::pair<cudaEvent_t, cudaEvent_t> ev;
     int rc;
     if ((rc = timing_begin(ctx, s, &ev))) return rc;
-    RT_CUDA(ctx, cudaLaunchKernel(rhs_fn(ctx), dim3(ctx->small_grid), dim3(small_threads(ctx)), args,
-                                  small_smem(ctx->real_size, S, false), s));
+    RT_CUDA(ctx, launch_pdl_fn(rhs_fn(ctx), dim3(ctx->small_grid), dim3(small_threads(ctx)),
+                               small_smem(ctx->real_size, S, false), s, args));
     ctx->launches++;
     return timing_end(ctx, s, ev);
 }
