@@ -67,15 +67,21 @@ template <class R> struct GroupView {
     int lg;  // lanes per item = 1 << lg
 };
 
-// Entry loads of one item on a sub-warp of 1 << lg lanes: VPL vectors of 4 entries per lane
-// (16-byte streaming loads, or cached ones where the entries are read again by the same kernel);
-// sl is the lane's index in its sub-warp.
+// How items and entries are loaded: streaming or ordinary loads from global memory (items always
+// ordinary), or generic ones from shared memory.
+enum { LOAD_STREAM = 0, LOAD_CACHED = 1, LOAD_SHARED = 2 };
+template <int LOAD, class T> __device__ __forceinline__ T load16(const T *p) {
+    return LOAD == LOAD_STREAM ? __ldcs(p) : LOAD == LOAD_CACHED ? __ldg(p) : *p;
+}
+
+// Entry loads of one item on a sub-warp of 1 << lg lanes: VPL vectors of 4 entries per lane, 16
+// bytes a load; sl is the lane's index in its sub-warp.
 template <class R, int VPL> struct Batch;
 template <int VPL> struct Batch<float, VPL> {
     uint4 iv[VPL];
     float4 wv[VPL];
     float Np;  // ph-e destination population, loaded with the entries
-    template <bool CACHED = false>
+    template <int LOAD = LOAD_STREAM>
     __device__ __forceinline__ void issue(const GroupView<float> &V, const Item &it, int sl, int lg) {
         const int nv = it.len >> 2;
         if (V.part == PART_PHE) Np = V.Nglob[it.dest];
@@ -85,8 +91,8 @@ template <int VPL> struct Batch<float, VPL> {
         for (int j = 0; j < VPL; ++j) {
             const int v = sl + (j << lg);
             if (v < nv) {
-                iv[j] = CACHED ? __ldg(ip + v) : __ldcs(ip + v);
-                wv[j] = CACHED ? __ldg(wp + v) : __ldcs(wp + v);
+                iv[j] = load16<LOAD>(ip + v);
+                wv[j] = load16<LOAD>(wp + v);
             }
         }
     }
@@ -98,7 +104,7 @@ template <int VPL> struct Batch<double, VPL> {
     uint4 iv[VPL];
     double2 wa[VPL], wb[VPL];
     double Np;  // ph-e destination population, loaded with the entries
-    template <bool CACHED = false>
+    template <int LOAD = LOAD_STREAM>
     __device__ __forceinline__ void issue(const GroupView<double> &V, const Item &it, int sl, int lg) {
         const int nv = it.len >> 2;
         if (V.part == PART_PHE) Np = V.Nglob[it.dest];
@@ -108,9 +114,9 @@ template <int VPL> struct Batch<double, VPL> {
         for (int j = 0; j < VPL; ++j) {
             const int v = sl + (j << lg);
             if (v < nv) {
-                iv[j] = CACHED ? __ldg(ip + v) : __ldcs(ip + v);
-                wa[j] = CACHED ? __ldg(wp + 2 * v) : __ldcs(wp + 2 * v);
-                wb[j] = CACHED ? __ldg(wp + 2 * v + 1) : __ldcs(wp + 2 * v + 1);
+                iv[j] = load16<LOAD>(ip + v);
+                wa[j] = load16<LOAD>(wp + 2 * v);
+                wb[j] = load16<LOAD>(wp + 2 * v + 1);
             }
         }
     }
@@ -276,7 +282,7 @@ struct ItemSum4 {
 // and eight shuffles an item), bounds tests on full items and separate emission / absorption
 // branches, graphene 180 took 395 us (full RHS, 2.27 GB), silicon 32 470 us and a 64-instance
 // ensemble 1.76 ms; without them 363, 430 and 1.42 ms.
-template <class R, bool WIDE, bool CACHED = false>
+template <class R, bool WIDE, int LOAD>
 __device__ __forceinline__ void run_range(const KParams &P, const GroupView<R> &V, int a, int b, int warp, int nwarps,
                                           int lane) {
     const int lg = WIDE ? 5 : V.lg;
@@ -288,9 +294,11 @@ __device__ __forceinline__ void run_range(const KParams &P, const GroupView<R> &
     int k = kb + (lane >> lg);
     const int4 *items = reinterpret_cast<const int4 *>(P.items);
     // (unsigned: an index past INT_MAX near the end of a very long list is out of range, not negative)
-    auto fetch = [&](unsigned i) { return i < (unsigned)b ? __ldg(items + i) : make_int4(0, 0, 0, 0); };
+    auto fetch = [&](unsigned i) {
+        return i < (unsigned)b ? load16<LOAD == LOAD_SHARED ? LOAD_SHARED : LOAD_CACHED>(items + i) : make_int4(0, 0, 0, 0);
+    };
     const int pf = P.pf_dist;  // packets ahead whose entries are prefetched into L2 (0: none)
-    const bool lead = sl == 0 && pf > 0;
+    const bool lead = LOAD != LOAD_SHARED && sl == 0 && pf > 0;
     int4 d = fetch(k), dn = fetch(k + step), dp = make_int4(0, 0, 0, 0);
     if (lead) {
         for (int j = 1; j < pf; ++j) prefetch_item(V, fetch((unsigned)k + j * step));
@@ -302,7 +310,7 @@ __device__ __forceinline__ void run_range(const KParams &P, const GroupView<R> &
         d = dn;
         dn = fetch((unsigned)k + 2 * step);
         Batch<R, 4> B;
-        B.template issue<CACHED>(V, it, sl, lg);
+        B.template issue<LOAD>(V, it, sl, lg);
         if (lead) {
             prefetch_item(V, dp);
             dp = fetch((unsigned)k + (pf + 1) * step);

@@ -311,9 +311,9 @@ struct rtbte_ctx {
     bool staged = false;
     bool wide = true;  // every group uses whole-warp items (the kernel variant without sub-warps)
     // one-launch kernels of a small single instance (small.cu); small_grid 0: not taken
-    rtbte::DevBuf small_tab, small_pops, small_sync;  // small_tab: items, runs, rows, row offsets at small_at[0..3]
-    size_t small_at[4] = {0, 0, 0, 0};
-    int small_grid = 0, small_max_items = 0, small_max_rows = 0, small_max_runs = 0;
+    rtbte::DevBuf small_tab, small_pops, small_sync;  // small_tab: items, runs, rows, row offsets, entry places at small_at[]
+    size_t small_at[5] = {0, 0, 0, 0, 0};
+    int small_grid = 0, small_max_items = 0, small_max_rows = 0, small_max_runs = 0, small_max_entries = 0;
     void *small_sync_host = nullptr;  // pinned mirror of small_sync
     int num_sms = 0;
     size_t smem_optin = 0;

@@ -103,7 +103,7 @@ __global__ void __launch_bounds__(NT, MINB) rhs_kernel(KParams P) {
             if (a < b && !(P.ctl && P.ctl[G.inst].done)) {  // (done: the instance is at its t_out)
                 GroupView<R> V;
                 enter_group<R, STAGED>(P, g, sm, staged, V);
-                run_range<R, WIDE, CACHED>(P, V, a, b, warp, nwarps, lane);
+                run_range<R, WIDE, CACHED ? LOAD_CACHED : LOAD_STREAM>(P, V, a, b, warp, nwarps, lane);
             }
             if (end <= G.item_end) break;
             g = P.act[++at];

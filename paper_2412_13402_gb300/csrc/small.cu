@@ -7,14 +7,20 @@
 // populations, runs every work item of its rows -- whatever their part and mode -- and sums them
 // itself, so no partial leaves the SM and the only exchange between CTAs is the new populations.
 //   - rhs_small: one launch per RHS, populations straight from y, rows straight to ydot;
-//   - attempts_small: up to `cap` attempted steps per launch on a cooperative grid, two grid
-//     barriers per stage less one: S - 1 to exchange stage populations, one before and one after
-//     the chunk sums of the WRMS norm; every CTA then runs the controller on its own copy.
+//   - attempts_small: up to `cap` attempted steps per launch on a cooperative grid: S grid barriers
+//     an attempt to exchange populations (the last one the squared errors too, one more where the
+//     norm's chunks exceed 8 rows); every CTA runs the controller on its own copy, beside the first
+//     stage of the next attempt.  Where they fit, the CTA's items and entries stay in shared memory
+//     for the launch: a barrier's acquire drops L1, so each stage would fetch them from L2 again
+//     (toy 12 x 12 FP64 31.1 -> 30.2 us an attempt, graphene 36 FP32 64 -> 62 us).
 // Items, their lanes and entry order, the order of a row's items, the norm's chunks and the
 // controller are those of the launch sequence (collide.cuh, rows.cuh, step.cuh), so both give the
-// same results bit for bit.  The 12 x 12 toy model in FP64 (15 174 entries): RHS 18.9 -> 8.2 us a
-// call, Bogacki-Shampine attempts 62 -> 31 us.  What is left of an attempt is latency: a grid barrier
-// 2.5 us, the items of a stage 2 us, its rows 0.9 us, the populations' copy 0.6 us.
+// same results bit for bit.  The 12 x 12 toy model in FP64 (15 174 entries), launch sequence and one
+// launch: RHS 18.9 and 4.9 us a call, Bogacki-Shampine attempts 62 and 30.2 us.  What is left of an
+// attempt is latency: about 2.4 us of each stage's 7.5 in the barrier, 2 in its items and 2 in its rows
+// (chains of FP64 operations), 0.6 in the populations' copy.  Messages in place of the barriers
+// (values with a sequence number beside them, polled by every CTA) took 38 us an attempt: the
+// polling of all CTAs on the same few lines costs more than the barrier saves.
 #include <algorithm>
 #include <cstring>
 #include <memory>
@@ -50,6 +56,8 @@ struct SmallPlan {
     int max_runs, max_items, max_rows;  // largest CTA's
     int n_f, n_N, n_P;     // populations held: f, all modes' N (mode stride N_q_pad), sub-lattice N
     const int *pp_full;    // [M] phonon of each sub-lattice state
+    const int *item_at;    // [items] where an item's entries go in its CTA's copy of the lists
+    int max_entries;       // largest CTA's entries; 0: the attempts' lists are not held
 };
 
 template <class R> struct SmallMem {  // shared memory of a CTA
@@ -59,6 +67,9 @@ template <class R> struct SmallMem {  // shared memory of a CTA
     SmallRow *rows;
     double *y;  // [2][max_rows] state of the owned rows: current and attempted, in turn
     double *K;  // [stages][max_rows]
+    ItemRec *items;  // [max_items], if the lists are held
+    R *W;            // [max_entries]
+    uint32_t *idx;
     __device__ __forceinline__ SmallMem(unsigned char *raw, const SmallPlan &S) {
         runs = reinterpret_cast<SmallRun *>(raw);
         f = reinterpret_cast<R *>(runs + S.max_runs);
@@ -68,11 +79,15 @@ template <class R> struct SmallMem {  // shared memory of a CTA
         rows = reinterpret_cast<SmallRow *>(partials + S.max_items);
         y = reinterpret_cast<double *>(rows + S.max_rows);
         K = y + 2 * S.max_rows;
+        items = reinterpret_cast<ItemRec *>(K + kMaxStages * S.max_rows);
+        W = reinterpret_cast<R *>(items + S.max_items);
+        idx = reinterpret_cast<uint32_t *>(W + S.max_entries);
     }
 };
 size_t small_smem(size_t R, const SmallPlan &S, bool attempts) {  // every array a multiple of 16 bytes
     return sizeof(SmallRun) * S.max_runs + R * (size_t)(S.n_f + S.n_N + S.n_P + S.max_items) +
-           (attempts ? (sizeof(SmallRow) + sizeof(double) * (2 + kMaxStages)) * S.max_rows : 0);
+           (attempts ? (sizeof(SmallRow) + sizeof(double) * (2 + kMaxStages)) * S.max_rows : 0) +
+           (attempts && S.max_entries > 0 ? sizeof(ItemRec) * S.max_items + (4 + R) * (size_t)S.max_entries : 0);
 }
 
 template <class T> __device__ __forceinline__ void copy_in(T *dst, const T *src, int n) {  // 16-byte units
@@ -84,12 +99,13 @@ template <class T> __device__ __forceinline__ void copy_in(T *dst, const T *src,
 // Every item of this CTA's rows whose part is in the mask, by `nwarps` warps of which this is
 // number `warp`.  Warps take packets in turn across the runs, so short runs do not all fall to the
 // first warps.
-template <class R, bool CACHED>
+template <class R, int LOAD>
 __device__ __forceinline__ void own_items(const KParams &P, const SmallPlan &S, const SmallMem<R> &M, unsigned parts,
                                           int warp, int nwarps) {
     const int lane = threadIdx.x & 31;
     KParams L = P;
     L.partials = M.partials;
+    if (LOAD == LOAD_SHARED) L.items = M.items;
     for (int u = 0; u < S.max_runs; ++u) {
         const SmallRun &run = M.runs[u];
         const int a = run.a, b = run.b;
@@ -104,7 +120,7 @@ __device__ __forceinline__ void own_items(const KParams &P, const SmallPlan &S, 
         V.s0 = V.part == PART_PP ? M.P : M.f;
         V.s1 = M.N + run.N_at;
         V.Nglob = M.N;
-        run_range<R, false, CACHED>(L, V, a, b, warp, nwarps, lane);
+        run_range<R, false, LOAD>(L, V, a, b, warp, nwarps, lane);
         const int packets = (b - a + (32 >> V.lg) - 1) >> (5 - V.lg);
         warp -= packets;
         while (warp < 0) warp += nwarps;
@@ -152,7 +168,7 @@ __global__ void __launch_bounds__(NT) rhs_small(KParams P, SmallPlan S, const In
     if (parts & RTBTE_PHPH)
         for (int a = threadIdx.x; a < I.M; a += NT) M.P[a] = (R)yN[__ldg(S.pp_full + a)];
     __syncthreads();
-    own_items<R, false>(P, S, M, parts, threadIdx.x >> 5, NT / 32);
+    own_items<R, LOAD_STREAM>(P, S, M, parts, threadIdx.x >> 5, NT / 32);
     __syncthreads();
     for (int r = r0; r < r1; r += NT) {
         const SmallRow row = S.rows[r];
@@ -221,7 +237,38 @@ __device__ __forceinline__ double small_wrms(const double *wsq, long long ni, in
     return t < 32 ? ((ws[0] + ws[1]) + ws[2]) + ws[3] : 0.0;
 }
 
+// Copies the CTA's items and their entries into shared memory and points its runs at them.
 template <class R, int NT>
+__device__ __forceinline__ void hold_lists(const KParams &P, const SmallPlan &S, const SmallMem<R> &M) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int item0 = M.runs[0].a;
+    for (int u = 0; u < S.max_runs; ++u) {
+        const SmallRun &run = M.runs[u];
+        for (int k = run.a + warp; k < run.b; k += NT / 32) {
+            const int4 d = __ldg(reinterpret_cast<const int4 *>(P.items) + k);
+            const Item it = item_from(d);
+            const int at = __ldg(S.item_at + k), vw = (int)(it.len * sizeof(R) / 16);
+            const uint4 *ip = reinterpret_cast<const uint4 *>(run.idx + it.begin);
+            const uint4 *wp = reinterpret_cast<const uint4 *>(reinterpret_cast<const R *>(run.W) + it.begin);
+            for (int v = lane; v < it.len >> 2; v += 32) reinterpret_cast<uint4 *>(M.idx + at)[v] = __ldg(ip + v);
+            for (int v = lane; v < vw; v += 32) reinterpret_cast<uint4 *>(M.W + at)[v] = __ldg(wp + v);
+            if (lane == 0) reinterpret_cast<int4 *>(M.items)[k - item0] = make_int4(at, d.y, d.z, d.w & 0xffffff);
+        }
+    }
+    __syncthreads();
+    for (int u = threadIdx.x; u < S.max_runs; u += NT) {
+        SmallRun &run = M.runs[u];
+        if (run.a < run.b) {
+            run.a -= item0;
+            run.b -= item0;
+        }
+        run.idx = M.idx;
+        run.W = M.W;
+    }
+}
+
+// LOAD: LOAD_SHARED where the CTAs' lists fit in shared memory, else LOAD_CACHED.
+template <class R, int NT, int LOAD>
 __global__ void __launch_bounds__(NT) attempts_small(KParams P, SmallPlan S, SmallPops B, StageArgs a, double *chunks,
                                                      int cap, SmallSync *sync) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -234,6 +281,7 @@ __global__ void __launch_bounds__(NT) attempts_small(KParams P, SmallPlan S, Sma
     copy_in(M.rows, S.rows + row0, nrows);
     __syncthreads();
     if (C.done) return;  // (alike in every CTA)
+    if (LOAD == LOAD_SHARED) hold_lists<R, NT>(P, S, M);
     const long long ni = a.n;
     const int L = (int)((ni + kWrmsChunks - 1) / kWrmsChunks);  // rows of a chunk
     const int warp = threadIdx.x >> 5;
@@ -281,7 +329,7 @@ __global__ void __launch_bounds__(NT) attempts_small(KParams P, SmallPlan S, Sma
                 asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;\n" ::: "memory");
                 if (split) asm volatile("bar.sync 1, %0;\n" ::"n"(NT - 32) : "memory");
                 else __syncthreads();
-                own_items<R, true>(P, S, M, a.parts, warp - t0 / 32, (NT - t0) / 32);
+                own_items<R, LOAD>(P, S, M, a.parts, warp - t0 / 32, (NT - t0) / 32);
             }
             __syncthreads();
             if (split) {
@@ -381,6 +429,8 @@ SmallPlan small_plan(rtbte_ctx *ctx) {
     S.n_N = I.d.nmodes * I.N_q_pad;
     S.n_P = I.M_pad;
     S.pp_full = I.t_ppfull.as<int>();
+    S.item_at = reinterpret_cast<const int *>(tab + ctx->small_at[4]);
+    S.max_entries = ctx->small_max_entries;
     return S;
 }
 
@@ -389,8 +439,11 @@ const void *rhs_fn(const rtbte_ctx *ctx) {
                                              : (const void *)rhs_small<float, kSmallThreads>;
 }
 const void *attempts_fn(const rtbte_ctx *ctx) {
-    return ctx->precision == RTBTE_PREC_FP64 ? (const void *)attempts_small<double, kSmallThreads64>
-                                             : (const void *)attempts_small<float, kSmallThreads64>;
+    if (ctx->small_max_entries > 0)
+        return ctx->precision == RTBTE_PREC_FP64 ? (const void *)attempts_small<double, kSmallThreads64, LOAD_SHARED>
+                                                 : (const void *)attempts_small<float, kSmallThreads64, LOAD_SHARED>;
+    return ctx->precision == RTBTE_PREC_FP64 ? (const void *)attempts_small<double, kSmallThreads64, LOAD_CACHED>
+                                             : (const void *)attempts_small<float, kSmallThreads64, LOAD_CACHED>;
 }
 int small_threads(const rtbte_ctx *ctx) {
     return ctx->precision == RTBTE_PREC_FP64 ? kSmallThreads64 : kSmallThreads;
@@ -466,11 +519,11 @@ int make_small_plan(rtbte_ctx *ctx, const ItemRec *items, int n, const std::vect
         max_items = std::max(max_items, m);
         max_rows = std::max(max_rows, (int)own[b].size());
     }
-    // one buffer, copied at once: items, runs, rows, row offsets
-    const size_t len[4] = {sizeof(ItemRec) * n, sizeof(SmallRun) * (size_t)G * ng, sizeof(SmallRow) * ny,
-                           sizeof(int) * (G + 1)};
+    // one buffer, copied at once: items, runs, rows, row offsets, places of the items' entries
+    const size_t len[5] = {sizeof(ItemRec) * n, sizeof(SmallRun) * (size_t)G * ng, sizeof(SmallRow) * ny,
+                           sizeof(int) * (G + 1), sizeof(int) * n};
     size_t bytes = 0;
-    for (int k = 0; k < 4; ++k) {
+    for (int k = 0; k < 5; ++k) {
         ctx->small_at[k] = bytes;
         bytes += (len[k] + 15) / 16 * 16;
     }
@@ -478,11 +531,13 @@ int make_small_plan(rtbte_ctx *ctx, const ItemRec *items, int n, const std::vect
     ItemRec *out = reinterpret_cast<ItemRec *>(tab.get() + ctx->small_at[0]);
     SmallRun *runs = reinterpret_cast<SmallRun *>(tab.get() + ctx->small_at[1]);
     SmallRow *rows = reinterpret_cast<SmallRow *>(tab.get() + ctx->small_at[2]);
+    int *item_at = reinterpret_cast<int *>(tab.get() + ctx->small_at[4]);
     std::memcpy(tab.get() + ctx->small_at[3], off.data(), len[3]);
     std::memset(runs, 0, len[1]);
     // a CTA's items by group and, within it, alike ones together (the packets of order_packets in
     // rhs.cu): counting sort over (group, process, vectors per lane)
     std::unique_ptr<int[]> counts(new int[(size_t)G * (8 * ng + 1)]), keys(new int[n]);
+    std::vector<int> entries(G);
     parallel_for(G, threads, [&](int b) {
         int *count = counts.get() + (size_t)b * (8 * ng + 1), *key = keys.get() + first[b];
         std::fill(count, count + 8 * ng + 1, 0);
@@ -528,7 +583,14 @@ int make_small_plan(rtbte_ctx *ctx, const ItemRec *items, int n, const std::vect
                 it = items[by_slot[s]];
                 it.slot = (unsigned)m;
             }
+        int e = 0;
+        for (int k = first[b]; k < first[b + 1]; ++k) {
+            item_at[k] = e;
+            e += out[k].len;
+        }
+        entries[b] = e;
     });
+    ctx->small_max_entries = *std::max_element(entries.begin(), entries.end());
     ctx->small_max_items = (int)round_up(max_items, 4);
     ctx->small_max_rows = (int)round_up(max_rows, 2);
     ctx->small_max_runs = ng;
@@ -540,6 +602,7 @@ int make_small_plan(rtbte_ctx *ctx, const ItemRec *items, int n, const std::vect
     RT_CUDA(ctx, cudaMemcpyAsync(ctx->small_tab.p, tab.get(), bytes, cudaMemcpyHostToDevice, ctx->stream));
     ctx->small_grid = G;
     SmallPlan S = small_plan(ctx);
+    if (small_smem(R, S, true) + 2048 > ctx->smem_optin) S.max_entries = ctx->small_max_entries = 0;
     if (small_smem(R, S, true) + 2048 > ctx->smem_optin) {
         ctx->small_grid = 0;
         return RTBTE_OK;

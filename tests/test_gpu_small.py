@@ -14,6 +14,7 @@ MODELS = {
     "toy30": lambda: ri.toy2d(30),      # 3600 rows: more than 8 rows to a chunk of the error norm
     "graphene27": lambda: ri.graphene(27, sigma_eph=0.05, sigma_pp=0.006),
     "ladder3d": lambda: ri.ladder3d(4),  # folded grid
+    "graphene66": lambda: ri.graphene(66, sigma_eph=0.0075, sigma_pp=0.00075),  # lists and populations past a CTA's memory
 }
 
 
