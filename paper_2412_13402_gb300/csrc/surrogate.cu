@@ -40,7 +40,7 @@ constexpr int kLayers = 4;
 // C + z*M*ldc.  Epilogue (split 1 only): + bias[n], tanh if act, times 1 - back^2 (the gradient
 // through tanh), BF16 copy if Cb.
 template <bool TA, bool TB>
-__global__ void __launch_bounds__(kGemmThreads) gemm_bf16(const bf16 *A, int lda, const bf16 *B, int ldb, float *C,
+__global__ void __launch_bounds__(kGemmThreads, 4) gemm_bf16(const bf16 *A, int lda, const bf16 *B, int ldb, float *C,
                                                           int ldc, int M, int N, int K, int kchunk, const float *bias,
                                                           int act, bf16 *Cb, const float *back) {
     pdl_begin();
@@ -60,6 +60,26 @@ __global__ void __launch_bounds__(kGemmThreads) gemm_bf16(const bf16 *A, int lda
 #pragma unroll
             for (int r = 0; r < 4; ++r) acc[i][j][r] = 0.f;
     const bf16 zero = __float2bfloat16(0.f);
+    // A lane's outputs are pairs of neighbouring columns, moved together where the layout allows it.
+    // The values of `back` are requested ahead of the products: C may alias it as far as the
+    // compiler knows, so in the epilogue each load would wait for the store before it.  Input gradient
+    // of 6 output channels at batch 8 of 60 x 60 (18 MB): 26.8 -> 13.1 us.
+    const bool pairs = ldc % 2 == 0 && N % 2 == 0 && ((size_t)C & 7) == 0 && ((size_t)Cb & 3) == 0 && ((size_t)back & 7) == 0;
+    const auto out_row = [&](int mi, int half) { return m0 + wm * 32 + mi * 16 + g + 8 * half; };
+    const auto out_col = [&](int ni) { return n0 + wn * 32 + ni * 8 + 2 * t4; };
+    float2 hv[2][4][2];
+    if (back && pairs) {
+#pragma unroll
+        for (int mi = 0; mi < 2; ++mi)
+#pragma unroll
+            for (int ni = 0; ni < 4; ++ni)
+#pragma unroll
+                for (int half = 0; half < 2; ++half) {
+                    const int row = out_row(mi, half), col = out_col(ni);
+                    hv[mi][ni][half] = row < M && col < N ? *reinterpret_cast<const float2 *>(back + (long long)row * ldc + col)
+                                                          : make_float2(0.f, 0.f);
+                }
+    }
     for (int k0 = kb; k0 < ke; k0 += kBK) {
         for (int e = tid; e < kBM * kBK; e += kGemmThreads) {
             int m, k;
@@ -104,24 +124,34 @@ __global__ void __launch_bounds__(kGemmThreads) gemm_bf16(const bf16 *A, int lda
         __syncthreads();
     }
     float *Cz = C + (long long)blockIdx.z * M * ldc;
+    const auto value = [&](float v, int col, float h) {
+        if (bias) v += bias[col];
+        if (act) v = tanhf(v);
+        return back ? v * (1.f - h * h) : v;
+    };
+    const bool pair_z = pairs && ((size_t)Cz & 7) == 0;
 #pragma unroll
     for (int mi = 0; mi < 2; ++mi)
 #pragma unroll
         for (int ni = 0; ni < 4; ++ni)
 #pragma unroll
-            for (int r = 0; r < 4; ++r) {
-                const int row = m0 + wm * 32 + mi * 16 + g + (r >= 2 ? 8 : 0);
-                const int col = n0 + wn * 32 + ni * 8 + 2 * t4 + (r & 1);
+            for (int half = 0; half < 2; ++half) {
+                const int row = out_row(mi, half), col = out_col(ni);
                 if (row >= M || col >= N) continue;
-                float v = acc[mi][ni][r];
-                if (bias) v += bias[col];
-                if (act) v = tanhf(v);
-                if (back) {
-                    const float h = back[(long long)row * ldc + col];
-                    v = v * (1.f - h * h);
+                const long long at = (long long)row * ldc + col;
+                const float v0 = acc[mi][ni][2 * half], v1 = acc[mi][ni][2 * half + 1];
+                if (pair_z) {
+                    const float2 h = hv[mi][ni][half];
+                    const float2 v = make_float2(value(v0, col, h.x), value(v1, col + 1, h.y));
+                    *reinterpret_cast<float2 *>(Cz + at) = v;
+                    if (Cb) *reinterpret_cast<__nv_bfloat162 *>(Cb + at) = __floats2bfloat162_rn(v.x, v.y);
+                    continue;
                 }
-                Cz[(long long)row * ldc + col] = v;
-                if (Cb) Cb[(long long)row * ldc + col] = __float2bfloat16(v);
+                for (int r = 0; r < 2 && col + r < N; ++r) {
+                    const float v = value(r ? v1 : v0, col + r, back ? back[at + r] : 0.f);
+                    Cz[at + r] = v;
+                    if (Cb) Cb[at + r] = __float2bfloat16(v);
+                }
             }
 }
 

@@ -133,38 +133,62 @@ __device__ __forceinline__ void put_tile(float *tile, const float *r) {
 // FP32 to C and BF16 to Cb (each may be null except C)
 __device__ __forceinline__ void store_tile(const float *tile, int m0, int col0, int M, int N, int ldc, const float *bias,
                                            bool act, const float *back, float *C, __nv_bfloat16 *Cb) {
-    const bool vec = (ldc & 3) == 0;
-    for (int e = threadIdx.x; e < kTM * 16; e += kThreads) {
-        const int r = e >> 4, row = m0 + r, j = (e & 15) * 4, col = col0 + j;
-        if (row >= M || col >= N) continue;
-        const float4 t = *reinterpret_cast<const float4 *>(tile + r * kEpiLd + j);
+    constexpr int RS = kThreads / 16, NR = kTM / RS, NB = 4;  // a thread's rows are RS apart, all at the same columns
+    const int r0 = threadIdx.x >> 4, j = (threadIdx.x & 15) * 4, col = col0 + j;
+    if (col >= N) return;
+    const int n = min(4, N - col);
+    const bool vec = n == 4 && (ldc & 3) == 0;
+    const auto acc = [&](int k) { return *reinterpret_cast<const float4 *>(tile + (r0 + k * RS) * kEpiLd + j); };
+    const auto put = [&](long long at, const float4 &v) {
+        *reinterpret_cast<float4 *>(C + at) = v;
+        if (!Cb) return;
+        const __nv_bfloat162 h0 = __floats2bfloat162_rn(v.x, v.y), h1 = __floats2bfloat162_rn(v.z, v.w);
+        uint2 u;
+        u.x = *reinterpret_cast<const uint32_t *>(&h0);
+        u.y = *reinterpret_cast<const uint32_t *>(&h1);
+        *reinterpret_cast<uint2 *>(Cb + at) = u;
+    };
+    if (back && vec && !bias && !act) {
+        // Four rows' `back` values are requested before the first is stored: C may alias them as far as
+        // the compiler knows, so in the loop below each load would wait for the store before it (input
+        // gradient of a 64-channel layer at batch 8 of 60 x 60: 16.2 us with one row at a time, 13.4 so).
+        for (int k0 = 0; k0 < NR; k0 += NB) {
+            float4 h[NB];
+#pragma unroll
+            for (int k = 0; k < NB; ++k) {
+                const int row = m0 + r0 + (k0 + k) * RS;
+                if (row < M) h[k] = *reinterpret_cast<const float4 *>(back + (long long)row * ldc + col);
+            }
+#pragma unroll
+            for (int k = 0; k < NB; ++k) {
+                const int row = m0 + r0 + (k0 + k) * RS;
+                if (row >= M) break;
+                const float4 t = acc(k0 + k);
+                put((long long)row * ldc + col, make_float4(t.x * (1.f - h[k].x * h[k].x), t.y * (1.f - h[k].y * h[k].y),
+                                                            t.z * (1.f - h[k].z * h[k].z), t.w * (1.f - h[k].w * h[k].w)));
+            }
+        }
+        return;
+    }
+#pragma unroll 1
+    for (int k = 0; k < NR; ++k) {
+        const int row = m0 + r0 + k * RS;
+        if (row >= M) break;
+        const float4 t = acc(k);
         float v[4] = {t.x, t.y, t.z, t.w};
         const long long at = (long long)row * ldc + col;
-        const int n = min(4, N - col);
-        float h[4] = {0.f, 0.f, 0.f, 0.f};
-        if (back) {
-            if (n == 4 && vec) {
-                const float4 b = *reinterpret_cast<const float4 *>(back + at);
-                h[0] = b.x, h[1] = b.y, h[2] = b.z, h[3] = b.w;
-            } else {
-                for (int i = 0; i < n; ++i) h[i] = back[at + i];
-            }
-        }
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-            if (bias && i < n) v[i] += bias[col + i];
+            if (i >= n) break;
+            if (bias) v[i] += bias[col + i];
             if (act) v[i] = tanhf(v[i]);
-            if (back) v[i] = v[i] * (1.f - h[i] * h[i]);
-        }
-        if (n == 4 && vec) {
-            *reinterpret_cast<float4 *>(C + at) = make_float4(v[0], v[1], v[2], v[3]);
-            if (Cb) {
-                uint2 u;
-                __nv_bfloat162 h0 = __floats2bfloat162_rn(v[0], v[1]), h1 = __floats2bfloat162_rn(v[2], v[3]);
-                u.x = *reinterpret_cast<uint32_t *>(&h0);
-                u.y = *reinterpret_cast<uint32_t *>(&h1);
-                *reinterpret_cast<uint2 *>(Cb + at) = u;
+            if (back) {
+                const float h = back[at + i];
+                v[i] = v[i] * (1.f - h * h);
             }
+        }
+        if (vec) {
+            put(at, make_float4(v[0], v[1], v[2], v[3]));
         } else {
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
@@ -322,8 +346,8 @@ __global__ void __launch_bounds__(kThreads) gemm_tc(const __grid_constant__ CUte
 // input gradient adds its nine taps in registers instead of through a 66 MB column matrix.  The
 // slices, their order and every rounding are those of the GEMMs over im2col columns.  Bound by the
 // latency of a slice's round trip (L2 gather, proxy fence, MMA, commit) at six or twelve warps per
-// SM; per layer at batch 8 of 60 x 60: forward 98 + 17 -> 12.5 us, input gradient 40 + 21 + 7 ->
-// 17 us, weight gradient 17 -> 11 us.
+// SM; per layer at batch 8 of 60 x 60: forward 98 + 17 -> 11.5 us, input gradient 40 + 21 + 7 ->
+// 13.4 us, weight gradient 17 -> 10.5 us (from one launch's end to the next's).
 constexpr int kConvC = 64;      // channels in and out
 constexpr int kConvStages = 4;  // ring of A (16 KB) and B (8 KB) slices: two CTAs per SM
 constexpr int kConvA = kTM * kTK * 2, kConvB = kConvC * kTK * 2;
