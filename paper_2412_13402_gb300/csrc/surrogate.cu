@@ -1171,7 +1171,10 @@ int backward_conv(rtbte_surrogate *s, int B) {
     q.bias[kLayers + 1] = g + s->off_c2;
     q.chains = s->chains.as<float>();
     q.P = P;
-    S_CUDA(s, launch_pdl(bias_chains, dim3(64, kLayers + 2), dim3(256), 0, st, q));
+    // an ordinary launch: blocks placed beside the running GEMM's fill some SMs and leave others idle
+    // (20.5 us after it instead of 13.9, and finish_grads 11.8 instead of 7.9)
+    bias_chains<<<dim3(64, kLayers + 2), 256, 0, st>>>(q);
+    S_CUDA(s, cudaGetLastError());
     int nbias = 0, elems = 0;
     for (int l = 0; l < kLayers + 2; ++l) {
         nbias += q.cols[l];
