@@ -375,10 +375,10 @@ class ClockSampler:
 
 def kernel_sources_sha():
     """Hash of the sources that decide the collision kernel's memory traffic: the kernel and
-    plan (rhs.cu), their constants and layouts (internal.cuh) and the channel builder that lays
-    out the entries it streams (builder.cu)."""
+    plan (rhs.cu, collide.cuh), their constants and layouts (internal.cuh) and the channel builder
+    that lays out the entries it streams (builder.cu)."""
     h = hashlib.sha256()
-    for f in ("rhs.cu", "internal.cuh", "builder.cu"):
+    for f in ("rhs.cu", "collide.cuh", "internal.cuh", "builder.cu"):
         h.update(open(os.path.join(ROOT, "paper_2412_13402_gb300", "csrc", f), "rb").read())
     return h.hexdigest()[:16]
 

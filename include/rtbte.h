@@ -326,10 +326,8 @@ int rtbte_set_stream(rtbte_ctx *ctx, void *stream);
  * among CTAs by weight = (entries + w) x c_part per item, w being the fixed cost of an item in
  * entry equivalents and c_part the calibrated cost of an entry of each part; a share s of the
  * weight is split statically, the rest is taken in chunks by CTAs that finish early; each
- * warp prefetches the entry arrays of the item d positions ahead of its sequence into L2.
- * In FP32 the kernel also has two launch forms, two register buffers of entries per warp at 16
- * warps per SM or one buffer at 24 warps per SM, chosen per parts mask.
- * This call times the kernel for `parts` over the forms and candidates of w, c_part, d and s and
+ * warp prefetches the entry arrays d packets of items ahead in its sequence into L2.
+ * This call times the kernel for `parts` over candidates of w, c_part, d and s and
  * keeps the fastest for that parts mask (w in *chosen when not NULL); masks never tuned
  * themselves take its w, c_part, d and s.  Each parts mask keeps its own parameters, so tuning
  * the fast and slow masks of MRI does not change the full-RHS launch.  Synchronises the stream;

@@ -40,7 +40,7 @@ struct KParams {
     const void *popf, *popN, *popP;
     const Ctl *ctl;  // per-instance controllers: launches inside an integrator skip finished instances
     int *tail_ctr;     // [0] next dynamic unit, [1] CTAs finished (reset by the last one)
-    int pf_dist;       // L2 prefetch distance in items of a warp's sequence (0: off)
+    int pf_dist;       // L2 prefetch distance in packets of a warp's sequence (0: off)
 };
 
 // n elements (a multiple of 16 bytes) from global to shared memory, asynchronously, by the threads

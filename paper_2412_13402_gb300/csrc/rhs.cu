@@ -778,8 +778,8 @@ int make_plan(rtbte_ctx *ctx) {
         D.compact_base = (long long)compact.size();
         compact.insert(compact.end(), I.compact.begin(), I.compact.end());
     }
-    // staging decision and launch shape: 16 warps per SM, as 1, 2 or 4 CTAs -- several CTAs
-    // per SM when their staging fits, so one CTA's group change (barrier + staging copy)
+    // staging decision and launch shape: 24 (FP32) or 16 (FP64) warps per SM, as 1, 2 or 4 CTAs --
+    // several CTAs per SM when their staging fits, so one CTA's group change (barrier + staging copy)
     // overlaps the others' streaming
     ctx->staged = max_stage + 64 <= ctx->smem_optin;  // 64 B left for the kernel's static shared memory
     ctx->smem_bytes = ctx->staged ? std::max<size_t>(max_stage, 16) : 0;
