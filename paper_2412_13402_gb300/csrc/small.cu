@@ -132,7 +132,18 @@ template <class R>
 __device__ __forceinline__ double own_row(const R *partials, const SmallRow &row, unsigned parts) {
     RowAcc<R> A;
     auto sum = [&](int i0, int i1) {
-        for (int i = i0; i < i1; ++i) A.add(partials[i]);
+        if constexpr (sizeof(R) == 8) {
+            for (int i = i0; i < i1; ++i) A.add(partials[i]);
+        } else {  // eight loads at a time (graphene 36: 9.8 -> 9.5 us an RHS; in FP64 the toy's 4.9 -> 5.3)
+            for (int i = i0; i < i1; i += 8) {
+                R v[8];
+#pragma unroll
+                for (int j = 0; j < 8; ++j) v[j] = i + j < i1 ? partials[i + j] : R(0);
+#pragma unroll
+                for (int j = 0; j < 8; ++j)
+                    if (i + j < i1) A.add(v[j]);
+            }
+        }
     };
     if (row.f >= 0) {
         if (!(parts & RTBTE_EPH)) return 0.0;
