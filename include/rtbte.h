@@ -291,7 +291,8 @@ int rtbte_phph_rates(rtbte_ctx *ctx, const double *y, double *rates);
  * norms once per slow attempt and decides it).  On success y holds the
  * solution at t_out; on failure y holds the last accepted state and st->t its time.
  * Synchronises the stream.  Errors: INVALID_ARG, STATE, TOO_MANY_STEPS, STEP_UNDERFLOW,
- * ERR_TEST_FAIL, NONFINITE, CUDA. */
+ * ERR_TEST_FAIL, NONFINITE, TIMEOUT (a device wait gave up: y is the state before the launch
+ * that held it), CUDA. */
 int rtbte_advance_to(rtbte_ctx *ctx, double t_out, double *y, const rtbte_integ *opt, rtbte_stats *st);
 
 /* Sizes of instance `inst` (channel counts are 0 before rtbte_upload_channels). */
@@ -344,6 +345,10 @@ int rtbte_get_tuning(const rtbte_ctx *ctx, int32_t *item_weight, int32_t *prefet
  * slower; for per-kernel profiling tools that do not descend into graph loops).
  * Errors: INVALID_ARG. */
 int rtbte_set_graph_mode(rtbte_ctx *ctx, int use_graphs);
+
+/* Polls after which a grid barrier of a small instance's attempt loop gives up (negative: the
+ * default, seconds); rtbte_advance_to then returns RTBTE_E_TIMEOUT.  Errors: INVALID_ARG. */
+int rtbte_set_wait_limit(rtbte_ctx *ctx, int polls);
 
 /* Kernel timing.  While enabled, every launch of the collision kernel enqueued outside a
  * CUDA graph (rtbte_rhs and the first-step estimate) is bracketed by CUDA events recorded on

@@ -692,6 +692,12 @@ int rtbte_set_graph_mode(rtbte_ctx *ctx, int use_graphs) {
     return RTBTE_OK;
 }
 
+int rtbte_set_wait_limit(rtbte_ctx *ctx, int polls) {
+    if (!ctx) return RTBTE_E_INVALID_ARG;
+    ctx->wait_polls = polls < 0 ? rtbte::kBarrierPolls : polls;
+    return RTBTE_OK;
+}
+
 int rtbte_set_kernel_timing(rtbte_ctx *ctx, int enable) {
     if (!ctx) return RTBTE_E_INVALID_ARG;
     ctx->timing = enable != 0;

@@ -523,8 +523,11 @@ int run_attempts(rtbte_ctx *ctx, int method, const CtlParams &cp, unsigned parts
         for (;;) {
             if ((rc = launch_small_attempts(ctx, &a, cap, ctx->stream)) || (rc = read_small(ctx))) return rc;
             if ((rc = read_ctl(ctx))) return rc;
+            if (small_give_up(ctx, ctx->ctl_host)) {
+                if ((rc = write_ctl(ctx))) return rc;
+                break;
+            }
             if (all_done(ctx)) break;
-            if (small_attempts_run(ctx) <= 0) return fail(ctx, RTBTE_E_TIMEOUT, "a grid barrier gave up");
         }
         if (attempts_out) *attempts_out = sum_attempts(ctx) - a0;
         return RTBTE_OK;

@@ -44,6 +44,7 @@ constexpr int kWrmsBlocks = 512;
 constexpr int kWrmsChunks = 128;  // per-instance blocks of the WRMS reduction before the controller
 constexpr int kMaxBatch = 1024;  // instances per context (shared-memory tables of the batched kernels)
 constexpr int kLoopCap = 64;     // attempts per launch of an attempt loop (default)
+constexpr int kBarrierPolls = 1 << 22;  // of a grid barrier (default): seconds
 
 enum { PART_EPH = 0, PART_PHE = 1, PART_PP = 2 };
 // Lanes working on one item are chosen per staging group (Group::lanes_log2): 4, 8, 16 or 32 lanes,
@@ -315,6 +316,7 @@ struct rtbte_ctx {
     size_t small_at[5] = {0, 0, 0, 0, 0};
     int small_grid = 0, small_max_items = 0, small_max_rows = 0, small_max_runs = 0, small_max_entries = 0;
     void *small_sync_host = nullptr;  // pinned mirror of small_sync
+    int wait_polls = rtbte::kBarrierPolls;  // polls of a grid barrier before its wait gives up
     int num_sms = 0;
     size_t smem_optin = 0;
     // integrator work buffers
@@ -361,8 +363,10 @@ int make_small_plan(rtbte_ctx *ctx, const ItemRec *items, int n, const std::vect
                     const std::vector<int> &rowoff, const std::vector<int> &rowmid);
 int launch_small_rhs(rtbte_ctx *ctx, unsigned parts, const double *y, double *ydot, cudaStream_t s);
 int launch_small_attempts(rtbte_ctx *ctx, const void *stage_args, int cap, cudaStream_t s);
-int small_attempts_run(const rtbte_ctx *ctx);  // by the last launch, once its counters were read back
-int read_small(rtbte_ctx *ctx);                // enqueue that read-back
+int read_small(rtbte_ctx *ctx);  // enqueue the read-back of the last launch's barrier block
+// Whether a wait of that launch gave up (after the read-back); then *c is the controller it started
+// from, stopped with RTBTE_E_TIMEOUT.
+bool small_give_up(const rtbte_ctx *ctx, Ctl *c);
 // integrate.cu
 int advance_to(rtbte_ctx *ctx, double t_out, double *y, const rtbte_integ *opt, rtbte_stats *st);
 void destroy_graphs(rtbte_ctx *ctx);

@@ -10,7 +10,8 @@
 //   - attempts_small: up to `cap` attempted steps per launch on a cooperative grid: S grid barriers
 //     an attempt to exchange populations (the last one the squared errors too, one more where the
 //     norm's chunks exceed 8 rows); every CTA runs the controller on its own copy, beside the first
-//     stage of the next attempt.  Where they fit, the CTA's items and entries stay in shared memory
+//     stage of the next attempt.  The state the launch started from is kept beside the one it writes,
+//     so that a barrier wait that gives up leaves a whole state to go back to.  Where they fit, the CTA's items and entries stay in shared memory
 //     for the launch: a barrier's acquire drops L1, so each stage would fetch them from L2 again
 //     (toy 12 x 12 FP64 31.1 -> 30.2 us an attempt, graphene 36 FP32 64 -> 62 us).
 // Items, their lanes and entry order, the order of a row's items, the norm's chunks and the
@@ -192,19 +193,17 @@ struct SmallSync {
     unsigned arrived;          // barrier arrivals so far
     int failed;                // a barrier wait gave up
     unsigned long long range;  // rows out of range in all attempts so far
-    int attempts;              // attempts run
-    int pad;
+    Ctl start;                 // the controller the launch started from
 };
-constexpr int kBarrierPolls = 1 << 22;
 
-// Grid barrier (arrivals reach `target`); false in every thread if the wait gave up.
-__device__ __forceinline__ bool grid_barrier(SmallSync *sync, unsigned target) {
+// Grid barrier (arrivals reach `target`); false in every thread if it was not seen in `polls` polls.
+__device__ __forceinline__ bool grid_barrier(SmallSync *sync, unsigned target, int polls) {
     __shared__ int s_ok;
     __syncthreads();
     if (threadIdx.x == 0) {
         int ok = 0;
         asm volatile("red.release.gpu.global.add.u32 [%0], 1;\n" ::"l"(&sync->arrived) : "memory");
-        for (int i = 0; i < kBarrierPolls; ++i) {
+        for (int i = 0; i < polls; ++i) {
             unsigned v;
             asm volatile("ld.acquire.gpu.global.u32 %0, [%1];\n" : "=r"(v) : "l"(&sync->arrived) : "memory");
             if ((int)(v - target) >= 0) {
@@ -281,7 +280,7 @@ __device__ __forceinline__ void hold_lists(const KParams &P, const SmallPlan &S,
 // LOAD: LOAD_SHARED where the CTAs' lists fit in shared memory, else LOAD_CACHED.
 template <class R, int NT, int LOAD>
 __global__ void __launch_bounds__(NT) attempts_small(KParams P, SmallPlan S, SmallPops B, StageArgs a, double *chunks,
-                                                     int cap, SmallSync *sync) {
+                                                     int cap, int polls, SmallSync *sync) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ Ctl C;
     __shared__ int s_accept;
@@ -292,6 +291,8 @@ __global__ void __launch_bounds__(NT) attempts_small(KParams P, SmallPlan S, Sma
     copy_in(M.rows, S.rows + row0, nrows);
     __syncthreads();
     if (C.done) return;  // (alike in every CTA)
+    const int cur0 = C.cur;
+    if (blockIdx.x == 0 && threadIdx.x == 0) sync->start = C;
     if (LOAD == LOAD_SHARED) hold_lists<R, NT>(P, S, M);
     const long long ni = a.n;
     const int L = (int)((ni + kWrmsChunks - 1) / kWrmsChunks);  // rows of a chunk
@@ -310,13 +311,13 @@ __global__ void __launch_bounds__(NT) attempts_small(KParams P, SmallPlan S, Sma
         }
     };
     {
-        const double *y = C.cur ? a.Y1 : a.Y0;
+        const double *y = cur0 ? a.Y1 : a.Y0;
         for (int r = threadIdx.x; r < nrows; r += NT) {
             const double v = y[M.rows[r].row];
             M.y[r] = v;
             put(0, M.rows[r], (R)v);
         }
-        ok = grid_barrier(sync, ++barriers * gridDim.x);
+        ok = grid_barrier(sync, ++barriers * gridDim.x, polls);
     }
     bool pending = false;  // the last attempt's controller runs beside the first stage of the next
     double sum = 0.0;
@@ -374,7 +375,7 @@ __global__ void __launch_bounds__(NT) attempts_small(KParams P, SmallPlan S, Sma
                 put(out, row, (R)z);
             }
             in = out;
-            ok = grid_barrier(sync, ++barriers * gridDim.x);
+            ok = grid_barrier(sync, ++barriers * gridDim.x, polls);
         }
         if (!ok) break;
         if (L <= 8) {
@@ -385,7 +386,7 @@ __global__ void __launch_bounds__(NT) attempts_small(KParams P, SmallPlan S, Sma
                 const double s = block_sum<true>(a.wsq, b, e > b ? e - b : 0);
                 if (threadIdx.x == 0) chunks[ch] = s;
             }
-            if (!(ok = grid_barrier(sync, ++barriers * gridDim.x))) break;
+            if (!(ok = grid_barrier(sync, ++barriers * gridDim.x, polls))) break;
             sum = small_wrms(chunks, kWrmsChunks, 1);
         }
         // accepted or not decides which state the next attempt starts from; the rest of the
@@ -403,15 +404,14 @@ __global__ void __launch_bounds__(NT) attempts_small(KParams P, SmallPlan S, Sma
         ++n;
     }
     __syncthreads();
-    if (!C.done && n != cap && blockIdx.x == 0 && threadIdx.x == 0) {  // a barrier wait gave up
-        C.status = RTBTE_E_TIMEOUT;
-        C.done = 1;
-    }
-    double *y = C.cur ? a.Y1 : a.Y0;
+    // The result goes into the other buffer, whichever the attempts' count would name: where some CTA's
+    // wait gave up, CTAs have left at different attempts (and others not at all), and the host goes back to
+    // the state and controller at the start (small_give_up).
+    double *y = cur0 ? a.Y0 : a.Y1;
     for (int r = threadIdx.x; r < nrows; r += NT) y[M.rows[r].row] = M.y[yc * S.max_rows + r];
     if (blockIdx.x == 0 && threadIdx.x == 0) {
+        C.cur = cur0 ^ 1;
         a.ctl[0] = C;
-        sync->attempts = n;
     }
 }
 
@@ -643,7 +643,14 @@ int read_small(rtbte_ctx *ctx) {
                                  ctx->stream));
     return RTBTE_OK;
 }
-int small_attempts_run(const rtbte_ctx *ctx) { return reinterpret_cast<const SmallSync *>(ctx->small_sync_host)->attempts; }
+bool small_give_up(const rtbte_ctx *ctx, Ctl *c) {
+    const SmallSync *sync = reinterpret_cast<const SmallSync *>(ctx->small_sync_host);
+    if (!sync->failed) return false;
+    *c = sync->start;
+    c->status = RTBTE_E_TIMEOUT;
+    c->done = 1;
+    return true;
+}
 
 namespace {
 // Buffers of the attempt loop, made on its first use.
@@ -688,7 +695,8 @@ int launch_small_attempts(rtbte_ctx *ctx, const void *stage_args, int cap, cudaS
     double *chunks = ctx->wrms_part.as<double>() + 2 * ctx->n_y;
     SmallSync *sync = ctx->small_sync.as<SmallSync>();
     RT_CUDA(ctx, cudaMemsetAsync(sync, 0, sizeof(SmallSync), s));
-    void *args[] = {&P, &S, &B, &a, &chunks, &cap, &sync};
+    int polls = ctx->wait_polls;
+    void *args[] = {&P, &S, &B, &a, &chunks, &cap, &polls, &sync};
     RT_CUDA(ctx, cudaLaunchCooperativeKernel(attempts_fn(ctx), dim3(ctx->small_grid), dim3(kSmallThreads64), args,
                                              small_smem(R, S, true), s));
     ctx->launches++;
