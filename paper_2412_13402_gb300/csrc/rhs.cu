@@ -1080,21 +1080,52 @@ int autotune(rtbte_ctx *ctx, unsigned parts, int *chosen) {
 // pair and absorption factors included), from the compute-precision sub-lattice copy popP,
 // summed in FP64 per lane then a fixed butterfly; written to rates[y_off + n_c + full(a)].
 // The FP64 pipe bounds it (2 or 3 operations per entry: 0.35 ms for graphene 180's 8.8e7 entries;
-// the list streams in 0.16 ms).  STAGED: one CTA per SM holds the populations in shared memory;
-// lanes read four entries with a 16-byte load, four such vectors in flight, and the next
-// destination's entries are prefetched into L2 (graphene 180, FP64 lists: 1043 us with one entry
-// per lane and load and gathers from global memory, 489 us so).
+// the list streams in 0.16 ms).  STAGED: one CTA per SM holds the populations in shared memory,
+// widened to FP64 (S) where they fit so; lanes read four entries with a 16-byte load, four such
+// vectors in flight, and the next destination's entries are prefetched into L2 (graphene 180, FP64
+// lists: 1043 us with one entry per lane and load and gathers from global memory, 489 us so; FP32
+// lists, whose weights are widened one by one: 1586 us before, 508 us so).
 constexpr int kRateThreads = 512;
-template <class R, bool STAGED>
+// x in FP64 where it is zero or a normal number, by integer operations: the bias of the exponent grows
+// by 1023 - 127, the fraction moves up by 29 bits.  (The conversion instruction shares the FP64 pipe;
+// with it the FP32 lists of graphene 180 take 686 us.)
+__device__ __forceinline__ bool zero_or_normal(float x) {
+    const unsigned u = __float_as_uint(x);
+    return (u << 1) == 0u || (u & 0x7f800000u) - 0x00800000u < 0x7f000000u;
+}
+__device__ __forceinline__ double widen(float x) {
+    const unsigned u = __float_as_uint(x);
+    const unsigned hi = (u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + (896u << 20));
+    return __hiloint2double((int)((u << 1) == 0u ? u : hi), (int)(u << 29));
+}
+// the four weights of a vector, exactly
+__device__ __forceinline__ void weights4(const Batch<float, 4> &B, int j, double (&w)[4]) {
+    if (zero_or_normal(B.w(j, 0)) && zero_or_normal(B.w(j, 1)) && zero_or_normal(B.w(j, 2)) && zero_or_normal(B.w(j, 3))) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) w[k] = widen(B.w(j, k));
+    } else {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) w[k] = (double)B.w(j, k);
+    }
+}
+__device__ __forceinline__ void weights4(const Batch<double, 4> &B, int j, double (&w)[4]) {
+#pragma unroll
+    for (int k = 0; k < 4; ++k) w[k] = B.w(j, k);
+}
+template <class R, class S, bool STAGED>
 __global__ void __launch_bounds__(kRateThreads) pp_rates_kernel(const uint32_t *idx, const R *W, const long long *off,
                                                                 const R *popP, int n_stage, const int *pp_full,
                                                                 int pp_bits, int M, long long row0, double *rates) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    const R *P = popP;
-    if (STAGED) {
-        R *sm = reinterpret_cast<R *>(smem_raw);
-        stage_copy<R>(sm, popP, n_stage);
-        asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;\n" ::: "memory");
+    const S *P = reinterpret_cast<const S *>(popP);
+    if constexpr (STAGED) {
+        S *sm = reinterpret_cast<S *>(smem_raw);
+        if constexpr (sizeof(S) == sizeof(R)) {
+            stage_copy<R>(sm, popP, n_stage);
+            asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;\n" ::: "memory");
+        } else {
+            for (int i = threadIdx.x; i < n_stage; i += kRateThreads) sm[i] = (S)popP[i];
+        }
         __syncthreads();
         P = sm;
     }
@@ -1114,10 +1145,7 @@ __global__ void __launch_bounds__(kRateThreads) pp_rates_kernel(const uint32_t *
             }
         }
         double acc = 0.0;
-        // sum of W (N' + N'' + 1), or W (N'' - N'), over a segment: FP64 lists in FP64; FP32 lists
-        // as exact sums and products in FP32 head/tail pairs (two-sum, FMA residual), widened once
-        // per 16 entries -- converting every value cost more than the arithmetic (graphene 180, FP32
-        // lists: 1579 us before, 1046 with conversions, 237 so)
+        // adds W (N' + N'' + 1), or W (N'' - N'), over a segment, in FP64 whatever the lists' precision
         auto segment = [&](long long b, long long e, auto emission) {
             constexpr bool EM = decltype(emission)::value;
             const int nv = (int)((e - b) >> 2);  // segments are padded to whole vectors
@@ -1132,28 +1160,18 @@ __global__ void __launch_bounds__(kRateThreads) pp_rates_kernel(const uint32_t *
                 it.len = (unsigned short)(4 * min(nv - v0, 128));
                 Batch<R, 4> B;
                 B.issue(V, it, lane, 5);
-                [[maybe_unused]] R hi = R(0), lo = R(0);
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
                     if (lane + 32 * j >= (it.len >> 2)) break;
+                    double w[4];
+                    weights4(B, j, w);
 #pragma unroll
                     for (int k = 0; k < 4; ++k) {
                         const unsigned x = comp4(B.iv[j], k);
-                        const R w = B.w(j, k), Nb = P[x & pmask], Nc = P[x >> pp_bits];
-                        if constexpr (sizeof(R) == 8) {
-                            acc = fma(w, EM ? Nb + Nc + 1.0 : Nc - Nb, acc);
-                        } else {
-                            R t = Nc, c = R(0);
-                            two_sum(t, c, EM ? Nb : -Nb);
-                            if (EM) two_sum(t, c, R(1));
-                            const R p = w * t;
-                            two_sum(hi, lo, p);
-                            lo += fma(w, c, fma(w, t, -p));
-                        }
+                        const double Nb = (double)P[x & pmask], Nc = (double)P[x >> pp_bits];
+                        acc = fma(w[k], EM ? Nb + Nc + 1.0 : Nc - Nb, acc);
                     }
                 }
-                // (an infinite sum has no tail: its two-sum residual is not a number)
-                if constexpr (sizeof(R) == 4) acc += (double)hi + (isfinite(hi) ? (double)lo : 0.0);
             }
         };
         segment(o0, o1, std::true_type{});
@@ -1164,22 +1182,15 @@ __global__ void __launch_bounds__(kRateThreads) pp_rates_kernel(const uint32_t *
     }
 }
 
-template <class R> static int launch_pp_rates_t(rtbte_ctx *ctx, InstHost &I, double *rates, cudaStream_t s) {
-    const size_t bytes = sizeof(R) * (size_t)I.M_pad;
-    const bool staged = bytes + 64 <= ctx->smem_optin;
-    const uint32_t *idx = I.pp_idx.as<uint32_t>();
-    const R *P = reinterpret_cast<const R *>(ctx->popP.p) + I.P_off;
+template <class R, class S, bool STAGED>
+static int launch_pp_rates_t(rtbte_ctx *ctx, InstHost &I, double *rates, cudaStream_t s) {
     const int grid = (int)std::min<long long>((I.M + 7) / 8, (long long)ctx->num_sms);
-    if (staged) {
-        RT_CUDA(ctx, allow_max_dynamic_smem((const void *)pp_rates_kernel<R, true>));
-        pp_rates_kernel<R, true><<<grid, kRateThreads, bytes, s>>>(idx, I.pp_W.as<R>(), I.pp_off_dev.as<long long>(), P,
-                                                                   I.M_pad, I.t_ppfull.as<int>(), I.pp_bits, (int)I.M,
-                                                                   I.y_off + I.d.n_c, rates);
-    } else {
-        pp_rates_kernel<R, false><<<grid, kRateThreads, 0, s>>>(idx, I.pp_W.as<R>(), I.pp_off_dev.as<long long>(), P, 0,
-                                                                I.t_ppfull.as<int>(), I.pp_bits, (int)I.M,
-                                                                I.y_off + I.d.n_c, rates);
-    }
+    const auto fn = pp_rates_kernel<R, S, STAGED>;
+    if (STAGED) RT_CUDA(ctx, allow_max_dynamic_smem((const void *)fn));
+    fn<<<grid, kRateThreads, STAGED ? sizeof(S) * (size_t)I.M_pad : 0, s>>>(
+        I.pp_idx.as<uint32_t>(), I.pp_W.as<R>(), I.pp_off_dev.as<long long>(),
+        reinterpret_cast<const R *>(ctx->popP.p) + I.P_off, STAGED ? I.M_pad : 0, I.t_ppfull.as<int>(), I.pp_bits,
+        (int)I.M, I.y_off + I.d.n_c, rates);
     RT_CUDA(ctx, cudaGetLastError());
     ctx->launches++;
     return RTBTE_OK;
@@ -1193,8 +1204,13 @@ int launch_pp_rates(rtbte_ctx *ctx, int inst, double *rates, cudaStream_t s) {
         I.pp_off_dev.bytes = sizeof(long long) * I.pp_off.size();
         RT_CUDA(ctx, cudaMemcpyAsync(I.pp_off_dev.p, I.pp_off.data(), I.pp_off_dev.bytes, cudaMemcpyHostToDevice, s));
     }
-    return ctx->precision == RTBTE_PREC_FP64 ? launch_pp_rates_t<double>(ctx, I, rates, s)
-                                             : launch_pp_rates_t<float>(ctx, I, rates, s);
+    const auto fits = [&](size_t size) { return size * (size_t)I.M_pad + 64 <= ctx->smem_optin; };
+    if (ctx->precision == RTBTE_PREC_FP64)
+        return fits(8) ? launch_pp_rates_t<double, double, true>(ctx, I, rates, s)
+                       : launch_pp_rates_t<double, double, false>(ctx, I, rates, s);
+    return fits(8)   ? launch_pp_rates_t<float, double, true>(ctx, I, rates, s)
+           : fits(4) ? launch_pp_rates_t<float, float, true>(ctx, I, rates, s)
+                     : launch_pp_rates_t<float, float, false>(ctx, I, rates, s);
 }
 
 int launch_rows(rtbte_ctx *ctx, unsigned parts, double *out, const double *forcing, cudaStream_t s) {
