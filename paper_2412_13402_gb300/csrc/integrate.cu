@@ -518,7 +518,7 @@ int run_attempts(rtbte_ctx *ctx, int method, const CtlParams &cp, unsigned parts
         if (attempts_out) *attempts_out = sum_attempts(ctx) - a0;
         return RTBTE_OK;
     }
-    if (ctx->small_grid > 0) {  // a small instance: up to cap attempts in one launch
+    if (ctx->small_fold > 0) {  // a small instance: up to cap attempts in one launch
         const StageArgs a = stage_args(ctx, tableau_of(method), cp, parts, forcing);
         for (;;) {
             if ((rc = launch_small_attempts(ctx, &a, cap, ctx->stream)) || (rc = read_small(ctx))) return rc;

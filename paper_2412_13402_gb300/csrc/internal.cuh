@@ -107,6 +107,10 @@ struct __align__(16) Ctl {
     int cur, last, fixed, pad_i0;
 };
 
+struct SmallCtaMax {
+    int items = 0, rows = 0, entries = 0;
+};
+
 // What an item costs the warp that runs it.
 struct ItemCost {
     unsigned short slots;  // entry slots: vectors per lane x lanes x 4
@@ -312,9 +316,11 @@ struct rtbte_ctx {
     bool staged = false;
     bool wide = true;  // every group uses whole-warp items (the kernel variant without sub-warps)
     // one-launch kernels of a small single instance (small.cu); small_grid 0: not taken
-    rtbte::DevBuf small_tab, small_pops, small_sync;  // small_tab: items, runs, rows, row offsets, entry places at small_at[]
-    size_t small_at[5] = {0, 0, 0, 0, 0};
-    int small_grid = 0, small_max_items = 0, small_max_rows = 0, small_max_runs = 0, small_max_entries = 0;
+    rtbte::DevBuf small_tab, small_pops, small_sync;  // small_tab: items, runs, rows, row offsets, entry places,
+    size_t small_at[6] = {0, 0, 0, 0, 0, 0};          //   slot offsets at small_at[]
+    int small_grid = 0;               // shares of the plan, one per CTA of an RHS
+    int small_fold = 0;               // shares per CTA of the attempt loop; 0: attempts take the launch sequence
+    rtbte::SmallCtaMax small_max[2];  // largest CTA of an RHS, of the attempt loop
     void *small_sync_host = nullptr;  // pinned mirror of small_sync
     int wait_polls = rtbte::kBarrierPolls;  // polls of a grid barrier before its wait gives up
     int num_sms = 0;

@@ -7,8 +7,8 @@
 // populations, runs every work item of its rows -- whatever their part and mode -- and sums them
 // itself, so no partial leaves the SM and the only exchange between CTAs is the new populations.
 //   - rhs_small: one launch per RHS, populations straight from y, rows straight to ydot;
-//   - attempts_small: up to `cap` attempted steps per launch on a cooperative grid: S grid barriers
-//     an attempt to exchange populations (the last one the squared errors too, one more where the
+//   - attempts_small: up to `cap` attempted steps per launch on a cooperative grid of at most half the
+//     SMs (see kSmallQuarter): S grid barriers an attempt to exchange populations (the last one the squared errors too, one more where the
 //     norm's chunks exceed 8 rows); every CTA runs the controller on its own copy, beside the first
 //     stage of the next attempt.  The state the launch started from is kept beside the one it writes,
 //     so that a barrier wait that gives up leaves a whole state to go back to.  Where they fit, the CTA's items and entries stay in shared memory
@@ -50,19 +50,28 @@ struct __align__(16) SmallRow {
     int row, p0, mid, p1;
     int f, N, P, pad;  // index in f / N / the sub-lattice N, or -1
 };
+// Rows and their items come in shares, one per SM.  A CTA of the RHS takes one, a CTA of the attempt
+// loop `fold` neighbouring ones, whose items are kept together by group.
 struct SmallPlan {
     const SmallRun *runs;  // [CTA][max_runs] (empty runs fill up)
     const SmallRow *rows;
-    const int *row_off;    // [CTAs + 1]
+    const int *row_off;    // [shares + 1]
+    const int *slot_off;   // [shares + 1] first partial slot, which for a CTA is its first item too
+    int shares, fold;
     int max_runs, max_items, max_rows;  // largest CTA's
     int n_f, n_N, n_P;     // populations held: f, all modes' N (mode stride N_q_pad), sub-lattice N
     const int *pp_full;    // [M] phonon of each sub-lattice state
-    const int *item_at;    // [items] where an item's entries go in its CTA's copy of the lists
+    const int *item_at;    // [items] entries of the items before this one
     int max_entries;       // largest CTA's entries; 0: the attempts' lists are not held
+    __device__ __forceinline__ int share0() const { return blockIdx.x * fold; }
+    __device__ __forceinline__ int row0() const { return __ldg(row_off + share0()); }
+    __device__ __forceinline__ int row1() const { return __ldg(row_off + min(share0() + fold, shares)); }
+    __device__ __forceinline__ int slot0() const { return __ldg(slot_off + share0()); }
 };
 
 template <class R> struct SmallMem {  // shared memory of a CTA
-    R *f, *N, *P, *partials;
+    R *f, *N, *P;
+    R *partials;  // indexed by slot: the CTA's first one's is slot0
     SmallRun *runs;
     // attempts only:
     SmallRow *rows;
@@ -71,13 +80,13 @@ template <class R> struct SmallMem {  // shared memory of a CTA
     ItemRec *items;  // [max_items], if the lists are held
     R *W;            // [max_entries]
     uint32_t *idx;
-    __device__ __forceinline__ SmallMem(unsigned char *raw, const SmallPlan &S) {
+    __device__ __forceinline__ SmallMem(unsigned char *raw, const SmallPlan &S, int slot0) {
         runs = reinterpret_cast<SmallRun *>(raw);
         f = reinterpret_cast<R *>(runs + S.max_runs);
         N = f + S.n_f;
         P = N + S.n_N;
-        partials = P + S.n_P;
-        rows = reinterpret_cast<SmallRow *>(partials + S.max_items);
+        partials = P + S.n_P - slot0;
+        rows = reinterpret_cast<SmallRow *>(P + S.n_P + S.max_items);
         y = reinterpret_cast<double *>(rows + S.max_rows);
         K = y + 2 * S.max_rows;
         items = reinterpret_cast<ItemRec *>(K + kMaxStages * S.max_rows);
@@ -161,9 +170,9 @@ template <class R, int NT>
 __global__ void __launch_bounds__(NT) rhs_small(KParams P, SmallPlan S, const InstDev *inst, unsigned parts,
                                                 const double *y, double *ydot) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    const SmallMem<R> M(smem_raw, S);
+    const SmallMem<R> M(smem_raw, S, S.slot0());
     copy_in(M.runs, S.runs + (long long)blockIdx.x * S.max_runs, S.max_runs);
-    const int r0 = __ldg(S.row_off + blockIdx.x) + threadIdx.x, r1 = __ldg(S.row_off + blockIdx.x + 1);
+    const int r0 = S.row0() + threadIdx.x, r1 = S.row1();
     const InstDev I = *inst;
     pdl_begin();
     pdl_wait();
@@ -249,15 +258,14 @@ __device__ __forceinline__ double small_wrms(const double *wsq, long long ni, in
 
 // Copies the CTA's items and their entries into shared memory and points its runs at them.
 template <class R, int NT>
-__device__ __forceinline__ void hold_lists(const KParams &P, const SmallPlan &S, const SmallMem<R> &M) {
+__device__ __forceinline__ void hold_lists(const KParams &P, const SmallPlan &S, const SmallMem<R> &M, int item0) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int item0 = M.runs[0].a;
     for (int u = 0; u < S.max_runs; ++u) {
         const SmallRun &run = M.runs[u];
         for (int k = run.a + warp; k < run.b; k += NT / 32) {
             const int4 d = __ldg(reinterpret_cast<const int4 *>(P.items) + k);
             const Item it = item_from(d);
-            const int at = __ldg(S.item_at + k), vw = (int)(it.len * sizeof(R) / 16);
+            const int at = __ldg(S.item_at + k) - __ldg(S.item_at + item0), vw = (int)(it.len * sizeof(R) / 16);
             const uint4 *ip = reinterpret_cast<const uint4 *>(run.idx + it.begin);
             const uint4 *wp = reinterpret_cast<const uint4 *>(reinterpret_cast<const R *>(run.W) + it.begin);
             for (int v = lane; v < it.len >> 2; v += 32) reinterpret_cast<uint4 *>(M.idx + at)[v] = __ldg(ip + v);
@@ -284,8 +292,8 @@ __global__ void __launch_bounds__(NT) attempts_small(KParams P, SmallPlan S, Sma
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ Ctl C;
     __shared__ int s_accept;
-    const SmallMem<R> M(smem_raw, S);
-    const int row0 = __ldg(S.row_off + blockIdx.x), nrows = __ldg(S.row_off + blockIdx.x + 1) - row0;
+    const int slot0 = S.slot0(), row0 = S.row0(), nrows = S.row1() - row0;
+    const SmallMem<R> M(smem_raw, S, slot0);
     if (threadIdx.x == 0) C = a.ctl[0];
     copy_in(M.runs, S.runs + (long long)blockIdx.x * S.max_runs, S.max_runs);
     copy_in(M.rows, S.rows + row0, nrows);
@@ -293,7 +301,7 @@ __global__ void __launch_bounds__(NT) attempts_small(KParams P, SmallPlan S, Sma
     if (C.done) return;  // (alike in every CTA)
     const int cur0 = C.cur;
     if (blockIdx.x == 0 && threadIdx.x == 0) sync->start = C;
-    if (LOAD == LOAD_SHARED) hold_lists<R, NT>(P, S, M);
+    if (LOAD == LOAD_SHARED) hold_lists<R, NT>(P, S, M, slot0);
     const long long ni = a.n;
     const int L = (int)((ni + kWrmsChunks - 1) / kWrmsChunks);  // rows of a chunk
     const int warp = threadIdx.x >> 5;
@@ -426,22 +434,27 @@ KParams small_params(rtbte_ctx *ctx) {
     return P;
 }
 
-SmallPlan small_plan(rtbte_ctx *ctx) {
+SmallPlan small_plan(rtbte_ctx *ctx, bool attempts) {
     SmallPlan S;
+    const SmallCtaMax &Z = ctx->small_max[attempts];
     const InstHost &I = ctx->inst[0];
     const char *tab = ctx->small_tab.as<char>();
-    S.runs = reinterpret_cast<const SmallRun *>(tab + ctx->small_at[1]);
+    S.runs = reinterpret_cast<const SmallRun *>(tab + ctx->small_at[1]) +
+             (attempts ? (size_t)ctx->small_grid * ctx->n_groups : 0);
     S.rows = reinterpret_cast<const SmallRow *>(tab + ctx->small_at[2]);
     S.row_off = reinterpret_cast<const int *>(tab + ctx->small_at[3]);
-    S.max_runs = ctx->small_max_runs;
-    S.max_items = ctx->small_max_items;
-    S.max_rows = ctx->small_max_rows;
+    S.slot_off = reinterpret_cast<const int *>(tab + ctx->small_at[5]);
+    S.shares = ctx->small_grid;
+    S.fold = attempts ? ctx->small_fold : 1;
+    S.max_runs = ctx->n_groups;
+    S.max_items = Z.items;
+    S.max_rows = Z.rows;
     S.n_f = I.n_c_pad;
     S.n_N = I.d.nmodes * I.N_q_pad;
     S.n_P = I.M_pad;
     S.pp_full = I.t_ppfull.as<int>();
     S.item_at = reinterpret_cast<const int *>(tab + ctx->small_at[4]);
-    S.max_entries = ctx->small_max_entries;
+    S.max_entries = Z.entries;
     return S;
 }
 
@@ -450,7 +463,7 @@ const void *rhs_fn(const rtbte_ctx *ctx) {
                                              : (const void *)rhs_small<float, kSmallThreads>;
 }
 const void *attempts_fn(const rtbte_ctx *ctx) {
-    if (ctx->small_max_entries > 0)
+    if (ctx->small_max[1].entries > 0)
         return ctx->precision == RTBTE_PREC_FP64 ? (const void *)attempts_small<double, kSmallThreads64, LOAD_SHARED>
                                                  : (const void *)attempts_small<float, kSmallThreads64, LOAD_SHARED>;
     return ctx->precision == RTBTE_PREC_FP64 ? (const void *)attempts_small<double, kSmallThreads64, LOAD_CACHED>
@@ -471,28 +484,41 @@ int small_threads(const rtbte_ctx *ctx) {
 // 237 / 224 us).
 constexpr double kSmallSlots = 2e6, kSmallSlots64 = 1.5e6;
 
+// The attempt loop holds whole SMs (its registers fill one) for as many as 64 attempts, about 2 ms, so it
+// takes half of them at most and leaves the rest to other streams; a quarter for the smallest lists, which
+// are as fast there.  Beside a 12 x 12 FP64 integration a 108 us RHS of graphene 120 takes 171 us and a copy
+// of 1 GB 174 instead of 162 us (1290 us with every SM taken; 167 and 167 by the launch sequence it was
+// before).  us per attempt of all contexts, 1 / 4 / 8 of them on their own streams:
+//                             launch sequence        every SM             half (toy 12: a quarter)
+//   toy 12 FP64               58.8 / 21.4 / 16.2     29.9 / 29.8 / 30.0   29.2 /  7.4 /  7.5
+//   toy 20 FP64               64.8 / 24.5 / 19.7     37.2 / 36.9 / 36.9   46.0 / 23.2 / 23.2
+//   graphene 24, 0.23M        76.0 / 30.0 / 21.2     53.9 / 46.4 / 45.0   52.8 / 24.0 / 23.3
+//   graphene 36, 0.96M        78.1 / 36.0 / 26.5     57.1 / 51.7 / 51.0   63.4 / 29.5 / 29.4
+//   graphene 42, 1.71M        89.9 / 41.6 / 35.3     -                    87.0 / 41.8 / 40.8
+//   graphene 24 FP64, 0.23M   93.7 / 40.0 / 29.5     -                    97.0 / 45.9 / 45.1
+// so FP64 attempts, bound by the FP64 pipes of their SMs, take the launch sequence from 0.2M slots on.
+constexpr double kSmallQuarter = 6e4, kSmallAttempts64 = 2e5;
+
 // Row ownership of a single small instance, or none (ctx->small_grid = 0).  `items` in launch
 // order with their row-major slots, `rowoff` / `rowmid` the rows' slots.
 int make_small_plan(rtbte_ctx *ctx, const ItemRec *items, int n, const std::vector<Group> &groups,
                     const std::vector<int> &rowoff, const std::vector<int> &rowmid) {
-    ctx->small_grid = 0;
+    ctx->small_grid = ctx->small_fold = 0;
     if (ctx->inst.size() != 1 || ctx->sliced || n == 0) return RTBTE_OK;
     const InstHost &I = ctx->inst[0];
     const size_t R = ctx->real_size;
     const size_t pops = R * ((size_t)I.n_c_pad + (size_t)I.d.nmodes * I.N_q_pad + I.M_pad);
     const double slots = (double)(ctx->part_slots[0] + ctx->part_slots[1] + ctx->part_slots[2]);
     if (pops > 160 * 1024 || slots > (R == 8 ? kSmallSlots64 : kSmallSlots) || groups.size() > 64) return RTBTE_OK;
-    constexpr bool threads = false;  // (starting threads takes longer than these plans)
     std::unique_ptr<int[]> by_slot(new int[n]);
     std::unique_ptr<short[]> group_of(new short[n]);
-    parallel_for((int)groups.size(), threads, [&](int g) {
+    for (int g = 0; g < (int)groups.size(); ++g)
         for (int k = groups[g].item_begin; k < groups[g].item_end; ++k) {
             by_slot[items[k].slot] = k;
             group_of[k] = (short)g;
         }
-    });
-    // Rows dealt to the CTAs family by family (electrons, sub-lattice phonons, other phonons: so
-    // every parts mask is spread evenly), back and forth; dearest first where a CTA gets only a few
+    // Rows dealt to the shares family by family (electrons, sub-lattice phonons, other phonons: so
+    // every parts mask is spread evenly), back and forth; dearest first where a share gets only a few
     // (many rows average out, and sorting them would cost more than it evens).
     const int ny = (int)ctx->n_y, nc = I.d.n_c, Nq = (int)I.N_q, ng = (int)groups.size();
     const int G = (int)std::max(1.0, std::min((double)ctx->num_sms, std::ceil(slots / 64.0)));
@@ -519,22 +545,23 @@ int make_small_plan(rtbte_ctx *ctx, const ItemRec *items, int n, const std::vect
             }
         }
     }
-    // where each CTA's rows and items start; items [first[b], first[b + 1]) are CTA b's
+    // shares per CTA of the attempt loop (0: attempts take the launch sequence), and where each share's
+    // rows and slots start; the slots of its rows follow each other
+    ctx->small_fold = R == 8 && slots > kSmallAttempts64 ? 0 : slots <= kSmallQuarter ? 4 : 2;
+    const int F = std::max(ctx->small_fold, 1), nb = (G + F - 1) / F;
     std::vector<int> off(G + 1, 0), first(G + 1, 0);
-    int max_items = 0, max_rows = 0;
     for (int b = 0; b < G; ++b) {
         int m = 0;
         for (int c : own[b]) m += rowoff[c + 1] - rowoff[c];
         off[b + 1] = off[b] + (int)own[b].size();
         first[b + 1] = first[b] + m;
-        max_items = std::max(max_items, m);
-        max_rows = std::max(max_rows, (int)own[b].size());
     }
-    // one buffer, copied at once: items, runs, rows, row offsets, places of the items' entries
-    const size_t len[5] = {sizeof(ItemRec) * n, sizeof(SmallRun) * (size_t)G * ng, sizeof(SmallRow) * ny,
-                           sizeof(int) * (G + 1), sizeof(int) * n};
+    // one buffer, copied at once: items, runs of the RHS and of the attempt loop, rows, row offsets, places of
+    // the items' entries, slot offsets
+    const size_t len[6] = {sizeof(ItemRec) * n, sizeof(SmallRun) * (size_t)(G + nb) * ng, sizeof(SmallRow) * ny,
+                           sizeof(int) * (G + 1), sizeof(int) * n, sizeof(int) * (G + 1)};
     size_t bytes = 0;
-    for (int k = 0; k < 5; ++k) {
+    for (int k = 0; k < 6; ++k) {
         ctx->small_at[k] = bytes;
         bytes += (len[k] + 15) / 16 * 16;
     }
@@ -544,67 +571,79 @@ int make_small_plan(rtbte_ctx *ctx, const ItemRec *items, int n, const std::vect
     SmallRow *rows = reinterpret_cast<SmallRow *>(tab.get() + ctx->small_at[2]);
     int *item_at = reinterpret_cast<int *>(tab.get() + ctx->small_at[4]);
     std::memcpy(tab.get() + ctx->small_at[3], off.data(), len[3]);
+    std::memcpy(tab.get() + ctx->small_at[5], first.data(), len[5]);
     std::memset(runs, 0, len[1]);
-    // a CTA's items by group and, within it, alike ones together (the packets of order_packets in
-    // rhs.cu): counting sort over (group, process, vectors per lane)
-    std::unique_ptr<int[]> counts(new int[(size_t)G * (8 * ng + 1)]), keys(new int[n]);
-    std::vector<int> entries(G);
-    parallel_for(G, threads, [&](int b) {
-        int *count = counts.get() + (size_t)b * (8 * ng + 1), *key = keys.get() + first[b];
-        std::fill(count, count + 8 * ng + 1, 0);
-        int m = 0;
-        SmallRow *r = rows + off[b];
-        for (int c : own[b]) {
-            r->row = c;
-            r->p0 = m;
-            r->mid = m + rowmid[c] - rowoff[c];
-            for (int s = rowoff[c]; s < rowoff[c + 1]; ++s, ++m) {
-                const int k = by_slot[s];
-                key[m] = 8 * group_of[k] + 4 * (items[k].proc != 0) + 4 - cost[k].slots / (4 * cost[k].lanes);
-                ++count[key[m] + 1];
+    // Items of F shares by group, within a group by share and, within a share, alike ones together (the
+    // packets of order_packets in rhs.cu): counting sort over (group, share, process, vectors per lane)
+    std::unique_ptr<int[]> count(new int[(size_t)8 * F * ng + 1]), key(new int[n]);
+    for (int b0 = 0; b0 < G; b0 += F) {
+        const int b1 = std::min(b0 + F, G), i0 = first[b0];
+        std::fill(count.get(), count.get() + (size_t)8 * F * ng + 1, 0);
+        int m = i0;  // slot
+        for (int b = b0; b < b1; ++b) {
+            SmallRow *r = rows + off[b];
+            for (int c : own[b]) {
+                r->row = c;
+                r->p0 = m;
+                r->mid = m + rowmid[c] - rowoff[c];
+                for (int s = rowoff[c]; s < rowoff[c + 1]; ++s, ++m) {
+                    const int k = by_slot[s];
+                    key[m] = 8 * (F * group_of[k] + b - b0) + 4 * (items[k].proc != 0) + 4 -
+                             cost[k].slots / (4 * cost[k].lanes);
+                    ++count[key[m] + 1];
+                }
+                r->p1 = m;
+                const int p = c - nc;
+                r->f = c < nc ? c : -1;
+                r->N = c < nc ? -1 : p / Nq * I.N_q_pad + p % Nq;
+                r->P = c < nc || I.M == 0 ? -1 : I.compact[p];
+                r->pad = 0;
+                ++r;
             }
-            r->p1 = m;
-            const int p = c - nc;
-            r->f = c < nc ? c : -1;
-            r->N = c < nc ? -1 : p / Nq * I.N_q_pad + p % Nq;
-            r->P = c < nc || I.M == 0 ? -1 : I.compact[p];
-            r->pad = 0;
-            ++r;
         }
-        for (int k = 0; k < 8 * ng; ++k) count[k + 1] += count[k];
-        SmallRun *q = runs + (size_t)b * ng;
-        for (int g = 0; g < ng; ++g) {
-            if (count[8 * (g + 1)] == count[8 * g]) continue;
+        for (int k = 0; k < 8 * F * ng; ++k) count[k + 1] += count[k];
+        auto add_run = [&](SmallRun *&q, int g, int a, int b) {
+            if (a == b) return;
             const Group &Q = groups[g];
             q->idx = Q.idx;
             q->W = Q.W;
-            q->a = first[b] + count[8 * g];
-            q->b = first[b] + count[8 * (g + 1)];
+            q->a = i0 + a;
+            q->b = i0 + b;
             q->part = (short)Q.part;
             q->sb = (short)Q.s_bits;
             q->pb = (short)Q.pp_bits;
             q->lg = (short)Q.lanes_log2;
             q->N_at = Q.nu * Q.n_q_pad;
             ++q;
+        };
+        for (int b = b0; b < b1; ++b) {
+            SmallRun *q = runs + (size_t)b * ng;
+            for (int g = 0; g < ng; ++g) add_run(q, g, count[8 * (F * g + b - b0)], count[8 * (F * g + b - b0 + 1)]);
         }
-        m = 0;
-        for (int c : own[b])
-            for (int s = rowoff[c]; s < rowoff[c + 1]; ++s, ++m) {
-                ItemRec &it = out[first[b] + count[key[m]]++];
-                it = items[by_slot[s]];
-                it.slot = (unsigned)m;
-            }
-        int e = 0;
-        for (int k = first[b]; k < first[b + 1]; ++k) {
-            item_at[k] = e;
-            e += out[k].len;
+        SmallRun *q = runs + (size_t)(G + b0 / F) * ng;
+        for (int g = 0; g < ng; ++g) add_run(q, g, count[8 * F * g], count[8 * F * (g + 1)]);
+        m = i0;
+        for (int b = b0; b < b1; ++b)
+            for (int c : own[b])
+                for (int s = rowoff[c]; s < rowoff[c + 1]; ++s, ++m) {
+                    ItemRec &it = out[i0 + count[key[m]]++];
+                    it = items[by_slot[s]];
+                    it.slot = (unsigned)m;
+                }
+    }
+    for (int k = 0, e = 0; k < n; e += out[k++].len) item_at[k] = e;
+    auto largest = [&](int fold) {  // CTA of `fold` shares
+        SmallCtaMax Z;
+        for (int b0 = 0; b0 < G; b0 += fold) {
+            const int b1 = std::min(b0 + fold, G), i0 = first[b0], i1 = first[b1];
+            Z.items = std::max(Z.items, (int)round_up(i1 - i0, 4));
+            Z.rows = std::max(Z.rows, (int)round_up(off[b1] - off[b0], 2));
+            if (fold == F && i1 > i0) Z.entries = std::max(Z.entries, item_at[i1 - 1] + out[i1 - 1].len - item_at[i0]);
         }
-        entries[b] = e;
-    });
-    ctx->small_max_entries = *std::max_element(entries.begin(), entries.end());
-    ctx->small_max_items = (int)round_up(max_items, 4);
-    ctx->small_max_rows = (int)round_up(max_rows, 2);
-    ctx->small_max_runs = ng;
+        return Z;
+    };
+    ctx->small_max[0] = largest(1);
+    ctx->small_max[1] = largest(F);
     if (ctx->small_tab.bytes < bytes) {
         ctx->small_tab.release();
         RT_CUDA(ctx, cudaMalloc(&ctx->small_tab.p, bytes));
@@ -612,10 +651,15 @@ int make_small_plan(rtbte_ctx *ctx, const ItemRec *items, int n, const std::vect
     }
     RT_CUDA(ctx, cudaMemcpyAsync(ctx->small_tab.p, tab.get(), bytes, cudaMemcpyHostToDevice, ctx->stream));
     ctx->small_grid = G;
-    SmallPlan S = small_plan(ctx);
-    if (small_smem(R, S, true) + 2048 > ctx->smem_optin) S.max_entries = ctx->small_max_entries = 0;
-    if (small_smem(R, S, true) + 2048 > ctx->smem_optin) {
-        ctx->small_grid = 0;
+    const auto fits = [&](bool attempts) {
+        return small_smem(R, small_plan(ctx, attempts), attempts) + 2048 <= ctx->smem_optin;
+    };
+    if (ctx->small_fold > 0 && !fits(true)) {
+        ctx->small_max[1].entries = 0;
+        if (!fits(true)) ctx->small_fold = 0;
+    }
+    if (!fits(false)) {
+        ctx->small_grid = ctx->small_fold = 0;
         return RTBTE_OK;
     }
     for (const void *f : {rhs_fn(ctx), attempts_fn(ctx)}) RT_CUDA(ctx, allow_max_dynamic_smem(f));
@@ -626,7 +670,7 @@ int make_small_plan(rtbte_ctx *ctx, const ItemRec *items, int n, const std::vect
 
 int launch_small_rhs(rtbte_ctx *ctx, unsigned parts, const double *y, double *ydot, cudaStream_t s) {
     KParams P = small_params(ctx);
-    SmallPlan S = small_plan(ctx);
+    SmallPlan S = small_plan(ctx, false);
     const InstDev *inst = ctx->instdev.as<InstDev>();
     void *args[] = {&P, &S, &inst, &parts, &y, &ydot};
     std::pair<cudaEvent_t, cudaEvent_t> ev;
@@ -676,7 +720,7 @@ int launch_small_attempts(rtbte_ctx *ctx, const void *stage_args, int cap, cudaS
     int rc;
     if ((rc = ensure_attempts(ctx))) return rc;
     KParams P = small_params(ctx);
-    SmallPlan S = small_plan(ctx);
+    SmallPlan S = small_plan(ctx, true);
     StageArgs a = *reinterpret_cast<const StageArgs *>(stage_args);
     const size_t R = ctx->real_size, al = 256;
     SmallPops B;
@@ -697,7 +741,7 @@ int launch_small_attempts(rtbte_ctx *ctx, const void *stage_args, int cap, cudaS
     RT_CUDA(ctx, cudaMemsetAsync(sync, 0, sizeof(SmallSync), s));
     int polls = ctx->wait_polls;
     void *args[] = {&P, &S, &B, &a, &chunks, &cap, &polls, &sync};
-    RT_CUDA(ctx, cudaLaunchCooperativeKernel(attempts_fn(ctx), dim3(ctx->small_grid), dim3(kSmallThreads64), args,
+    RT_CUDA(ctx, cudaLaunchCooperativeKernel(attempts_fn(ctx), dim3((S.shares + S.fold - 1) / S.fold), dim3(kSmallThreads64), args,
                                              small_smem(R, S, true), s));
     ctx->launches++;
     return RTBTE_OK;

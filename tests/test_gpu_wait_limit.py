@@ -22,7 +22,7 @@ def _advance(ctx, y, t, **opts):
     return st.status, st
 
 
-@pytest.mark.parametrize("n", [12, 30])  # up to 8 rows to a chunk of the error norm, and more (one more barrier)
+@pytest.mark.parametrize("n", [12, 18])  # up to 8 rows to a chunk of the error norm, and more (one more barrier)
 @pytest.mark.parametrize("precision", ["fp32", "fp64"])
 def test_a_wait_that_gives_up_fails_with_the_state_before(n, precision):
     import paper_2412_13402_gb300 as rt
