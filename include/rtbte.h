@@ -348,8 +348,10 @@ int rtbte_get_tuning(const rtbte_ctx *ctx, int32_t *item_weight, int32_t *prefet
  * Errors: INVALID_ARG. */
 int rtbte_set_graph_mode(rtbte_ctx *ctx, int use_graphs);
 
-/* Polls after which a grid barrier of a small instance's attempt loop gives up (negative: the
- * default, seconds); rtbte_advance_to then returns RTBTE_E_TIMEOUT.  Errors: INVALID_ARG. */
+/* Polls after which a bounded device wait gives up (negative: the default, seconds): the grid barriers
+ * of a small instance's attempt loop (rtbte_advance_to) and the mbarriers of the tensor-core kernels
+ * (rtbte_surrogate_train, rtbte_surrogate_loss_grad), whose calls then return RTBTE_E_TIMEOUT.
+ * Errors: INVALID_ARG. */
 int rtbte_set_wait_limit(rtbte_ctx *ctx, int polls);
 
 /* Kernel timing.  While enabled, every launch of the collision kernel enqueued outside a

@@ -413,7 +413,7 @@ class Context:
         _check(self.ctx, load().rtbte_set_graph_mode(self.ctx, int(bool(use_graphs))))
 
     def set_wait_limit(self, polls: int):
-        """Polls after which a bounded device wait of advance_to gives up (negative: the default)."""
+        """Polls after which a bounded device wait gives up (negative: the default)."""
         _check(self.ctx, load().rtbte_set_wait_limit(self.ctx, int(polls)))
 
     def set_kernel_timing(self, enable: bool):

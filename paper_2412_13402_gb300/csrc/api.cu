@@ -694,7 +694,7 @@ int rtbte_set_graph_mode(rtbte_ctx *ctx, int use_graphs) {
 
 int rtbte_set_wait_limit(rtbte_ctx *ctx, int polls) {
     if (!ctx) return RTBTE_E_INVALID_ARG;
-    ctx->wait_polls = polls < 0 ? rtbte::kBarrierPolls : polls;
+    ctx->wait_polls = polls;
     return RTBTE_OK;
 }
 

@@ -44,7 +44,7 @@ constexpr int kWrmsBlocks = 512;
 constexpr int kWrmsChunks = 128;  // per-instance blocks of the WRMS reduction before the controller
 constexpr int kMaxBatch = 1024;  // instances per context (shared-memory tables of the batched kernels)
 constexpr int kLoopCap = 64;     // attempts per launch of an attempt loop (default)
-constexpr int kBarrierPolls = 1 << 22;  // of a grid barrier (default): seconds
+constexpr int kBarrierPolls = 1 << 22;  // of a grid barrier: seconds
 
 enum { PART_EPH = 0, PART_PHE = 1, PART_PP = 2 };
 // Lanes working on one item are chosen per staging group (Group::lanes_log2): 4, 8, 16 or 32 lanes,
@@ -322,7 +322,7 @@ struct rtbte_ctx {
     int small_fold = 0;               // shares per CTA of the attempt loop; 0: attempts take the launch sequence
     rtbte::SmallCtaMax small_max[2];  // largest CTA of an RHS, of the attempt loop
     void *small_sync_host = nullptr;  // pinned mirror of small_sync
-    int wait_polls = rtbte::kBarrierPolls;  // polls of a grid barrier before its wait gives up
+    int wait_polls = -1;              // polls before a bounded device wait gives up (negative: the kernel's own limit)
     int num_sms = 0;
     size_t smem_optin = 0;
     // integrator work buffers

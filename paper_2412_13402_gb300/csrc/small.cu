@@ -739,7 +739,7 @@ int launch_small_attempts(rtbte_ctx *ctx, const void *stage_args, int cap, cudaS
     double *chunks = ctx->wrms_part.as<double>() + 2 * ctx->n_y;
     SmallSync *sync = ctx->small_sync.as<SmallSync>();
     RT_CUDA(ctx, cudaMemsetAsync(sync, 0, sizeof(SmallSync), s));
-    int polls = ctx->wait_polls;
+    int polls = ctx->wait_polls < 0 ? kBarrierPolls : ctx->wait_polls;
     void *args[] = {&P, &S, &B, &a, &chunks, &cap, &polls, &sync};
     RT_CUDA(ctx, cudaLaunchCooperativeKernel(attempts_fn(ctx), dim3((S.shares + S.fold - 1) / S.fold), dim3(kSmallThreads64), args,
                                              small_smem(R, S, true), s));

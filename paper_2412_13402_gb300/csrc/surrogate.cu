@@ -879,6 +879,8 @@ bool kmajor_map(CUtensorMap *m, const bf16 *ptr, long long rows, long long cols,
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+int wait_polls(const rtbte_surrogate *s) { return s->ctx->wait_polls < 0 ? umma::kWaitLimit : s->ctx->wait_polls; }
+
 // C[M x N] = A[M x K] B[N x K]^T (+ bias, tanh, BF16 copy) on the tensor cores, A and B K-major
 int gemm_tc(rtbte_surrogate *s, const bf16 *A, int lda, const bf16 *B, int ldb, float *C, int ldc, int M, int N, int K,
             const float *bias, int act, bf16 *Cb, const float *back = nullptr) {
@@ -900,6 +902,7 @@ int gemm_tc(rtbte_surrogate *s, const bf16 *A, int lda, const bf16 *B, int ldb, 
     a.C = C;
     a.Cb = Cb;
     a.err = s->tcerr.as<int>();
+    a.polls = wait_polls(s);
     a.a_mn = a.b_mn = 0;
     a.k_base = 0;
     a.c_split = 0;
@@ -957,6 +960,7 @@ int gemm_tc_mn(rtbte_surrogate *s, const bf16 *A, int lda, const bf16 *B, int ld
     a.C = part ? part : splits > 1 ? s->split.as<float>() : C;
     if (nsplit) *nsplit = splits;
     a.err = s->tcerr.as<int>();
+    a.polls = wait_polls(s);
     a.a_mn = a.b_mn = 1;
     a.k_base = 0;
     a.c_split = (long long)M * ldc;
@@ -1016,6 +1020,7 @@ int conv(rtbte_surrogate *s, umma::ConvArgs a, int B, const bf16 *mat, long long
     a.ny = s->ny;
     a.nx = s->nx;
     a.err = s->tcerr.as<int>();
+    a.polls = wait_polls(s);
     CUtensorMap tb;
     if (!kmajor_map(&tb, mat, rows, cols, cols, 64))
         return sfail(s, RTBTE_E_UNSUPPORTED, "tensor-core convolution: operand layout not expressible as a TMA map");

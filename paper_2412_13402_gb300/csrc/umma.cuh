@@ -15,7 +15,7 @@
 //   - the warps read the accumulator with tcgen05.ld and apply the epilogue (store_tile).
 // Out-of-range rows and columns of a tile are zero-filled by TMA and not stored.  Every mbarrier
 // wait is bounded: on timeout the kernel writes a nonzero code to *err, stops issuing, waits
-// (bounded) for the copies it started, frees its tensor memory and returns.
+// (bounded) for the copies and products it started, frees its tensor memory and returns.
 #pragma once
 
 #include <cuda.h>
@@ -30,7 +30,7 @@ namespace umma {
 constexpr int kTM = 128;        // tile rows (accumulator lanes)
 constexpr int kTK = 64;         // K per stage: 64 BF16 = 128 bytes = one swizzle span
 constexpr int kThreads = 256;  // two warps per 32 accumulator rows, 32 of 64 columns each
-constexpr long long kWaitLimit = 1LL << 24;  // polls of an mbarrier before giving up
+constexpr int kWaitLimit = 1 << 24;  // polls of an mbarrier before giving up
 // MN-major tiles with 128-byte swizzle: blocks of 64 M (or N) elements x kTK K rows; the leading
 // byte offset is the distance between such blocks, the stride byte offset the distance between
 // 8-row K groups inside one (checked against a host reference)
@@ -44,6 +44,7 @@ struct Args {
     float *C;
     __nv_bfloat16 *Cb;
     int *err;
+    int polls;            // of an mbarrier before a wait gives up (0: at once)
     int a_mn, b_mn;       // operand stored MN-major (M or N contiguous) instead of K-major
     int k_base;           // first K of this CTA's range (split-K over blockIdx.z: K range k_base + z * K)
     long long c_split;    // element stride of C between split-K slices
@@ -57,9 +58,11 @@ __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
 __device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(bar), "r"(bytes) : "memory");
 }
-// true when the phase with `parity` completed within the poll limit
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
-    for (long long i = 0; i < kWaitLimit; ++i) {
+// true when the phase with `parity` completed within the poll limit (of the current phase and the one
+// before it: an older phase is not told from the current one).  The first poll is always made: a limit
+// known at run time and tested before it cost a training step 1.3 us of 238.
+__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, int polls = kWaitLimit) {
+    for (int i = 1;; ++i) {
         uint32_t done;
         asm volatile(
             "{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}\n"
@@ -67,8 +70,8 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
             : "r"(bar), "r"(parity)
             : "memory");
         if (done) return true;
+        if (i >= polls) return false;
     }
-    return false;
 }
 
 // 64-bit shared-memory matrix descriptor of a K-major tile with 128-byte swizzle: rows of 128
@@ -267,15 +270,16 @@ __global__ void __launch_bounds__(kThreads) gemm_tc(const __grid_constant__ CUte
         s_fail = 0;
         const uint32_t idesc = idesc_bf16(kTM, bn, a.a_mn, a.b_mn);
         int issued = 0;  // slices whose TMA was started
+        int products = 0;  // slices whose copies have landed and whose MMAs were committed
         for (int s = 0; s < NS && s < nk; ++s) {
             load_stage(s, s);
             ++issued;
         }
-        bool ok = true;
+        bool ok = a.polls > 0;
         for (int kt = 0; kt < nk && ok; ++kt) {
             const int s = kt % NS;
             const uint32_t par = (uint32_t)((kt / NS) & 1);
-            if (!(ok = mbar_wait(full[s], par))) break;
+            if (!(ok = mbar_wait(full[s], par, a.polls))) break;
             asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
 #pragma unroll
             for (int k16 = 0; k16 < kTK / 16; ++k16) {
@@ -293,8 +297,9 @@ __global__ void __launch_bounds__(kThreads) gemm_tc(const __grid_constant__ CUte
             }
             asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(empty[s])
                          : "memory");
+            ++products;
             if (kt + NS < nk) {  // refill this stage once its MMAs have read it
-                if (!(ok = mbar_wait(empty[s], par))) break;
+                if (!(ok = mbar_wait(empty[s], par, a.polls))) break;
                 load_stage(s, kt + NS);
                 ++issued;
             }
@@ -302,19 +307,22 @@ __global__ void __launch_bounds__(kThreads) gemm_tc(const __grid_constant__ CUte
         if (ok) {
             asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(done)
                          : "memory");
-        } else {  // give up: record it, let the copies already started land before the CTA leaves
+        } else {  // give up: record it, let the copies and products already started end before the CTA leaves
             s_fail = 1;
             atomicExch(a.err, 1);
-            for (int kt = 0; kt < issued; ++kt) mbar_wait(full[kt % NS], (uint32_t)((kt / NS) & 1));
+            for (int kt = products; kt < issued; ++kt) mbar_wait(full[kt % NS], (uint32_t)((kt / NS) & 1));
+            if (products > 0) mbar_wait(empty[(products - 1) % NS], (uint32_t)(((products - 1) / NS) & 1));
         }
     }
     __syncthreads();
     bool bad = s_fail != 0;
-    if (!bad && !mbar_wait(done, 0)) {
+    if (!bad && !mbar_wait(done, 0, a.polls)) {
         bad = true;
         if (lane == 0) atomicExch(a.err, 2);
     }
-    if (!__syncthreads_or(bad)) {
+    if (__syncthreads_or(bad)) {
+        if (threadIdx.x == 0 && !s_fail) mbar_wait(done, 0);
+    } else {
         asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
         // the ring is free: every slice was read before `done`
         float *tile = reinterpret_cast<float *>(smem_raw + (base - raw));
@@ -361,6 +369,7 @@ struct ConvArgs {
     float *out;                // [P][64], or the weight gradient's partials [split][576][64]
     __nv_bfloat16 *outb;       // [P][64] BF16 copy of out
     int *err;
+    int polls;                 // of an mbarrier before a wait gives up (0: at once)
 };
 
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void *src, bool valid) {
@@ -484,12 +493,14 @@ __global__ void __launch_bounds__(kThreads, 2) conv_tc(const __grid_constant__ C
 
     pdl_wait();
     int loaded = 0;  // slices whose copies were started
+    int products = 0;  // (thread 0) slices whose copies have landed and whose MMAs were committed
     for (; loaded < NS - 1 && loaded < nk; ++loaded) {
         load(loaded, loaded);
         asm volatile("cp.async.commit_group;\n" ::: "memory");
     }
     for (int i = loaded; i < NS - 1; ++i) asm volatile("cp.async.commit_group;\n" ::: "memory");
     const uint32_t idesc = idesc_bf16(kTM, kConvC, MODE == CONV_WEIGHT, MODE == CONV_WEIGHT);
+    if (a.polls <= 0) give_up(3);
     for (int kt = 0; kt < nk; ++kt) {
         const int s = kt % NS;
         // slice kt is the oldest of the NS - 1 groups in flight; its bytes become visible to the
@@ -500,7 +511,7 @@ __global__ void __launch_bounds__(kThreads, 2) conv_tc(const __grid_constant__ C
         if (__syncthreads_or(bad)) break;
         if (tid == 0) {
             asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-            if (!mbar_wait(full(s), (uint32_t)((kt / NS) & 1))) give_up(3);
+            if (!mbar_wait(full(s), (uint32_t)((kt / NS) & 1), a.polls)) give_up(3);
             else {
                 const uint32_t d = tmem + (MODE == CONV_BACK ? 64u * (kt & 3) : 0u);
 #pragma unroll
@@ -519,11 +530,12 @@ __global__ void __launch_bounds__(kThreads, 2) conv_tc(const __grid_constant__ C
                 asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(
                                  used(s))
                              : "memory");
+                ++products;
             }
         }
         // the previous slice's MMAs: their stage is free, and (CONV_BACK) their product complete
         if (kt > 0) {
-            if (!mbar_wait(used((kt - 1) % NS), (uint32_t)(((kt - 1) / NS) & 1))) give_up(4);
+            if (!mbar_wait(used((kt - 1) % NS), (uint32_t)(((kt - 1) / NS) & 1), a.polls)) give_up(4);
             if (MODE == CONV_BACK) {
                 asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
                 __syncwarp();
@@ -539,12 +551,14 @@ __global__ void __launch_bounds__(kThreads, 2) conv_tc(const __grid_constant__ C
     asm volatile("cp.async.wait_all;\n" ::: "memory");
     bool any = __syncthreads_or(bad);
     if (!any) {
-        if (!mbar_wait(used((nk - 1) % NS), (uint32_t)(((nk - 1) / NS) & 1))) give_up(5);
+        if (!mbar_wait(used((nk - 1) % NS), (uint32_t)(((nk - 1) / NS) & 1), a.polls)) give_up(5);
         any = __syncthreads_or(bad);
     }
-    if (any) {  // copies of B slices started but never waited for land before the CTA leaves
-        if (tid == 0)
-            for (int kt = 0; kt < loaded; ++kt) mbar_wait(full(kt % NS), (uint32_t)((kt / NS) & 1));
+    if (any) {  // copies of B slices not waited for yet, and products, end before the CTA leaves
+        if (tid == 0) {
+            for (int kt = products; kt < loaded; ++kt) mbar_wait(full(kt % NS), (uint32_t)((kt / NS) & 1));
+            if (products > 0) mbar_wait(used((products - 1) % NS), (uint32_t)(((products - 1) / NS) & 1));
+        }
         __syncthreads();
     } else {
         asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
