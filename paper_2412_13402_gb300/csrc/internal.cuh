@@ -316,8 +316,8 @@ struct rtbte_ctx {
     bool staged = false;
     bool wide = true;  // every group uses whole-warp items (the kernel variant without sub-warps)
     // one-launch kernels of a small single instance (small.cu); small_grid 0: not taken
-    rtbte::DevBuf small_tab, small_pops, small_sync;  // small_tab: items, runs, rows, row offsets, entry places,
-    size_t small_at[6] = {0, 0, 0, 0, 0, 0};          //   slot offsets at small_at[]
+    rtbte::DevBuf small_tab, small_pops, small_sync;  // small_tab: items, runs, rows, shares' offsets, entry places
+    size_t small_at[5] = {0, 0, 0, 0, 0};             //   at small_at[]
     int small_grid = 0;               // shares of the plan, one per CTA of an RHS
     int small_fold = 0;               // shares per CTA of the attempt loop; 0: attempts take the launch sequence
     rtbte::SmallCtaMax small_max[2];  // largest CTA of an RHS, of the attempt loop

@@ -55,18 +55,15 @@ struct __align__(16) SmallRow {
 struct SmallPlan {
     const SmallRun *runs;  // [CTA][max_runs] (empty runs fill up)
     const SmallRow *rows;
-    const int *row_off;    // [shares + 1]
-    const int *slot_off;   // [shares + 1] first partial slot, which for a CTA is its first item too
+    const int2 *off;       // [shares + 1] first row and first partial slot (for a CTA its first item too)
     int shares, fold;
     int max_runs, max_items, max_rows;  // largest CTA's
     int n_f, n_N, n_P;     // populations held: f, all modes' N (mode stride N_q_pad), sub-lattice N
     const int *pp_full;    // [M] phonon of each sub-lattice state
     const int *item_at;    // [items] entries of the items before this one
     int max_entries;       // largest CTA's entries; 0: the attempts' lists are not held
-    __device__ __forceinline__ int share0() const { return blockIdx.x * fold; }
-    __device__ __forceinline__ int row0() const { return __ldg(row_off + share0()); }
-    __device__ __forceinline__ int row1() const { return __ldg(row_off + min(share0() + fold, shares)); }
-    __device__ __forceinline__ int slot0() const { return __ldg(slot_off + share0()); }
+    __device__ __forceinline__ int2 begin() const { return __ldg(off + blockIdx.x * fold); }
+    __device__ __forceinline__ int2 end() const { return __ldg(off + min((int)(blockIdx.x + 1) * fold, shares)); }
 };
 
 template <class R> struct SmallMem {  // shared memory of a CTA
@@ -170,9 +167,10 @@ template <class R, int NT>
 __global__ void __launch_bounds__(NT) rhs_small(KParams P, SmallPlan S, const InstDev *inst, unsigned parts,
                                                 const double *y, double *ydot) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    const SmallMem<R> M(smem_raw, S, S.slot0());
+    const int2 from = S.begin();
+    const SmallMem<R> M(smem_raw, S, from.y);
     copy_in(M.runs, S.runs + (long long)blockIdx.x * S.max_runs, S.max_runs);
-    const int r0 = S.row0() + threadIdx.x, r1 = S.row1();
+    const int r0 = from.x + threadIdx.x, r1 = S.end().x;
     const InstDev I = *inst;
     pdl_begin();
     pdl_wait();
@@ -292,7 +290,8 @@ __global__ void __launch_bounds__(NT) attempts_small(KParams P, SmallPlan S, Sma
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ Ctl C;
     __shared__ int s_accept;
-    const int slot0 = S.slot0(), row0 = S.row0(), nrows = S.row1() - row0;
+    const int2 from = S.begin();
+    const int slot0 = from.y, row0 = from.x, nrows = S.end().x - row0;
     const SmallMem<R> M(smem_raw, S, slot0);
     if (threadIdx.x == 0) C = a.ctl[0];
     copy_in(M.runs, S.runs + (long long)blockIdx.x * S.max_runs, S.max_runs);
@@ -442,8 +441,7 @@ SmallPlan small_plan(rtbte_ctx *ctx, bool attempts) {
     S.runs = reinterpret_cast<const SmallRun *>(tab + ctx->small_at[1]) +
              (attempts ? (size_t)ctx->small_grid * ctx->n_groups : 0);
     S.rows = reinterpret_cast<const SmallRow *>(tab + ctx->small_at[2]);
-    S.row_off = reinterpret_cast<const int *>(tab + ctx->small_at[3]);
-    S.slot_off = reinterpret_cast<const int *>(tab + ctx->small_at[5]);
+    S.off = reinterpret_cast<const int2 *>(tab + ctx->small_at[3]);
     S.shares = ctx->small_grid;
     S.fold = attempts ? ctx->small_fold : 1;
     S.max_runs = ctx->n_groups;
@@ -549,19 +547,18 @@ int make_small_plan(rtbte_ctx *ctx, const ItemRec *items, int n, const std::vect
     // rows and slots start; the slots of its rows follow each other
     ctx->small_fold = R == 8 && slots > kSmallAttempts64 ? 0 : slots <= kSmallQuarter ? 4 : 2;
     const int F = std::max(ctx->small_fold, 1), nb = (G + F - 1) / F;
-    std::vector<int> off(G + 1, 0), first(G + 1, 0);
+    std::vector<int2> off(G + 1, make_int2(0, 0));
     for (int b = 0; b < G; ++b) {
         int m = 0;
         for (int c : own[b]) m += rowoff[c + 1] - rowoff[c];
-        off[b + 1] = off[b] + (int)own[b].size();
-        first[b + 1] = first[b] + m;
+        off[b + 1] = make_int2(off[b].x + (int)own[b].size(), off[b].y + m);
     }
-    // one buffer, copied at once: items, runs of the RHS and of the attempt loop, rows, row offsets, places of
-    // the items' entries, slot offsets
-    const size_t len[6] = {sizeof(ItemRec) * n, sizeof(SmallRun) * (size_t)(G + nb) * ng, sizeof(SmallRow) * ny,
-                           sizeof(int) * (G + 1), sizeof(int) * n, sizeof(int) * (G + 1)};
+    // one buffer, copied at once: items, runs of the RHS and of the attempt loop, rows, the shares' offsets, places
+    // of the items' entries
+    const size_t len[5] = {sizeof(ItemRec) * n, sizeof(SmallRun) * (size_t)(G + nb) * ng, sizeof(SmallRow) * ny,
+                           sizeof(int2) * (G + 1), sizeof(int) * n};
     size_t bytes = 0;
-    for (int k = 0; k < 6; ++k) {
+    for (int k = 0; k < 5; ++k) {
         ctx->small_at[k] = bytes;
         bytes += (len[k] + 15) / 16 * 16;
     }
@@ -571,17 +568,16 @@ int make_small_plan(rtbte_ctx *ctx, const ItemRec *items, int n, const std::vect
     SmallRow *rows = reinterpret_cast<SmallRow *>(tab.get() + ctx->small_at[2]);
     int *item_at = reinterpret_cast<int *>(tab.get() + ctx->small_at[4]);
     std::memcpy(tab.get() + ctx->small_at[3], off.data(), len[3]);
-    std::memcpy(tab.get() + ctx->small_at[5], first.data(), len[5]);
     std::memset(runs, 0, len[1]);
     // Items of F shares by group, within a group by share and, within a share, alike ones together (the
     // packets of order_packets in rhs.cu): counting sort over (group, share, process, vectors per lane)
     std::unique_ptr<int[]> count(new int[(size_t)8 * F * ng + 1]), key(new int[n]);
     for (int b0 = 0; b0 < G; b0 += F) {
-        const int b1 = std::min(b0 + F, G), i0 = first[b0];
+        const int b1 = std::min(b0 + F, G), i0 = off[b0].y;
         std::fill(count.get(), count.get() + (size_t)8 * F * ng + 1, 0);
         int m = i0;  // slot
         for (int b = b0; b < b1; ++b) {
-            SmallRow *r = rows + off[b];
+            SmallRow *r = rows + off[b].x;
             for (int c : own[b]) {
                 r->row = c;
                 r->p0 = m;
@@ -635,9 +631,9 @@ int make_small_plan(rtbte_ctx *ctx, const ItemRec *items, int n, const std::vect
     auto largest = [&](int fold) {  // CTA of `fold` shares
         SmallCtaMax Z;
         for (int b0 = 0; b0 < G; b0 += fold) {
-            const int b1 = std::min(b0 + fold, G), i0 = first[b0], i1 = first[b1];
+            const int b1 = std::min(b0 + fold, G), i0 = off[b0].y, i1 = off[b1].y;
             Z.items = std::max(Z.items, (int)round_up(i1 - i0, 4));
-            Z.rows = std::max(Z.rows, (int)round_up(off[b1] - off[b0], 2));
+            Z.rows = std::max(Z.rows, (int)round_up(off[b1].x - off[b0].x, 2));
             if (fold == F && i1 > i0) Z.entries = std::max(Z.entries, item_at[i1 - 1] + out[i1 - 1].len - item_at[i0]);
         }
         return Z;
