@@ -849,19 +849,16 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t
                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
 EncodeTiledFn encode_tiled() {
-    static EncodeTiledFn fn = nullptr;
-    static bool tried = false;
-    if (!tried) {
-        tried = true;
+    static const EncodeTiledFn fn = []() -> EncodeTiledFn {  // (initialised once, whatever threads ask)
         void *p = nullptr;
         cudaDriverEntryPointQueryResult q;
         if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) ==
                 cudaSuccess &&
             q == cudaDriverEntryPointSuccess)
-            fn = (EncodeTiledFn)p;
-        else
-            cudaGetLastError();
-    }
+            return (EncodeTiledFn)p;
+        cudaGetLastError();
+        return nullptr;
+    }();
     return fn;
 }
 
@@ -909,13 +906,6 @@ int gemm_tc(rtbte_surrogate *s, const bf16 *A, int lda, const bf16 *B, int ldb, 
     const dim3 grid((M + umma::kTM - 1) / umma::kTM, (N + bn - 1) / bn);
     const size_t sm = umma::smem_bytes(bn);
     cudaStream_t st = s->ctx->stream;
-    static bool attr_set = false;  // the shared-memory limit is a per-function attribute: set once
-    if (!attr_set) {
-        const void *fns[4] = {(const void *)umma::gemm_tc<32, 4>, (const void *)umma::gemm_tc<64, 4>,
-                              (const void *)umma::gemm_tc<128, 4>, (const void *)umma::gemm_tc<256, 2>};
-        for (const void *f : fns) S_CUDA(s, allow_max_dynamic_smem(f));
-        attr_set = true;
-    }
     static_assert(umma::kTM * umma::kTK * 2 + 128 * umma::kTK * 2 <= 32768, "four stages for bn <= 128");
     cudaError_t e;
     if (bn <= 32) e = launch_pdl(umma::gemm_tc<32, 4>, grid, dim3(umma::kThreads), sm, st, ta, tb, a);
@@ -1013,6 +1003,21 @@ int check_tc(rtbte_surrogate *s) {
 // slice of 64 lies within a tap: 64 channels on the tcgen05 engine.  Other widths take im2col.
 bool implicit_conv(const rtbte_surrogate *s) { return s->engine == 0 && s->width == umma::kConvC; }
 
+// Dynamic shared memory of the tensor-core training kernels: an attribute of a function on one device, so
+// every surrogate sets it on its own.
+int allow_training_smem(rtbte_surrogate *s) {
+    const void *fns[] = {(const void *)umma::gemm_tc<32, 4>,
+                         (const void *)umma::gemm_tc<64, 4>,
+                         (const void *)umma::gemm_tc<128, 4>,
+                         (const void *)umma::gemm_tc<256, 2>,
+                         (const void *)umma::conv_tc<umma::CONV_FORWARD>,
+                         (const void *)umma::conv_tc<umma::CONV_BACK>,
+                         (const void *)umma::conv_tc<umma::CONV_WEIGHT>,
+                         (const void *)head_grad};
+    for (const void *f : fns) S_CUDA(s, allow_max_dynamic_smem(f));
+    return RTBTE_OK;
+}
+
 // One implicit convolution over B samples; `mat` is the kernel's TMA operand [rows][cols].
 template <int MODE>
 int conv(rtbte_surrogate *s, umma::ConvArgs a, int B, const bf16 *mat, long long rows, long long cols, int splits = 1) {
@@ -1024,11 +1029,6 @@ int conv(rtbte_surrogate *s, umma::ConvArgs a, int B, const bf16 *mat, long long
     CUtensorMap tb;
     if (!kmajor_map(&tb, mat, rows, cols, cols, 64))
         return sfail(s, RTBTE_E_UNSUPPORTED, "tensor-core convolution: operand layout not expressible as a TMA map");
-    static bool attr_set = false;  // the shared-memory limit is a per-function attribute: set once
-    if (!attr_set) {
-        S_CUDA(s, allow_max_dynamic_smem((const void *)umma::conv_tc<MODE>));
-        attr_set = true;
-    }
     const int mrows = MODE == umma::CONV_WEIGHT ? 9 * umma::kConvC : a.P;
     const dim3 grid((mrows + umma::kTM - 1) / umma::kTM, splits);
     S_CUDA(s, launch_pdl(umma::conv_tc<MODE>, grid, dim3(umma::kThreads), umma::conv_smem_bytes(), s->ctx->stream, tb, a));
@@ -1122,11 +1122,6 @@ int backward_conv(rtbte_surrogate *s, int B) {
     int splits = (int)std::min<long long>(64, std::max<long long>(1, P / 1024));
     const int kchunk = (int)(((P + splits - 1) / splits + kBK - 1) / kBK * kBK);
     splits = (int)((P + kchunk - 1) / kchunk);
-    static bool attr_set = false;
-    if (!attr_set) {
-        S_CUDA(s, allow_max_dynamic_smem((const void *)head_grad));
-        attr_set = true;
-    }
     S_CUDA(s, launch_pdl(head_grad, dim3(splits), dim3(kHeadThreads), kHeadSmem, st, s->actb[0].as<bf16>(), s->goutb.as<bf16>(), C,
                          (int)P, kchunk, part));
     sums(part, splits, Wd * C, g + s->off_M2);
@@ -1587,6 +1582,7 @@ int rtbte_surrogate_create(rtbte_ctx *ctx, int inst, int width, int capacity, ui
         int cc = 0;
         cudaDeviceGetAttribute(&cc, cudaDevAttrComputeCapabilityMajor, ctx->device);
         s->engine = (cc >= 10 && encode_tiled()) ? 0 : 1;
+        if (s->engine == 0 && (rc = allow_training_smem(s))) return bail(rc);
         long long t = 0;
         for (int l = 0; l < kLayers; ++l) {
             s->off_tt[l] = t;
