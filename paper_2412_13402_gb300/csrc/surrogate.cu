@@ -1312,8 +1312,8 @@ int ensure_batch(rtbte_surrogate *s, int B) {
     int rc;
     if ((rc = salloc(s, s->xb, sizeof(bf16) * P * s->C)) || (rc = salloc(s, s->t, sizeof(float) * P * s->C)) ||
         (rc = salloc(s, s->out, sizeof(float) * P * s->C)) || (rc = salloc(s, s->gout, sizeof(float) * P * s->C)) ||
-        (rc = salloc(s, s->goutb, sizeof(bf16) * P * s->C)) || (rc = salloc(s, s->ga, sizeof(float) * P * Wd)) ||
-        (rc = salloc(s, s->gz, sizeof(float) * P * Wd)) || (rc = salloc(s, s->gzb, sizeof(bf16) * 2 * P * Wd)) ||
+        (rc = salloc(s, s->goutb, sizeof(bf16) * P * s->C)) || (rc = salloc(s, s->ga, conv ? 0 : sizeof(float) * P * Wd)) ||
+        (rc = salloc(s, s->gz, conv ? 0 : sizeof(float) * P * Wd)) || (rc = salloc(s, s->gzb, sizeof(bf16) * 2 * P * Wd)) ||
         (rc = salloc(s, s->gcol, conv ? 0 : sizeof(float) * P * s->kpad[1])) ||
         (rc = salloc(s, s->gzl, conv ? sizeof(float) * (kLayers + 1) * P * Wd : 0)) ||
         (rc = salloc(s, s->chains, conv ? sizeof(float) * 6 * 256 * 64 : 0)) ||
