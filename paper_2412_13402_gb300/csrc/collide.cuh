@@ -11,11 +11,6 @@ namespace {
 
 constexpr unsigned kFull = 0xffffffffu;
 
-template <class R> __device__ __forceinline__ R Fem(R f, R fp, R N) { return f * (R(1) - fp) + N * (f - fp); }
-template <class R> __device__ __forceinline__ R Fab(R f, R fp, R N) { return N * (f - fp) - fp * (R(1) - f); }
-template <class R> __device__ __forceinline__ R Gem(R Na, R Nb, R Nc) { return Na * (Nb + Nc + R(1)) - Nb * Nc; }
-template <class R> __device__ __forceinline__ R Gab(R Na, R Nb, R Nc) { return Na * (Nc - Nb) - Nb * (Nc + R(1)); }
-
 // s + c += x with the rounding error of the addition kept in c (Knuth two-sum).
 template <class R> __device__ __forceinline__ void two_sum(R &s, R &c, R x) {
     R t = s + x;
@@ -28,7 +23,6 @@ template <class R> __device__ __forceinline__ void two_sum(R &s, R &c, R x) {
 struct KParams {
     const ItemRec *items;
     const Group *groups;
-    int n_groups;
     // Work units: unit u is the items from bound[u] up to bound[u + 1] of the groups listed in act,
     // in order (parts not evaluated and finished instances are not in the list).  Units 0..grid-1
     // are the CTAs' static ranges, units grid.. are taken from a counter.

@@ -910,7 +910,6 @@ static int launch_core_t(rtbte_ctx *ctx, unsigned parts, const Ctl *ctl, cudaStr
     std::memset(&P, 0, sizeof(P));
     P.items = ctx->items.as<ItemRec>();
     P.groups = ctx->groups.as<Group>();
-    P.n_groups = ctx->n_groups;
     P.pf_dist = ctx->lt[parts].pf;
     P.tail_ctr = ctx->tail_ctr.as<int>();
     if (ctl && ctx->inst.size() > 1) {  // batched integration: units over the active instances (launch_resplit)

@@ -428,8 +428,6 @@ KParams small_params(rtbte_ctx *ctx) {
     KParams P;
     std::memset(&P, 0, sizeof(P));
     P.items = reinterpret_cast<const ItemRec *>(ctx->small_tab.as<char>() + ctx->small_at[0]);
-    P.groups = ctx->groups.as<Group>();
-    P.n_groups = ctx->n_groups;
     return P;
 }
 
