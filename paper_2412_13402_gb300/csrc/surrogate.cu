@@ -1306,6 +1306,7 @@ long long split_elems(const rtbte_surrogate *s, bool all) {
 
 int ensure_batch(rtbte_surrogate *s, int B) {
     if (B <= s->max_batch) return RTBTE_OK;
+    s->max_batch = 0;  // until every buffer is there: an allocation below may fail
     const long long P = (long long)B * s->Pq;
     const int Wd = s->width;
     const bool conv = implicit_conv(s);
