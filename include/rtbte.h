@@ -287,7 +287,7 @@ int rtbte_phph_rates(rtbte_ctx *ctx, const double *y, double *rates);
  * back before it returns.  All stepping, error norms and step-size control run on the device:
  * each integration span is one launch of a CUDA graph whose WHILE node repeats the attempt
  * kernels until every instance is done (at most opt->chunk attempts per launch), and the host
- * reads the status block once per launch; a small single instance (up to 2e6 entries, 2e5 in FP64)
+ * reads the status block once per launch; a small single instance (up to 2e6 entry slots, 2e5 in FP64)
  * runs up to opt->chunk attempts in one cooperative launch, which holds a quarter or half of the SMs
  * meanwhile and leaves the others to other streams (MRI_ADAPT: the host also reads the slow error
  * norms once per slow attempt and decides it).  On success y holds the

@@ -481,13 +481,16 @@ template <bool CACHED> const void *collision_kernel_of(const rtbte_ctx *ctx) {
                      : (const void *)rhs_kernel<float, true, false, CACHED, 1, kRhsThreads>;
 }
 // Ordinary or streaming loads of the lists.  Inside an integration the same lists are read again
-// at once: below kKeepBytes they stay in L2 (129 MB) with ordinary loads (57 MB: 22.4 -> 20.7 us a
-// launch, 79 MB: 27.0 -> 25.0), and several instances take ordinary loads whatever their size, since
+// at once: below kKeepBytes, two thirds of L2's 129 MB, they stay there with ordinary loads (57 MB: 156 ->
+// 138 us an attempt, 79 MB: 27.0 -> 25.0 us a launch; but 105 MB: 205 -> 226 us an attempt), and several
+// instances take ordinary loads whatever their size, since
 // what is read shrinks as they finish (16-instance window: 32.2 -> 31.1 ms of collision time).
 // Otherwise streaming loads, whose lines are evicted first, keep a part of the stream for the next
-// reading where ordinary ones would evict all of it (105 MB: 33.0 us, 37.1 with ordinary loads; three
-// contexts of 57 MB in turn: 31.1 / 32.2 us a call), up to sizes where no part matters and ordinary
-// loads are 1-2% faster again (2.27 GB: 348.6 -> 345.0 us, 2.78 GB: 413 -> 406).
+// reading where ordinary ones would evict all of it (streaming / ordinary loads, us an RHS: 105 MB
+// 34.6 / 36.5, 154 MB 41.9 / 44.7, 345 MB 73.7 / 74.3, 546 MB 108.8 / 110.6, 827 MB 146.9 / 148.8; three
+// contexts of 57 MB in turn 31.1 / 32.2), up to sizes where no part matters and ordinary loads are as
+// fast or 1-2% faster (1.20 GB 201.4 / 200.6, 1.68 GB 270.5 / 268.6, 2.27 GB 348.6 / 345.0, 2.78 GB 413 /
+// 406).
 constexpr double kKeepBytes = 85e6, kStreamBytes = 1e9;
 const void *collision_kernel(const rtbte_ctx *ctx, unsigned parts, bool integrating) {
     double bytes = 0;

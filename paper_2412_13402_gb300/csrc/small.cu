@@ -471,13 +471,16 @@ int small_threads(const rtbte_ctx *ctx) {
 
 }  // namespace
 
-// Entry slots up to which a single instance takes the one-launch kernels: about where what they
-// save over a few evaluations no longer covers building their plan (FP32 one-launch / launch
-// sequence, per RHS and per Zonneveld attempt: graphene 24, 0.23M entries, 10.3 / 16.5 and 59 / 80 us;
-// graphene 36, 0.96M, 12.4 / 19.5 and 65 / 89 us, plan 0.27 ms; graphene 48, 2.6M, 16.5 / 22.6 and
-// 88 / 111 us, plan 0.6 ms beside 0.6; graphene 63, 7.1M, 26.8 / 28.5 and 130 / 147 us; FP64, where the
-// arithmetic dominates sooner: graphene 36, 20.6 / 26.7 and 126 / 135 us; graphene 48, 41 / 45 and
-// 237 / 224 us).
+// Entry slots up to which a single instance takes the one-launch kernels.  In FP32 about where the 3 us
+// that they save an RHS take some hundred of them to cover building their plan; in FP64, where the
+// arithmetic dominates sooner, where they save nothing any more.  us per RHS, one launch / launch sequence:
+//   FP32  graphene 24, 0.23M entries  7.0 / 10.8    graphene 48, 2.65M  13.6 / 15.1 (plan 0.7 ms)
+//         graphene 36, 0.96M          9.5 / 11.2    graphene 54, 4.17M  17.2 / 17.2
+//         graphene 42, 1.71M         10.9 / 14.1    graphene 60, 6.00M  20.9 / 20.1
+//         (plan 0.5 ms beside 0.5)                  silicon 12, 4.70M   10.9 / 15.2
+//   FP64  graphene 24, 0.23M         12.5 / 15.0    graphene 42, 1.71M  29.5 / 28.3
+//         graphene 36, 0.96M         19.0 / 21.7    graphene 48, 2.65M  39.0 / 36.9
+//         graphene 39, 1.28M         23.3 / 25.9    silicon 10, 1.77M   22.1 / 26.4
 constexpr double kSmallSlots = 2e6, kSmallSlots64 = 1.5e6;
 
 // The attempt loop holds whole SMs (its registers fill one) for as many as 64 attempts, about 2 ms, so it

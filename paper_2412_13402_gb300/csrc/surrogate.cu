@@ -999,8 +999,9 @@ int check_tc(rtbte_surrogate *s) {
     return RTBTE_OK;
 }
 
-// Convolutions of layers 1..3 gather their operand slices themselves (umma::conv_tc) where a K
-// slice of 64 lies within a tap: 64 channels on the tcgen05 engine.  Other widths take im2col.
+// Convolutions of layers 1..3 gather their operand slices themselves (umma::conv_tc) on the tcgen05
+// engine at 64 channels, the default width: conv_tc has one K slice to a tap and one tile of output
+// channels.  Other widths take im2col.
 bool implicit_conv(const rtbte_surrogate *s) { return s->engine == 0 && s->width == umma::kConvC; }
 
 // Dynamic shared memory of the tensor-core training kernels: an attribute of a function on one device, so
