@@ -8,20 +8,21 @@
 // itself, so no partial leaves the SM and the only exchange between CTAs is the new populations.
 //   - rhs_small: one launch per RHS, populations straight from y, rows straight to ydot;
 //   - attempts_small: up to `cap` attempted steps per launch on a cooperative grid of at most half the
-//     SMs (see kSmallQuarter): S grid barriers an attempt to exchange populations (the last one the squared errors too, one more where the
-//     norm's chunks exceed 8 rows); every CTA runs the controller on its own copy, beside the first
-//     stage of the next attempt.  The state the launch started from is kept beside the one it writes,
-//     so that a barrier wait that gives up leaves a whole state to go back to.  Where they fit, the CTA's items and entries stay in shared memory
+//     SMs (see kSmallQuarter): S grid barriers an attempt to exchange populations (the last one the
+//     squared errors too, one more where the norm's chunks exceed 8 rows); every CTA runs the
+//     controller on its own copy, beside the first stage of the next attempt.  The state the launch
+//     started from is kept beside the one it writes, so that a barrier wait that gives up leaves a
+//     whole state to go back to.  Where they fit, the CTA's items and entries stay in shared memory
 //     for the launch: a barrier's acquire drops L1, so each stage would fetch them from L2 again
-//     (toy 12 x 12 FP64 31.1 -> 30.2 us an attempt, graphene 36 FP32 64 -> 62 us).
+//     (with a CTA on every SM, toy 12 x 12 FP64 31.1 -> 30.2 us an attempt, graphene 36 FP32 64 -> 62).
 // Items, their lanes and entry order, the order of a row's items, the norm's chunks and the
 // controller are those of the launch sequence (collide.cuh, rows.cuh, step.cuh), so both give the
 // same results bit for bit.  The 12 x 12 toy model in FP64 (15 174 entries), launch sequence and one
-// launch: RHS 18.9 and 4.9 us a call, Bogacki-Shampine attempts 62 and 30.2 us.  What is left of an
-// attempt is latency: about 2.4 us of each stage's 7.5 in the barrier, 2 in its items and 2 in its rows
-// (chains of FP64 operations), 0.6 in the populations' copy.  Messages in place of the barriers
-// (values with a sequence number beside them, polled by every CTA) took 38 us an attempt: the
-// polling of all CTAs on the same few lines costs more than the barrier saves.
+// launch: RHS 12.1 and 4.8 us a call, Bogacki-Shampine attempts 58.8 and 29.2 us.  What is left of an
+// attempt is latency (measured with a CTA on every SM: of a stage's 7.5 us 2.4 in the barrier, 2 in
+// the items, 2 in the rows' chains of FP64 operations, 0.6 in the populations' copy).  Messages in
+// place of the barriers (values with a sequence number beside them, polled by every CTA) took 38 us
+// an attempt: the polling of all CTAs on the same few lines costs more than the barrier saves.
 #include <algorithm>
 #include <cstring>
 #include <memory>
